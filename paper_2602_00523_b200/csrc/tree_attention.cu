@@ -165,6 +165,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, Shared
         }
     }
 }
+// The same for a whole converged warp: every lane polls, so that the warp never splits over the answer.
+template <bool kCluster = false>
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, Shared* sh, const AttnParams& p) {
+    if (__all_sync(0xffffffffu, mbar_try<kCluster>(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait<kCluster>(bar, parity, sh, p));
+}
 // Used on the abort path only: gives up silently after the budget.
 __device__ __forceinline__ void mbar_wait_quiet(uint64_t* bar, uint32_t parity, long long budget) {
     const long long t0 = clock64();
@@ -188,49 +194,63 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
 // ---- tcgen05 --------------------------------------------------------------------
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// Issued by the one thread that issues the MMAs.
+// One lane of a converged warp; the same lane every time for a full mask.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e != 0;
+}
+// The helpers below are called by a whole converged warp, so that their operands stay in uniform registers, and
+// carry the elected lane as a predicate of the instruction itself: a branch around it (`if (lane == 0)`) makes the
+// compiler move every operand back into uniform registers first, 73 to 84 clocks per 128 x 128 x 16 MMA instead of
+// the 64 that the tensor pipe needs (measured with eight P V and eight score MMAs per block).
 // Pair form: the arrival goes to the barrier at this offset in both CTAs, or (`both` false) in this one only.
 template <bool kPair>
-__device__ __forceinline__ void tc_commit_to(uint64_t* bar, bool both = true) {
+__device__ __forceinline__ void tc_commit_to(uint32_t leader, uint64_t* bar, bool both = true) {
     if (!kPair) {
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+                     "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                     ::"r"(smem_u32(bar)), "r"(leader) : "memory");
     } else if (both) {
         const uint16_t mask = 3;
-        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                     ::"r"(smem_u32(bar)), "h"(mask) : "memory");
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+                     "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
+                     ::"r"(smem_u32(bar)), "h"(mask), "r"(leader) : "memory");
     } else {
-        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+                     "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                     ::"r"(smem_u32(bar)), "r"(leader) : "memory");
     }
 }
-// Shared-memory matrix descriptors are passed as (low word, high word): only the low word (start
-// address and leading byte offset) varies between the MMAs of a kernel, so the issuing thread keeps
-// 32-bit values and the 64-bit operand is assembled next to the instruction.
+// Shared-memory matrix descriptors are passed as their low word: the high word (kDescHi) is the same everywhere.
+// Pair form: M = 256, each CTA supplies its 128 rows of A and its half of B's N extent.
 // D[tmem] (+)= A[smem desc] * B[smem desc]
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
-                 "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
-                 ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc) : "memory");
-}
-// The same two for a CTA pair: M = 256, each CTA supplies its 128 rows of A and its half of B's N extent.
-__device__ __forceinline__ void mma2_ss(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
-                 "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-                 "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}"
-                 ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void mma2_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
-                 "mov.b64 db, {%2, %3};\n\t"
-                 "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], db, %4, p;\n\t}"
-                 ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc) : "memory");
+template <bool kPair, uint32_t kHi, uint32_t kIdesc>
+__device__ __forceinline__ void mma_ss(uint32_t leader, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t acc) {
+    if (kPair)
+        asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+                     "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+                     "@q tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}"
+                     ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "n"(kHi), "n"(kIdesc), "r"(acc), "r"(leader) : "memory");
+    else
+        asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+                     "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+                     "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
+                     ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "n"(kHi), "n"(kIdesc), "r"(acc), "r"(leader) : "memory");
 }
 // D[tmem] (+)= A[tmem] * B[smem desc]
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
-                 "mov.b64 db, {%2, %3};\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}"
-                 ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc) : "memory");
+template <bool kPair, uint32_t kHi, uint32_t kIdesc>
+__device__ __forceinline__ void mma_ts(uint32_t leader, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t acc) {
+    if (kPair)
+        asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+                     "mov.b64 db, {%2, %3};\n\t"
+                     "@q tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], db, %4, p;\n\t}"
+                     ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "n"(kHi), "n"(kIdesc), "r"(acc), "r"(leader) : "memory");
+    else
+        asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+                     "mov.b64 db, {%2, %3};\n\t"
+                     "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}"
+                     ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "n"(kHi), "n"(kIdesc), "r"(acc), "r"(leader) : "memory");
 }
 // 32 lanes x 32 consecutive 32-bit columns: thread i of the warp gets lane (quadrant*32 + i)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
@@ -743,85 +763,82 @@ tree_attention_kernel(const AttnParams p, const __grid_constant__ CUtensorMap qm
         }
     } else if (warp == 9) {
         // =========================== MMA issuer ===========================
-        // One thread issues for both slots, in blocks [P V of step i-2, scores of step i]: step i belongs to
+        // One warp issues for both slots, in blocks [P V of step i-2, scores of step i]: step i belongs to
         // slot i & 1, so a slot's block runs on the tensor pipe while the other slot's warpgroup is in its
-        // softmax, and the blocks never interleave.  The whole instruction stream sits in one single-thread
-        // region: a predicated branch around every MMA costs more issue time than the MMA takes to execute.
-        if (lane == 0 && is_lead) {
+        // softmax, and the blocks never interleave.  The whole warp walks the loop and the elected lane is a
+        // predicate of each MMA (see mma_ss).
+        if (is_lead) {
+            const uint32_t leader = elect_one() ? 1u : 0u;
+            const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);      // (a broadcast: known to be the same in all lanes)
             // descriptors differ only in their 14-bit start-address field (bytes >> 4); shared memory ends below 256 KB
             // (pair form: the same offsets hold the partner's parts in its shared memory)
             const uint32_t dq = desc_lo(smem_u32(sQ), 16);
             const uint32_t dk = desc_lo(smem_u32(sK), 16);
             const uint32_t dv = desc_lo(smem_u32(sV), kTileHalfBytes);
+            constexpr uint32_t kQK = kPair ? kIdescQK2 : kIdescQK, kPV = kPair ? kIdescPV2 : kIdescPV;
             auto issue_qk = [&](int t, int slot) {
                 // S_t = Q K^T: 8 slices of K = 16 over d = 128 (4 per 64-wide half)
                 const uint32_t dks = dk + ((slot * kTile) >> 4);
-                const uint32_t s_tmem = tmem + t * 128;
+                const uint32_t s_tmem = tm + t * 128;
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint32_t a = dq + (((ks >> 2) * kQHalfBytes + (ks & 3) * 32) >> 4);
-                    const uint32_t b = dks + (((ks >> 2) * kKHalf + (ks & 3) * 32) >> 4);
-                    if (kPair) mma2_ss(s_tmem, a, b, kDescHi, kIdescQK2, ks > 0 ? 1u : 0u);
-                    else mma_ss(s_tmem, a, b, kDescHi, kIdescQK, ks > 0 ? 1u : 0u);
-                }
+                for (int ks = 0; ks < 8; ++ks)
+                    mma_ss<kPair, kDescHi, kQK>(leader, s_tmem, dq + (((ks >> 2) * kQHalfBytes + (ks & 3) * 32) >> 4),
+                                                dks + (((ks >> 2) * kKHalf + (ks & 3) * 32) >> 4), ks > 0 ? 1u : 0u);
             };
             auto issue_pv = [&](int t, int slot, bool first) {
                 // O_t += P_t V: 8 slices of K = 16 keys; P in TMEM (8 columns per slice), V MN-major
                 const uint32_t dvs = dv + ((slot * kTile) >> 4);
-                const uint32_t s_tmem = tmem + t * 128, o_tmem = tmem + 256 + t * 128;
+                const uint32_t s_tmem = tm + t * 128, o_tmem = tm + 256 + t * 128;
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    if (kPair) mma2_ts(o_tmem, s_tmem + ks * 8, dvs + ((ks * 2048) >> 4), kDescHi, kIdescPV2, (first && ks == 0) ? 0u : 1u);
-                    else mma_ts(o_tmem, s_tmem + ks * 8, dvs + ((ks * 2048) >> 4), kDescHi, kIdescPV, (first && ks == 0) ? 0u : 1u);
-                }
+                for (int ks = 0; ks < 8; ++ks)
+                    mma_ts<kPair, kDescHi, kPV>(leader, o_tmem, s_tmem + ks * 8, dvs + ((ks * 2048) >> 4), (first && ks == 0) ? 0u : 1u);
             };
             SegIter it;
             it.init(sh);
             Seg sg;
-            int rc = 0, kc = 0, vc = 0, nseg = 0;           // ring steps, K tiles, V tiles consumed; segments started
+            int rc = 0, kslot = 0, vslot = 0, nseg = 0;     // ring steps consumed, slots of the next K and V tile; segments started
             int np[2] = {0, 0};                             // steps of each slot whose probabilities were consumed
             bool ok = true;
-            // Every synchronisation instruction costs this thread a couple of hundred clocks, during which
-            // at most a few queued MMAs keep the pipe busy: the loop holds as few of them as the protocol
-            // allows (one wait and one commit per ring step for the tiles, one of each for the step's slot).
+            // The loop holds as few synchronisation instructions as the protocol allows: one wait and one commit
+            // per ring step for the tiles, one of each for the step's slot.
             while (ok && it.next(p, sg)) {
                 if (member0 >= sg.rp) continue;
-                const int n = sg.s1 - sg.s0;
-                ok = mbar_wait<kPair>(&sh->q_ready, nseg & 1, sh, p);
+                const int n = __shfl_sync(0xffffffffu, sg.s1 - sg.s0, 0);
+                ok = mbar_wait_warp<kPair>(&sh->q_ready, nseg & 1, sh, p);
                 for (int i = 0; ok && i < n + 2; ++i) {
-                    ok = mbar_wait<kPair>(&sh->kv_full[rc % kRing], (rc / kRing) & 1, sh, p);
+                    ok = mbar_wait_warp<kPair>(&sh->kv_full[rc % kRing], (rc / kRing) & 1, sh, p);
                     if (!ok) break;
                     const int t = i & 1;
                     if (i >= 2) {
                         // (the warpgroup zeroed the V rows past the end of the sequence before it arrived)
-                        ok = mbar_wait<kPair>(&sh->p_full[t], np[t] & 1, sh, p);
+                        ok = mbar_wait_warp<kPair>(&sh->p_full[t], np[t] & 1, sh, p);
                         if (!ok) break;
                         ++np[t];
                         // the segment's first P V products overwrite both accumulators, which the softmax warps
                         // read in the epilogue of the segment before
                         if (i == 2 && nseg > 0) {
-                            ok = mbar_wait<kPair>(&sh->epi_done, (nseg - 1) & 1, sh, p);
+                            ok = mbar_wait_warp<kPair>(&sh->epi_done, (nseg - 1) & 1, sh, p);
                             if (!ok) break;
                         }
                         tc_fence_after();
-                        issue_pv(t, vc % kStages, i < 4);
-                        ++vc;
-                        if (i >= n) tc_commit_to<kPair>(&sh->o_full[t]);    // the slot's last step of the segment
+                        issue_pv(t, vslot, i < 4);
+                        vslot = (vslot == kStages - 1) ? 0 : vslot + 1;
+                        if (i >= n) tc_commit_to<kPair>(leader, &sh->o_full[t]);    // the slot's last step of the segment
                     }
                     if (i < n) {
-                        issue_qk(t, kc % kStages);
-                        ++kc;
-                        tc_commit_to<kPair>(&sh->s_full[t]);
+                        issue_qk(t, kslot);
+                        kslot = (kslot == kStages - 1) ? 0 : kslot + 1;
+                        tc_commit_to<kPair>(leader, &sh->s_full[t]);
                     }
-                    tc_commit_to<kPair>(&sh->kv_done[rc % kRing]);
+                    tc_commit_to<kPair>(leader, &sh->kv_done[rc % kRing]);
                     ++rc;
-                    if (i == n - 1) tc_commit_to<kPair>(&sh->q_free);   // the segment's last score MMAs read the query tile
+                    if (i == n - 1) tc_commit_to<kPair>(leader, &sh->q_free);   // the segment's last score MMAs read the query tile
                 }
                 ++nseg;
             }
             if (!ok) {
-                // abort: everything this thread has issued must retire before the TMEM and the tiles go away
-                tc_commit_to<kPair>(&sh->drain, false);
+                // abort: everything this warp has issued must retire before the TMEM and the tiles go away
+                tc_commit_to<kPair>(leader, &sh->drain, false);
                 mbar_wait_quiet(&sh->drain, 0, p.wait_cycles);
             }
         }

@@ -117,6 +117,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, Shared
         }
     }
 }
+// The same for a whole converged warp: every lane polls, so that the warp never splits over the answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, Shared* sh, const AttnParams& p) {
+    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, sh, p));
+}
 // Used on the abort path only: gives up silently after the budget.
 __device__ __forceinline__ void mbar_wait_quiet(uint64_t* bar, uint32_t parity, long long budget) {
     const long long t0 = clock64();
@@ -146,28 +151,31 @@ __device__ __forceinline__ bool elect_one() {
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
     return e != 0;
 }
-// The helpers below are called by a whole converged warp so that their operands stay warp-uniform;
-// only the `leader` lane executes the instruction.
-__device__ __forceinline__ void tc_commit(bool leader, uint64_t* bar) {
-    if (leader)
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+// The helpers below are called by a whole converged warp, so that their operands stay in uniform registers, and
+// carry the elected lane as a predicate of the instruction itself: a branch around it (`if (lane == 0)`) makes the
+// compiler move every operand back into uniform registers first, 73 to 84 clocks per 128 x 128 x 16 MMA instead of
+// the 64 that the tensor pipe needs (measured with eight P V and eight score MMAs per block).
+__device__ __forceinline__ void tc_commit(uint32_t leader, uint64_t* bar) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+                 "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                 ::"r"(smem_u32(bar)), "r"(leader) : "memory");
 }
-// Shared-memory matrix descriptors are passed as (low word, high word): only the low word (start
-// address and leading byte offset) varies between the MMAs of a kernel, so the issuing thread keeps
-// 32-bit values and the 64-bit operand is assembled next to the instruction.
+// Shared-memory matrix descriptors are passed as their low word: the high word (kDescHi) is the same everywhere.
 // D[tmem] (+)= A[smem desc] * B[smem desc]
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+template <uint32_t kHi, uint32_t kIdesc>
+__device__ __forceinline__ void mma_ss(uint32_t leader, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t acc) {
+    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
                  "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
-                 ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc) : "memory");
+                 "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "n"(kHi), "n"(kIdesc), "r"(acc), "r"(leader) : "memory");
 }
 // D[tmem] (+)= A[tmem] * B[smem desc]
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+template <uint32_t kHi, uint32_t kIdesc>
+__device__ __forceinline__ void mma_ts(uint32_t leader, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t acc) {
+    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
                  "mov.b64 db, {%2, %3};\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}"
-                 ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc) : "memory");
+                 "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "n"(kHi), "n"(kIdesc), "r"(acc), "r"(leader) : "memory");
 }
 // 32 lanes x 32 consecutive 32-bit columns: thread i of the warp gets lane (quadrant*32 + i)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
@@ -625,86 +633,83 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
         }
     } else if (warp == 9) {
         // =========================== MMA issuer ===========================
-        // One thread issues for both row tiles, in blocks [P V of step j-1, scores of step j] per tile:
+        // One warp issues for both row tiles, in blocks [P V of step j-1, scores of step j] per tile:
         // a tile's block runs on the tensor pipe while the other tile's warpgroup is in its softmax, and
         // the blocks of the two tiles never interleave (two issuers would finish both tiles' scores at
-        // the same moment and leave the pipe idle during both softmaxes).  The whole instruction stream
-        // sits in one single-thread region: a predicated branch around every MMA costs more issue time
-        // than the MMA takes to execute.
-        if (lane == 0) {
-            // descriptors differ only in their 14-bit start-address field (bytes >> 4); shared memory ends below 256 KB
-            const uint32_t dq = desc_lo(smem_u32(sQ), 16);
-            const uint32_t dk = desc_lo(smem_u32(sK), 16);
-            const uint32_t dv = desc_lo(smem_u32(sV), kTileHalfBytes);
-            auto issue_qk = [&](int t, int slot) {
-                // S_t = Q_t K^T: 8 slices of K = 16 over d = 128 (4 per 64-wide half)
-                const uint32_t dqt = dq + ((t * kQTileBytes) >> 4);
-                const uint32_t dks = dk + ((slot * kTileBytes) >> 4);
-                const uint32_t s_tmem = tmem + t * 128;
+        // the same moment and leave the pipe idle during both softmaxes).  The whole warp walks the loop and
+        // the elected lane is a predicate of each MMA (see mma_ss): 80 layers x 16k keys, 24 nodes: 1349 -> 1257 us.
+        const uint32_t leader = elect_one() ? 1u : 0u;
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);      // (a broadcast: known to be the same in all lanes)
+        // descriptors differ only in their 14-bit start-address field (bytes >> 4); shared memory ends below 256 KB
+        const uint32_t dq = desc_lo(smem_u32(sQ), 16);
+        const uint32_t dk = desc_lo(smem_u32(sK), 16);
+        const uint32_t dv = desc_lo(smem_u32(sV), kTileHalfBytes);
+        auto issue_qk = [&](int t, int slot) {
+            // S_t = Q_t K^T: 8 slices of K = 16 over d = 128 (4 per 64-wide half)
+            const uint32_t dqt = dq + ((t * kQTileBytes) >> 4);
+            const uint32_t dks = dk + ((slot * kTileBytes) >> 4);
+            const uint32_t s_tmem = tm + t * 128;
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    mma_ss(s_tmem, dqt + (((ks >> 2) * kQHalfBytes + (ks & 3) * 32) >> 4),
-                           dks + (((ks >> 2) * kTileHalfBytes + (ks & 3) * 32) >> 4), kDescHi, kIdescQK, ks > 0 ? 1u : 0u);
-            };
-            auto issue_pv = [&](int t, int slot, bool first) {
-                // O_t += P_t V: 8 slices of K = 16 keys; P in TMEM (8 columns per slice), V MN-major
-                const uint32_t dvs = dv + ((slot * kTileBytes) >> 4);
-                const uint32_t s_tmem = tmem + t * 128, o_tmem = tmem + 256 + t * 128;
+            for (int ks = 0; ks < 8; ++ks)
+                mma_ss<kDescHi, kIdescQK>(leader, s_tmem, dqt + (((ks >> 2) * kQHalfBytes + (ks & 3) * 32) >> 4),
+                                          dks + (((ks >> 2) * kTileHalfBytes + (ks & 3) * 32) >> 4), ks > 0 ? 1u : 0u);
+        };
+        auto issue_pv = [&](int t, int slot, bool first) {
+            // O_t += P_t V: 8 slices of K = 16 keys; P in TMEM (8 columns per slice), V MN-major
+            const uint32_t dvs = dv + ((slot * kTileBytes) >> 4);
+            const uint32_t s_tmem = tm + t * 128, o_tmem = tm + 256 + t * 128;
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    mma_ts(o_tmem, s_tmem + ks * 8, dvs + ((ks * 2048) >> 4), kDescHi, kIdescPV, (first && ks == 0) ? 0u : 1u);
-            };
-            SegIter it;
-            it.init(sh);
-            Seg sg;
-            int rc = 0, kc = 0, vc = 0, nq = 0;             // ring steps, K tiles, V tiles consumed; segments started
-            int np[2] = {0, 0};                             // steps of each row tile whose probabilities were consumed
-            bool ok = true;
-            // Every synchronisation instruction costs this thread a couple of hundred clocks, during which
-            // at most a few queued MMAs keep the pipe busy: the loop holds as few of them as the protocol
-            // allows (one wait and one commit per ring step for the tiles, one of each per row tile).
-            while (ok && it.next(p, sg)) {
-                if (member >= sg.rp) continue;
-                const int n_rt = (sg.N * p.G - member * kRowsPerCta > kRowTile) ? 2 : 1;
-                const int s0 = sg.s0, s1 = sg.s1;
-                ok = mbar_wait(&sh->q_ready, nq & 1, sh, p);
-                ++nq;
-                // ring step: the P V products of step j - 1 (when j > s0) and the scores of step j (when j < s1)
-                for (int j = s0; ok && j <= s1; ++j) {
-                    ok = mbar_wait(&sh->kv_full[rc % kRing], (rc / kRing) & 1, sh, p);
-                    if (!ok) break;
-                    const int kslot = kc % kKStages, vslot = vc % kVStages;
-                    if (j < s1) ++kc;
-                    if (j > s0) ++vc;
+            for (int ks = 0; ks < 8; ++ks)
+                mma_ts<kDescHi, kIdescPV>(leader, o_tmem, s_tmem + ks * 8, dvs + ((ks * 2048) >> 4), (first && ks == 0) ? 0u : 1u);
+        };
+        SegIter it;
+        it.init(sh);
+        Seg sg;
+        int rc = 0, kslot = 0, vslot = 0, nq = 0;       // ring steps consumed, slots of the next K and V tile; segments started
+        int np[2] = {0, 0};                             // steps of each row tile whose probabilities were consumed
+        bool ok = true;
+        // The loop holds as few synchronisation instructions as the protocol allows: one wait and one commit
+        // per ring step for the tiles, one of each per row tile.
+        while (ok && it.next(p, sg)) {
+            if (member >= sg.rp) continue;
+            const int n_rt = __shfl_sync(0xffffffffu, (sg.N * p.G - member * kRowsPerCta > kRowTile) ? 2 : 1, 0);
+            const int n = __shfl_sync(0xffffffffu, sg.s1 - sg.s0, 0);
+            ok = mbar_wait_warp(&sh->q_ready, nq & 1, sh, p);
+            ++nq;
+            // ring step i: the P V products of step i - 1 (when i > 0) and the scores of step i (when i < n)
+            for (int i = 0; ok && i <= n; ++i) {
+                ok = mbar_wait_warp(&sh->kv_full[rc % kRing], (rc / kRing) & 1, sh, p);
+                if (!ok) break;
 #pragma unroll
-                    for (int t = 0; t < 2; ++t) {
-                        if (t < n_rt) {
-                            if (j > s0) {
-                                // (the warpgroup zeroed the V rows past the end of the sequence before it arrived)
-                                ok = mbar_wait(&sh->p_full[t], np[t] & 1, sh, p);
-                                if (!ok) break;
-                                ++np[t];
-                                tc_fence_after();
-                                issue_pv(t, vslot, j - 1 == s0);
-                                if (j == s1) tc_commit(true, &sh->o_full[t]);   // every MMA of this tile's segment has been issued
-                            }
-                            if (j < s1) {
-                                issue_qk(t, kslot);
-                                tc_commit(true, &sh->s_full[t]);
-                            }
+                for (int t = 0; t < 2; ++t) {
+                    if (t < n_rt) {
+                        if (i > 0) {
+                            // (the warpgroup zeroed the V rows past the end of the sequence before it arrived)
+                            ok = mbar_wait_warp(&sh->p_full[t], np[t] & 1, sh, p);
+                            if (!ok) break;
+                            ++np[t];
+                            tc_fence_after();
+                            issue_pv(t, vslot, i == 1);
+                            if (i == n) tc_commit(leader, &sh->o_full[t]);  // every MMA of this tile's segment has been issued
+                        }
+                        if (i < n) {
+                            issue_qk(t, kslot);
+                            tc_commit(leader, &sh->s_full[t]);
                         }
                     }
-                    if (!ok) break;
-                    tc_commit(true, &sh->kv_done[rc % kRing]);
-                    ++rc;
-                    if (j == s1 - 1) tc_commit(true, &sh->q_free);          // the segment's last score MMAs read the query tiles
                 }
+                if (!ok) break;
+                tc_commit(leader, &sh->kv_done[rc % kRing]);
+                ++rc;
+                if (i < n) kslot = (kslot == kKStages - 1) ? 0 : kslot + 1;
+                if (i > 0) vslot = (vslot == kVStages - 1) ? 0 : vslot + 1;
+                if (i == n - 1) tc_commit(leader, &sh->q_free);             // the segment's last score MMAs read the query tiles
             }
-            if (!ok) {
-                // abort: everything this thread has issued must retire before the TMEM and the tiles go away
-                tc_commit(true, &sh->drain);
-                mbar_wait_quiet(&sh->drain, 0, p.wait_cycles);
-            }
+        }
+        if (!ok) {
+            // abort: everything this warp has issued must retire before the TMEM and the tiles go away
+            tc_commit(leader, &sh->drain);
+            mbar_wait_quiet(&sh->drain, 0, p.wait_cycles);
         }
         __syncwarp();
     }

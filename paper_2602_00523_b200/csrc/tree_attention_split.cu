@@ -120,26 +120,30 @@ __device__ __forceinline__ bool elect_one() {
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
     return e != 0;
 }
-// The helpers below are called by a whole converged warp so that their operands stay warp-uniform;
-// only the `leader` lane executes the instruction.
-__device__ __forceinline__ void tc_commit(bool leader, uint64_t* bar) {
-    if (leader)
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+// The helpers below are called by a whole converged warp, so that their operands stay in uniform registers, and
+// carry the elected lane as a predicate of the instruction itself (a branch around it costs more issue time than
+// the MMA takes to execute).
+__device__ __forceinline__ void tc_commit(uint32_t leader, uint64_t* bar) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+                 "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                 ::"r"(smem_u32(bar)), "r"(leader) : "memory");
 }
+// Shared-memory matrix descriptors are passed as their low word: the high word (kDescHi) is the same everywhere.
 // D[tmem] (+)= A[smem desc] * B[smem desc]
-template <bool kAcc>
-__device__ __forceinline__ void mma_ss(bool leader, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc) {
-    if (leader)
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                     ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "n"(kAcc ? 1 : 0) : "memory");
+template <uint32_t kHi, uint32_t kIdesc>
+__device__ __forceinline__ void mma_ss(uint32_t leader, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t acc) {
+    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+                 "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+                 "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "n"(kHi), "n"(kIdesc), "r"(acc), "r"(leader) : "memory");
 }
 // D[tmem] (+)= A[tmem] * B[smem desc]
-__device__ __forceinline__ void mma_ts(bool leader, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t acc) {
-    if (leader)
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                     "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-                     ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
+template <uint32_t kHi, uint32_t kIdesc>
+__device__ __forceinline__ void mma_ts(uint32_t leader, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t acc) {
+    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 db;\n\tsetp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+                 "mov.b64 db, {%2, %3};\n\t"
+                 "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "n"(kHi), "n"(kIdesc), "r"(acc), "r"(leader) : "memory");
 }
 // 32 lanes x 32 consecutive 32-bit columns: thread i of the warp gets lane (quadrant*32 + i)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
@@ -181,11 +185,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 }
 
 // Shared-memory matrix descriptor (sm_100 format): start address, leading / stride byte
-// offsets in 16-byte units, version 1, 128-byte swizzle.
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) |
-           ((uint64_t)(sbo_bytes >> 4) << 32) | (1ull << 46) | (2ull << 61);
+// offsets in 16-byte units, version 1, 128-byte swizzle.  Low word: address and leading offset;
+// high word: stride offset (1024 bytes between 8-row groups everywhere here), version, swizzle.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes) {
+    return ((saddr & 0x3FFFFu) >> 4) | ((lbo_bytes >> 4) << 16);
 }
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 // Instruction descriptor, kind::f16: D fp32, A and B bf16, M = 128, N as given.
 constexpr uint32_t idesc_f16(uint32_t n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((128u >> 4) << 24);
@@ -468,35 +473,33 @@ tree_attention_split_kernel(const AttnParams p, const __grid_constant__ CUtensor
         const int n_rtiles = __shfl_sync(0xffffffffu, (M - rpair * kRowsPerCta > kRowTile) ? 2 : 1, 0);
         const int first_pos = __shfl_sync(0xffffffffu, pg_begin * kPageSize, 0);
         const int T = __shfl_sync(0xffffffffu, L + N, 0);
-        const bool leader = elect_one();
-        // lane 0 polls, the result is broadcast so that the warp never diverges on a wait
+        const uint32_t leader = elect_one() ? 1u : 0u;
+        // every lane polls, so that the warp never splits over the answer
         auto wait_all = [&](uint64_t* bar, uint32_t parity) {
-            int r = 1;
-            if (lane == 0) r = mbar_wait(bar, parity, bars, p.status, p.wait_cycles) ? 1 : 0;
-            return __shfl_sync(0xffffffffu, r, 0) != 0;
+            if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+            return __all_sync(0xffffffffu, mbar_wait(bar, parity, bars, p.status, p.wait_cycles)) != 0;
         };
         // descriptors differ only in their 14-bit start-address field (bytes >> 4); shared memory ends below 256 KB
-        const uint64_t dq = make_desc(smem_u32(sQ) + t * kQTileBytes, 16, 1024);
-        const uint64_t dk = make_desc(smem_u32(sK), 16, 1024);
-        const uint64_t dv = make_desc(smem_u32(sV), kPageHalfBytes, 1024);
+        const uint32_t dq = desc_lo(smem_u32(sQ) + t * kQTileBytes, 16);
+        const uint32_t dk = desc_lo(smem_u32(sK), 16);
+        const uint32_t dv = desc_lo(smem_u32(sV), kPageHalfBytes);
         const uint32_t s_tmem = tmem + t * 128, o_tmem = tmem + 256 + t * 128;
         auto issue_qk = [&](int x, int slot) {
             // S_t,x = Q_t K^T: 8 steps of K = 16 over d = 128 (4 per 64-wide half)
-            const uint64_t dks = dk + (uint64_t)((slot * kPageBytes) >> 4);
+            const uint32_t dks = dk + ((slot * kPageBytes) >> 4);
             const uint32_t d = s_tmem + x * 64;
-            mma_ss<false>(leader, d, dq, dks, kIdescQK);
 #pragma unroll
-            for (int ks = 1; ks < 8; ++ks)
-                mma_ss<true>(leader, d, dq + (uint64_t)(((ks >> 2) * kQHalfBytes + (ks & 3) * 32) >> 4),
-                             dks + (uint64_t)(((ks >> 2) * kPageHalfBytes + (ks & 3) * 32) >> 4), kIdescQK);
+            for (int ks = 0; ks < 8; ++ks)
+                mma_ss<kDescHi, kIdescQK>(leader, d, dq + (((ks >> 2) * kQHalfBytes + (ks & 3) * 32) >> 4),
+                                          dks + (((ks >> 2) * kPageHalfBytes + (ks & 3) * 32) >> 4), ks > 0 ? 1u : 0u);
         };
         auto issue_pv = [&](int x, int slot, bool first) {
             // O_t += P_t,x V: 4 steps of K = 16 keys; P in TMEM (8 columns per step), V MN-major
-            const uint64_t dvs = dv + (uint64_t)((slot * kPageBytes) >> 4);
+            const uint32_t dvs = dv + ((slot * kPageBytes) >> 4);
             const uint32_t a = s_tmem + x * 64;
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-                mma_ts(leader, o_tmem, a + ks * 8, dvs + (uint64_t)((ks * 2048) >> 4), kIdescPV, (!first || ks > 0) ? 1u : 0u);
+                mma_ts<kDescHi, kIdescPV>(leader, o_tmem, a + ks * 8, dvs + ((ks * 2048) >> 4), (!first || ks > 0) ? 1u : 0u);
         };
         bool ok = ns > 0 && t < n_rtiles;
         if (ok) ok = wait_all(&bars->q_ready, 0);
