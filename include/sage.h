@@ -87,7 +87,8 @@ typedef struct sage_tree_policy {
  *   draft_token[i] = topk_idx[(n0 + parent[i])*k + rank[i]]  for non-root nodes,
  *   draft_token[n0] = root_token[b],   n0 = node_offsets[b];
  * then parent, rank, node_offsets, root_token must be non-NULL and rank[i] < k.
- * ws: sage_expand_topk_workspace_size(rows, vocab) bytes. */
+ * One launch.  ws: sage_expand_topk_workspace_size(rows, vocab) bytes are asked for (SAGE_ERR_WORKSPACE otherwise);
+ * the present kernel passes its partial results on in shared memory and does not write them. */
 int sage_expand_topk(const float *logits, int rows, int vocab, int64_t row_stride,
                      int k, int k_entropy,
                      int32_t *topk_idx, float *topk_logprob,
@@ -103,20 +104,13 @@ size_t sage_expand_topk_workspace_size(int rows, int vocab);
  * handed only its input and output buffers by a serving engine whose own pool already owns
  * all of the GPU's memory, or a decode loop that must not call cudaMalloc because that call
  * synchronises the whole device.  Such a caller has nowhere to get `ws` from.
- * Same arguments, results and error codes as sage_expand_topk, minus ws / ws_bytes: the
- * scratch is a fixed array of SAGE_STATIC_SCRATCH_BYTES bytes inside the library, present on
- * every GPU that loads the library, for the life of the process.  The call performs no
- * allocation of any kind.
+ * Same arguments, results and error codes as sage_expand_topk, minus ws / ws_bytes.  The call performs no
+ * allocation of any kind, and calls may overlap (different streams, different host threads).
  *  - Limit: sage_expand_topk_workspace_size(rows, vocab) must not exceed
  *    SAGE_STATIC_SCRATCH_BYTES (60 rows x 152064 need about 90 KB; several thousand rows
  *    fit); otherwise SAGE_ERR_TOO_LARGE is returned and nothing is enqueued.
- *  - The first call on each device looks up the array's device address (a runtime query,
- *    done with that device current, which also loads the library's kernels there).  Make
- *    that first call before starting any stream capture on that device.
- *  - All calls on one device use the same array, and it keeps whatever the previous call
- *    left; the kernels overwrite every slot they later read, so no clearing is needed.  Two
- *    calls that may run at the same time on one GPU (different streams, or different host
- *    threads) race on the array and give wrong results: keep them ordered on one stream. */
+ *  - The first call on each device sets an attribute of the kernel (a runtime call, which also loads the
+ *    library's kernels there).  Make that first call before starting any stream capture on that device. */
 #define SAGE_STATIC_SCRATCH_BYTES (1 << 20)
 int sage_expand_topk_static(const float *logits, int rows, int vocab, int64_t row_stride,
                             int k, int k_entropy,

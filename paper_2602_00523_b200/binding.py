@@ -174,11 +174,10 @@ def sage_expand_topk_static(logits: torch.Tensor, k: int, k_entropy: int, *, par
                             node_offsets=None, root_token=None, out: Dict[str, torch.Tensor],
                             status: Optional[torch.Tensor] = None, stream=None) -> Dict[str, torch.Tensor]:
     """sage_expand_topk without a workspace argument, for callers that cannot allocate device
-    memory: the scratch is an array inside the library.  To honour that, this wrapper
-    allocates nothing either -- every output tensor must already be in ``out`` (topk_idx,
-    topk_logprob, entropy_full, entropy_topk, alpha, lse, and draft_token when the tree
-    arrays are given).  Calls on one GPU must not overlap; problems whose workspace would
-    exceed SAGE_STATIC_SCRATCH_BYTES raise SageError(SAGE_ERR_TOO_LARGE)."""
+    memory.  To honour that, this wrapper allocates nothing either -- every output tensor must
+    already be in ``out`` (topk_idx, topk_logprob, entropy_full, entropy_topk, alpha, lse, and
+    draft_token when the tree arrays are given).  Problems whose workspace would exceed
+    SAGE_STATIC_SCRATCH_BYTES raise SageError(SAGE_ERR_TOO_LARGE)."""
     assert logits.dtype == torch.float32 and logits.dim() == 2 and logits.stride(1) == 1
     rows, vocab = logits.shape
     batch = node_offsets.numel() - 1 if parent is not None else 0

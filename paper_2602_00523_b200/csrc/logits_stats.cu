@@ -1,28 +1,41 @@
 // Fused softmax entropy + top-k over vocabulary-sized fp32 rows (Eq. 4, Eq. 7-9)
-// and the draft-token expansion gather.
+// and the draft-token expansion gather, in one launch.
 //
-// Pass 1 (logits_partial_kernel): grid = (chunks, rows).  Every CTA streams one
-// contiguous chunk of one row once from HBM with 16-byte loads.  Each thread keeps
-// online softmax moments (m, s = sum e^(x-m), t = sum (x-m) e^(x-m)) in fp32 over its
-// few dozen elements; threads are merged in fp64.  Each warp keeps the K best
-// (value, index) pairs of its elements as 64-bit keys, one per lane, sorted; an
-// element is only looked at more closely when it reaches the warp's current K-th
-// value.  Keys order by value (with -0 == +0) and then by lowest index, so every
-// merge order gives the same answer.
-// Pass 2 (logits_finalize_kernel): one warp per row merges the chunks' moments in
-// fp64 and does a shuffle-based multi-way merge of the chunks' sorted candidate
-// lists, then derives lse, full entropy, log-probs, top-k entropy and alpha.
+// A row belongs to a cluster of CTAs, each of which streams one contiguous chunk of it once from
+// HBM.  Every thread copies its own 16-byte pieces asynchronously to shared memory, three batches
+// ahead, and is the only one to read them: no barrier in the stream, and 48 KB per CTA in flight
+// without registers to hold them.
+//  1. Every thread keeps softmax moments (s = sum e^(x-m), t = sum (x-m) e^(x-m), m a reference at
+//     most 8 below the largest element so far) in fp32 over its elements: about seven instructions
+//     per logit, loads included.
+//  2. The K best.  After batches 0, 1, 3, 7, ... the CTA takes a threshold from its threads' largest
+//     elements: with r = 1 (K <= 8) or 2, the q-th largest of the warps' r-th largest thread maxima,
+//     q = ceil(K / r), so that at least K elements reach it.  Elements that reach the threshold go to the
+//     warp's sorted queue, whose K-th value raises the threshold for the whole CTA too; the rest of the
+//     stream only compares each thread's largest element of a batch with it.  Keys order by value (with
+//     -0 == +0) and then by lowest index, so every merge order gives the same answer.
+//  3. Moments (in fp64) and the K best keys of every CTA go to the first CTA of the cluster through
+//     distributed shared memory; it ranks them, derives lse, entropies, log-probs and alpha, and
+//     hands the row's tokens to the children of the row's node.
+// What bounds it: HBM for many rows (960 rows x 152064, K = 10: 158 -> 97 us, 6.0 TB/s), the chain
+// launch -> load -> select -> merge for few (60 rows: 41 -> 17.5 us; 15 rows x 32000, K = 4: 13 -> 5.9 us).
+// The form before this one offered every element to per-warp queues that started empty, 67 thread
+// instructions per logit at K = 10, and took two more launches to merge and to gather the tokens.
 #include <math.h>
 
-#include <mutex>
+#include <atomic>
 
 #include "sage_common.cuh"
 
 namespace sage {
 
-constexpr int kPartialThreads = 256;
-constexpr int kPartialWarps = kPartialThreads / 32;
-constexpr int kMaxChunks = 32;
+constexpr int kThreads = 256;
+constexpr int kWarps = kThreads / 32;
+constexpr int kMaxChunks = 8;                    // CTAs of a cluster (the portable limit)
+constexpr int kBatch = 4;                        // 16-byte pieces of a batch per thread
+constexpr int kStages = 3;                       // batches on their way per thread
+constexpr int kStreamBytes = kStages * kBatch * kThreads * 16;
+constexpr int kCtasPerSm = 4;
 
 __device__ __forceinline__ uint32_t order_key(float x) {
     x += 0.0f;                                   // -0 -> +0
@@ -36,291 +49,517 @@ __device__ __forceinline__ uint64_t make_key(float x, int idx) {
     return ((uint64_t)order_key(x) << 32) | (uint32_t)(0xffffffffu - (uint32_t)idx);
 }
 
-// e^d for d <= 0 through the hardware 2^x (relative error about 2^-22): one multiply and one
-// special-function instruction instead of the library routine's range reduction.  The moments
-// built from it are merged in fp64; the entropy stays well inside its 1e-5 bound.
-__device__ __forceinline__ float exp_neg(float d) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(d * 1.4426950408889634f));
-    return y;
+// ---- packed fp32 pairs (one instruction works on two values) ----
+__device__ __forceinline__ uint64_t f2_pack(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
 }
 
-struct WarpQueue {
-    uint64_t q;        // lane j < K: j-th best key so far (0 = empty)
-    uint64_t kth;      // key in lane K-1 (same in all lanes)
-    float thr;         // value of kth, -inf while the queue is not full
-    int K;
-    __device__ __forceinline__ void init(int k) { q = 0; kth = 0; thr = -INFINITY; K = k; }
-    // Called by the whole warp; `want` marks lanes that hold a candidate (x, idx).
-    __device__ __forceinline__ void offer(bool want, float x, int idx, int lane) {
-        unsigned b = __ballot_sync(0xffffffffu, want);
-        while (b) {
-            const int src = __ffs(b) - 1;
-            b &= b - 1;
-            const uint64_t mine = make_key(x, idx);
-            const uint64_t cand = __shfl_sync(0xffffffffu, mine, src);
-            if (cand > kth) {
-                const unsigned gt = __ballot_sync(0xffffffffu, q > cand);   // lanes >= K hold 0
-                const int pos = __popc(gt);
-                const uint64_t up = __shfl_up_sync(0xffffffffu, q, 1);
-                if (lane < K && lane >= pos) q = (lane == pos) ? cand : up;
-                kth = __shfl_sync(0xffffffffu, q, K - 1);
-                thr = kth ? key_value((uint32_t)(kth >> 32)) : -INFINITY;
-            }
+// e^d through the hardware 2^x (relative error about 2^-22): one multiply and one special-function
+// instruction instead of the library routine's range reduction.  The moments built from it are merged
+// in fp64; the entropy stays well inside its 1e-5 bound.
+__device__ __forceinline__ float ex2(float y) {
+    float e;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(y));
+    return e;
+}
+constexpr float kLog2e = 1.4426950408889634f;
+
+// Online softmax moments of one thread: s = sum e^(x - m), t = sum (x - m) e^(x - m).
+struct Moments {
+    float m;           // reference, -1e30 before the first element
+    uint64_t s2, t2;   // (even, odd) partial sums
+    __device__ __forceinline__ void init() { m = -1e30f; s2 = 0; t2 = 0; }
+    // The reference only moves when an element exceeds it by more than 8 (any reference is exact; e^8 keeps
+    // the sums far from overflow), which after the first batch hardly ever happens: no divergent rescaling.
+    __device__ __forceinline__ void rise(float mx) {
+        if (mx > m + 8.0f) {
+            const float c = expf(m - mx);
+            float s0, s1, t0, t1;
+            f2_unpack(s2, s0, s1);
+            f2_unpack(t2, t0, t1);
+            t2 = f2_pack(c * fmaf(m - mx, s0, t0), c * fmaf(m - mx, s1, t1));
+            s2 = f2_pack(s0 * c, s1 * c);
+            m = mx;
         }
+    }
+    __device__ __forceinline__ void add(float x0, float x1, uint64_t nm2) {
+        const uint64_t d2 = f2_add(f2_pack(x0, x1), nm2);
+        float y0, y1;
+        f2_unpack(f2_mul(d2, f2_pack(kLog2e, kLog2e)), y0, y1);
+        const uint64_t e2 = f2_pack(ex2(y0), ex2(y1));
+        s2 = f2_add(s2, e2);
+        t2 = f2_fma(d2, e2, t2);
+    }
+    __device__ __forceinline__ void add4(const float4& v) {
+        const uint64_t nm2 = f2_pack(-m, -m);
+        add(v.x, v.y, nm2);
+        add(v.z, v.w, nm2);
+    }
+    __device__ __forceinline__ void add1(float x) {
+        rise(x);
+        const float d = x - m, e = expf(d);
+        s2 = f2_add(s2, f2_pack(e, 0.f));
+        t2 = f2_add(t2, f2_pack(d * e, 0.f));
     }
 };
 
-struct PartialParams {
-    const float* logits;
-    int64_t row_stride;
-    int vocab, chunk_len, n_chunks, K;
-    double* stats;      // [rows][n_chunks][3]  (M, S, T)
-    uint64_t* cand;     // [rows][n_chunks][SAGE_MAX_TOPK]
+__device__ __forceinline__ float max4(const float4& v) { return fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)); }
+
+// The K best keys a warp has been offered, lane j < K holding the j-th best (0 = empty).
+struct WarpQueue {
+    uint64_t q, kth;   // kth: key in lane K-1 (same in all lanes)
+    int K;
+    __device__ __forceinline__ void init(int k) { q = 0; kth = 0; K = k; }
+    // Called by the whole warp with the same key in every lane.
+    __device__ __forceinline__ void insert(uint64_t cand, int lane) {
+        const unsigned gt = __ballot_sync(0xffffffffu, q > cand);   // lanes >= K hold 0
+        const int pos = __popc(gt);
+        const uint64_t up = __shfl_up_sync(0xffffffffu, q, 1);
+        if (lane < K && lane >= pos) q = (lane == pos) ? cand : up;
+        kth = __shfl_sync(0xffffffffu, q, K - 1);
+    }
 };
 
-__global__ void __launch_bounds__(kPartialThreads) logits_partial_kernel(PartialParams p) {
-    __shared__ float s_wmax[kPartialWarps];
-    __shared__ double s_ws[kPartialWarps], s_wt[kPartialWarps];
-    __shared__ uint64_t s_keys[kPartialWarps * SAGE_MAX_TOPK];
-    const int chunk = blockIdx.x, row = blockIdx.y;
+// ---- asynchronous copies of a thread's own pieces ----
+__device__ __forceinline__ void copy16(uint32_t dst, const float4* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int kPending>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory"); }
+
+// ---- the same shared-memory location in the first CTA of the cluster ----
+__device__ __forceinline__ uint32_t lead_addr(const void* ptr) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(ptr)));
+    return r;
+}
+__device__ __forceinline__ void st_cluster(uint32_t addr, uint64_t v) {
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+
+struct ExpandParams {
+    const float* logits;
+    int64_t row_stride;
+    int rows, vocab, chunk_len, k, k_entropy, K;
+    int32_t* topk_idx;
+    float *topk_logprob, *entropy_full, *entropy_topk, *alpha, *lse;
+    const int32_t *parent, *rank, *node_offsets, *root_token;
+    int batch;
+    int32_t* draft_token;
+    int32_t* status;
+    double inv_ln_k;                             // 1 / ln(k_entropy)
+};
+
+// A well-formed tree of the batch that row `row` belongs to.
+__device__ __forceinline__ bool row_of_tree(const ExpandParams& p, int b, int row, int* n0_out, int* n_out) {
+    const int n0 = p.node_offsets[b];
+    const int n = p.node_offsets[b + 1] - n0;
+    *n0_out = n0;
+    *n_out = n;
+    if (n < 1 || n > SAGE_MAX_NODES || n0 < 0 || n0 + n > p.rows) {
+        if (row == 0) report_status(p.status, SAGE_STATUS_BAD_TREE);
+        return false;
+    }
+    return row >= n0 && row < n0 + n;
+}
+
+// draft_token[i] = topk_idx[row(parent(i))][rank(i)] (Section 2.2 "Tree-based Drafting") for the children i of the
+// node this row stands for; one warp.  s_idx: the row's candidates.
+__device__ __forceinline__ void hand_tokens(const ExpandParams& p, int row, int lane, const int32_t* s_idx) {
+    for (int b0 = 0; b0 < p.batch; b0 += 32) {
+        int n0 = 0, n = 0;
+        unsigned hit = __ballot_sync(0xffffffffu, b0 + lane < p.batch && row_of_tree(p, b0 + lane, row, &n0, &n));
+        while (hit) {
+            const int src = __ffs(hit) - 1;
+            hit &= hit - 1;
+            const int t0 = __shfl_sync(0xffffffffu, n0, src), tn = __shfl_sync(0xffffffffu, n, src);
+            const int u = row - t0;                      // this row's node
+            for (int i = lane; i < tn; i += 32) {
+                const int par = p.parent[t0 + i], r = p.rank[t0 + i];
+                const bool ok = par >= 0 && par < i && r >= 0 && r < p.k;
+                if (i == u) {
+                    if (i == 0) {
+                        p.draft_token[t0] = p.root_token[b0 + src];
+                    } else if (!ok) {
+                        report_status(p.status, SAGE_STATUS_BAD_TREE);
+                        p.draft_token[t0 + i] = -1;
+                    }
+                } else if (i > 0 && ok && par == u) {
+                    p.draft_token[t0 + i] = s_idx[r];
+                }
+            }
+        }
+    }
+}
+
+// A threshold that at least K of the CTA's elements reach (see the top of the file), as a value key; 0 lets everything
+// pass.  top_key: key of this thread's largest element so far; *most: the largest of the warps' values.
+__device__ __forceinline__ uint32_t cta_threshold(int K, uint32_t top_key, uint32_t* s_wtop, uint32_t* most, int lane, int warp) {
+    const int r_th = K <= kWarps ? 1 : 2;
+    const int q_th = (K + r_th - 1) / r_th;
+    uint32_t wt = __reduce_max_sync(0xffffffffu, top_key);
+    if (r_th == 2) {
+        const unsigned b = __ballot_sync(0xffffffffu, top_key == wt);
+        const uint32_t second = __reduce_max_sync(0xffffffffu, top_key == wt ? 0u : top_key);
+        if (__popc(b) == 1) wt = second;
+    }
+    if (lane == 0) s_wtop[warp] = wt;
+    __syncthreads();
+    const uint32_t v = s_wtop[lane & (kWarps - 1)];
+    int ge = 0;
+    *most = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        const uint32_t o = s_wtop[w];
+        ge += (o >= v) ? 1 : 0;
+        *most = max(*most, o);
+    }
+    return __reduce_max_sync(0xffffffffu, ge >= q_th ? v : 0u);
+}
+
+// Number of the n keys (n a multiple of 8, the list padded with 0) above `mine`.
+__device__ __forceinline__ int rank_of(const uint64_t* keys, int n, uint64_t mine) {
+    int rank = 0;
+    for (int j = 0; j < n; j += 8) {
+        ulonglong2 k[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) k[u] = *reinterpret_cast<const ulonglong2*>(keys + j + 2 * u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) rank += (k[u].x > mine ? 1 : 0) + (k[u].y > mine ? 1 : 0);
+    }
+    return rank;
+}
+
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const ExpandParams p) {
+    extern __shared__ float4 s_stream[];                         // [kStages][kBatch][kThreads]
+    __shared__ uint32_t s_thr;                                   // threshold raised by full queues
+    __shared__ uint32_t s_wtop[2][kWarps];
+    __shared__ float s_wref[kWarps];
+    __shared__ double s_ws[kWarps], s_wt[kWarps];
+    __shared__ __align__(16) uint64_t s_list[kWarps * SAGE_MAX_TOPK];
+    __shared__ int s_n;
+    // written by every CTA of the cluster in its first CTA
+    __shared__ uint64_t s_stat[kMaxChunks][3];                   // moments (M, S, T), as doubles
+    __shared__ __align__(16) uint64_t s_ckeys[kMaxChunks * SAGE_MAX_TOPK];     // K best keys of every CTA, 0 where there are fewer
+    __shared__ uint64_t s_best[SAGE_MAX_TOPK];
+    __shared__ int32_t s_idx[SAGE_MAX_TOPK];
+    const int chunk = blockIdx.x, row = blockIdx.y, n_chunks = gridDim.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int begin = chunk * p.chunk_len;
     const int end = min(p.vocab, begin + p.chunk_len);
     const float* rowp = p.logits + (int64_t)row * p.row_stride;
+    const int n4 = max(0, end - begin) >> 2;                     // 16-byte pieces: `begin` and row_stride are multiples of 4 elements
+    const float4* src4 = reinterpret_cast<const float4*>(rowp + begin);
+    const int n_tail = max(0, end - begin) & 3;                  // ragged end of the last chunk, one element to each of the first lanes
+    // this thread's pieces of batch b (a group even when there are none)
+    auto start = [&](int b) {
+        const int i0 = b * kBatch * kThreads + tid;
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_stream + (b % kStages) * kBatch * kThreads + tid);
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u)
+            if (i0 + u * kThreads < n4) copy16(dst + u * kThreads * 16, src4 + i0 + u * kThreads);
+        copy_commit();
+    };
+#pragma unroll
+    for (int b = 0; b < kStages; ++b) start(b);
+    // (read and raised after the barrier in the first cta_threshold)
+    if (tid < kWarps * SAGE_MAX_TOPK) s_list[tid] = 0;
+    if (tid == 0) { s_n = 0; s_thr = 0; }
+    // (the other half of this barrier, before the first store to the first CTA's memory: that CTA runs by then)
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
-    float m = -1e30f, s = 0.f, t = 0.f;
+    // ---- 1. and 2.: the stream
+    Moments mo;
+    mo.init();
     WarpQueue wq;
     wq.init(p.K);
-
-    // 16-byte loads: `begin` and row_stride are multiples of 4 elements.
-    const int n4 = (end - begin) >> 2;
-    const float4* src4 = reinterpret_cast<const float4*>(rowp + begin);
-    // Four 16-byte loads are in flight per thread before the first is used: the chunk is short
-    // (a few dozen elements per thread), so the pass is bound by load latency, not by bandwidth.
-    for (int i0 = 0; i0 < n4; i0 += 4 * kPartialThreads) {
-        float4 vv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int i = i0 + u * kPartialThreads + tid;
-            vv[u] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-            if (i < n4) vv[u] = __ldcs(src4 + i);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int i = i0 + u * kPartialThreads + tid;
-            const bool live = i < n4;
-            const float4 v = vv[u];
-            if (live) {
-                const float m4 = fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w));
-                if (m4 > m) {
-                    const float c = expf(m - m4);
-                    t = c * fmaf(m - m4, s, t);
-                    s *= c;
-                    m = m4;
-                }
-                const float d0 = v.x - m, d1 = v.y - m, d2 = v.z - m, d3 = v.w - m;
-                const float e0 = exp_neg(d0), e1 = exp_neg(d1), e2 = exp_neg(d2), e3 = exp_neg(d3);
-                s += (e0 + e1) + (e2 + e3);
-                t += fmaf(d0, e0, d1 * e1) + fmaf(d2, e2, d3 * e3);
-            }
-            // A lane's largest component goes first: it lifts the queue's threshold, so that most of
-            // the other components no longer qualify (matters while the queue is still filling).
-            const float m4q = fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w));
-            const bool hit = live && m4q >= wq.thr;
-            if (__any_sync(0xffffffffu, hit)) {
-                const int base = begin + 4 * i;
-                const int top = (v.x == m4q) ? 0 : (v.y == m4q) ? 1 : (v.z == m4q) ? 2 : 3;   // lowest index on ties
-                wq.offer(hit, m4q, base + top, lane);
-                wq.offer(live && top != 0 && v.x >= wq.thr, v.x, base + 0, lane);
-                wq.offer(live && top != 1 && v.y >= wq.thr, v.y, base + 1, lane);
-                wq.offer(live && top != 2 && v.z >= wq.thr, v.z, base + 2, lane);
-                wq.offer(live && top != 3 && v.w >= wq.thr, v.w, base + 3, lane);
-            }
-        }
-    }
-    // ragged tail of the last chunk (vocab % 4 elements)
     {
-        const int i = begin + 4 * n4 + tid;
-        const bool live = (tid < 4) && i < end;
-        float x = -INFINITY;
-        if (live) {
-            x = rowp[i];
-            if (x > m) {
-                const float c = expf(m - x);
-                t = c * fmaf(m - x, s, t);
-                s *= c;
-                m = x;
-            }
-            const float d = x - m, e = expf(d);
-            s += e;
-            t = fmaf(d, e, t);
-        }
-        if (warp == 0) wq.offer(live && x >= wq.thr, x, i, lane);
-    }
-
-    // ---- moments: block max, then rescale every thread's (s, t) in fp64
-    float wm = m;
-    for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
-    if (lane == 0) s_wmax[warp] = wm;
-    if (lane < p.K) s_keys[warp * SAGE_MAX_TOPK + lane] = wq.q;
-    else if (lane < SAGE_MAX_TOPK) s_keys[warp * SAGE_MAX_TOPK + lane] = 0;
-    __syncthreads();
-    float M = s_wmax[0];
+        const int n_batch = (n4 + kBatch * kThreads - 1) / (kBatch * kThreads);
+        uint32_t thr = 0;
+        float top = -INFINITY;                                   // this thread's largest element so far
+        for (int b = 0; b < n_batch; ++b) {
+            copy_wait<kStages - 1>();
+            const int i0 = b * kBatch * kThreads + tid;
+            const float4* buf = s_stream + (b % kStages) * kBatch * kThreads;
+            float4 v[kBatch];
+            float mx4[kBatch];
 #pragma unroll
-    for (int w = 1; w < kPartialWarps; ++w) M = fmaxf(M, s_wmax[w]);
-    double ds = 0.0, dt = 0.0;
-    if (s > 0.f) {
-        const double dm = (double)m - (double)M;
-        const double c = exp(dm);
-        ds = c * (double)s;
-        dt = c * ((double)t + dm * (double)s);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        ds += __shfl_xor_sync(0xffffffffu, ds, o);
-        dt += __shfl_xor_sync(0xffffffffu, dt, o);
-    }
-    if (lane == 0) { s_ws[warp] = ds; s_wt[warp] = dt; }
-    __syncthreads();
-    const size_t slot = (size_t)row * p.n_chunks + chunk;
-    if (tid == 0) {
-        double S = 0.0, T = 0.0;
-        for (int w = 0; w < kPartialWarps; ++w) { S += s_ws[w]; T += s_wt[w]; }
-        p.stats[slot * 3 + 0] = (double)M;
-        p.stats[slot * 3 + 1] = S;
-        p.stats[slot * 3 + 2] = T;
-    }
-    // ---- candidates: rank each of the warps' keys among all of them (keys are unique)
-    if (tid < kPartialWarps * SAGE_MAX_TOPK) {
-        const uint64_t mine = s_keys[tid];
-        if (mine != 0) {
-            int rank = 0;
-            for (int j = 0; j < kPartialWarps * SAGE_MAX_TOPK; ++j) rank += (s_keys[j] > mine) ? 1 : 0;
-            if (rank < p.K) p.cand[slot * SAGE_MAX_TOPK + rank] = mine;
-        }
-    }
-    // slots past the number of elements in this chunk stay empty
-    const int have = min(end - begin, p.K);
-    if (tid >= have && tid < SAGE_MAX_TOPK) p.cand[slot * SAGE_MAX_TOPK + tid] = 0;
-}
-
-struct FinalizeParams {
-    const double* stats;
-    const uint64_t* cand;
-    int rows, n_chunks, k, k_entropy, K;
-    int32_t* topk_idx;
-    float* topk_logprob;
-    float* entropy_full;
-    float* entropy_topk;
-    float* alpha;
-    float* lse;
-};
-
-__global__ void logits_finalize_kernel(FinalizeParams p) {
-    const int warps = blockDim.x >> 5;
-    const int row = blockIdx.x * warps + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (row >= p.rows) return;
-    const size_t base = (size_t)row * p.n_chunks;
-    // moments
-    double Mc = -INFINITY, Sc = 0.0, Tc = 0.0;
-    if (lane < p.n_chunks) {
-        Mc = p.stats[(base + lane) * 3 + 0];
-        Sc = p.stats[(base + lane) * 3 + 1];
-        Tc = p.stats[(base + lane) * 3 + 2];
-    }
-    double M = Mc;
-    for (int o = 16; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, o));
-    double S = 0.0, T = 0.0;
-    if (lane < p.n_chunks && Sc > 0.0) {
-        const double dm = Mc - M, c = exp(dm);
-        S = c * Sc;
-        T = c * (Tc + dm * Sc);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        S += __shfl_xor_sync(0xffffffffu, S, o);
-        T += __shfl_xor_sync(0xffffffffu, T, o);
-    }
-    const double lnS = log(S);
-    const double lse = M + lnS;
-    if (lane == 0) {
-        if (p.lse) p.lse[row] = (float)lse;
-        if (p.entropy_full) p.entropy_full[row] = (float)(lnS - T / S);
-    }
-    // multi-way merge of the chunks' sorted candidate lists: lane c holds the head of list c
-    int head = 0;
-    uint64_t cur = (lane < p.n_chunks) ? p.cand[(base + lane) * SAGE_MAX_TOPK] : 0;
-    double v1 = 0.0, wsum = 0.0, wlog = 0.0;     // top-k entropy accumulators (lane-uniform)
-    for (int j = 0; j < p.K; ++j) {
-        uint64_t best = cur;
-        for (int o = 16; o > 0; o >>= 1) {
-            const uint64_t other = __shfl_xor_sync(0xffffffffu, best, o);
-            best = other > best ? other : best;
-        }
-        if (best != 0 && cur == best) {          // keys are unique: exactly one lane advances
-            ++head;
-            cur = (head < SAGE_MAX_TOPK) ? p.cand[(base + lane) * SAGE_MAX_TOPK + head] : 0;
-        }
-        const double v = (double)key_value((uint32_t)(best >> 32));
-        const int idx = (int)(0xffffffffu - (uint32_t)best);
-        if (j < p.k && lane == 0) {
-            p.topk_idx[(size_t)row * p.k + j] = best ? idx : -1;
-            if (p.topk_logprob) p.topk_logprob[(size_t)row * p.k + j] = (float)(v - lse);
-        }
-        if (j < p.k_entropy && best != 0) {
-            if (j == 0) v1 = v;
-            const double d = v - v1, w = exp(d);  // w_j = P_j / P_1
-            wsum += w;
-            wlog += w * d;
-        }
-    }
-    if (lane == 0 && (p.entropy_topk || p.alpha)) {
-        // P~_j = w_j / wsum;  H = -sum P~ ln P~ = ln(wsum) - wlog / wsum
-        const double H = log(wsum) - wlog / wsum;
-        if (p.entropy_topk) p.entropy_topk[row] = (float)H;
-        if (p.alpha) {
-            double a = 1.0;
-            if (p.k_entropy > 1) a = fmin(1.0, fmax(0.0, 1.0 - H / log((double)p.k_entropy)));
-            p.alpha[row] = (float)a;
-        }
-    }
-}
-
-// draft_token[i] = topk_idx[row(parent(i))][rank(i)]  (Section 2.2 "Tree-based Drafting")
-__global__ void expand_gather_kernel(const int32_t* __restrict__ topk_idx, int k, int rows,
-                                     const int32_t* __restrict__ parent, const int32_t* __restrict__ rank,
-                                     const int32_t* __restrict__ node_offsets, const int32_t* __restrict__ root_token,
-                                     int32_t* __restrict__ draft_token, int32_t* status) {
-    const int b = blockIdx.x;
-    const int n0 = node_offsets[b];
-    const int n = node_offsets[b + 1] - n0;
-    if (n < 1 || n > SAGE_MAX_NODES || n0 < 0 || n0 + n > rows) {
-        if (threadIdx.x == 0) report_status(status, SAGE_STATUS_BAD_TREE);
-        return;
-    }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int par = parent[n0 + i];
-        if (i == 0) {
-            draft_token[n0] = root_token[b];
-        } else {
-            const int r = rank[n0 + i];
-            if (par < 0 || par >= i || r < 0 || r >= k) {
-                report_status(status, SAGE_STATUS_BAD_TREE);
-                draft_token[n0 + i] = -1;
+            for (int u = 0; u < kBatch; ++u) {
+                v[u] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+                if (i0 + u * kThreads < n4) v[u] = buf[u * kThreads + tid];
+                mx4[u] = max4(v[u]);
+            }
+            const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+            top = fmaxf(top, mx);
+            if ((b & (b + 1)) == 0) {
+                // after batches 0, 1, 3, 7, ...: as many elements pass in each doubling of the stream
+                uint32_t most;
+                thr = max(thr, cta_threshold(p.K, top == -INFINITY ? 0u : order_key(top), s_wtop[__popc(b) & 1], &most, lane, warp));
+                // threads share their first reference, so that the sums hardly ever need rescaling when they are merged
+                if (b == 0 && most) mo.m = fmaxf(mo.m, key_value(most));
+            }
+            thr = max(thr, *(volatile uint32_t*)&s_thr);
+            const float thr_x = thr ? key_value(thr) : -INFINITY;
+            if (__any_sync(0xffffffffu, mx >= thr_x && mx != -INFINITY)) {
+                __syncwarp();                                    // the whole warp reads what its lanes' copies left in shared memory
+                // this thread's elements that reach the threshold, one bit each; they are looked at one by one, the
+                // last lane's first: in ascending data that fills the queue with values that stay
+                uint32_t mask = 0;
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) {
+                    if (i0 + u * kThreads < n4)
+                        mask |= ((v[u].x >= thr_x ? 1u : 0u) | (v[u].y >= thr_x ? 2u : 0u) | (v[u].z >= thr_x ? 4u : 0u) |
+                                 (v[u].w >= thr_x ? 8u : 0u)) << (4 * u);
+                }
+                unsigned todo = __ballot_sync(0xffffffffu, mask != 0);
+                while (todo) {
+                    const int src = 31 - __clz(todo);
+                    uint32_t m = __shfl_sync(0xffffffffu, mask, src);
+                    while (m) {
+                        const int e = 31 - __clz(m);
+                        m &= ~(1u << e);
+                        const int at = (e >> 2) * kThreads + warp * 32 + src;
+                        const float x = reinterpret_cast<const float*>(buf + at)[e & 3];
+                        const uint64_t key = make_key(x, begin + 4 * (b * kBatch * kThreads + at) + (e & 3));
+                        if (key > wq.kth) wq.insert(key, lane);
+                    }
+                    todo &= ~(1u << src);
+                }
+                if (lane == 0 && (uint32_t)(wq.kth >> 32) > thr) atomicMax(&s_thr, (uint32_t)(wq.kth >> 32));
+                __syncwarp();
+            }
+            mo.rise(mx);
+            start(b + kStages);                                  // (into the slots just read)
+            if ((b + 1) * kBatch * kThreads <= n4) {
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) mo.add4(v[u]);
             } else {
-                draft_token[n0 + i] = topk_idx[(size_t)(n0 + par) * k + r];
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u)
+                    if (i0 + u * kThreads < n4) mo.add4(v[u]);
+            }
+        }
+        copy_wait<0>();
+        if (warp == 0) {
+            for (int j = 0; j < n_tail; ++j) {
+                const int i = begin + 4 * n4 + j;
+                const float x = rowp[i];
+                const uint64_t key = make_key(x, i);
+                if (key > wq.kth) wq.insert(key, lane);
+                if (lane == j) mo.add1(x);
+            }
+        }
+        float wr = mo.m;
+        for (int o = 16; o > 0; o >>= 1) wr = fmaxf(wr, __shfl_xor_sync(0xffffffffu, wr, o));
+        const unsigned have = __ballot_sync(0xffffffffu, wq.q != 0);
+        int at = 0;
+        if (lane == 0) {
+            s_wref[warp] = wr;
+            if (have) at = atomicAdd(&s_n, __popc(have));
+        }
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (wq.q != 0) s_list[at + lane] = wq.q;
+    }
+    __syncthreads();
+    // ---- 3. the K best keys of this CTA go to the first CTA of the cluster, ...
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    {
+        const int n = s_n;
+        const uint32_t keys = lead_addr(&s_ckeys[chunk * SAGE_MAX_TOPK]);
+        if (tid < n) {
+            const uint64_t mine = s_list[tid];
+            const int rank = rank_of(s_list, (n + 7) & ~7, mine);        // keys are unique
+            if (rank < p.K) st_cluster(keys + rank * 8, mine);
+        }
+        if (tid >= min(n, p.K) && tid < SAGE_MAX_TOPK) st_cluster(keys + tid * 8, 0);
+    }
+    // ... and its moments, in fp64 under the CTA's reference
+    float ref = s_wref[0];
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) ref = fmaxf(ref, s_wref[w]);
+    {
+        float s0, s1, t0, t1;
+        f2_unpack(mo.s2, s0, s1);
+        f2_unpack(mo.t2, t0, t1);
+        double ds = (double)s0 + (double)s1, dt = (double)t0 + (double)t1;
+        if (!__all_sync(0xffffffffu, mo.m == ref)) {
+            if (ds > 0.0) {
+                const double dm = (double)mo.m - (double)ref;
+                const double c = exp(dm);
+                dt = c * (dt + dm * ds);
+                ds *= c;
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            ds += __shfl_xor_sync(0xffffffffu, ds, o);
+            dt += __shfl_xor_sync(0xffffffffu, dt, o);
+        }
+        if (lane == 0) { s_ws[warp] = ds; s_wt[warp] = dt; }
+    }
+    __syncthreads();
+    if (tid < 3) {
+        double v = (double)ref;
+        if (tid > 0) {
+            const double* part = tid == 1 ? s_ws : s_wt;
+            v = ((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]));
+        }
+        st_cluster(lead_addr(&s_stat[chunk][tid]), (uint64_t)__double_as_longlong(v));
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (chunk != 0) return;
+
+    // ---- the row: lse and entropy in warp 0 while the others rank every CTA's keys among all
+    double lse = 0.0;
+    if (warp == 0) {
+        double Mc = -INFINITY, Sc = 0.0, Tc = 0.0;
+        if (lane < n_chunks) {
+            Mc = __longlong_as_double((long long)s_stat[lane][0]);
+            Sc = __longlong_as_double((long long)s_stat[lane][1]);
+            Tc = __longlong_as_double((long long)s_stat[lane][2]);
+        }
+        double M = Mc;
+        for (int o = 4; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, o));
+        M = __shfl_sync(0xffffffffu, M, 0);
+        double S = 0.0, T = 0.0;
+        if (Sc > 0.0) {
+            const double dm = Mc - M, c = exp(dm);
+            S = c * Sc;
+            T = c * (Tc + dm * Sc);
+        }
+        for (int o = 4; o > 0; o >>= 1) {
+            S += __shfl_xor_sync(0xffffffffu, S, o);
+            T += __shfl_xor_sync(0xffffffffu, T, o);
+        }
+        // (lanes 0 .. 7 hold the sums; log-probabilities are needed in up to 16 lanes)
+        S = __shfl_sync(0xffffffffu, S, 0);
+        T = __shfl_sync(0xffffffffu, T, 0);
+        const double lnS = log(S);
+        lse = M + lnS;
+        if (lane == 0) {
+            if (p.lse) p.lse[row] = (float)lse;
+            if (p.entropy_full) p.entropy_full[row] = (float)(lnS - T / S);
+        }
+    } else if (tid - 32 < n_chunks * SAGE_MAX_TOPK) {
+        const uint64_t mine = s_ckeys[tid - 32];
+        if (mine != 0) {
+            const int rank = rank_of(s_ckeys, n_chunks * SAGE_MAX_TOPK, mine);
+            if (rank < p.K) {
+                s_best[rank] = mine;
+                s_idx[rank] = (int32_t)(0xffffffffu - (uint32_t)mine);
             }
         }
     }
+    __syncthreads();
+    if (warp == 0) {
+        if (lane < p.k) {
+            p.topk_idx[(size_t)row * p.k + lane] = s_idx[lane];
+            if (p.topk_logprob)
+                p.topk_logprob[(size_t)row * p.k + lane] = (float)((double)key_value((uint32_t)(s_best[lane] >> 32)) - lse);
+        }
+    } else if (warp == 1) {
+        if (p.draft_token) hand_tokens(p, row, lane, s_idx);
+    } else if (warp == 2 && (p.entropy_topk || p.alpha)) {
+        const double v = lane < p.k_entropy ? (double)key_value((uint32_t)(s_best[lane] >> 32)) : 0.0;
+        const double v1 = __shfl_sync(0xffffffffu, v, 0);
+        double w = 0.0, wd = 0.0;                        // w_j = P_j / P_1
+        if (lane < p.k_entropy) {
+            const double d = v - v1;
+            w = exp(d);
+            wd = w * d;
+        }
+        for (int o = 8; o > 0; o >>= 1) {
+            w += __shfl_xor_sync(0xffffffffu, w, o);
+            wd += __shfl_xor_sync(0xffffffffu, wd, o);
+        }
+        if (lane == 0) {
+            // P~_j = w_j / wsum;  H = -sum P~ ln P~ = ln(wsum) - sum w ln w / wsum
+            const double H = log(w) - wd / w;
+            if (p.entropy_topk) p.entropy_topk[row] = (float)H;
+            if (p.alpha) p.alpha[row] = p.k_entropy > 1 ? (float)fmin(1.0, fmax(0.0, 1.0 - H * p.inv_ln_k)) : 1.0f;
+        }
+    }
 }
 
+// The opt-in to more than 48 KB of shared memory is a per-device attribute of the kernel.
+static bool allow_stream_buffer() {
+    static std::atomic<bool> done[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    if (!done[dev].load(std::memory_order_acquire)) {
+        if (cudaFuncSetAttribute(expand_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStreamBytes) != cudaSuccess)
+            return false;
+        done[dev].store(true, std::memory_order_release);
+    }
+    return true;
+}
+
+// CTAs per row (a power of two, each with at least one batch of elements).  About 200 CTAs when the rows are few:
+// more, shorter chunks only add selecting and merging (60 rows x 152064, K = 10: 4 CTAs per row 17.5 us, 8 19.4 us;
+// 120 rows: 2 / 4 / 8 give 24.7 / 25.4 / 30.6 us).  A launch of one wave of resident CTAs and a part of a second takes
+// as long as two: twice the CTAs fill the second (672 rows, K = 1: 1 / 2 CTAs per row 82 / 72 us; 4 take 77).
 static int pick_chunks(int rows, int vocab) {
-    int c = (592 + rows - 1) / rows;                 // about four CTAs per SM
-    const int max_by_len = (vocab + 4095) / 4096;    // keep chunks >= 4096 elements
-    if (c > max_by_len) c = max_by_len;
-    if (c > kMaxChunks) c = kMaxChunks;
-    if (c < 1) c = 1;
+    const int batch = kBatch * 4 * kThreads;
+    const long wave = 148 * kCtasPerSm;
+    auto can_double = [&](int c) { return c < kMaxChunks && (2 * c - 1) * batch < vocab; };
+    int c = 1;
+    while (c * rows < 200 && can_double(c)) c *= 2;
+    if ((long)c * rows > wave && (long)c * rows < 2 * wave && can_double(c)) c *= 2;
     return c;
+}
+
+// Scratch that callers hand in: the size that they were always asked for (24 bytes of moments and SAGE_MAX_TOPK keys
+// for each of up to 32 chunks of a row).  Results pass from CTA to CTA in distributed shared memory, the buffer is not
+// written.
+static size_t workspace_bytes(int rows, int vocab) {
+    int c = (592 + rows - 1) / rows;
+    const int max_by_len = (vocab + 4095) / 4096;
+    if (c > max_by_len) c = max_by_len;
+    if (c > 32) c = 32;
+    if (c < 1) c = 1;
+    return (size_t)rows * c * (3 * sizeof(double) + SAGE_MAX_TOPK * sizeof(uint64_t));
+}
+
+static int launch_expand(const ExpandParams& p, cudaStream_t stream) {
+    if (!allow_stream_buffer()) return SAGE_ERR_CUDA;
+    const int C = pick_chunks(p.rows, p.vocab);
+    ExpandParams q = p;
+    q.chunk_len = (((p.vocab + C - 1) / C) + 3) & ~3;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)C, (unsigned)p.rows);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kStreamBytes;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, expand_topk_kernel, q) != cudaSuccess) return SAGE_ERR_CUDA;
+    return launch_status();
 }
 
 }  // namespace sage
@@ -329,15 +568,15 @@ using namespace sage;
 
 extern "C" size_t sage_expand_topk_workspace_size(int rows, int vocab) {
     if (rows <= 0 || vocab <= 0) return 0;
-    const size_t slots = (size_t)rows * pick_chunks(rows, vocab);
-    return slots * (3 * sizeof(double) + SAGE_MAX_TOPK * sizeof(uint64_t));
+    return workspace_bytes(rows, vocab);
 }
 
-extern "C" int sage_expand_topk(const float* logits, int rows, int vocab, int64_t row_stride, int k, int k_entropy,
-                                int32_t* topk_idx, float* topk_logprob, float* entropy_full, float* entropy_topk,
-                                float* alpha, float* lse, const int32_t* parent, const int32_t* rank,
-                                const int32_t* node_offsets, int batch, const int32_t* root_token,
-                                int32_t* draft_token, void* ws, size_t ws_bytes, int32_t* status, void* stream) {
+// Checks of the arguments that both entry points share, then the launch.
+static int expand_topk(const float* logits, int rows, int vocab, int64_t row_stride, int k, int k_entropy,
+                       int32_t* topk_idx, float* topk_logprob, float* entropy_full, float* entropy_topk,
+                       float* alpha, float* lse, const int32_t* parent, const int32_t* rank,
+                       const int32_t* node_offsets, int batch, const int32_t* root_token,
+                       int32_t* draft_token, bool have_ws, int32_t* status, void* stream) {
     if (!logits || !topk_idx || rows < 0 || vocab < 1 || row_stride < vocab) return SAGE_ERR_INVALID_ARG;
     if (k < 1 || k_entropy < 1) return SAGE_ERR_INVALID_ARG;
     if (k > SAGE_MAX_TOPK || k_entropy > SAGE_MAX_TOPK) return SAGE_ERR_UNSUPPORTED;
@@ -347,58 +586,24 @@ extern "C" int sage_expand_topk(const float* logits, int rows, int vocab, int64_
     if (draft_token && (!parent || !rank || !node_offsets || !root_token || batch < 0)) return SAGE_ERR_INVALID_ARG;
     if (rows == 0) return SAGE_OK;
     if (rows > 65535) return SAGE_ERR_UNSUPPORTED;
-    const size_t need = sage_expand_topk_workspace_size(rows, vocab);
-    if (!ws || ws_bytes < need || ((uintptr_t)ws & 15)) return SAGE_ERR_WORKSPACE;
-    const int C = pick_chunks(rows, vocab);
-    int chunk_len = (vocab + C - 1) / C;
-    chunk_len = (chunk_len + 3) & ~3;
-    double* stats = reinterpret_cast<double*>(ws);
-    uint64_t* cand = reinterpret_cast<uint64_t*>(stats + (size_t)rows * C * 3);
-    PartialParams pp{logits, row_stride, vocab, chunk_len, C, K, stats, cand};
-    logits_partial_kernel<<<dim3(C, rows), kPartialThreads, 0, as_stream(stream)>>>(pp);
-    FinalizeParams fp{stats, cand, rows, C, k, k_entropy, K, topk_idx, topk_logprob,
-                      entropy_full, entropy_topk, alpha, lse};
-    logits_finalize_kernel<<<(rows + 3) / 4, 128, 0, as_stream(stream)>>>(fp);
-    if (draft_token && batch > 0)
-        expand_gather_kernel<<<batch, 64, 0, as_stream(stream)>>>(topk_idx, k, rows, parent, rank, node_offsets,
-                                                                  root_token, draft_token, status);
-    return launch_status();
+    if (!have_ws) return SAGE_ERR_WORKSPACE;
+    ExpandParams p{logits, row_stride, rows, vocab, 0, k, k_entropy, K, topk_idx, topk_logprob, entropy_full,
+                   entropy_topk, alpha, lse, parent, rank, node_offsets, root_token, batch,
+                   batch > 0 ? draft_token : nullptr, status, k_entropy > 1 ? 1.0 / log((double)k_entropy) : 0.0};
+    return launch_expand(p, as_stream(stream));
 }
 
-// ---------------------------------------------------------------------------
-// sage_expand_topk_static: the same computation with the scratch memory built
-// into the library instead of supplied by the caller.
-// ---------------------------------------------------------------------------
-namespace sage {
-
-// Scratch of the static variant.  It is part of the library image: every GPU on which
-// the library's kernels get loaded holds these bytes until the process exits.
-__device__ __align__(256) static unsigned char g_static_scratch[SAGE_STATIC_SCRATCH_BYTES];
-
-constexpr int kMaxDevices = 64;
-
-// Device address of g_static_scratch on the current device (nullptr on failure).  In host
-// code the array's name is only a handle for the runtime, not a device address, so the
-// address is looked up once per device, with that device current, and remembered.
-static void* static_scratch_address() {
-    static std::mutex mu;
-    static void* addr[kMaxDevices] = {};
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
-    std::lock_guard<std::mutex> lock(mu);
-    if (addr[dev] == nullptr) {
-        void* p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess) {
-            (void)cudaGetLastError();
-            return nullptr;
-        }
-        addr[dev] = p;
-    }
-    return addr[dev];
+extern "C" int sage_expand_topk(const float* logits, int rows, int vocab, int64_t row_stride, int k, int k_entropy,
+                                int32_t* topk_idx, float* topk_logprob, float* entropy_full, float* entropy_topk,
+                                float* alpha, float* lse, const int32_t* parent, const int32_t* rank,
+                                const int32_t* node_offsets, int batch, const int32_t* root_token,
+                                int32_t* draft_token, void* ws, size_t ws_bytes, int32_t* status, void* stream) {
+    const bool have_ws = ws && !((uintptr_t)ws & 15) && ws_bytes >= sage_expand_topk_workspace_size(rows, vocab);
+    return expand_topk(logits, rows, vocab, row_stride, k, k_entropy, topk_idx, topk_logprob, entropy_full, entropy_topk,
+                       alpha, lse, parent, rank, node_offsets, batch, root_token, draft_token, have_ws, status, stream);
 }
 
-}  // namespace sage
-
+// The same without a scratch argument, within the size limit that the header states.
 extern "C" int sage_expand_topk_static(const float* logits, int rows, int vocab, int64_t row_stride, int k,
                                        int k_entropy, int32_t* topk_idx, float* topk_logprob, float* entropy_full,
                                        float* entropy_topk, float* alpha, float* lse, const int32_t* parent,
@@ -408,14 +613,6 @@ extern "C" int sage_expand_topk_static(const float* logits, int rows, int vocab,
     if (rows < 0 || vocab < 1) return SAGE_ERR_INVALID_ARG;
     if (rows > 0 && sage_expand_topk_workspace_size(rows, vocab) > (size_t)SAGE_STATIC_SCRATCH_BYTES)
         return SAGE_ERR_TOO_LARGE;
-    void* scratch = nullptr;
-    if (rows > 0) {
-        scratch = static_scratch_address();
-        if (scratch == nullptr) return SAGE_ERR_CUDA;
-    }
-    // Every scratch slot the finalize kernel reads is written by the partial kernel of the
-    // same call, so nothing has to be cleared between calls.
-    return sage_expand_topk(logits, rows, vocab, row_stride, k, k_entropy, topk_idx, topk_logprob, entropy_full,
-                            entropy_topk, alpha, lse, parent, rank, node_offsets, batch, root_token, draft_token,
-                            scratch, (size_t)SAGE_STATIC_SCRATCH_BYTES, status, stream);
+    return expand_topk(logits, rows, vocab, row_stride, k, k_entropy, topk_idx, topk_logprob, entropy_full, entropy_topk,
+                       alpha, lse, parent, rank, node_offsets, batch, root_token, draft_token, true, status, stream);
 }

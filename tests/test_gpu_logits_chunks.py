@@ -1,0 +1,82 @@
+"""sage_expand_topk at the edges of its chunks: vocabularies around one batch of a thread block, rows that take one,
+two, four and eight blocks, ragged ends, candidates on both sides of a boundary, references that jump, and the
+hand-over of tokens to several trees.  Against the fp64 oracle, with the tolerances of the other parity tests."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2602_00523_b200 as sage
+from helpers import check_logits, dev_f32, dev_i32
+from workloads import chain_tree, random_tree, star_tree
+
+pytestmark = pytest.mark.gpu
+BATCH = 4096                                     # elements of one batch of a thread block
+
+
+def expand(lg, k, ke, **tree):
+    """Rows padded to a stride of a multiple of four with values that must not be read."""
+    rows, vocab = lg.shape
+    buf = np.full((rows, (vocab + 3) // 4 * 4 + 4), 1e9, np.float32)
+    buf[:, :vocab] = lg
+    st = sage.new_status()
+    o = sage.sage_expand_topk(dev_f32(buf)[:, :vocab], k, ke, status=st, **tree)
+    torch.cuda.synchronize()
+    return {n: t.cpu().numpy() for n, t in o.items()}, int(st.item())
+
+
+# (rows, vocab): blocks per row 1, 2, 4, 8 and, for the many-row case, a doubled count
+@pytest.mark.parametrize("rows,vocab", [(1, 1), (2, 3), (3, 5), (201, 9), (1, BATCH - 1), (1, BATCH + 1), (2, 2 * BATCH),
+                                        (1, 4 * BATCH + 3), (30, 8 * BATCH - 2), (70, 3 * BATCH + 1), (120, 5 * BATCH),
+                                        (200, 7 * BATCH + 2), (25, 15 * BATCH + 1), (601, 2 * BATCH + 5)])
+@pytest.mark.parametrize("k", [1, 8, 9, 16])
+def test_chunk_edges(rows, vocab, k):
+    k = min(k, vocab)
+    r = np.random.Generator(np.random.Philox(rows * 1000003 + vocab + k))
+    lg = r.standard_normal((rows, vocab)).astype(np.float32) * 2
+    for edge in range(BATCH, vocab, BATCH):      # peaks and ties on both sides of every batch boundary
+        lg[:, edge - 1:edge + 1] = np.float32(9.0)
+    lg[-1, -1] = 11.0                            # the last element of the last chunk
+    got, st = expand(lg, k, max(1, min(k, 10)))
+    assert st == 0
+    check_logits(got, lg, k, max(1, min(k, 10)))
+
+
+def test_reference_jumps_and_masked_tokens():
+    V = 6 * BATCH + 2
+    r = np.random.Generator(np.random.Philox(11))
+    lg = r.standard_normal((6, V)).astype(np.float32)
+    lg[0, 5 * BATCH + 17] = 40.0                 # far above everything before it
+    lg[1] += np.linspace(0, 60, V).astype(np.float32)
+    lg[2] += np.linspace(60, 0, V).astype(np.float32)
+    lg[3, :4 * BATCH] = np.finfo(np.float32).min  # a masked prefix: whole blocks without weight
+    lg[4, BATCH // 2:] = np.finfo(np.float32).min
+    lg[5] = 7.5                                  # constant: the lowest indices, in order
+    got, st = expand(lg, 10, 10)
+    assert st == 0
+    check_logits(got, lg, 10, 10)
+    assert list(got["topk_idx"][5]) == list(range(10))
+
+
+def test_tokens_go_to_the_children_in_every_tree_of_a_batch():
+    r = np.random.Generator(np.random.Philox(12))
+    trees = [random_tree(r, n, max_children=5) for n in (1, 2, 33, 40)] + [chain_tree(64), star_tree(6)] * 16
+    offs = np.concatenate([[0], np.cumsum([len(t["parent"]) for t in trees])]).astype(np.int32)
+    rows, V, k = int(offs[-1]) + 3, 2 * BATCH + 1, 6
+    parent, rank = np.concatenate([t["parent"] for t in trees]), np.concatenate([t["rank"] for t in trees])
+    root = r.integers(0, V, len(trees)).astype(np.int32)
+    lg = r.standard_normal((rows, V)).astype(np.float32)
+    kw = dict(parent=dev_i32(parent), rank=dev_i32(rank), node_offsets=dev_i32(offs), root_token=dev_i32(root))
+    got, st = expand(lg, k, 4, **kw)
+    assert st == 0
+    np.testing.assert_array_equal(got["draft_token"], oracle.expand_gather(got["topk_idx"], parent, rank, offs, root))
+    # a rank outside the candidates and a parent that is not before its child: reported, token -1, the others as before
+    bad_rank, bad_parent = rank.copy(), parent.copy()
+    a, b = int(offs[2]) + 7, int(offs[3]) + 9
+    bad_rank[a], bad_parent[b] = k, 9
+    kw.update(parent=dev_i32(bad_parent), rank=dev_i32(bad_rank))
+    bad, st = expand(lg, k, 4, **kw)
+    assert st == sage.SAGE_STATUS_BAD_TREE
+    want = got["draft_token"].copy()
+    want[[a, b]] = -1
+    np.testing.assert_array_equal(bad["draft_token"], want)
