@@ -2,7 +2,7 @@
 round: fused softmax-entropy + top-k, entropy -> tree template, tree-masked
 verification attention over a paged bf16 KV cache, greedy acceptance and KV
 compaction.  The product is the C-ABI library ``libsage.so`` (include/sage.h);
-this package is its thin ctypes binding.  Build it with
+this package is its thin Python binding.  Build it with
 ``python -m paper_2602_00523_b200.build``.
 
 The binding is loaded on first use of any of its names, so that the ``build``
