@@ -264,6 +264,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
     __shared__ __align__(16) uint64_t s_ckeys[kMaxChunks * SAGE_MAX_TOPK];     // K best keys of every CTA, 0 where there are fewer
     __shared__ uint64_t s_best[SAGE_MAX_TOPK];
     __shared__ int32_t s_idx[SAGE_MAX_TOPK];
+    after_previous_kernel();
     const int chunk = blockIdx.x, row = blockIdx.y, n_chunks = gridDim.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int begin = chunk * p.chunk_len;
@@ -546,19 +547,8 @@ static int launch_expand(const ExpandParams& p, cudaStream_t stream) {
     const int C = pick_chunks(p.rows, p.vocab);
     ExpandParams q = p;
     q.chunk_len = (((p.vocab + C - 1) / C) + 3) & ~3;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)C, (unsigned)p.rows);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kStreamBytes;
-    cfg.stream = stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)C;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, expand_topk_kernel, q) != cudaSuccess) return SAGE_ERR_CUDA;
+    if (launch(expand_topk_kernel, dim3((unsigned)C, (unsigned)p.rows), kThreads, kStreamBytes, stream, C, q) != cudaSuccess)
+        return SAGE_ERR_CUDA;
     return launch_status();
 }
 

@@ -553,6 +553,7 @@ template <bool kPair>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 tree_attention_kernel(const AttnParams p, const __grid_constant__ CUtensorMap qmap,
                       const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap) {
+    after_previous_kernel();
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte alignment: the 128B swizzle pattern repeats every 1024 bytes of address
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -1103,6 +1104,7 @@ tree_attention_kernel(const AttnParams p, const __grid_constant__ CUtensorMap qm
 // item's segments: which gangs hold them, and in which of their two partial slots, follows from
 // the positions alone.
 __global__ void __launch_bounds__(256) attention_merge_kernel(AttnParams p) {
+    after_previous_kernel();
     __shared__ int s_Wb, s_b, s_s0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k_cut = blockIdx.x + 1;                   // boundary between gang k_cut - 1 and gang k_cut
@@ -1434,26 +1436,13 @@ extern "C" int sage_tree_attention(const void* q, const void* k_pool, const void
             return SAGE_ERR_CUDA;
         attr_set[dev] = true;
     }
-    if (pair) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(p.n_gangs * p.n_rp));
-        cfg.blockDim = dim3(kAttnThreads);
-        cfg.dynamicSmemBytes = kSmemBytes;
-        cfg.stream = as_stream(stream);
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 2;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, tree_attention_kernel<true>, p, qmap, kmap, vmap) != cudaSuccess) return SAGE_ERR_CUDA;
-    } else {
-        tree_attention_kernel<false><<<p.n_gangs * p.n_rp, kAttnThreads, kSmemBytes, as_stream(stream)>>>(p, qmap, kmap, vmap);
-    }
+    const dim3 grid((unsigned)(p.n_gangs * p.n_rp));
+    if ((pair ? launch(tree_attention_kernel<true>, grid, kAttnThreads, kSmemBytes, as_stream(stream), 2, p, qmap, kmap, vmap)
+              : launch(tree_attention_kernel<false>, grid, kAttnThreads, kSmemBytes, as_stream(stream), 0, p, qmap, kmap, vmap)) != cudaSuccess)
+        return SAGE_ERR_CUDA;
     if (p.n_gangs > 1) {
         dim3 mg((unsigned)(p.n_gangs - 1), (unsigned)((p.n_rp * kRowsPerCta + 31) / 32));
-        attention_merge_kernel<<<mg, 256, 0, as_stream(stream)>>>(p);
+        if (launch(attention_merge_kernel, mg, 256, 0, as_stream(stream), 0, p) != cudaSuccess) return SAGE_ERR_CUDA;
     }
     return launch_status();
 }

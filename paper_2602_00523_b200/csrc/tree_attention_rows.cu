@@ -482,6 +482,7 @@ struct SegIter {
 __global__ void __launch_bounds__(kAttnThreads, 1)
 tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorMap qmap,
                       const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap) {
+    after_previous_kernel();
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte alignment: the 128B swizzle pattern repeats every 1024 bytes of address
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -884,6 +885,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
 // item's segments: which gangs hold them, and in which of their two partial slots, follows from
 // the positions alone.
 __global__ void __launch_bounds__(256) attention_rows_merge_kernel(AttnParams p) {
+    after_previous_kernel();
     __shared__ int s_Wb, s_b, s_s0, s_n_rp;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int k_cut = blockIdx.x + 1;                   // boundary between gang k_cut - 1 and gang k_cut
@@ -992,11 +994,12 @@ int launch(int n_ctas, int select, int n_layers, int n_pages, const int32_t* pag
             return SAGE_ERR_CUDA;
         attr_set[dev] = true;
     }
-    tree_attention_rows_kernel<<<p.n_ctas, kAttnThreads, kSmemBytes, stream>>>(p, qmap, kmap, vmap);
+    if (sage::launch(tree_attention_rows_kernel, dim3(p.n_ctas), kAttnThreads, kSmemBytes, stream, 0, p, qmap, kmap, vmap) != cudaSuccess)
+        return SAGE_ERR_CUDA;
     if (p.n_ctas > 1) {
         // one block per possible boundary between two gangs' ranges and 32-row chunk; those that find no cut item leave
         dim3 mg((unsigned)(p.n_ctas - 1), (unsigned)((p.n_rp * kRowsPerCta + 31) / 32));
-        attention_rows_merge_kernel<<<mg, 256, 0, stream>>>(p);
+        if (sage::launch(attention_rows_merge_kernel, mg, 256, 0, stream, 0, p) != cudaSuccess) return SAGE_ERR_CUDA;
     }
     return launch_status();
 }

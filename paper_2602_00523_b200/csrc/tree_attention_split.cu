@@ -307,6 +307,7 @@ __device__ __noinline__ void rescale_o_rows(uint32_t o_taddr, float alpha) {
 
 __global__ void __launch_bounds__(kAttnThreads, 1)
 tree_attention_split_kernel(const AttnParams p, const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap) {
+    after_previous_kernel();
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t s_anc[SAGE_MAX_NODES];
     __shared__ int32_t s_parent[SAGE_MAX_NODES];
@@ -697,6 +698,7 @@ tree_attention_split_kernel(const AttnParams p, const __grid_constant__ CUtensor
 // Split-K merge: one warp per (layer, node, head) row.  Lanes first reduce (m, l) over
 // the slices with shuffles, then each lane combines its four output columns.
 __global__ void attention_split_merge_kernel(AttnParams p) {
+    after_previous_kernel();
     const int warps = blockDim.x >> 5;
     const size_t rows_total = (size_t)p.sum_nodes * p.Hq;
     const size_t row = (size_t)blockIdx.x * warps + (threadIdx.x >> 5);
@@ -794,11 +796,11 @@ int launch(const void* q, int n_layers, int n_pages, const int32_t* page_table, 
         attr_set[dev] = true;
     }
     dim3 grid(S, row_pairs_for(sum_nodes, G), n_layers * batch * n_kv_heads);
-    tree_attention_split_kernel<<<grid, kAttnThreads, kSmemBytes, stream>>>(p, kmap, vmap);
+    if (sage::launch(tree_attention_split_kernel, grid, kAttnThreads, kSmemBytes, stream, 0, p, kmap, vmap) != cudaSuccess) return SAGE_ERR_CUDA;
     if (S > 1) {
         const size_t rows_total = (size_t)sum_nodes * n_q_heads;
         dim3 mg((unsigned)((rows_total + 7) / 8), n_layers);
-        attention_split_merge_kernel<<<mg, 256, 0, stream>>>(p);
+        if (sage::launch(attention_split_merge_kernel, mg, 256, 0, stream, 0, p) != cudaSuccess) return SAGE_ERR_CUDA;
     }
     return launch_status();
 }

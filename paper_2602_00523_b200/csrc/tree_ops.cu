@@ -36,6 +36,7 @@ __device__ __forceinline__ int pick_template(const SelectParams& p, int b, float
 }
 
 __global__ void select_tree_kernel(SelectParams p) {
+    after_previous_kernel();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= p.batch) return;
     float a;
@@ -47,6 +48,7 @@ __global__ void select_tree_kernel(SelectParams p) {
 
 // One block: offsets are a running sum over the batch, then every tree is copied.
 __global__ void handover_trees_kernel(SelectParams p) {
+    after_previous_kernel();
     __shared__ int s_bad;
     if (threadIdx.x == 0) {
         int off = 0, bad = 0;
@@ -78,6 +80,7 @@ __global__ void handover_trees_kernel(SelectParams p) {
 // ---------------------------------------------------------------------------
 __global__ void ancestor_mask_kernel(const int32_t* __restrict__ parent, const int32_t* __restrict__ node_offsets,
                                      uint64_t* __restrict__ anc, int32_t* status) {
+    after_previous_kernel();
     const int b = blockIdx.x;
     const int n0 = node_offsets[b];
     const int n = node_offsets[b + 1] - n0;
@@ -105,6 +108,7 @@ __global__ void accept_kernel(const int32_t* __restrict__ parent, const int32_t*
                               const int32_t* __restrict__ target_argmax, const int32_t* __restrict__ node_offsets,
                               int batch, int max_path, int32_t* __restrict__ path, int32_t* __restrict__ path_len,
                               int32_t* __restrict__ bonus_token, int32_t* status) {
+    after_previous_kernel();
     const int warps_per_block = blockDim.x >> 5;
     const int b = blockIdx.x * warps_per_block + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -208,6 +212,7 @@ constexpr int kColumns = 3;                      // columns a thread works on at
 constexpr int kMoves = 4;                        // moves of a batch
 
 __global__ void __launch_bounds__(kCompactThreads) compact_kv_kernel(const CompactParams p) {
+    after_previous_kernel();
     __shared__ int64_t s_src[SAGE_MAX_NODES];    // element offsets of the (page, head 0, slot) rows to move
     __shared__ int64_t s_dst[SAGE_MAX_NODES];
     __shared__ int s_moves, s_len;               // s_len: the sequence's new length, -1 if it does not advance
@@ -327,6 +332,7 @@ struct GrowParams {
 };
 
 __global__ void __launch_bounds__(SAGE_MAX_NODES) grow_tree_kernel(GrowParams p) {
+    after_previous_kernel();
     __shared__ int s_count[SAGE_MAX_NODES];
     const int b = blockIdx.x, tid = threadIdx.x;
     const int base = b * SAGE_MAX_NODES;
@@ -399,6 +405,7 @@ __global__ void __launch_bounds__(SAGE_MAX_NODES) grow_tree_kernel(GrowParams p)
 __global__ void update_history_kernel(const int32_t* __restrict__ path_len, int batch, sage_history_policy pol,
                                       int32_t* __restrict__ window_buf, int32_t* __restrict__ count,
                                       float* __restrict__ d_max, int32_t* status) {
+    after_previous_kernel();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= batch) return;
     const int pl = path_len[b];
@@ -440,8 +447,8 @@ extern "C" int sage_select_tree(const float* alpha, const int32_t* alpha_row, in
     if (batch == 0) return SAGE_OK;
     SelectParams p{alpha, alpha_row, batch, *policy, template_id, depth_cont, width_cont, bank_parent,
                    bank_rank, bank_n_nodes, next_parent, next_rank, next_node_offsets, status};
-    select_tree_kernel<<<(batch + 127) / 128, 128, 0, as_stream(stream)>>>(p);
-    if (handover) handover_trees_kernel<<<1, 256, 0, as_stream(stream)>>>(p);
+    (void)launch(select_tree_kernel, dim3((batch + 127) / 128), 128, 0, as_stream(stream), 0, p);
+    if (handover) (void)launch(handover_trees_kernel, dim3(1), 256, 0, as_stream(stream), 0, p);
     return launch_status();
 }
 
@@ -449,7 +456,7 @@ extern "C" int sage_build_ancestor_mask(const int32_t* parent, const int32_t* no
                                         uint64_t* anc, int32_t* status, void* stream) {
     if (!parent || !node_offsets || !anc || batch < 0) return SAGE_ERR_INVALID_ARG;
     if (batch == 0) return SAGE_OK;
-    ancestor_mask_kernel<<<batch, SAGE_MAX_NODES, 0, as_stream(stream)>>>(parent, node_offsets, anc, status);
+    (void)launch(ancestor_mask_kernel, dim3(batch), SAGE_MAX_NODES, 0, as_stream(stream), 0, parent, node_offsets, anc, status);
     return launch_status();
 }
 
@@ -461,8 +468,8 @@ extern "C" int sage_accept(const int32_t* parent, const int32_t* draft_token, co
     if (batch < 0 || max_path < 1) return SAGE_ERR_INVALID_ARG;
     if (batch == 0) return SAGE_OK;
     const int wpb = 4;
-    accept_kernel<<<(batch + wpb - 1) / wpb, wpb * 32, 0, as_stream(stream)>>>(
-        parent, draft_token, target_argmax, node_offsets, batch, max_path, path, path_len, bonus_token, status);
+    (void)launch(accept_kernel, dim3((batch + wpb - 1) / wpb), wpb * 32, 0, as_stream(stream), 0, parent, draft_token,
+                 target_argmax, node_offsets, batch, max_path, path, path_len, bonus_token, status);
     return launch_status();
 }
 
@@ -484,18 +491,8 @@ extern "C" int sage_compact_kv(void* k_pool, void* v_pool, int64_t layer_stride_
     while (blocks < kCompactCluster && (int64_t)blocks * kCompactThreads < columns) blocks *= 2;
     CompactParams p{(__nv_bfloat16*)k_pool, (__nv_bfloat16*)v_pool, layer_stride_elems, n_layers, n_pages,
                     max_pages_per_seq, max_path, n_kv_heads, blocks, page_table, seq_len, path, path_len, status};
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(blocks * batch));
-    cfg.blockDim = dim3(kCompactThreads);
-    cfg.stream = as_stream(stream);
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)blocks;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, compact_kv_kernel, p) != cudaSuccess) return SAGE_ERR_CUDA;
+    if (launch(compact_kv_kernel, dim3((unsigned)(blocks * batch)), kCompactThreads, 0, as_stream(stream), blocks, p) != cudaSuccess)
+        return SAGE_ERR_CUDA;
     return launch_status();
 }
 
@@ -515,7 +512,7 @@ extern "C" int sage_grow_tree(const int32_t* topk_idx, const float* topk_logprob
     if (batch == 0) return SAGE_OK;
     GrowParams p{topk_idx, topk_logprob, k, alpha, alpha_row, *policy, n_max, parent, rank, depth, token,
                  cum_logprob, n_nodes, frontier_begin, d_max_seq, status};
-    grow_tree_kernel<<<batch, SAGE_MAX_NODES, 0, as_stream(stream)>>>(p);
+    (void)launch(grow_tree_kernel, dim3(batch), SAGE_MAX_NODES, 0, as_stream(stream), 0, p);
     return launch_status();
 }
 
@@ -528,8 +525,8 @@ extern "C" int sage_update_history(const int32_t* path_len, int batch, const sag
         return SAGE_ERR_INVALID_ARG;
     if (policy->window > 1024) return SAGE_ERR_UNSUPPORTED;
     if (batch == 0) return SAGE_OK;
-    update_history_kernel<<<(batch + 127) / 128, 128, 0, as_stream(stream)>>>(path_len, batch, *policy, window_buf,
-                                                                              count, d_max, status);
+    (void)launch(update_history_kernel, dim3((batch + 127) / 128), 128, 0, as_stream(stream), 0, path_len, batch, *policy,
+                 window_buf, count, d_max, status);
     return launch_status();
 }
 
