@@ -50,8 +50,11 @@ constexpr int kMinSteps = 2;                   // no range shorter than this (sh
 
 struct AttnParams {
     __nv_bfloat16* out;
-    float* part_o;     // [gang][2][gang member][256 rows][128]   unnormalised
-    float* part_ml;    // [gang][2][gang member][256 rows][2]     (reference max in log2 units, l)
+    // Partial results, one slot per CTA for the head and one for the tail of its range.  Four output columns of
+    // consecutive rows lie side by side: a warp (one thread per row) writes 512 contiguous bytes per instruction, where
+    // row-major slots took 32 separate lines (an epilogue of 6 000 to 10 000 clocks; now KEPI).
+    float4* part_o;    // [CTA][2][32 column quads][256 rows]   unnormalised
+    float2* part_ml;   // [CTA][2][256 rows]                    (reference in log2 units, l)
     const int32_t* page_table;
     const int32_t* seq_len;
     const int32_t* parent;
@@ -66,6 +69,7 @@ struct AttnParams {
     int producer_off;          // diagnostics: the TMA warp issues no copies (every consumer wait then runs out)
 };
 
+struct Place { int layer, u, b, s0; };     // layer, unit, sequence and step of a position in the launch's work
 struct __align__(16) Shared {
     uint64_t kv_full[kRing];   // ring step r: the K tile of its step and the V tile of the step before have landed
     uint64_t kv_done[kRing];   // ring step r: every MMA that reads those tiles has finished
@@ -76,8 +80,8 @@ struct __align__(16) Shared {
     uint64_t q_ready;          // the query tiles of the segment are in shared memory
     uint64_t drain;            // abort path: everything issued so far has retired
     long long range_begin, range_end;
-    int first_lg, first_b, first_s0;
-    int n_rp, n_gangs;         // CTAs per gang (row pairs of the largest tree of this batch) and gangs, found on the device
+    Place first;               // where the range begins
+    int n_rp, heads_all;       // of the plan
     uint32_t tmem_base;
     volatile int abort;
 };
@@ -368,7 +372,7 @@ __device__ __noinline__ void rescale_o_rows(uint32_t o_taddr, float alpha) {
 }
 
 // ---- schedule: items, ranges, segments ---------------------------------------------------
-struct Item { int n0, N, L, steps, rp; };     // steps == 0: the sequence is skipped (and reported)
+struct Item { int n0, N, L, steps, rp; };     // steps == 0: the sequence is skipped (and reported); rp: row pairs
 
 __device__ __forceinline__ Item load_item(const AttnParams& p, int b, int* err) {
     Item it;
@@ -390,35 +394,75 @@ __device__ __forceinline__ Item load_item(const AttnParams& p, int b, int* err) 
     return it;
 }
 
-// Steps of all sequences of one (layer, KV head); called by a whole warp.
-__device__ __forceinline__ int steps_per_head(const AttnParams& p, int lane, int* err) {
-    int total = 0;
+// The work of a launch, laid end to end in steps: layer by layer, unit by unit, sequence by sequence.  With one CTA per
+// gang a unit is a KV head.  With two (some tree of the batch has more than 256 rows) it is a KV head for the trees of
+// two row pairs, one per CTA, and two KV heads, one per CTA, for the trees of one: both CTAs always have rows to work on
+// (with a head per unit throughout, one of them idled through the small trees of a mixed batch).
+struct Plan {
+    int n_rp;               // CTAs per gang
+    int heads_all;          // units that every sequence takes part in; the others are for trees of two row pairs only
+    int steps_all, steps_big;   // steps of all sequences, and of those with two row pairs
+    int n_act;              // gangs with work
+    long long steps_layer, W;   // steps of a layer, of the launch
+};
+// Called by a whole warp; the same answer in every CTA and in the merge kernel.
+__device__ __forceinline__ Plan make_plan(const AttnParams& p, int lane, int* err) {
+    Plan pl;
+    int mx = 0, all = 0, big = 0;
     for (int b0 = 0; b0 < p.batch; b0 += 32) {
-        int s = 0;
-        if (b0 + lane < p.batch) s = load_item(p, b0 + lane, err).steps;
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        total += s;
+        Item it{0, 0, 0, 0, 0};
+        if (b0 + lane < p.batch) it = load_item(p, b0 + lane, err);
+        // (whatever its length is: the kernels of a launch agree on the largest tree)
+        if (it.N >= 1 && it.N <= SAGE_MAX_NODES && it.n0 >= 0 && it.n0 + it.N <= p.sum_nodes) mx = max(mx, it.N * p.G);
+        all += it.steps;
+        big += it.rp > 1 ? it.steps : 0;
     }
-    return total;
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    pl.steps_all = __reduce_add_sync(0xffffffffu, all);
+    pl.steps_big = __reduce_add_sync(0xffffffffu, big);
+    pl.n_rp = mx > kRowsPerCta ? 2 : 1;
+    pl.heads_all = pl.n_rp == 2 ? (p.Hkv + 1) / 2 : p.Hkv;
+    pl.steps_layer = (long long)pl.heads_all * pl.steps_all + (long long)(p.Hkv - pl.heads_all) * pl.steps_big;
+    pl.W = schedule_selected(p.select, mx) ? pl.steps_layer * p.n_layers : 0;
+    const long long a = pl.W / kMinSteps;
+    const int gangs = p.n_ctas / pl.n_rp;
+    pl.n_act = a < 1 ? 1 : a < gangs ? (int)a : gangs;
+    return pl;
 }
-__device__ __forceinline__ int active_gangs(long long W, int n_gangs) {
-    long long a = W / kMinSteps;
-    if (a < 1) a = 1;
-    return a < n_gangs ? (int)a : n_gangs;
+// First step of a gang's range.  (32-bit division where the numbers allow it: the 64-bit one takes some hundred clocks.)
+__device__ __forceinline__ long long gang_begin(const Plan& pl, int gang) {
+    if (pl.W < (1 << 23)) return (unsigned)gang * (unsigned)pl.W / (unsigned)pl.n_act;      // gang <= 148 < 2^9
+    return (long long)gang * pl.W / pl.n_act;
 }
-__device__ __forceinline__ long long gang_begin(long long W, int n_act, int gang) { return (long long)gang * W / n_act; }
 // Gang whose range holds position pos: the largest k with gang_begin(k) <= pos.
-__device__ __forceinline__ int gang_of(long long W, int n_act, long long pos) {
-    return (int)(((pos + 1) * n_act - 1) / W);
-}
-// Sequence b and step s0 inside it for offset `off` into one (layer, KV head); whole warp.
-__device__ __forceinline__ void locate(const AttnParams& p, int lane, int off, int* b_out, int* s0_out) {
+__device__ __forceinline__ int gang_of(const Plan& pl, long long pos) { return (int)(((pos + 1) * pl.n_act - 1) / pl.W); }
+
+// Layer, unit, sequence and step inside it of position pos < W; whole warp.
+__device__ __forceinline__ Place locate(const AttnParams& p, const Plan& pl, int lane, long long pos) {
+    Place at;
+    unsigned r;
+    if (pl.W < (1ll << 31)) {
+        at.layer = (int)((unsigned)pos / (unsigned)pl.steps_layer);
+        r = (unsigned)pos % (unsigned)pl.steps_layer;
+    } else {
+        at.layer = (int)(pos / pl.steps_layer);
+        r = (unsigned)(pos % pl.steps_layer);
+    }
+    const unsigned first = (unsigned)pl.heads_all * (unsigned)pl.steps_all;
+    const bool big_only = r >= first;
+    if (big_only) r -= first;
+    const unsigned per_unit = (unsigned)(big_only ? pl.steps_big : pl.steps_all);
+    at.u = (int)(r / per_unit) + (big_only ? pl.heads_all : 0);
+    const int off = (int)(r % per_unit);
     int run = 0, err = 0;
-    *b_out = p.batch;
-    *s0_out = 0;
+    at.b = p.batch;
+    at.s0 = 0;
     for (int b0 = 0; b0 < p.batch; b0 += 32) {
         int s = 0;
-        if (b0 + lane < p.batch) s = load_item(p, b0 + lane, &err).steps;
+        if (b0 + lane < p.batch) {
+            const Item it = load_item(p, b0 + lane, &err);
+            if (!big_only || it.rp > 1) s = it.steps;
+        }
         int inc = s;
         for (int o = 1; o < 32; o <<= 1) {
             const int v = __shfl_up_sync(0xffffffffu, inc, o);
@@ -428,52 +472,66 @@ __device__ __forceinline__ void locate(const AttnParams& p, int lane, int off, i
         if (hit) {
             const int l = __ffs(hit) - 1;
             const int incl = __shfl_sync(0xffffffffu, inc, l), sl = __shfl_sync(0xffffffffu, s, l);
-            *b_out = b0 + l;
-            *s0_out = off - (run + incl - sl);
-            return;
+            at.b = b0 + l;
+            at.s0 = off - (run + incl - sl);
+            break;
         }
         run += __shfl_sync(0xffffffffu, inc, 31);
     }
+    return at;
 }
+// Which 256 rows of a tree of two row pairs a gang member takes: alternates, so that the member with the smaller
+// share of one tree (36 and 48 nodes leave 32 and 128 rows) has the larger one of the next.
+__device__ __forceinline__ int row_pair_of(int member, int u, int b) { return (member + u + b) & 1; }
 
-struct Seg { int layer, g, b, n0, N, L, s0, s1, steps, rp; bool at_range_begin; };
+struct Seg { int layer, g, b, n0, N, L, s0, s1, steps, row0; bool at_range_begin; };   // g: KV head, row0: first row of this CTA
 
-// Walks the segments of a range; every thread that needs them runs its own copy.
+// Walks the segments of a CTA's range; every thread that needs them runs its own copy.
 struct SegIter {
     int remaining;      // steps of the range still to hand out
-    int lg, b, s0;
+    int layer, u, b, s0;
+    int n_rp, heads_all, member;
     bool fresh;         // nothing handed out yet
     __device__ __forceinline__ void init(const Shared* sh) {
         remaining = (int)(sh->range_end - sh->range_begin);
-        lg = sh->first_lg;
-        b = sh->first_b;
-        s0 = sh->first_s0;
+        layer = sh->first.layer;
+        u = sh->first.u;
+        b = sh->first.b;
+        s0 = sh->first.s0;
+        n_rp = sh->n_rp;
+        heads_all = sh->heads_all;
+        member = n_rp == 2 ? (blockIdx.x & 1) : 0;
         fresh = true;
     }
+    __device__ __forceinline__ void next_sequence(const AttnParams& p) {
+        s0 = 0;
+        if (++b == p.batch) {
+            b = 0;
+            if (++u == p.Hkv) { u = 0; ++layer; }
+        }
+    }
+    // The next segment that has rows for this CTA.
     __device__ __forceinline__ bool next(const AttnParams& p, Seg& sg) {
-        int skipped = 0;
-        while (remaining > 0 && b < p.batch && skipped <= p.batch) {
+        while (remaining > 0 && layer < p.n_layers) {
             int err = 0;
             const Item it = load_item(p, b, &err);
-            if (it.steps == 0) {
-                ++skipped;
-                if (++b == p.batch) { b = 0; ++lg; }
+            if (it.steps == 0 || (u >= heads_all && it.rp < 2)) {
+                next_sequence(p);
                 continue;
             }
             const int s1 = (it.steps - s0 <= remaining) ? it.steps : s0 + remaining;
-            sg.layer = lg / p.Hkv; sg.g = lg % p.Hkv; sg.b = b;
+            const bool pair = n_rp == 2 && it.rp == 1;              // two heads of a small tree, one per CTA
+            sg.layer = layer; sg.b = b;
+            sg.g = pair ? 2 * u + member : u;
+            sg.row0 = it.rp == 2 ? row_pair_of(member, u, b) * kRowsPerCta : 0;
             sg.n0 = it.n0; sg.N = it.N; sg.L = it.L;
-            sg.s0 = s0; sg.s1 = s1; sg.steps = it.steps; sg.rp = it.rp;
+            sg.s0 = s0; sg.s1 = s1; sg.steps = it.steps;
             sg.at_range_begin = fresh;
             fresh = false;
             remaining -= s1 - s0;
-            if (s1 == it.steps) {
-                s0 = 0;
-                if (++b == p.batch) { b = 0; ++lg; }
-            } else {
-                s0 = s1;
-            }
-            return true;
+            if (s1 == it.steps) next_sequence(p);
+            else s0 = s1;
+            if (sg.g < p.Hkv) return true;
         }
         return false;
     }
@@ -493,58 +551,43 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    // ---- the gangs of this launch and this gang's range of steps (warp 0 computes, everybody reads).
-    // A gang has as many CTAs as the largest tree of the batch has row pairs, which only the device knows
-    // when the caller's node arrays are larger than the trees in them.
+    // ---- set-up, side by side: warp 0 works out the CTA's range of steps, another warp allocates tensor memory
+    // (512 columns: nothing else is resident), a thread prepares the barriers and fetches the tensor maps.
     if (warp == 0) {
         int err = 0;
-        const int rows_max = max_tree_rows(p.node_offsets, p.batch, p.sum_nodes, p.G, lane);
-        const bool mine = schedule_selected(p.select, rows_max);
-        const int n_rp = min(p.n_rp, max(1, (rows_max + kRowsPerCta - 1) / kRowsPerCta));
-        const int n_gangs = p.n_ctas / n_rp;
-        const int gang = blockIdx.x / n_rp;
-        const int Wb = mine ? steps_per_head(p, lane, &err) : 0;
+        const Plan pl = make_plan(p, lane, &err);
         if (err) report_status(p.status, err);
-        const long long W = (long long)p.n_layers * p.Hkv * Wb;
+        const int gang = pl.n_rp == 2 ? blockIdx.x >> 1 : blockIdx.x;
         long long begin = 0, end = 0;
-        int lg = 0, b = 0, s0 = 0;
-        if (W > 0) {
-            const int n_act = active_gangs(W, n_gangs);
-            if (gang < n_act) {
-                begin = gang_begin(W, n_act, gang);
-                end = gang_begin(W, n_act, gang + 1);
-            }
-            if (end > begin) {
-                lg = (int)(begin / Wb);
-                locate(p, lane, (int)(begin % Wb), &b, &s0);
-            }
+        Place at{0, 0, 0, 0};
+        if (pl.W > 0 && gang < pl.n_act) {
+            begin = gang_begin(pl, gang);
+            end = gang_begin(pl, gang + 1);
+            if (end > begin) at = locate(p, pl, lane, begin);
         }
         if (lane == 0) {
             sh->range_begin = begin; sh->range_end = end;
-            sh->first_lg = lg; sh->first_b = b; sh->first_s0 = s0;
-            sh->n_rp = n_rp; sh->n_gangs = n_gangs;
+            sh->first = at;
+            sh->n_rp = pl.n_rp; sh->heads_all = pl.heads_all;
         }
-    }
-    __syncthreads();
-    if (sh->range_end <= sh->range_begin) return;       // uniform: nothing to do, nothing allocated yet
-    const int n_rp = sh->n_rp;
-    const int member = blockIdx.x % n_rp, gang = blockIdx.x / n_rp;
-
-    // ---- set-up: barriers, TMEM
-    if (tid == 0) {
-        for (int i = 0; i < kRing; ++i) { mbar_init(&sh->kv_full[i], 1); mbar_init(&sh->kv_done[i], 1); }
-        for (int t = 0; t < 2; ++t) {
-            mbar_init(&sh->s_full[t], 1);
-            mbar_init(&sh->p_full[t], 4);               // one arrival per softmax warp
-            mbar_init(&sh->o_full[t], 1);
+    } else if (warp == 8) {
+        if (lane == 0) {
+            asm volatile("prefetch.tensormap [%0];" ::"l"(&kmap) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"(&vmap) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"(&qmap) : "memory");
+            for (int i = 0; i < kRing; ++i) { mbar_init(&sh->kv_full[i], 1); mbar_init(&sh->kv_done[i], 1); }
+            for (int t = 0; t < 2; ++t) {
+                mbar_init(&sh->s_full[t], 1);
+                mbar_init(&sh->p_full[t], 4);               // one arrival per softmax warp
+                mbar_init(&sh->o_full[t], 1);
+            }
+            mbar_init(&sh->q_free, 1);
+            mbar_init(&sh->drain, 1);
+            mbar_init(&sh->q_ready, 1);
+            sh->abort = 0;
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
-        mbar_init(&sh->q_free, 1);
-        mbar_init(&sh->drain, 1);
-        mbar_init(&sh->q_ready, 1);
-        sh->abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 9) {
+    } else if (warp == 9) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(&sh->tmem_base)), "r"(512) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -553,6 +596,10 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
+    if (sh->range_end <= sh->range_begin) {                 // uniform: nothing to do
+        if (warp == 9) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+        return;
+    }
 
     // Registers move from the copy / MMA warpgroup (which needs few) to the softmax warpgroups:
     // 4 warps give up 168 - 72 registers per thread, 8 warps take 216 - 168 each.
@@ -570,9 +617,8 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
             int rc = 0, kc = 0, vc = 0, nq = 0;          // ring steps, K tiles, V tiles, query loads issued so far
             bool ok = !p.producer_off;
             while (ok && it.next(p, sg)) {
-                if (member >= sg.rp) continue;
                 const int M = sg.N * p.G;
-                const int n_rt = (M - member * kRowsPerCta > kRowTile) ? 2 : 1;
+                const int n_rt = (M - sg.row0 > kRowTile) ? 2 : 1;
                 const int32_t* pages = p.page_table + (size_t)sg.b * p.max_pages;
                 const int n_pages_seq = (sg.L + sg.N + kPageSize - 1) / kPageSize;
                 const int n = sg.s1 - sg.s0;
@@ -619,7 +665,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                         for (int t = 0; t < n_rt; ++t)
                             for (int h = 0; h < 2; ++h)
                                 tma_load_5d(smem_u32(sQ + t * kQTileBytes + h * kQHalfBytes), &qmap, h * 64, 0, sg.g,
-                                            sg.n0 + (member * kRowsPerCta + t * kRowTile) / p.G, sg.layer, &sh->q_ready);
+                                            sg.n0 + (sg.row0 + t * kRowTile) / p.G, sg.layer, &sh->q_ready);
                         ++nq;
                     }
                     ids_prev[0] = ids[0]; ids_prev[1] = ids[1]; npg_prev = npg;
@@ -672,8 +718,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
         // The loop holds as few synchronisation instructions as the protocol allows: one wait and one commit
         // per ring step for the tiles, one of each per row tile.
         while (ok && it.next(p, sg)) {
-            if (member >= sg.rp) continue;
-            const int n_rt = __shfl_sync(0xffffffffu, (sg.N * p.G - member * kRowsPerCta > kRowTile) ? 2 : 1, 0);
+            const int n_rt = __shfl_sync(0xffffffffu, (sg.N * p.G - sg.row0 > kRowTile) ? 2 : 1, 0);
             const int n = __shfl_sync(0xffffffffu, sg.s1 - sg.s0, 0);
             ok = mbar_wait_warp(&sh->q_ready, nq & 1, sh, p);
             ++nq;
@@ -729,16 +774,15 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
         int rc0 = 0, vc0 = 0;                           // ring steps / V tiles of the CTA before the current segment
         bool ok = true;
         while (ok && it.next(p, sg)) {
-            if (member >= sg.rp) continue;
             const int M = sg.N * p.G;
             const int rc_seg = rc0, vc_seg = vc0;       // this segment's first ring step / V tile
             rc0 += sg.s1 - sg.s0 + 1;
             vc0 += sg.s1 - sg.s0;
-            if (t == 1 && M - member * kRowsPerCta <= kRowTile) continue;
-            const int R = member * kRowsPerCta + t * kRowTile + r;
+            if (t == 1 && M - sg.row0 <= kRowTile) continue;
+            const int R = sg.row0 + t * kRowTile + r;
             const bool row_ok = R < M;
             const int node = row_ok ? R / p.G : 0;
-            const bool warp_live = member * kRowsPerCta + t * kRowTile + (warp & 3) * 32 < M;
+            const bool warp_live = sg.row0 + t * kRowTile + (warp & 3) * 32 < M;
             uint64_t anc = 0;
             if (sg.s1 * kStepKeys > sg.L && row_ok) {
                 // the segment reaches the tree part: this row's ancestor bitset (the G rows of a node
@@ -829,16 +873,15 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
             tc_fence_after();
             const bool whole = (sg.s0 == 0 && sg.s1 == sg.steps);
             const float inv = (l_sum > 0.f) ? 1.0f / l_sum : 0.f;
-            float* po = nullptr;
+            float4* po = nullptr;
             __nv_bfloat16* oo = nullptr;
             if (whole) {
                 const size_t row = (size_t)(sg.n0 + node) * p.Hq + sg.g * p.G + (row_ok ? R % p.G : 0);
                 oo = p.out + ((size_t)sg.layer * p.sum_nodes * p.Hq + row) * kHeadDim;
             } else {
-                const size_t pr = (((size_t)gang * 2 + (sg.at_range_begin ? 0 : 1)) * n_rp + member) * kRowsPerCta +
-                                  t * kRowTile + r;
-                po = p.part_o + pr * kHeadDim;
-                if (row_ok) { p.part_ml[pr * 2] = m_ref; p.part_ml[pr * 2 + 1] = l_sum; }
+                const size_t slot = (size_t)blockIdx.x * 2 + (sg.at_range_begin ? 0 : 1);
+                po = p.part_o + slot * (kHeadDim / 4) * kRowsPerCta + t * kRowTile + r;
+                if (row_ok) p.part_ml[slot * kRowsPerCta + t * kRowTile + r] = make_float2(m_ref, l_sum);
             }
             if (warp_live) {
 #pragma unroll
@@ -860,8 +903,9 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                         } else {
 #pragma unroll
                             for (int i = 0; i < 8; ++i)
-                                *reinterpret_cast<uint4*>(po + c * 32 + i * 4) =
-                                    make_uint4(orr[4 * i], orr[4 * i + 1], orr[4 * i + 2], orr[4 * i + 3]);
+                                po[(c * 8 + i) * kRowsPerCta] =
+                                    make_float4(__uint_as_float(orr[4 * i]), __uint_as_float(orr[4 * i + 1]),
+                                                __uint_as_float(orr[4 * i + 2]), __uint_as_float(orr[4 * i + 3]));
                         }
                     }
                 }
@@ -878,81 +922,87 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
     }
 }
 
-// Merge of the items that a range boundary cut into segments.  Only a boundary between two gangs'
-// ranges can cut an item, so the grid is (x = boundary, y = 32-row chunk): the block finds the item
-// its boundary falls into, leaves if the boundary coincides with the item's start or if an earlier
-// boundary already lies inside the same item (that block does the work), and otherwise combines the
-// item's segments: which gangs hold them, and in which of their two partial slots, follows from
-// the positions alone.
+// Merge of the items that a range boundary cut into segments.  Only a boundary between two gangs' ranges can cut an
+// item, so the grid holds a block per boundary and 32 rows of a gang's CTAs: the block finds the item its boundary falls into,
+// leaves if the boundary coincides with the item's start or if an earlier boundary already lies inside the same item
+// (that block does the work), and otherwise combines the item's segments: which gangs hold them, and in which of their
+// two partial slots, follows from the positions alone.  One lane per row, 16 output columns per warp; the loads of four
+// segments are in flight together (one segment after the other took 20 us for one layer at 16k keys).
 __global__ void __launch_bounds__(256) attention_rows_merge_kernel(AttnParams p) {
     after_previous_kernel();
-    __shared__ int s_Wb, s_b, s_s0, s_n_rp;
+    __shared__ Plan s_plan;
+    __shared__ Place s_at;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int k_cut = blockIdx.x + 1;                   // boundary between gang k_cut - 1 and gang k_cut
     if (warp == 0) {
-        int err = 0, b = 0, s0 = 0;
-        // the same gang layout as the attention kernel worked out
-        const int rows_max = max_tree_rows(p.node_offsets, p.batch, p.sum_nodes, p.G, lane);
-        const bool mine = schedule_selected(p.select, rows_max);
-        const int n_rp = min(p.n_rp, max(1, (rows_max + kRowsPerCta - 1) / kRowsPerCta));
-        const int Wb = mine ? steps_per_head(p, lane, &err) : 0;
-        if (Wb > 0) {
-            const long long W = (long long)p.n_layers * p.Hkv * Wb;
-            const int n_act = active_gangs(W, p.n_ctas / n_rp);
-            if (k_cut < n_act) locate(p, lane, (int)(gang_begin(W, n_act, k_cut) % Wb), &b, &s0);
-        }
-        if (lane == 0) { s_Wb = Wb; s_b = b; s_s0 = s0; s_n_rp = n_rp; }
+        int err = 0;
+        const Plan pl = make_plan(p, lane, &err);
+        const int k = blockIdx.x / (pl.n_rp * (kRowsPerCta / 32)) + 1;
+        Place at{0, 0, 0, 0};
+        if (pl.W > 0 && k < pl.n_act) at = locate(p, pl, lane, gang_begin(pl, k));
+        if (lane == 0) { s_plan = pl; s_at = at; }
     }
     __syncthreads();
-    const int Wb = s_Wb;
-    if (Wb <= 0) return;
-    const int n_rp = s_n_rp;
-    const long long W = (long long)p.n_layers * p.Hkv * Wb;
-    const int n_act = active_gangs(W, p.n_ctas / n_rp);
-    if (k_cut >= n_act || s_s0 == 0) return;            // no such boundary, or it falls between two items
-    const long long cut = gang_begin(W, n_act, k_cut);
-    const int lg = (int)(cut / Wb), b = s_b;
+    const Plan pl = s_plan;
+    const Place at = s_at;
+    const int k_cut = blockIdx.x / (pl.n_rp * (kRowsPerCta / 32)) + 1;  // boundary between gang k_cut - 1 and gang k_cut
+    if (pl.W <= 0 || k_cut >= pl.n_act || at.s0 == 0) return;           // no such boundary, or it falls between two items
+    const int chunk = blockIdx.x % (pl.n_rp * (kRowsPerCta / 32));
+    const int member = chunk / (kRowsPerCta / 32), row = chunk % (kRowsPerCta / 32) * 32 + lane;
     int err = 0;
-    const Item it = load_item(p, b, &err);
-    const long long a = cut - s_s0;                     // position of the item's first step
-    const int k_first = gang_of(W, n_act, a), k_last = gang_of(W, n_act, a + it.steps - 1);
+    const Item it = load_item(p, at.b, &err);
+    const long long a = gang_begin(pl, k_cut) - at.s0;  // position of the item's first step
+    const int k_first = gang_of(pl, a), k_last = gang_of(pl, a + it.steps - 1);
     if (k_first != k_cut - 1) return;                   // an earlier boundary cuts the same item
-    const bool first_mid_range = (a != gang_begin(W, n_act, k_first));
-    const int M = it.N * p.G;
-    const int layer = lg / p.Hkv, g = lg % p.Hkv;
-    for (int i = 0; i < 4; ++i) {
-        const int R = blockIdx.y * 32 + warp * 4 + i;
-        if (R >= M) break;
-        const int member = R / kRowsPerCta, Rl = R % kRowsPerCta;
-        auto slot_row = [&](int k) -> size_t {
-            const int slot = (k == k_first && first_mid_range) ? 1 : 0;
-            return (((size_t)k * 2 + slot) * n_rp + member) * kRowsPerCta + Rl;
-        };
-        float mx = -INFINITY;
-        for (int k = k_first + lane; k <= k_last; k += 32) {
-            const size_t pr = slot_row(k);
-            if (p.part_ml[pr * 2 + 1] > 0.f) mx = fmaxf(mx, p.part_ml[pr * 2]);
-        }
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        float lsum = 0.f;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int k = k_first; k <= k_last; ++k) {
-            const size_t pr = slot_row(k);
-            const float l = p.part_ml[pr * 2 + 1];
-            if (!(l > 0.f)) continue;
-            const float w = exp2f(p.part_ml[pr * 2] - mx);
-            lsum = fmaf(l, w, lsum);
-            const float4 v = reinterpret_cast<const float4*>(p.part_o + pr * kHeadDim)[lane];
-            acc.x = fmaf(w, v.x, acc.x); acc.y = fmaf(w, v.y, acc.y);
-            acc.z = fmaf(w, v.z, acc.z); acc.w = fmaf(w, v.w, acc.w);
-        }
-        const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
-        uint2 packed;
-        packed.x = pack_bf16(acc.x * inv, acc.y * inv);
-        packed.y = pack_bf16(acc.z * inv, acc.w * inv);
-        const size_t row = (size_t)(it.n0 + R / p.G) * p.Hq + g * p.G + R % p.G;
-        reinterpret_cast<uint2*>(p.out + ((size_t)layer * p.sum_nodes * p.Hq + row) * kHeadDim)[lane] = packed;
+    const bool first_mid_range = (a != gang_begin(pl, k_first));
+    const bool pair = pl.n_rp == 2 && it.rp == 1;
+    const int g = pair ? 2 * at.u + member : at.u;
+    const int R = row + (it.rp == 2 ? row_pair_of(member, at.u, at.b) * kRowsPerCta : 0);
+    if (g >= p.Hkv) return;
+    const bool row_ok = R < it.N * p.G;
+    if (!__any_sync(0xffffffffu, row_ok)) return;
+    auto slot_of = [&](int k) { return (size_t)(k * pl.n_rp + member) * 2 + (k == k_first && first_mid_range ? 1 : 0); };
+    // (rows past the tree were not written: they are read all the same, as lanes of a warp with live rows, and dropped)
+    float mx = -INFINITY;
+    for (int k = k_first; k <= k_last; ++k) {
+        const float2 ml = p.part_ml[slot_of(k) * kRowsPerCta + row];
+        if (row_ok && ml.y > 0.f) mx = fmaxf(mx, ml.x);
     }
+    float lsum = 0.f;
+    float4 acc[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k0 = k_first; k0 <= k_last; k0 += 4) {
+        float w[4];
+        float4 v[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const size_t slot = slot_of(min(k0 + u, k_last));
+            const float2 ml = p.part_ml[slot * kRowsPerCta + row];
+            w[u] = (row_ok && k0 + u <= k_last && ml.y > 0.f) ? exp2f(ml.x - mx) : 0.f;
+            lsum = fmaf(w[u] > 0.f ? ml.y : 0.f, w[u], lsum);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[u][i] = p.part_o[(slot * (kHeadDim / 4) + warp * 4 + i) * kRowsPerCta + row];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (w[u] > 0.f) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    acc[i].x = fmaf(w[u], v[u][i].x, acc[i].x); acc[i].y = fmaf(w[u], v[u][i].y, acc[i].y);
+                    acc[i].z = fmaf(w[u], v[u][i].z, acc[i].z); acc[i].w = fmaf(w[u], v[u][i].w, acc[i].w);
+                }
+            }
+        }
+    }
+    if (!row_ok) return;
+    const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
+    const size_t orow = (size_t)(it.n0 + R / p.G) * p.Hq + g * p.G + R % p.G;
+    uint4* out = reinterpret_cast<uint4*>(p.out + ((size_t)at.layer * p.sum_nodes * p.Hq + orow) * kHeadDim + warp * 16);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        out[h] = make_uint4(pack_bf16(acc[2 * h].x * inv, acc[2 * h].y * inv), pack_bf16(acc[2 * h].z * inv, acc[2 * h].w * inv),
+                            pack_bf16(acc[2 * h + 1].x * inv, acc[2 * h + 1].y * inv),
+                            pack_bf16(acc[2 * h + 1].z * inv, acc[2 * h + 1].w * inv));
 }
 
 // ---- host side ------------------------------------------------------------------------------
@@ -975,8 +1025,8 @@ int launch(int n_ctas, int select, int n_layers, int n_pages, const int32_t* pag
     p.n_ctas = (n_ctas / p.n_rp) * p.n_rp;          // whole gangs whatever the gang size turns out to be (1 or 2)
     p.select = select;
     p.out = (__nv_bfloat16*)out;
-    p.part_o = (float*)ws;
-    p.part_ml = (float*)ws + (size_t)n_ctas * 2 * kRowsPerCta * kHeadDim;
+    p.part_o = (float4*)ws;
+    p.part_ml = (float2*)((float*)ws + (size_t)n_ctas * 2 * kRowsPerCta * kHeadDim);
     p.page_table = page_table; p.seq_len = seq_len; p.parent = parent; p.node_offsets = node_offsets;
     p.status = status;
     p.n_layers = n_layers; p.batch = batch; p.sum_nodes = sum_nodes; p.n_pages = n_pages;
@@ -997,8 +1047,8 @@ int launch(int n_ctas, int select, int n_layers, int n_pages, const int32_t* pag
     if (sage::launch(tree_attention_rows_kernel, dim3(p.n_ctas), kAttnThreads, kSmemBytes, stream, 0, p, qmap, kmap, vmap) != cudaSuccess)
         return SAGE_ERR_CUDA;
     if (p.n_ctas > 1) {
-        // one block per possible boundary between two gangs' ranges and 32-row chunk; those that find no cut item leave
-        dim3 mg((unsigned)(p.n_ctas - 1), (unsigned)((p.n_rp * kRowsPerCta + 31) / 32));
+        // one block per possible boundary between two gangs' ranges and 32 rows; those that find no cut item leave
+        dim3 mg((unsigned)(p.n_ctas * (kRowsPerCta / 32)));
         if (sage::launch(attention_rows_merge_kernel, mg, 256, 0, stream, 0, p) != cudaSuccess) return SAGE_ERR_CUDA;
     }
     return launch_status();
