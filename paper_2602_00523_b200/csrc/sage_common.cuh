@@ -57,10 +57,9 @@ __device__ __forceinline__ int max_tree_rows(const int32_t* __restrict__ node_of
     return mx;
 }
 // select: 0 = the kernel runs whatever the trees look like; 1 = only for trees of one 128-row tile;
-// 2 = only for two row tiles; 3 = only for more.
+// 2 = only for more.
 __device__ __forceinline__ bool schedule_selected(int select, int rows) {
-    return select == 0 || (select == 1 && rows <= 128) || (select == 2 && rows > 128 && rows <= 256) ||
-           (select == 3 && rows > 256);
+    return select == 0 || (select == 1) == (rows <= 128);
 }
 
 // Every kernel is launched to overlap its launch with the end of the kernel before it (programmatic stream

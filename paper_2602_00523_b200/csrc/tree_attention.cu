@@ -1289,7 +1289,7 @@ size_t workspace_size(int n_layers, int batch, int sum_nodes, int n_q_heads, int
 int launch(const void* q, int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,
            const int32_t* seq_len, const int32_t* parent, const int32_t* node_offsets, int batch, int sum_nodes,
            int n_q_heads, int n_kv_heads, float sm_scale, void* out, void* ws, int32_t* status, long long wait_cycles,
-           int producer_off, int select, const CUtensorMap& kmap, const CUtensorMap& vmap, cudaStream_t stream);
+           int producer_off, const CUtensorMap& kmap, const CUtensorMap& vmap, cudaStream_t stream);
 }  // namespace split
 
 // The streaming schedule for trees of more than one row tile (tree_attention_rows.cu).
@@ -1387,7 +1387,7 @@ extern "C" int sage_tree_attention(const void* q, const void* k_pool, const void
     if (sched == kSplit)
         return split::launch(q, n_layers, n_pages, page_table, max_pages_per_seq, seq_len, parent, node_offsets, batch,
                              sum_nodes, n_q_heads, n_kv_heads, sm_scale, out, ws, status, g_wait_cycles, g_producer_off,
-                             0, kmap, vmap, as_stream(stream));
+                             kmap, vmap, as_stream(stream));
     if (!make_q_map(&qmap, q, n_layers, sum_nodes, n_kv_heads, G)) return SAGE_ERR_CUDA;
     if (sched == kRows)
         return rows::launch(resident_ctas(), 0, n_layers, n_pages, page_table, max_pages_per_seq, seq_len, parent,
@@ -1395,18 +1395,11 @@ extern "C" int sage_tree_attention(const void* q, const void* k_pool, const void
                             g_wait_cycles, g_producer_off, qmap, kmap, vmap, as_stream(stream));
     const int tiles = row_tiles(sum_nodes, G);
     if (sched == kOnDevice) {
-        // the kernels for two row tiles and (if the bound allows them) for more; the one for one row tile follows below
-        int rc = rows::launch(resident_ctas(), 2, n_layers, n_pages, page_table, max_pages_per_seq, seq_len, parent,
-                              node_offsets, batch, sum_nodes, n_q_heads, n_kv_heads, sm_scale, out, ws, status,
-                              g_wait_cycles, g_producer_off, qmap, kmap, vmap, as_stream(stream));
+        // the kernel for more than one row tile; the one for one row tile follows below
+        const int rc = rows::launch(resident_ctas(), 2, n_layers, n_pages, page_table, max_pages_per_seq, seq_len, parent,
+                                    node_offsets, batch, sum_nodes, n_q_heads, n_kv_heads, sm_scale, out, ws, status,
+                                    g_wait_cycles, g_producer_off, qmap, kmap, vmap, as_stream(stream));
         if (rc != SAGE_OK) return rc;
-        if (tiles > 2) {
-            if ((long long)n_layers * batch * n_kv_heads > 65535) return SAGE_ERR_UNSUPPORTED;    // grid limit of the split schedule
-            rc = split::launch(q, n_layers, n_pages, page_table, max_pages_per_seq, seq_len, parent, node_offsets, batch,
-                               sum_nodes, n_q_heads, n_kv_heads, sm_scale, out, ws, status, g_wait_cycles,
-                               g_producer_off, 3, kmap, vmap, as_stream(stream));
-            if (rc != SAGE_OK) return rc;
-        }
     }
     const int n_ctas = resident_ctas();
     AttnParams p{};

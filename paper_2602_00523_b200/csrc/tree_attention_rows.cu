@@ -46,13 +46,14 @@ constexpr int kTileBytes = 2 * kTileHalfBytes;              // K or V tile of on
 constexpr int kQTileBytes = kRowTile * kHeadDim * 2;        // 32 KB
 constexpr int kQHalfBytes = kRowTile * 64 * 2;              // one 64-wide d-half of a Q tile: 16 KB
 constexpr int kAttnThreads = 384;              // 2 softmax warpgroups + one warpgroup of TMA warp, MMA warp and two idle warps
+constexpr float kMaxSum = 1073741824.f;        // a step whose sum of probabilities stays below this keeps its reference
 constexpr int kMinSteps = 2;                   // no range shorter than this (short contexts are latency-bound)
 
 struct AttnParams {
     __nv_bfloat16* out;
     // Partial results, one slot per CTA for the head and one for the tail of its range.  Four output columns of
     // consecutive rows lie side by side: a warp (one thread per row) writes 512 contiguous bytes per instruction, where
-    // row-major slots took 32 separate lines (an epilogue of 6 000 to 10 000 clocks; now KEPI).
+    // row-major slots took 32 separate lines (an epilogue of 6 000 to 10 000 clocks; now 1 500 to 3 000).
     float4* part_o;    // [CTA][2][32 column quads][256 rows]   unnormalised
     float2* part_ml;   // [CTA][2][256 rows]                    (reference in log2 units, l)
     const int32_t* page_table;
@@ -208,6 +209,15 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
           "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// The wait, tied to the registers that a load filled: what uses them stays behind it, other loads need not.
+__device__ __forceinline__ void tmem_wait_ld_of(uint32_t (&r)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                   "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]),
+                   "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]),
+                   "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+                 :: "memory");
+}
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ float fast_exp2(float x) {
@@ -264,12 +274,12 @@ __device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
 // (which delivers only 16 results per clock per SM and would otherwise bound the softmax):
 // x = n + f with n = round(x), f in [-0.5, 0.5]; 2^f by a cubic fitted to 7.5e-5 relative error
 // (well below the 2^-9 rounding of the bf16 probabilities); n goes straight into the exponent bits.
-// Inputs are clamped at -125, so that 2^x never leaves the normal range; -inf does not come here.
+// Inputs are clamped to [-125, 127], so that 2^x never leaves the normal range; -inf does not come here.
 __device__ __forceinline__ void exp2_pair_fma(uint64_t x2, float& p0, float& p1) {
     constexpr float kMagic = 12582912.f;             // 1.5 * 2^23: adding it leaves round(x) in the low mantissa bits
     float x0, x1;
     f2_unpack(x2, x0, x1);
-    x2 = f2_pack(fmaxf(x0, -125.f), fmaxf(x1, -125.f));
+    x2 = f2_pack(fminf(fmaxf(x0, -125.f), 127.f), fminf(fmaxf(x1, -125.f), 127.f));
     const uint64_t t2 = f2_add(x2, f2_pack(kMagic, kMagic));
     const uint64_t n2 = f2_add(t2, f2_pack(-kMagic, -kMagic));
     const uint64_t f2 = f2_fma(n2, f2_pack(-1.f, -1.f), x2);
@@ -369,6 +379,25 @@ __device__ __noinline__ void rescale_o_rows(uint32_t o_taddr, float alpha) {
         tmem_st32(o_taddr + c * 32, orr);
     }
     tmem_wait_st();
+}
+
+// 4 x 4 transpose of 16-byte pieces among each four lanes: lane 4a + b gives its piece i to lane 4a + i and ends up with
+// piece b of rows 4a .. 4a + 3 in v[0 .. 3].
+__device__ __forceinline__ void transpose4(uint4 (&v)[4], int lane) {
+    auto swap = [&](uint4& keep_lo, uint4& keep_hi, bool hi, int mask) {      // lanes with `hi` send the first, the others the second
+        uint4 mine = hi ? keep_lo : keep_hi;
+        mine.x = __shfl_xor_sync(0xffffffffu, mine.x, mask);
+        mine.y = __shfl_xor_sync(0xffffffffu, mine.y, mask);
+        mine.z = __shfl_xor_sync(0xffffffffu, mine.z, mask);
+        mine.w = __shfl_xor_sync(0xffffffffu, mine.w, mask);
+        if (hi) keep_lo = mine;
+        else keep_hi = mine;
+    };
+    const bool h1 = lane & 1, h2 = lane & 2;
+    swap(v[0], v[1], h1, 1);
+    swap(v[2], v[3], h1, 1);
+    swap(v[0], v[2], h2, 2);
+    swap(v[1], v[3], h2, 2);
 }
 
 // ---- schedule: items, ranges, segments ---------------------------------------------------
@@ -622,6 +651,14 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                 const int32_t* pages = p.page_table + (size_t)sg.b * p.max_pages;
                 const int n_pages_seq = (sg.L + sg.N + kPageSize - 1) / kPageSize;
                 const int n = sg.s1 - sg.s0;
+                // the segment's query tiles, once the previous segment's score MMAs have read theirs
+                if (nq > 0 && !mbar_wait(&sh->q_free, (nq - 1) & 1, sh, p)) break;
+                mbar_expect_tx(&sh->q_ready, n_rt * kQTileBytes);
+                for (int t = 0; t < n_rt; ++t)
+                    for (int h = 0; h < 2; ++h)
+                        tma_load_5d(smem_u32(sQ + t * kQTileBytes + h * kQHalfBytes), &qmap, h * 64, 0, sg.g,
+                                    sg.n0 + (sg.row0 + t * kRowTile) / p.G, sg.layer, &sh->q_ready);
+                ++nq;
                 int ids_prev[2] = {0, 0}, npg_prev = 0;
                 for (int i = 0; i <= n; ++i) {
                     const int j = sg.s0 + i;
@@ -658,16 +695,6 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                         ++vc;
                     }
                     ++rc;
-                    if (i == 0) {
-                        // the segment's query tiles, once the previous segment's score MMAs have read theirs
-                        if (nq > 0 && !mbar_wait(&sh->q_free, (nq - 1) & 1, sh, p)) { ok = false; break; }
-                        mbar_expect_tx(&sh->q_ready, n_rt * kQTileBytes);
-                        for (int t = 0; t < n_rt; ++t)
-                            for (int h = 0; h < 2; ++h)
-                                tma_load_5d(smem_u32(sQ + t * kQTileBytes + h * kQHalfBytes), &qmap, h * 64, 0, sg.g,
-                                            sg.n0 + (sg.row0 + t * kRowTile) / p.G, sg.layer, &sh->q_ready);
-                        ++nq;
-                    }
                     ids_prev[0] = ids[0]; ids_prev[1] = ids[1]; npg_prev = npg;
                 }
             }
@@ -824,38 +851,55 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                 const int pos0 = j * kStepKeys;
                 const bool masked = pos0 + kStepKeys > sg.L;     // reaches into the tree part (or past the end)
                 uint32_t sr[128];
-                load_scores(s_taddr, sr);
-                if (masked) {
+                // Probabilities are taken against the row's reference of the steps before: any reference within some 2^60
+                // of the row's maximum gives the same result, so a step need not look for its maximum first.  It shows in
+                // the step's sum whether the reference still serves; the first step of a segment, steps with masked
+                // scores and steps whose sum has grown beyond 2^30 go through the maximum.
+                bool by_max = masked || j == sg.s0;
+                if (!by_max) {
+                    uint64_t acc[2] = {0ull, 0ull};
+                    tmem_ld32(s_taddr, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) mask_chunk(sr + 32 * c, pos0 + 32 * c, sg.L, sg.N, anc);
+                    for (int c = 0; c < 4; ++c) {
+                        tmem_wait_ld_of(*reinterpret_cast<uint32_t(*)[32]>(&sr[32 * c]));
+                        if (c < 3) tmem_ld32(s_taddr + 32 * (c + 1), *reinterpret_cast<uint32_t(*)[32]>(&sr[32 * (c + 1)]));
+                        exp_chunk<SAGE_EXP2_FMA_PAIRS>(sr + 32 * c, p.scale_log2, -m_ref, sr + 16 * c, acc);
+                    }
+                    float sum_a, sum_b;
+                    f2_unpack(f2_add(acc[0], acc[1]), sum_a, sum_b);
+                    const float sum = sum_a + sum_b;
+                    by_max = __any_sync(0xffffffffu, !(sum < kMaxSum));
+                    if (!by_max) l_sum += sum;
                 }
-                float mx = -INFINITY;
+                if (by_max) {
+                    load_scores(s_taddr, sr);
+                    if (masked) {
 #pragma unroll
-                for (int c = 0; c < 4; ++c) max_chunk(sr + 32 * c, mx);
-                // lazy rescale: the reference moves only when the row max grew by more than 2^8 over it
-                const float m_cand = mx * p.scale_log2;
-                const bool grow = m_cand > m_ref + 8.0f;
-                float alpha = 1.0f;
-                if (grow) {
-                    alpha = fast_exp2(m_ref - m_cand);              // 0 when m_ref was -inf
-                    m_ref = m_cand;
-                }
-                // O_t *= alpha.  The P V product of the step before has finished: the scores of this step were
-                // issued after it, and their completion is what this warp waited for above.
-                if (j > sg.s0 && __any_sync(0xffffffffu, grow)) rescale_o_rows(o_taddr, alpha);
-                const float neg_ref = (m_ref == -INFINITY) ? 0.f : -m_ref;
-                // probabilities, packed to bf16 in place: chunk c (32 scores) leaves its 16 words at sr[16c ..]
-                uint64_t acc[2] = {0ull, 0ull};
-                if (masked) {
+                        for (int c = 0; c < 4; ++c) mask_chunk(sr + 32 * c, pos0 + 32 * c, sg.L, sg.N, anc);
+                    }
+                    float mx = -INFINITY;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) max_chunk(sr + 32 * c, mx);
+                    // the reference moves only when the row max grew by more than 2^8 over it
+                    const float m_cand = mx * p.scale_log2;
+                    const bool grow = m_cand > m_ref + 8.0f;
+                    float alpha = 1.0f;
+                    if (grow) {
+                        alpha = fast_exp2(m_ref - m_cand);              // 0 when m_ref was -inf
+                        m_ref = m_cand;
+                    }
+                    // O_t *= alpha.  The P V product of the step before has finished: the scores of this step were
+                    // issued after it, and their completion is what this warp waited for above.
+                    if (j > sg.s0 && __any_sync(0xffffffffu, grow)) rescale_o_rows(o_taddr, alpha);
+                    const float neg_ref = (m_ref == -INFINITY) ? 0.f : -m_ref;
+                    uint64_t acc[2] = {0ull, 0ull};
 #pragma unroll
                     for (int c = 0; c < 4; ++c) exp_chunk<0>(sr + 32 * c, p.scale_log2, neg_ref, sr + 16 * c, acc);   // may hold -inf
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) exp_chunk<SAGE_EXP2_FMA_PAIRS>(sr + 32 * c, p.scale_log2, neg_ref, sr + 16 * c, acc);
+                    float sum_a, sum_b;
+                    f2_unpack(f2_add(acc[0], acc[1]), sum_a, sum_b);
+                    l_sum = l_sum * alpha + (sum_a + sum_b);
                 }
-                float sum_a, sum_b;
-                f2_unpack(f2_add(acc[0], acc[1]), sum_a, sum_b);
-                l_sum = l_sum * alpha + (sum_a + sum_b);
+                // (chunk c of 32 scores has left its 16 words of bf16 pairs at sr[16c ..])
                 uint32_t* pk = sr;
                 tmem_st32(s_taddr, pk);                 // P over the first 64 columns of S_t
                 tmem_st32(s_taddr + 32, pk + 32);
@@ -874,11 +918,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
             const bool whole = (sg.s0 == 0 && sg.s1 == sg.steps);
             const float inv = (l_sum > 0.f) ? 1.0f / l_sum : 0.f;
             float4* po = nullptr;
-            __nv_bfloat16* oo = nullptr;
-            if (whole) {
-                const size_t row = (size_t)(sg.n0 + node) * p.Hq + sg.g * p.G + (row_ok ? R % p.G : 0);
-                oo = p.out + ((size_t)sg.layer * p.sum_nodes * p.Hq + row) * kHeadDim;
-            } else {
+            if (!whole) {
                 const size_t slot = (size_t)blockIdx.x * 2 + (sg.at_range_begin ? 0 : 1);
                 po = p.part_o + slot * (kHeadDim / 4) * kRowsPerCta + t * kRowTile + r;
                 if (row_ok) p.part_ml[slot * kRowsPerCta + t * kRowTile + r] = make_float2(m_ref, l_sum);
@@ -889,24 +929,31 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                     uint32_t orr[32];
                     tmem_ld32(o_taddr + c * 32, orr);
                     tmem_wait_ld();
-                    if (row_ok) {
-                        if (oo) {
+                    if (whole) {
+                        // every lane holds 64 bytes of its row; four lanes exchange them, so that a store instruction writes
+                        // 64 contiguous bytes of eight rows instead of 16 bytes of 32
+                        uint4 v[4];
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                uint4 v;
-                                v.x = pack_bf16(__uint_as_float(orr[8 * i + 0]) * inv, __uint_as_float(orr[8 * i + 1]) * inv);
-                                v.y = pack_bf16(__uint_as_float(orr[8 * i + 2]) * inv, __uint_as_float(orr[8 * i + 3]) * inv);
-                                v.z = pack_bf16(__uint_as_float(orr[8 * i + 4]) * inv, __uint_as_float(orr[8 * i + 5]) * inv);
-                                v.w = pack_bf16(__uint_as_float(orr[8 * i + 6]) * inv, __uint_as_float(orr[8 * i + 7]) * inv);
-                                *reinterpret_cast<uint4*>(oo + c * 32 + i * 8) = v;
+                        for (int i = 0; i < 4; ++i)
+                            v[i] = make_uint4(pack_bf16(__uint_as_float(orr[8 * i + 0]) * inv, __uint_as_float(orr[8 * i + 1]) * inv),
+                                              pack_bf16(__uint_as_float(orr[8 * i + 2]) * inv, __uint_as_float(orr[8 * i + 3]) * inv),
+                                              pack_bf16(__uint_as_float(orr[8 * i + 4]) * inv, __uint_as_float(orr[8 * i + 5]) * inv),
+                                              pack_bf16(__uint_as_float(orr[8 * i + 6]) * inv, __uint_as_float(orr[8 * i + 7]) * inv));
+                        transpose4(v, lane);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int Ri = sg.row0 + t * kRowTile + (warp & 3) * 32 + (lane & ~3) + i;
+                            if (Ri < M) {
+                                const size_t row = (size_t)(sg.n0 + Ri / p.G) * p.Hq + sg.g * p.G + Ri % p.G;
+                                reinterpret_cast<uint4*>(p.out + ((size_t)sg.layer * p.sum_nodes * p.Hq + row) * kHeadDim + c * 32)[lane & 3] = v[i];
                             }
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 8; ++i)
-                                po[(c * 8 + i) * kRowsPerCta] =
-                                    make_float4(__uint_as_float(orr[4 * i]), __uint_as_float(orr[4 * i + 1]),
-                                                __uint_as_float(orr[4 * i + 2]), __uint_as_float(orr[4 * i + 3]));
                         }
+                    } else if (row_ok) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            po[(c * 8 + i) * kRowsPerCta] =
+                                make_float4(__uint_as_float(orr[4 * i]), __uint_as_float(orr[4 * i + 1]),
+                                            __uint_as_float(orr[4 * i + 2]), __uint_as_float(orr[4 * i + 3]));
                     }
                 }
             }
@@ -929,7 +976,6 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
 // two partial slots, follows from the positions alone.  One lane per row, 16 output columns per warp; the loads of four
 // segments are in flight together (one segment after the other took 20 us for one layer at 16k keys).
 __global__ void __launch_bounds__(256) attention_rows_merge_kernel(AttnParams p) {
-    after_previous_kernel();
     __shared__ Plan s_plan;
     __shared__ Place s_at;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -960,12 +1006,18 @@ __global__ void __launch_bounds__(256) attention_rows_merge_kernel(AttnParams p)
     if (g >= p.Hkv) return;
     const bool row_ok = R < it.N * p.G;
     if (!__any_sync(0xffffffffu, row_ok)) return;
+    // (up to here only inputs have been read, which were complete before the attention kernel let this one be brought up)
+    after_previous_kernel();
     auto slot_of = [&](int k) { return (size_t)(k * pl.n_rp + member) * 2 + (k == k_first && first_mid_range ? 1 : 0); };
     // (rows past the tree were not written: they are read all the same, as lanes of a warp with live rows, and dropped)
     float mx = -INFINITY;
-    for (int k = k_first; k <= k_last; ++k) {
-        const float2 ml = p.part_ml[slot_of(k) * kRowsPerCta + row];
-        if (row_ok && ml.y > 0.f) mx = fmaxf(mx, ml.x);
+    for (int k0 = k_first; k0 <= k_last; k0 += 8) {
+        float2 ml[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) ml[u] = p.part_ml[slot_of(min(k0 + u, k_last)) * kRowsPerCta + row];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (row_ok && ml[u].y > 0.f) mx = fmaxf(mx, ml[u].x);
     }
     float lsum = 0.f;
     float4 acc[4];
