@@ -1,7 +1,6 @@
 // Tree-masked verification attention over a paged bf16 KV cache (Section 2.2;
 // Algorithm 1, the target pass over all tree tokens; Section 3.3 Phase 2), sm_100a:
-// the streaming schedule for trees of more than 128 query rows per KV head.
-// tree_attention.cu holds the form for smaller trees, the dispatch and the C entry points.
+// the streaming schedule.  tree_attention.cu holds the dispatch and the C entry points.
 //
 // Work decomposition.  The N tree nodes x G query heads that share one KV head form
 // M = N*G query rows (<= 512).  An *item* is one (layer, sequence, KV head); its work
@@ -13,18 +12,23 @@
 // directly, items cut by a range boundary leave unnormalised partial results that
 // the merge kernel combines.  Nothing waits on another CTA.
 //
-// Inside a CTA (384 threads), per 128-key step and 128-row tile t:
-//   TMA      : K and V tiles (2 pages x 2 d-halves) -> 128B-swizzled shared memory, rings of
-//              3 K tiles and 2 V tiles, mbarriers; the two query tiles also arrive by TMA
-//   tcgen05  : S_t = Q_t K^T (128 x 128, fp32) into TMEM; one warp issues for both row tiles, through
-//              one elected lane, with warp-uniform descriptor arithmetic
-//   softmax  : one warpgroup per row tile, one thread per row: tcgen05.ld S in four 32-column
-//              chunks, online softmax in fp32 (log2 domain, lazy rescale), P -> bf16 back
-//              into TMEM over the first 64 columns of S_t
-//   tcgen05  : O_t += P_t V with P as the TMEM A operand, V MN-major from shared memory
-// The two row tiles alternate on the tensor pipe: while one tile's warpgroup runs its softmax,
-// the pipe works on the other tile.
-// TMEM map (512 columns): S_t [128t, 128t+128), O_t [256+128t, 384+128t).
+// Inside a CTA (384 threads): tensor memory holds two slots t of (S_t 128 x 128 fp32 scores,
+// O_t 128 x 128 fp32 accumulator): S_t in columns [128t, 128t+128), O_t in [256+128t, 384+128t).
+//   TMA      : K and V tiles of a step (2 pages x 2 d-halves) -> 128B-swizzled shared memory, rings of
+//              3 K tiles and 2 or 3 V tiles, mbarriers; the query tiles also arrive by TMA
+//   tcgen05  : S_t = Q K^T into TMEM, O_t += P_t V with P as the TMEM A operand (V MN-major); one warp
+//              issues for both slots, in blocks [P V of an earlier step, scores of a later one]
+//   softmax  : one warpgroup per slot, one thread per row: tcgen05.ld S in 32-column chunks,
+//              online softmax in fp32 (log2 domain, lazy rescale), P -> bf16 back into TMEM
+//              over the first 64 columns of S_t
+// The two slots alternate on the tensor pipe: while one's warpgroup runs its softmax, the pipe works on the
+// other.  What a slot is depends on the batch's largest tree, which the device works out:
+//   two tiles (more than 128 rows): slot = row tile; every step goes to both slots, K/V enters the SM once.
+//   alternating (up to 128 rows, kAlt): both slots belong to the same rows and take the even and the odd steps
+//     of a segment, each with its own accumulator and running (reference, sum); combined in the epilogue.
+//     (With one slot per row tile the chain scores -> softmax -> P V would be strictly serial.)
+// A 128 x 64 score MMA occupies the tensor pipe exactly as long as a 128 x 128 one (64 clocks
+// per K=16 slice, measured), hence the 128-key step.
 // All waits are bounded: on expiry the CTA records SAGE_STATUS_TIMEOUT, waits (bounded) for
 // its copies and MMAs in flight, frees its TMEM and returns.
 #include <cuda.h>
@@ -32,14 +36,22 @@
 #include "sage_common.cuh"
 
 namespace sage {
-namespace rows {
+namespace stream {
 
 constexpr int kRowTile = 128;                  // query rows per MMA tile
 constexpr int kRowsPerCta = 2 * kRowTile;
 constexpr int kStepKeys = 2 * kPageSize;       // keys per pipeline step
 constexpr int kKStages = 3;                    // K tiles in flight
-constexpr int kVStages = 2;                    // V tiles in flight
-constexpr int kRing = 4;                       // barrier pairs of the copy ring (ring steps in flight <= 2)
+constexpr int kRing = 4;                       // barrier pairs of the copy ring (> ring steps in flight)
+// Ring step i of a segment carries the K tile of its step i and the V tile of step i - kLag, which is what the MMA
+// warp consumes together.  Shared memory holds seven 32 KB tiles: two query tiles, 3 K and 2 V, or one, 3 and 3.
+template <bool kAlt>
+struct Mode {
+    static constexpr int kLag = kAlt ? 2 : 1;
+    static constexpr int kVStages = kAlt ? 3 : 2;
+    static constexpr int kDepth = kAlt ? 3 : 2;    // ring steps the copies run ahead of the MMAs
+    static constexpr int kQTiles = kAlt ? 1 : 2;
+};
 constexpr int kPageHalfBytes = kPageSize * 64 * 2;          // one TMA box: 64 keys x 64-wide d-half = 8 KB
 constexpr int kTileHalfBytes = kStepKeys * 64 * 2;          // one d-half of a 128-key tile: 16 KB
 constexpr int kTileBytes = 2 * kTileHalfBytes;              // K or V tile of one step: 32 KB
@@ -64,7 +76,6 @@ struct AttnParams {
     int n_layers, batch, sum_nodes, n_pages, max_pages;
     int Hq, Hkv, G;
     int n_ctas, n_rp;          // CTAs of the launch; most CTAs a gang can have (row pairs of the largest possible tree)
-    int select;                // which tree sizes this launch is for (schedule_selected)
     float scale_log2;          // sm_scale * log2(e)
     long long wait_cycles;     // budget of every on-device wait
     int producer_off;          // diagnostics: the TMA warp issues no copies (every consumer wait then runs out)
@@ -72,21 +83,23 @@ struct AttnParams {
 
 struct Place { int layer, u, b, s0; };     // layer, unit, sequence and step of a position in the launch's work
 struct __align__(16) Shared {
-    uint64_t kv_full[kRing];   // ring step r: the K tile of its step and the V tile of the step before have landed
+    uint64_t kv_full[kRing];   // ring step r: its K tile and its V tile have landed
     uint64_t kv_done[kRing];   // ring step r: every MMA that reads those tiles has finished
-    uint64_t s_full[2];        // [row tile]: scores of a step are in TMEM
-    uint64_t p_full[2];        // [row tile]: probabilities of a step are in TMEM
-    uint64_t o_full[2];        // [row tile]: every MMA of the segment has finished
+    uint64_t s_full[2];        // [slot]: scores of a step are in TMEM
+    uint64_t p_full[2];        // [slot]: probabilities of a step are in TMEM
+    uint64_t o_full[2];        // [slot]: every MMA of the slot's part of the segment has finished
+    uint64_t epi_done;         // alternating: the softmax warps have read both accumulators of the segment
     uint64_t q_free;           // the segment's last score MMAs have read the query tiles
     uint64_t q_ready;          // the query tiles of the segment are in shared memory
     uint64_t drain;            // abort path: everything issued so far has retired
+    volatile uint32_t eflag[2][4];     // alternating: [slot][quadrant] segment number whose (reference, sum) this warp has posted
     long long range_begin, range_end;
     Place first;               // where the range begins
-    int n_rp, heads_all;       // of the plan
+    int n_rp, heads_all, one_tile;     // of the plan
     uint32_t tmem_base;
     volatile int abort;
 };
-constexpr int kSmemBytes = 1024 /*align*/ + 2 * kQTileBytes + (kKStages + kVStages) * kTileBytes + (int)sizeof(Shared);
+constexpr int kSmemBytes = 1024 /*align*/ + 7 * kTileBytes + (int)sizeof(Shared);
 static_assert(kSmemBytes <= 232448, "shared memory budget of one CTA exceeded");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -207,6 +220,14 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
         ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
           "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
+}
+__device__ __forceinline__ void tmem_st2(uint32_t taddr, uint32_t a, uint32_t b) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(taddr), "r"(a), "r"(b) : "memory");
+}
+// two columns, waited for
+__device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t& a, uint32_t& b) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "r"(taddr) : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // The wait, tied to the registers that a load filled: what uses them stays behind it, other loads need not.
@@ -432,6 +453,7 @@ struct Plan {
     int heads_all;          // units that every sequence takes part in; the others are for trees of two row pairs only
     int steps_all, steps_big;   // steps of all sequences, and of those with two row pairs
     int n_act;              // gangs with work
+    int one_tile;           // no tree has more than one row tile
     long long steps_layer, W;   // steps of a layer, of the launch
 };
 // Called by a whole warp; the same answer in every CTA and in the merge kernel.
@@ -441,8 +463,7 @@ __device__ __forceinline__ Plan make_plan(const AttnParams& p, int lane, int* er
     for (int b0 = 0; b0 < p.batch; b0 += 32) {
         Item it{0, 0, 0, 0, 0};
         if (b0 + lane < p.batch) it = load_item(p, b0 + lane, err);
-        // (whatever its length is: the kernels of a launch agree on the largest tree)
-        if (it.N >= 1 && it.N <= SAGE_MAX_NODES && it.n0 >= 0 && it.n0 + it.N <= p.sum_nodes) mx = max(mx, it.N * p.G);
+        if (it.steps) mx = max(mx, it.N * p.G);
         all += it.steps;
         big += it.rp > 1 ? it.steps : 0;
     }
@@ -452,7 +473,8 @@ __device__ __forceinline__ Plan make_plan(const AttnParams& p, int lane, int* er
     pl.n_rp = mx > kRowsPerCta ? 2 : 1;
     pl.heads_all = pl.n_rp == 2 ? (p.Hkv + 1) / 2 : p.Hkv;
     pl.steps_layer = (long long)pl.heads_all * pl.steps_all + (long long)(p.Hkv - pl.heads_all) * pl.steps_big;
-    pl.W = schedule_selected(p.select, mx) ? pl.steps_layer * p.n_layers : 0;
+    pl.one_tile = mx <= kRowTile;
+    pl.W = pl.steps_layer * p.n_layers;
     const long long a = pl.W / kMinSteps;
     const int gangs = p.n_ctas / pl.n_rp;
     pl.n_act = a < 1 ? 1 : a < gangs ? (int)a : gangs;
@@ -566,17 +588,490 @@ struct SegIter {
     }
 };
 
+// =========================== TMA producer (one thread) ===========================
+template <bool kAlt>
+__device__ __forceinline__ void produce(const AttnParams& p, Shared* sh, uint8_t* smem, const CUtensorMap& qmap,
+                                        const CUtensorMap& kmap, const CUtensorMap& vmap) {
+    using C = Mode<kAlt>;
+    uint8_t* sQ = smem;
+    uint8_t* sK = sQ + C::kQTiles * kQTileBytes;
+    uint8_t* sV = sK + kKStages * kTileBytes;
+    SegIter it;
+    it.init(sh);
+    Seg sg;
+    int rc = 0, kslot = 0, vslot = 0, nq = 0;    // ring steps issued, slots of the next K and V tile, query loads issued
+    bool ok = !p.producer_off;
+    while (ok && it.next(p, sg)) {
+        const int n_rt = kAlt || sg.N * p.G - sg.row0 <= kRowTile ? 1 : 2;
+        const int32_t* pages = p.page_table + (size_t)sg.b * p.max_pages;
+        const int n_pages_seq = (sg.L + sg.N + kPageSize - 1) / kPageSize;
+        const int n = sg.s1 - sg.s0;
+        // the segment's query tiles, once the previous segment's score MMAs have read theirs
+        if (nq > 0 && !mbar_wait(&sh->q_free, (nq - 1) & 1, sh, p)) break;
+        mbar_expect_tx(&sh->q_ready, n_rt * kQTileBytes);
+        for (int t = 0; t < n_rt; ++t)
+            for (int h = 0; h < 2; ++h)
+                tma_load_5d(smem_u32(sQ + t * kQTileBytes + h * kQHalfBytes), &qmap, h * 64, 0, sg.g,
+                            sg.n0 + (sg.row0 + t * kRowTile) / p.G, sg.layer, &sh->q_ready);
+        ++nq;
+        int ids[C::kLag + 1][2] = {}, npg[C::kLag + 1] = {};       // pages of steps i, i - 1, ...
+        for (int i = 0; i < n + C::kLag; ++i) {
+            const int j = sg.s0 + i;
+#pragma unroll
+            for (int d = C::kLag; d > 0; --d) {
+                ids[d][0] = ids[d - 1][0]; ids[d][1] = ids[d - 1][1]; npg[d] = npg[d - 1];
+            }
+            // page ids of step j (checked: they become TMA coordinates)
+            npg[0] = 0;
+            if (i < n) {
+                npg[0] = (2 * j + 1 < n_pages_seq) ? 2 : 1;
+#pragma unroll
+                for (int pi = 0; pi < 2; ++pi) {
+                    if (pi < npg[0]) {
+                        ids[0][pi] = pages[2 * j + pi];
+                        if (ids[0][pi] < 0 || ids[0][pi] >= p.n_pages) {
+                            report_status(p.status, SAGE_STATUS_BAD_PAGE);
+                            ids[0][pi] = 0;
+                        }
+                    }
+                }
+            }
+            const int npv = i >= C::kLag ? npg[C::kLag] : 0;
+            // the tiles that ring step rc - kDepth used are free once its MMAs have finished
+            if (rc >= C::kDepth && !mbar_wait(&sh->kv_done[(rc - C::kDepth) % kRing], ((rc - C::kDepth) / kRing) & 1, sh, p)) { ok = false; break; }
+            uint64_t* full = &sh->kv_full[rc % kRing];
+            mbar_expect_tx(full, (npg[0] + npv) * 2 * kPageHalfBytes);
+            if (i < n) {
+#pragma unroll
+                for (int pi = 0; pi < 2; ++pi)
+                    if (pi < npg[0])
+                        for (int h = 0; h < 2; ++h)
+                            tma_load_4d(smem_u32(sK + kslot * kTileBytes + h * kTileHalfBytes + pi * kPageHalfBytes), &kmap, h * 64, 0,
+                                        ids[0][pi] * p.Hkv + sg.g, sg.layer, full);
+                kslot = kslot == kKStages - 1 ? 0 : kslot + 1;
+            }
+            if (i >= C::kLag) {
+#pragma unroll
+                for (int pi = 0; pi < 2; ++pi)
+                    if (pi < npv)
+                        for (int h = 0; h < 2; ++h)
+                            tma_load_4d(smem_u32(sV + vslot * kTileBytes + h * kTileHalfBytes + pi * kPageHalfBytes), &vmap, h * 64, 0,
+                                        ids[C::kLag][pi] * p.Hkv + sg.g, sg.layer, full);
+                vslot = vslot == C::kVStages - 1 ? 0 : vslot + 1;
+            }
+            ++rc;
+        }
+    }
+    if (sh->abort) {
+        // drain: every issued copy must land before the CTA may exit
+        for (int n = max(0, rc - C::kDepth); n < rc; ++n)
+            mbar_wait_quiet(&sh->kv_full[n % kRing], (n / kRing) & 1, p.wait_cycles);
+        if (nq > 0) mbar_wait_quiet(&sh->q_ready, (nq - 1) & 1, p.wait_cycles);
+    }
+}
+
+// Query rows past the tree (the box of a tile reaches into the next sequence's rows, or into spare capacity) become zero:
+// nothing reads their results, but the tensor cores draw less power on zeros, and long launches run at the power limit
+// (nine nodes in arrays of 64, 80 layers x 16k: KZERO us).  Called by the whole MMA warp.
+__device__ __forceinline__ void clear_query_rows(uint8_t* sQ, int rows, int n_rt, int lane) {
+    const int tile = n_rt - 1, live = rows - tile * kRowTile;       // of the last tile
+    if (live >= kRowTile) return;
+    uint8_t* q = sQ + tile * kQTileBytes;
+    for (int c = lane; c < (kRowTile - live) * 16; c += 32) {
+        const int r = live + c / 16, ch = c % 16;
+        *reinterpret_cast<uint4*>(q + (ch >> 3) * kQHalfBytes + r * 128 + ((ch & 7) << 4)) = make_uint4(0, 0, 0, 0);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");    // generic writes -> visible to the MMA unit
+    __syncwarp();
+}
+
+// =========================== MMA issuer (one warp) ===========================
+// One warp issues for both slots, in blocks [P V of step i - kLag, scores of step i] of a slot: a slot's block
+// runs on the tensor pipe while the other slot's warpgroup is in its softmax, and the blocks never interleave
+// (two issuers would finish both slots' scores at the same moment and leave the pipe idle during both
+// softmaxes).  The whole warp walks the loop and the elected lane is a predicate of each MMA (see mma_ss): 80
+// layers x 16k keys, 24 nodes: 1349 -> 1257 us.
+template <bool kAlt>
+__device__ __forceinline__ void issue(const AttnParams& p, Shared* sh, uint8_t* smem, uint32_t tmem, int lane) {
+    using C = Mode<kAlt>;
+    const uint32_t leader = elect_one() ? 1u : 0u;
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);      // (a broadcast: known to be the same in all lanes)
+    // descriptors differ only in their 14-bit start-address field (bytes >> 4); shared memory ends below 256 KB
+    const uint32_t dq = desc_lo(smem_u32(smem), 16);
+    const uint32_t dk = desc_lo(smem_u32(smem + C::kQTiles * kQTileBytes), 16);
+    const uint32_t dv = desc_lo(smem_u32(smem + C::kQTiles * kQTileBytes + kKStages * kTileBytes), kTileHalfBytes);
+    auto issue_qk = [&](int t, int slot) {
+        // S_t = Q_t K^T: 8 slices of K = 16 over d = 128 (4 per 64-wide half)
+        const uint32_t dqt = kAlt ? dq : dq + ((t * kQTileBytes) >> 4);
+        const uint32_t dks = dk + ((slot * kTileBytes) >> 4);
+        const uint32_t s_tmem = tm + t * 128;
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks)
+            mma_ss<kDescHi, kIdescQK>(leader, s_tmem, dqt + (((ks >> 2) * kQHalfBytes + (ks & 3) * 32) >> 4),
+                                      dks + (((ks >> 2) * kTileHalfBytes + (ks & 3) * 32) >> 4), ks > 0 ? 1u : 0u);
+    };
+    auto issue_pv = [&](int t, int slot, bool first) {
+        // O_t += P_t V: 8 slices of K = 16 keys; P in TMEM (8 columns per slice), V MN-major
+        const uint32_t dvs = dv + ((slot * kTileBytes) >> 4);
+        const uint32_t s_tmem = tm + t * 128, o_tmem = tm + 256 + t * 128;
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks)
+            mma_ts<kDescHi, kIdescPV>(leader, o_tmem, s_tmem + ks * 8, dvs + ((ks * 2048) >> 4), (first && ks == 0) ? 0u : 1u);
+    };
+    SegIter it;
+    it.init(sh);
+    Seg sg;
+    int rc = 0, kslot = 0, vslot = 0, nseg = 0;     // ring steps consumed, slots of the next K and V tile; segments started
+    int np[2] = {0, 0};                             // steps of each slot whose probabilities were consumed
+    bool ok = true;
+    // The loop holds as few synchronisation instructions as the protocol allows: one wait and one commit
+    // per ring step for the tiles, one of each per slot.
+    while (ok && it.next(p, sg)) {
+        const int rows = __shfl_sync(0xffffffffu, sg.N * p.G - sg.row0, 0);
+        const int n = __shfl_sync(0xffffffffu, sg.s1 - sg.s0, 0);
+        const int n_rt = kAlt || rows <= kRowTile ? 1 : 2;
+        ok = mbar_wait_warp(&sh->q_ready, nseg & 1, sh, p);
+        if (ok) clear_query_rows(smem, rows, n_rt, lane);
+        for (int i = 0; ok && i < n + C::kLag; ++i) {
+            ok = mbar_wait_warp(&sh->kv_full[rc % kRing], (rc / kRing) & 1, sh, p);
+            if (!ok) break;
+#pragma unroll
+            for (int tt = 0; tt < (kAlt ? 1 : 2); ++tt) {
+                const int t = kAlt ? i & 1 : tt;
+                if (tt < n_rt) {
+                    if (i >= C::kLag) {
+                        // (the warpgroup zeroed the V rows past the end of the sequence before it arrived)
+                        ok = mbar_wait_warp(&sh->p_full[t], np[t] & 1, sh, p);
+                        if (!ok) break;
+                        ++np[t];
+                        // the segment's first P V products overwrite both accumulators, which the softmax warps
+                        // read in the epilogue of the segment before
+                        if (kAlt && i == C::kLag && nseg > 0) {
+                            ok = mbar_wait_warp(&sh->epi_done, (nseg - 1) & 1, sh, p);
+                            if (!ok) break;
+                        }
+                        tc_fence_after();
+                        issue_pv(t, vslot, i < 2 * C::kLag);
+                        if (i >= n + C::kLag - (kAlt ? 2 : 1)) tc_commit(leader, &sh->o_full[t]);   // the slot's last step of the segment
+                    }
+                    if (i < n) {
+                        issue_qk(t, kslot);
+                        tc_commit(leader, &sh->s_full[t]);
+                    }
+                }
+            }
+            if (!ok) break;
+            tc_commit(leader, &sh->kv_done[rc % kRing]);
+            ++rc;
+            if (i < n) kslot = (kslot == kKStages - 1) ? 0 : kslot + 1;
+            if (i >= C::kLag) vslot = (vslot == C::kVStages - 1) ? 0 : vslot + 1;
+            if (i == n - 1) tc_commit(leader, &sh->q_free);             // the segment's last score MMAs read the query tiles
+        }
+        ++nseg;
+    }
+    if (!ok) {
+        // abort: everything this warp has issued must retire before the TMEM and the tiles go away
+        tc_commit(leader, &sh->drain);
+        mbar_wait_quiet(&sh->drain, 0, p.wait_cycles);
+    }
+    __syncwarp();
+}
+
+// =========================== softmax ===========================
+// One step of one query row per thread: scores of S_t -> probabilities (bf16, over the first 64 columns of S_t), running
+// reference and sum.  first: nothing has been accumulated yet; masked: the step reaches into the tree part (or past the end).
+__device__ __forceinline__ void softmax_step(uint32_t s_taddr, uint32_t o_taddr, float scale, bool first, bool masked, int pos0,
+                                             int L, int N, uint64_t anc, float& m_ref, float& l_sum) {
+    uint32_t sr[128];
+    // Probabilities are taken against the row's reference of the steps before: any reference within some 2^60
+    // of the row's maximum gives the same result, so a step need not look for its maximum first.  It shows in
+    // the step's sum whether the reference still serves; the first step of a segment, steps with masked
+    // scores and steps whose sum has grown beyond 2^30 go through the maximum.
+    bool by_max = masked || first;
+    if (!by_max) {
+        uint64_t acc[2] = {0ull, 0ull};
+        tmem_ld32(s_taddr, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            tmem_wait_ld_of(*reinterpret_cast<uint32_t(*)[32]>(&sr[32 * c]));
+            if (c < 3) tmem_ld32(s_taddr + 32 * (c + 1), *reinterpret_cast<uint32_t(*)[32]>(&sr[32 * (c + 1)]));
+            exp_chunk<SAGE_EXP2_FMA_PAIRS>(sr + 32 * c, scale, -m_ref, sr + 16 * c, acc);
+        }
+        float sum_a, sum_b;
+        f2_unpack(f2_add(acc[0], acc[1]), sum_a, sum_b);
+        const float sum = sum_a + sum_b;
+        by_max = __any_sync(0xffffffffu, !(sum < kMaxSum));
+        if (!by_max) l_sum += sum;
+    }
+    if (by_max) {
+        load_scores(s_taddr, sr);
+        if (masked) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) mask_chunk(sr + 32 * c, pos0 + 32 * c, L, N, anc);
+        }
+        float mx = -INFINITY;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) max_chunk(sr + 32 * c, mx);
+        // the reference moves only when the row max grew by more than 2^8 over it
+        const float m_cand = mx * scale;
+        const bool grow = m_cand > m_ref + 8.0f;
+        float alpha = 1.0f;
+        if (grow) {
+            alpha = fast_exp2(m_ref - m_cand);              // 0 when m_ref was -inf
+            m_ref = m_cand;
+        }
+        // O_t *= alpha.  The P V product of the step before has finished: the scores of this step were
+        // issued after it, and their completion is what this warp waited for above.
+        if (!first && __any_sync(0xffffffffu, grow)) rescale_o_rows(o_taddr, alpha);
+        const float neg_ref = (m_ref == -INFINITY) ? 0.f : -m_ref;
+        uint64_t acc[2] = {0ull, 0ull};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) exp_chunk<0>(sr + 32 * c, scale, neg_ref, sr + 16 * c, acc);   // may hold -inf
+        float sum_a, sum_b;
+        f2_unpack(f2_add(acc[0], acc[1]), sum_a, sum_b);
+        l_sum = l_sum * alpha + (sum_a + sum_b);
+    }
+    // (chunk c of 32 scores has left its 16 words of bf16 pairs at sr[16c ..])
+    uint32_t* pk = sr;
+    tmem_st32(s_taddr, pk);                 // P over the first 64 columns of S_t
+    tmem_st32(s_taddr + 32, pk + 32);
+    tmem_wait_st();
+    tc_fence_before();
+}
+
+// Four lanes exchange the 64 bytes of output that each has of its row, so that a store instruction writes 64 contiguous
+// bytes of eight rows instead of 16 bytes of 32.  v: 32 columns of the row as bf16; col: the first one; row0: row of lane 0.
+__device__ __forceinline__ void store_rows(const AttnParams& p, const Seg& sg, uint4 (&v)[4], int row0, int M, int col, int lane) {
+    transpose4(v, lane);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int R = row0 + (lane & ~3) + i;
+        if (R < M) {
+            const size_t row = (size_t)(sg.n0 + R / p.G) * p.Hq + sg.g * p.G + R % p.G;
+            reinterpret_cast<uint4*>(p.out + ((size_t)sg.layer * p.sum_nodes * p.Hq + row) * kHeadDim + col)[lane & 3] = v[i];
+        }
+    }
+}
+__device__ __forceinline__ void pack_rows(const uint32_t (&o)[32], float f, uint4 (&v)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        v[i] = make_uint4(pack_bf16(__uint_as_float(o[8 * i + 0]) * f, __uint_as_float(o[8 * i + 1]) * f),
+                          pack_bf16(__uint_as_float(o[8 * i + 2]) * f, __uint_as_float(o[8 * i + 3]) * f),
+                          pack_bf16(__uint_as_float(o[8 * i + 4]) * f, __uint_as_float(o[8 * i + 5]) * f),
+                          pack_bf16(__uint_as_float(o[8 * i + 6]) * f, __uint_as_float(o[8 * i + 7]) * f));
+}
+// 32 columns of a partial result; po: the thread's place in the first column quad.
+__device__ __forceinline__ void store_partial(float4* po, const uint32_t (&o)[32]) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        po[i * kRowsPerCta] = make_float4(__uint_as_float(o[4 * i]), __uint_as_float(o[4 * i + 1]), __uint_as_float(o[4 * i + 2]),
+                                          __uint_as_float(o[4 * i + 3]));
+}
+
+// Two tiles: O_t / l -> bf16 output, or unnormalised partials for the merge.
+__device__ __forceinline__ void finish_tile(const AttnParams& p, const Seg& sg, uint32_t o_taddr, int t, int r, int lane, float m_ref,
+                                            float l_sum) {
+    const int M = sg.N * p.G, R = sg.row0 + t * kRowTile + r;
+    const bool whole = (sg.s0 == 0 && sg.s1 == sg.steps);
+    const float inv = (l_sum > 0.f) ? 1.0f / l_sum : 0.f;
+    const size_t slot = (size_t)blockIdx.x * 2 + (sg.at_range_begin ? 0 : 1);
+    float4* po = p.part_o + slot * (kHeadDim / 4) * kRowsPerCta + t * kRowTile + r;
+    if (!whole && R < M) p.part_ml[slot * kRowsPerCta + t * kRowTile + r] = make_float2(m_ref, l_sum);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        uint32_t o[32];
+        tmem_ld32(o_taddr + c * 32, o);
+        tmem_wait_ld();
+        if (whole) {
+            uint4 v[4];
+            pack_rows(o, inv, v);
+            store_rows(p, sg, v, R - lane, M, c * 32, lane);
+        } else if (R < M) {
+            store_partial(po + c * 8 * kRowsPerCta, o);
+        }
+    }
+}
+
+// Alternating: the two slots combined, this warpgroup taking the output columns [64t, 64t + 64) of both accumulators.
+// Returns false when the CTA is aborting.
+__device__ __forceinline__ bool finish_slots(const AttnParams& p, Shared* sh, const Seg& sg, uint32_t tmem, uint32_t lane_base, int t, int q,
+                                             int r, int lane, bool has1, uint32_t eseq, float m_ref, float l_sum) {
+    const int M = sg.N * p.G;
+    // 64 columns of both accumulators, 32 at a time
+    const uint32_t o0 = tmem + lane_base + 256 + 64 * t, o1 = o0 + 128;
+    uint32_t oa[32], ob[32];
+    tmem_ld32(o0, oa);
+    if (has1) tmem_ld32(o1, ob);
+    tmem_wait_ld();
+    // The row's (reference, sum) of this slot goes to the other warpgroup through two columns of O_t
+    // that this thread has just read and nobody else reads: columns 64t and 64t + 1.
+    tmem_st2(tmem + lane_base + 256 + 128 * t + 64 * t, __float_as_uint(m_ref), __float_as_uint(l_sum));
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) {
+        __threadfence_block();
+        sh->eflag[t][q] = eseq;
+    }
+    // bounded wait for the partner warp (same rows, other slot)
+    volatile uint32_t* flag = &sh->eflag[1 - t][q];
+    bool seen = (*flag == eseq);
+    if (!seen) {
+        const long long t0 = clock64();
+        while (true) {
+            for (int k = 0; k < 64 && !seen; ++k) seen = (*flag == eseq);
+            if (seen || sh->abort) break;
+            if (clock64() - t0 > p.wait_cycles) {
+                sh->abort = 1;
+                report_status(p.status, SAGE_STATUS_TIMEOUT);
+                break;
+            }
+        }
+    }
+    if (!__all_sync(0xffffffffu, seen)) return false;
+    tc_fence_after();
+    uint32_t pm, pl;
+    tmem_ld2(tmem + lane_base + 256 + (1 - t) * 128 + 64 * (1 - t), pm, pl);
+    const float m_o = __uint_as_float(pm), l_o = __uint_as_float(pl);
+    // weights of the two slots under the common reference (a slot without visible keys has l = 0)
+    const float m_all = fmaxf(l_sum > 0.f ? m_ref : -INFINITY, l_o > 0.f ? m_o : -INFINITY);
+    const float w_me = l_sum > 0.f ? fast_exp2(m_ref - m_all) : 0.f;
+    const float w_ot = l_o > 0.f ? fast_exp2(m_o - m_all) : 0.f;
+    const float l_all = l_sum * w_me + l_o * w_ot;
+    const bool whole = (sg.s0 == 0 && sg.s1 == sg.steps);
+    // factors of O_0 and O_1: the slot weights, and 1 / l for a finished row
+    const float inv = whole ? ((l_all > 0.f) ? 1.0f / l_all : 0.f) : 1.0f;
+    const float f0 = (t == 0 ? w_me : w_ot) * inv, f1 = has1 ? (t == 0 ? w_ot : w_me) * inv : 0.f;
+    const size_t slot = (size_t)blockIdx.x * 2 + (sg.at_range_begin ? 0 : 1);
+    float4* po = p.part_o + (slot * (kHeadDim / 4) + 16 * t) * kRowsPerCta + r;
+    if (!whole && t == 0 && r < M) p.part_ml[slot * kRowsPerCta + r] = make_float2(m_all, l_all);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        if (c == 1) {
+            tmem_ld32(o0 + 32, oa);
+            if (has1) tmem_ld32(o1 + 32, ob);
+            tmem_wait_ld();
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            float v = __uint_as_float(oa[i]) * f0;
+            if (has1) v = fmaf(__uint_as_float(ob[i]), f1, v);
+            oa[i] = __float_as_uint(v);
+        }
+        if (whole) {
+            uint4 v[4];
+            pack_rows(oa, 1.0f, v);
+            store_rows(p, sg, v, r - lane, M, 64 * t + c * 32, lane);
+        } else if (r < M) {
+            store_partial(po + c * 8 * kRowsPerCta, oa);
+        }
+    }
+    return true;
+}
+
+// Warpgroup t owns slot t; one thread per query row.
+template <bool kAlt>
+__device__ __forceinline__ void softmax(const AttnParams& p, Shared* sh, uint8_t* smem, uint32_t tmem, int t, int q, int r, int lane) {
+    using C = Mode<kAlt>;
+    uint8_t* sV = smem + C::kQTiles * kQTileBytes + kKStages * kTileBytes;
+    const uint32_t lane_base = (uint32_t)(q * 32) << 16;            // r: row inside the tile == TMEM lane, q: its quadrant
+    const uint32_t s_taddr = tmem + lane_base + t * 128;
+    const uint32_t o_taddr = tmem + lane_base + 256 + t * 128;
+    SegIter it;
+    it.init(sh);
+    Seg sg;
+    int nsteps = 0, nseg = 0, nseg1 = 0;            // steps this slot has been through; segments; those with work for the slot (for slot 1, alternating)
+    int rc0 = 0, vc0 = 0;                           // ring steps / V tiles of the CTA before the current segment
+    bool ok = true;
+    while (ok && it.next(p, sg)) {
+        const int M = sg.N * p.G, n = sg.s1 - sg.s0;
+        const int rc_seg = rc0, vc_seg = vc0;       // this segment's first ring step / V tile
+        rc0 += n + C::kLag;
+        vc0 += n;
+        const int first_row = kAlt ? 0 : sg.row0 + t * kRowTile;
+        if (!kAlt && t == 1 && M <= first_row) continue;
+        const bool row_ok = first_row + r < M;
+        const int node = row_ok ? (first_row + r) / p.G : 0;
+        const bool warp_live = first_row + q * 32 < M;
+        uint64_t anc = 0;
+        if (sg.s1 * kStepKeys > sg.L && row_ok) {
+            // the segment reaches the tree part: this row's ancestor bitset (the G rows of a node
+            // walk the same parent chain, at most N - 1 cached loads deep)
+            bool bad = false;
+            anc = ancestor_bits(p.parent + sg.n0, sg.N, node, &bad);
+            if (bad) { report_status(p.status, SAGE_STATUS_BAD_TREE); anc = 1ull << node; }
+        }
+        float m_ref = -INFINITY, l_sum = 0.f;
+        for (int i = kAlt ? t : 0; i < n; i += kAlt ? 2 : 1) {
+            const int j = sg.s0 + i;
+            ok = mbar_wait(&sh->s_full[t], nsteps & 1, sh, p);
+            if (!ok) break;
+            ++nsteps;
+            const int valid = sg.L + sg.N - j * kStepKeys;      // keys of this step that exist
+            if (valid < kStepKeys) {
+                // V rows past the end of the sequence may hold anything (a missing second page was not even
+                // copied): zero them so that 0 * V stays 0.  Each warp of the warpgroup takes a quarter of
+                // the rows (two tiles: both warpgroups write the same zeros); the writes are ordered before this
+                // warp's arrival, which the P V product waits for.  The V tile of step s0 + i lands with ring
+                // step i + kLag of the segment.
+                const int rcv = rc_seg + i + C::kLag;
+                ok = mbar_wait(&sh->kv_full[rcv % kRing], (rcv / kRing) & 1, sh, p);
+                if (!ok) break;
+                uint8_t* vb = sV + ((vc_seg + i) % C::kVStages) * kTileBytes;
+                for (int c = q * 32 + lane; c < (kStepKeys - valid) * 16; c += 128) {
+                    const int vr = valid + c / 16, ch = c % 16;
+                    *reinterpret_cast<uint4*>(vb + (ch >> 3) * kTileHalfBytes + vr * 128 + ((ch & 7) << 4)) = make_uint4(0, 0, 0, 0);
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            }
+            // (a warp none of whose 32 rows exists keeps the barrier protocol going and leaves the scores of these
+            // rows, which are zero, as they are; their outputs are never stored)
+            if (warp_live) {
+                tc_fence_after();
+                const int pos0 = j * kStepKeys;
+                softmax_step(s_taddr, o_taddr, p.scale_log2, i < (kAlt ? 2 : 1), pos0 + kStepKeys > sg.L, pos0, sg.L, sg.N, anc, m_ref, l_sum);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh->p_full[t]);
+        }
+        if (!ok) break;
+        if (kAlt) {
+            const bool has1 = n >= 2;               // slot 1 took part in this segment
+            ok = mbar_wait(&sh->o_full[0], nseg & 1, sh, p);
+            if (ok && has1) ok = mbar_wait(&sh->o_full[1], nseg1 & 1, sh, p);
+            ++nseg;
+            if (has1) ++nseg1;
+            if (!ok) break;
+            if (warp_live) {
+                tc_fence_after();
+                ok = finish_slots(p, sh, sg, tmem, lane_base, t, q, r, lane, has1, (uint32_t)nseg, m_ref, l_sum);
+                if (!ok) break;
+            }
+            tc_fence_before();                      // the next segment's first P V products overwrite O_0 and O_1
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh->epi_done);
+        } else {
+            ok = mbar_wait(&sh->o_full[t], nseg & 1, sh, p);
+            ++nseg;
+            if (!ok) break;
+            if (warp_live) {
+                tc_fence_after();
+                finish_tile(p, sg, o_taddr, t, r, lane, m_ref, l_sum);
+            }
+            tc_fence_before();                      // the next segment's first P V overwrites O_t
+        }
+    }
+}
+
 __global__ void __launch_bounds__(kAttnThreads, 1)
-tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorMap qmap,
+tree_attention_stream_kernel(const AttnParams p, const __grid_constant__ CUtensorMap qmap,
                       const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap) {
     after_previous_kernel();
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte alignment: the 128B swizzle pattern repeats every 1024 bytes of address
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* sQ = smem;                                 // [2 tiles][2 d-halves][128 rows][128 B]
-    uint8_t* sK = sQ + 2 * kQTileBytes;                 // [kKStages][2 d-halves][128 keys][128 B]
-    uint8_t* sV = sK + kKStages * kTileBytes;           // [kVStages][2 d-halves][128 keys][128 B]
-    Shared* sh = reinterpret_cast<Shared*>(sV + kVStages * kTileBytes);
+    // query tiles [2 d-halves][128 rows][128 B], K ring and V ring [2 d-halves][128 keys][128 B] each (see Mode)
+    Shared* sh = reinterpret_cast<Shared*>(smem + 7 * kTileBytes);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
@@ -597,7 +1092,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
         if (lane == 0) {
             sh->range_begin = begin; sh->range_end = end;
             sh->first = at;
-            sh->n_rp = pl.n_rp; sh->heads_all = pl.heads_all;
+            sh->n_rp = pl.n_rp; sh->heads_all = pl.heads_all; sh->one_tile = pl.one_tile;
         }
     } else if (warp == 8) {
         if (lane == 0) {
@@ -610,6 +1105,8 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                 mbar_init(&sh->p_full[t], 4);               // one arrival per softmax warp
                 mbar_init(&sh->o_full[t], 1);
             }
+            mbar_init(&sh->epi_done, 8);                    // one arrival per softmax warp
+            for (int i = 0; i < 8; ++i) (&sh->eflag[0][0])[i] = 0;
             mbar_init(&sh->q_free, 1);
             mbar_init(&sh->drain, 1);
             mbar_init(&sh->q_ready, 1);
@@ -632,333 +1129,22 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
 
     // Registers move from the copy / MMA warpgroup (which needs few) to the softmax warpgroups:
     // 4 warps give up 168 - 72 registers per thread, 8 warps take 216 - 168 each.
+    const bool alt = sh->one_tile;
     if (warp >= 8) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
-    if (warp == 8) {
-        // =========================== TMA producer ===========================
-        if (lane == 0) {
-            SegIter it;
-            it.init(sh);
-            Seg sg;
-            // A segment of n steps takes n + 1 ring steps: ring step i carries the K tile of step s0 + i
-            // (i < n) and the V tile of step s0 + i - 1 (i > 0), which is what the MMA warp consumes together
-            // ([P V of the step before, scores of this step]); both land on one barrier.
-            int rc = 0, kc = 0, vc = 0, nq = 0;          // ring steps, K tiles, V tiles, query loads issued so far
-            bool ok = !p.producer_off;
-            while (ok && it.next(p, sg)) {
-                const int M = sg.N * p.G;
-                const int n_rt = (M - sg.row0 > kRowTile) ? 2 : 1;
-                const int32_t* pages = p.page_table + (size_t)sg.b * p.max_pages;
-                const int n_pages_seq = (sg.L + sg.N + kPageSize - 1) / kPageSize;
-                const int n = sg.s1 - sg.s0;
-                // the segment's query tiles, once the previous segment's score MMAs have read theirs
-                if (nq > 0 && !mbar_wait(&sh->q_free, (nq - 1) & 1, sh, p)) break;
-                mbar_expect_tx(&sh->q_ready, n_rt * kQTileBytes);
-                for (int t = 0; t < n_rt; ++t)
-                    for (int h = 0; h < 2; ++h)
-                        tma_load_5d(smem_u32(sQ + t * kQTileBytes + h * kQHalfBytes), &qmap, h * 64, 0, sg.g,
-                                    sg.n0 + (sg.row0 + t * kRowTile) / p.G, sg.layer, &sh->q_ready);
-                ++nq;
-                int ids_prev[2] = {0, 0}, npg_prev = 0;
-                for (int i = 0; i <= n; ++i) {
-                    const int j = sg.s0 + i;
-                    // page ids of step j (checked: they become TMA coordinates)
-                    int ids[2] = {0, 0}, npg = 0;
-                    if (i < n) {
-                        npg = (2 * j + 1 < n_pages_seq) ? 2 : 1;
-                        for (int pi = 0; pi < npg; ++pi) {
-                            ids[pi] = pages[2 * j + pi];
-                            if (ids[pi] < 0 || ids[pi] >= p.n_pages) {
-                                report_status(p.status, SAGE_STATUS_BAD_PAGE);
-                                ids[pi] = 0;
-                            }
-                        }
-                    }
-                    // the tiles that ring step rc - 2 used are free once its MMAs have finished
-                    if (rc >= 2 && !mbar_wait(&sh->kv_done[(rc - 2) % kRing], ((rc - 2) / kRing) & 1, sh, p)) { ok = false; break; }
-                    uint64_t* full = &sh->kv_full[rc % kRing];
-                    mbar_expect_tx(full, (npg + (i > 0 ? npg_prev : 0)) * 2 * kPageHalfBytes);
-                    if (i < n) {
-                        const int kslot = kc % kKStages;
-                        for (int pi = 0; pi < npg; ++pi)
-                            for (int h = 0; h < 2; ++h)
-                                tma_load_4d(smem_u32(sK + kslot * kTileBytes + h * kTileHalfBytes + pi * kPageHalfBytes), &kmap,
-                                            h * 64, 0, ids[pi] * p.Hkv + sg.g, sg.layer, full);
-                        ++kc;
-                    }
-                    if (i > 0) {
-                        const int vslot = vc % kVStages;
-                        for (int pi = 0; pi < npg_prev; ++pi)
-                            for (int h = 0; h < 2; ++h)
-                                tma_load_4d(smem_u32(sV + vslot * kTileBytes + h * kTileHalfBytes + pi * kPageHalfBytes), &vmap,
-                                            h * 64, 0, ids_prev[pi] * p.Hkv + sg.g, sg.layer, full);
-                        ++vc;
-                    }
-                    ++rc;
-                    ids_prev[0] = ids[0]; ids_prev[1] = ids[1]; npg_prev = npg;
-                }
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        if (warp == 8) {
+            if (lane == 0) {
+                if (alt) produce<true>(p, sh, smem, qmap, kmap, vmap);
+                else produce<false>(p, sh, smem, qmap, kmap, vmap);
             }
-            if (sh->abort) {
-                // drain: every issued copy must land before the CTA may exit
-                for (int n = max(0, rc - 2); n < rc; ++n)
-                    mbar_wait_quiet(&sh->kv_full[n % kRing], (n / kRing) & 1, p.wait_cycles);
-                if (nq > 0) mbar_wait_quiet(&sh->q_ready, (nq - 1) & 1, p.wait_cycles);
-            }
+        } else if (warp == 9) {
+            if (alt) issue<true>(p, sh, smem, tmem, lane);
+            else issue<false>(p, sh, smem, tmem, lane);
         }
-    } else if (warp == 9) {
-        // =========================== MMA issuer ===========================
-        // One warp issues for both row tiles, in blocks [P V of step j-1, scores of step j] per tile:
-        // a tile's block runs on the tensor pipe while the other tile's warpgroup is in its softmax, and
-        // the blocks of the two tiles never interleave (two issuers would finish both tiles' scores at
-        // the same moment and leave the pipe idle during both softmaxes).  The whole warp walks the loop and
-        // the elected lane is a predicate of each MMA (see mma_ss): 80 layers x 16k keys, 24 nodes: 1349 -> 1257 us.
-        const uint32_t leader = elect_one() ? 1u : 0u;
-        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);      // (a broadcast: known to be the same in all lanes)
-        // descriptors differ only in their 14-bit start-address field (bytes >> 4); shared memory ends below 256 KB
-        const uint32_t dq = desc_lo(smem_u32(sQ), 16);
-        const uint32_t dk = desc_lo(smem_u32(sK), 16);
-        const uint32_t dv = desc_lo(smem_u32(sV), kTileHalfBytes);
-        auto issue_qk = [&](int t, int slot) {
-            // S_t = Q_t K^T: 8 slices of K = 16 over d = 128 (4 per 64-wide half)
-            const uint32_t dqt = dq + ((t * kQTileBytes) >> 4);
-            const uint32_t dks = dk + ((slot * kTileBytes) >> 4);
-            const uint32_t s_tmem = tm + t * 128;
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks)
-                mma_ss<kDescHi, kIdescQK>(leader, s_tmem, dqt + (((ks >> 2) * kQHalfBytes + (ks & 3) * 32) >> 4),
-                                          dks + (((ks >> 2) * kTileHalfBytes + (ks & 3) * 32) >> 4), ks > 0 ? 1u : 0u);
-        };
-        auto issue_pv = [&](int t, int slot, bool first) {
-            // O_t += P_t V: 8 slices of K = 16 keys; P in TMEM (8 columns per slice), V MN-major
-            const uint32_t dvs = dv + ((slot * kTileBytes) >> 4);
-            const uint32_t s_tmem = tm + t * 128, o_tmem = tm + 256 + t * 128;
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks)
-                mma_ts<kDescHi, kIdescPV>(leader, o_tmem, s_tmem + ks * 8, dvs + ((ks * 2048) >> 4), (first && ks == 0) ? 0u : 1u);
-        };
-        SegIter it;
-        it.init(sh);
-        Seg sg;
-        int rc = 0, kslot = 0, vslot = 0, nq = 0;       // ring steps consumed, slots of the next K and V tile; segments started
-        int np[2] = {0, 0};                             // steps of each row tile whose probabilities were consumed
-        bool ok = true;
-        // The loop holds as few synchronisation instructions as the protocol allows: one wait and one commit
-        // per ring step for the tiles, one of each per row tile.
-        while (ok && it.next(p, sg)) {
-            const int n_rt = __shfl_sync(0xffffffffu, (sg.N * p.G - sg.row0 > kRowTile) ? 2 : 1, 0);
-            const int n = __shfl_sync(0xffffffffu, sg.s1 - sg.s0, 0);
-            ok = mbar_wait_warp(&sh->q_ready, nq & 1, sh, p);
-            ++nq;
-            // ring step i: the P V products of step i - 1 (when i > 0) and the scores of step i (when i < n)
-            for (int i = 0; ok && i <= n; ++i) {
-                ok = mbar_wait_warp(&sh->kv_full[rc % kRing], (rc / kRing) & 1, sh, p);
-                if (!ok) break;
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    if (t < n_rt) {
-                        if (i > 0) {
-                            // (the warpgroup zeroed the V rows past the end of the sequence before it arrived)
-                            ok = mbar_wait_warp(&sh->p_full[t], np[t] & 1, sh, p);
-                            if (!ok) break;
-                            ++np[t];
-                            tc_fence_after();
-                            issue_pv(t, vslot, i == 1);
-                            if (i == n) tc_commit(leader, &sh->o_full[t]);  // every MMA of this tile's segment has been issued
-                        }
-                        if (i < n) {
-                            issue_qk(t, kslot);
-                            tc_commit(leader, &sh->s_full[t]);
-                        }
-                    }
-                }
-                if (!ok) break;
-                tc_commit(leader, &sh->kv_done[rc % kRing]);
-                ++rc;
-                if (i < n) kslot = (kslot == kKStages - 1) ? 0 : kslot + 1;
-                if (i > 0) vslot = (vslot == kVStages - 1) ? 0 : vslot + 1;
-                if (i == n - 1) tc_commit(leader, &sh->q_free);             // the segment's last score MMAs read the query tiles
-            }
-        }
-        if (!ok) {
-            // abort: everything this warp has issued must retire before the TMEM and the tiles go away
-            tc_commit(leader, &sh->drain);
-            mbar_wait_quiet(&sh->drain, 0, p.wait_cycles);
-        }
-        __syncwarp();
-    }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
-        // =========================== softmax warpgroups ===========================
-        const int t = warp >> 2;                        // row tile of this warpgroup
-        const int r = tid & 127;                        // row inside the tile == TMEM lane
-        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t s_taddr = tmem + lane_base + t * 128;
-        const uint32_t o_taddr = tmem + lane_base + 256 + t * 128;
-        SegIter it;
-        it.init(sh);
-        Seg sg;
-        int nsteps = 0, nseg = 0;                       // steps / segments this row tile has been through
-        int rc0 = 0, vc0 = 0;                           // ring steps / V tiles of the CTA before the current segment
-        bool ok = true;
-        while (ok && it.next(p, sg)) {
-            const int M = sg.N * p.G;
-            const int rc_seg = rc0, vc_seg = vc0;       // this segment's first ring step / V tile
-            rc0 += sg.s1 - sg.s0 + 1;
-            vc0 += sg.s1 - sg.s0;
-            if (t == 1 && M - sg.row0 <= kRowTile) continue;
-            const int R = sg.row0 + t * kRowTile + r;
-            const bool row_ok = R < M;
-            const int node = row_ok ? R / p.G : 0;
-            const bool warp_live = sg.row0 + t * kRowTile + (warp & 3) * 32 < M;
-            uint64_t anc = 0;
-            if (sg.s1 * kStepKeys > sg.L && row_ok) {
-                // the segment reaches the tree part: this row's ancestor bitset (the G rows of a node
-                // walk the same parent chain, at most N - 1 cached loads deep)
-                bool bad = false;
-                anc = ancestor_bits(p.parent + sg.n0, sg.N, node, &bad);
-                if (bad) { report_status(p.status, SAGE_STATUS_BAD_TREE); anc = 1ull << node; }
-            }
-            float m_ref = -INFINITY, l_sum = 0.f;
-            for (int j = sg.s0; j < sg.s1; ++j) {
-                ok = mbar_wait(&sh->s_full[t], nsteps & 1, sh, p);
-                if (!ok) break;
-                const int valid = sg.L + sg.N - j * kStepKeys;      // keys of this step that exist
-                if (valid < kStepKeys) {
-                    // V rows past the end of the sequence may hold anything (a missing second page was not even
-                    // copied): zero them so that 0 * V stays 0.  Each warp of the warpgroup takes a quarter of
-                    // the rows (both warpgroups write the same zeros); the writes are ordered before this
-                    // warp's arrival, which the P V product waits for.  The V tile of step j lands with ring
-                    // step j - s0 + 1 of the segment.
-                    const int rcv = rc_seg + (j - sg.s0) + 1;
-                    ok = mbar_wait(&sh->kv_full[rcv % kRing], (rcv / kRing) & 1, sh, p);
-                    if (!ok) break;
-                    uint8_t* vb = sV + ((vc_seg + (j - sg.s0)) % kVStages) * kTileBytes;
-                    for (int c = (warp & 3) * 32 + lane; c < (kStepKeys - valid) * 16; c += 128) {
-                        const int vr = valid + c / 16, ch = c % 16;
-                        *reinterpret_cast<uint4*>(vb + (ch >> 3) * kTileHalfBytes + vr * 128 + ((ch & 7) << 4)) = make_uint4(0, 0, 0, 0);
-                    }
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                }
-                if (!warp_live) {
-                    // none of this warp's 32 rows exists (ragged last tile): keep the barrier protocol
-                    // going, leave the probabilities of these rows as they are; their outputs are never stored
-                    ++nsteps;
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&sh->p_full[t]);
-                    continue;
-                }
-                tc_fence_after();
-                const int pos0 = j * kStepKeys;
-                const bool masked = pos0 + kStepKeys > sg.L;     // reaches into the tree part (or past the end)
-                uint32_t sr[128];
-                // Probabilities are taken against the row's reference of the steps before: any reference within some 2^60
-                // of the row's maximum gives the same result, so a step need not look for its maximum first.  It shows in
-                // the step's sum whether the reference still serves; the first step of a segment, steps with masked
-                // scores and steps whose sum has grown beyond 2^30 go through the maximum.
-                bool by_max = masked || j == sg.s0;
-                if (!by_max) {
-                    uint64_t acc[2] = {0ull, 0ull};
-                    tmem_ld32(s_taddr, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        tmem_wait_ld_of(*reinterpret_cast<uint32_t(*)[32]>(&sr[32 * c]));
-                        if (c < 3) tmem_ld32(s_taddr + 32 * (c + 1), *reinterpret_cast<uint32_t(*)[32]>(&sr[32 * (c + 1)]));
-                        exp_chunk<SAGE_EXP2_FMA_PAIRS>(sr + 32 * c, p.scale_log2, -m_ref, sr + 16 * c, acc);
-                    }
-                    float sum_a, sum_b;
-                    f2_unpack(f2_add(acc[0], acc[1]), sum_a, sum_b);
-                    const float sum = sum_a + sum_b;
-                    by_max = __any_sync(0xffffffffu, !(sum < kMaxSum));
-                    if (!by_max) l_sum += sum;
-                }
-                if (by_max) {
-                    load_scores(s_taddr, sr);
-                    if (masked) {
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) mask_chunk(sr + 32 * c, pos0 + 32 * c, sg.L, sg.N, anc);
-                    }
-                    float mx = -INFINITY;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) max_chunk(sr + 32 * c, mx);
-                    // the reference moves only when the row max grew by more than 2^8 over it
-                    const float m_cand = mx * p.scale_log2;
-                    const bool grow = m_cand > m_ref + 8.0f;
-                    float alpha = 1.0f;
-                    if (grow) {
-                        alpha = fast_exp2(m_ref - m_cand);              // 0 when m_ref was -inf
-                        m_ref = m_cand;
-                    }
-                    // O_t *= alpha.  The P V product of the step before has finished: the scores of this step were
-                    // issued after it, and their completion is what this warp waited for above.
-                    if (j > sg.s0 && __any_sync(0xffffffffu, grow)) rescale_o_rows(o_taddr, alpha);
-                    const float neg_ref = (m_ref == -INFINITY) ? 0.f : -m_ref;
-                    uint64_t acc[2] = {0ull, 0ull};
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) exp_chunk<0>(sr + 32 * c, p.scale_log2, neg_ref, sr + 16 * c, acc);   // may hold -inf
-                    float sum_a, sum_b;
-                    f2_unpack(f2_add(acc[0], acc[1]), sum_a, sum_b);
-                    l_sum = l_sum * alpha + (sum_a + sum_b);
-                }
-                // (chunk c of 32 scores has left its 16 words of bf16 pairs at sr[16c ..])
-                uint32_t* pk = sr;
-                tmem_st32(s_taddr, pk);                 // P over the first 64 columns of S_t
-                tmem_st32(s_taddr + 32, pk + 32);
-                tmem_wait_st();
-                tc_fence_before();
-                ++nsteps;
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sh->p_full[t]);
-            }
-            if (!ok) break;
-            // ---- epilogue: O_t / l -> bf16 output, or unnormalised partials for the merge
-            ok = mbar_wait(&sh->o_full[t], nseg & 1, sh, p);
-            ++nseg;
-            if (!ok) break;
-            tc_fence_after();
-            const bool whole = (sg.s0 == 0 && sg.s1 == sg.steps);
-            const float inv = (l_sum > 0.f) ? 1.0f / l_sum : 0.f;
-            float4* po = nullptr;
-            if (!whole) {
-                const size_t slot = (size_t)blockIdx.x * 2 + (sg.at_range_begin ? 0 : 1);
-                po = p.part_o + slot * (kHeadDim / 4) * kRowsPerCta + t * kRowTile + r;
-                if (row_ok) p.part_ml[slot * kRowsPerCta + t * kRowTile + r] = make_float2(m_ref, l_sum);
-            }
-            if (warp_live) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    uint32_t orr[32];
-                    tmem_ld32(o_taddr + c * 32, orr);
-                    tmem_wait_ld();
-                    if (whole) {
-                        // every lane holds 64 bytes of its row; four lanes exchange them, so that a store instruction writes
-                        // 64 contiguous bytes of eight rows instead of 16 bytes of 32
-                        uint4 v[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            v[i] = make_uint4(pack_bf16(__uint_as_float(orr[8 * i + 0]) * inv, __uint_as_float(orr[8 * i + 1]) * inv),
-                                              pack_bf16(__uint_as_float(orr[8 * i + 2]) * inv, __uint_as_float(orr[8 * i + 3]) * inv),
-                                              pack_bf16(__uint_as_float(orr[8 * i + 4]) * inv, __uint_as_float(orr[8 * i + 5]) * inv),
-                                              pack_bf16(__uint_as_float(orr[8 * i + 6]) * inv, __uint_as_float(orr[8 * i + 7]) * inv));
-                        transpose4(v, lane);
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int Ri = sg.row0 + t * kRowTile + (warp & 3) * 32 + (lane & ~3) + i;
-                            if (Ri < M) {
-                                const size_t row = (size_t)(sg.n0 + Ri / p.G) * p.Hq + sg.g * p.G + Ri % p.G;
-                                reinterpret_cast<uint4*>(p.out + ((size_t)sg.layer * p.sum_nodes * p.Hq + row) * kHeadDim + c * 32)[lane & 3] = v[i];
-                            }
-                        }
-                    } else if (row_ok) {
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            po[(c * 8 + i) * kRowsPerCta] =
-                                make_float4(__uint_as_float(orr[4 * i]), __uint_as_float(orr[4 * i + 1]),
-                                            __uint_as_float(orr[4 * i + 2]), __uint_as_float(orr[4 * i + 3]));
-                    }
-                }
-            }
-            tc_fence_before();                          // the next segment's first P V overwrites O_t
-        }
+        if (alt) softmax<true>(p, sh, smem, tmem, warp >> 2, warp & 3, tid & 127, lane);
+        else softmax<false>(p, sh, smem, tmem, warp >> 2, warp & 3, tid & 127, lane);
     }
     // ---- teardown: every role is past its last TMEM access
     tc_fence_before();
@@ -975,7 +1161,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
 // (that block does the work), and otherwise combines the item's segments: which gangs hold them, and in which of their
 // two partial slots, follows from the positions alone.  One lane per row, 16 output columns per warp; the loads of four
 // segments are in flight together (one segment after the other took 20 us for one layer at 16k keys).
-__global__ void __launch_bounds__(256) attention_rows_merge_kernel(AttnParams p) {
+__global__ void __launch_bounds__(256) attention_merge_kernel(AttnParams p) {
     __shared__ Plan s_plan;
     __shared__ Place s_at;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1066,7 +1252,7 @@ static int row_pairs(int sum_nodes, int G) {
 // Two partial slots (head and tail of its range) per resident CTA, independent of the problem size.
 size_t workspace_size(int n_ctas) { return (size_t)n_ctas * 2 * kRowsPerCta * (kHeadDim + 2) * sizeof(float); }
 
-int launch(int n_ctas, int select, int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,
+int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,
            const int32_t* seq_len, const int32_t* parent, const int32_t* node_offsets, int batch, int sum_nodes,
            int n_q_heads, int n_kv_heads, float sm_scale, void* out, void* ws, int32_t* status, long long wait_cycles,
            int producer_off, const CUtensorMap& qmap, const CUtensorMap& kmap, const CUtensorMap& vmap,
@@ -1075,7 +1261,6 @@ int launch(int n_ctas, int select, int n_layers, int n_pages, const int32_t* pag
     AttnParams p{};
     p.n_rp = row_pairs(sum_nodes, G);
     p.n_ctas = (n_ctas / p.n_rp) * p.n_rp;          // whole gangs whatever the gang size turns out to be (1 or 2)
-    p.select = select;
     p.out = (__nv_bfloat16*)out;
     p.part_o = (float4*)ws;
     p.part_ml = (float2*)((float*)ws + (size_t)n_ctas * 2 * kRowsPerCta * kHeadDim);
@@ -1091,20 +1276,20 @@ int launch(int n_ctas, int select, int n_layers, int n_pages, const int32_t* pag
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SAGE_ERR_CUDA;
     if (!attr_set[dev]) {
-        if (cudaFuncSetAttribute(tree_attention_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) !=
+        if (cudaFuncSetAttribute(tree_attention_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) !=
             cudaSuccess)
             return SAGE_ERR_CUDA;
         attr_set[dev] = true;
     }
-    if (sage::launch(tree_attention_rows_kernel, dim3(p.n_ctas), kAttnThreads, kSmemBytes, stream, 0, p, qmap, kmap, vmap) != cudaSuccess)
+    if (sage::launch(tree_attention_stream_kernel, dim3(p.n_ctas), kAttnThreads, kSmemBytes, stream, 0, p, qmap, kmap, vmap) != cudaSuccess)
         return SAGE_ERR_CUDA;
     if (p.n_ctas > 1) {
         // one block per possible boundary between two gangs' ranges and 32 rows; those that find no cut item leave
         dim3 mg((unsigned)(p.n_ctas * (kRowsPerCta / 32)));
-        if (sage::launch(attention_rows_merge_kernel, mg, 256, 0, stream, 0, p) != cudaSuccess) return SAGE_ERR_CUDA;
+        if (sage::launch(attention_merge_kernel, mg, 256, 0, stream, 0, p) != cudaSuccess) return SAGE_ERR_CUDA;
     }
     return launch_status();
 }
 
-}  // namespace rows
+}  // namespace stream
 }  // namespace sage
