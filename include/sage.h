@@ -200,11 +200,10 @@ int sage_build_ancestor_mask(const int32_t *parent, const int32_t *node_offsets,
  * q, out: bf16 [n_layers][sum_nodes][n_q_heads][head_dim]; `sum_nodes` is the node
  * capacity of those buffers (>= node_offsets[batch]).  Softmax and accumulation in
  * fp32.  Rows of the cache beyond L_b+N_b may hold anything (NaN included).
- * Rows of q and out beyond node_offsets[batch] are neither read nor written.  The work is scheduled from
- * the trees actually present, not from the capacity: where the host cannot tell which of the library's
- * kernels suits them (a long launch whose capacity allows trees of more than 128 query rows per KV
- * head), every candidate is started, each finds the largest tree of the batch in node_offsets on the
- * device, and all but the right one leave at once.
+ * Rows of q and out beyond node_offsets[batch] have no effect and are not written.  The work is scheduled from
+ * the trees actually present, not from the capacity: where the host cannot tell which of the streaming
+ * kernels suits them (capacity for trees of more than 128 query rows per KV head), both are started, each
+ * finds the largest tree of the batch in node_offsets on the device, and one leaves at once.
  * ws: sage_tree_attention_workspace_size(...) bytes: partial results of the sequences that a work
  * boundary or a context slice cuts (the larger of a fixed amount per streaming multiprocessor and an
  * amount per layer, context slice and query row). */
@@ -255,12 +254,11 @@ void sage_debug_attention_waits(long long wait_cycles, int producer_off);
 
 /* sage_tree_attention picks a schedule per launch: a streaming one (one resident thread block per
  * multiprocessor walks an equal share of all the work in steps of 128 keys; trees of up to 128 query
- * rows per KV head alternate their steps between two accumulator slots, trees of up to 256 keep two row
- * tiles per block) for long, HBM-bound launches, and a split one (a grid over context slices, row pairs
- * and KV heads, plus a merge) for tensor-bound trees and short launches.  schedule = 1 forces the
- * streaming one, 2 the split one, 3 the streaming one on two-block clusters that share every K/V tile
- * (one tensor-core instruction stream per cluster; measured slower, kept for comparison), anything
- * else restores the automatic choice.  For tests and measurements (no counterpart in the paper). */
+ * rows per KV head alternate their steps between two accumulator slots, larger ones keep two row
+ * tiles per block) for long launches, and a split one (a grid over context slices, row pairs
+ * and KV heads, plus a merge) for short ones.  schedule = 1 or 3 forces the streaming one (3 was a form on
+ * two-block clusters that was never faster), 2 the split one, anything else restores the automatic
+ * choice.  For tests and measurements (no counterpart in the paper). */
 void sage_debug_attention_schedule(int schedule);
 
 #ifdef __cplusplus

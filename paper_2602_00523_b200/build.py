@@ -12,7 +12,7 @@ ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libsage.so")
 NATIVE_PATH = os.path.join(PKG_DIR, "_native" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
-SOURCES = ["tree_ops.cu", "logits_stats.cu", "tree_attention.cu", "tree_attention_stream.cu", "tree_attention_split.cu"]
+SOURCES = ["tree_ops.cu", "logits_stats.cu", "tree_attention.cu", "tree_attention_rows.cu", "tree_attention_alt.cu", "tree_attention_split.cu"]
 NATIVE_SOURCE = "binding.cpp"
 
 
