@@ -117,7 +117,8 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 // Bounded wait.  Returns false when the CTA is aborting (this wait or another one expired).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, Shared* sh, const AttnParams& p) {
+template <typename S, typename P>
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, S* sh, const P& p) {
     if (mbar_try(bar, parity)) return true;
     const long long t0 = clock64();
     while (true) {
@@ -132,7 +133,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, Shared
     }
 }
 // The same for a whole converged warp: every lane polls, so that the warp never splits over the answer.
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, Shared* sh, const AttnParams& p) {
+template <typename S, typename P>
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, S* sh, const P& p) {
     if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, sh, p));
 }
@@ -417,6 +419,15 @@ __device__ __forceinline__ void transpose4(uint4 (&v)[4], int lane) {
     swap(v[1], v[3], h2, 2);
 }
 
+__device__ __forceinline__ void pack_rows(const uint32_t (&o)[32], float f, uint4 (&v)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        v[i] = make_uint4(pack_bf16(__uint_as_float(o[8 * i + 0]) * f, __uint_as_float(o[8 * i + 1]) * f),
+                          pack_bf16(__uint_as_float(o[8 * i + 2]) * f, __uint_as_float(o[8 * i + 3]) * f),
+                          pack_bf16(__uint_as_float(o[8 * i + 4]) * f, __uint_as_float(o[8 * i + 5]) * f),
+                          pack_bf16(__uint_as_float(o[8 * i + 6]) * f, __uint_as_float(o[8 * i + 7]) * f));
+}
+
 // ---- schedule: items, ranges, segments ---------------------------------------------------
 struct Item { int n0, N, L, steps, rp; };     // steps == 0: the sequence is skipped (and reported); rp: row pairs
 
@@ -669,14 +680,15 @@ __device__ __forceinline__ void tear_down(uint32_t tmem, int warp) {
     }
 }
 
-// The opt-in to large dynamic shared memory is a per-device attribute of a kernel.
-template <void (*kKernel)(AttnParams, CUtensorMap, CUtensorMap, CUtensorMap)>
-inline bool allow_shared_memory() {
+// The opt-in to large dynamic shared memory is a per-device attribute of a kernel.  Internal linkage: two
+// kernels of the same type in different translation units must not share the flags (one such kernel per unit).
+template <int kBytes, typename K>
+static bool allow_shared_memory(K kernel) {
     static std::atomic<bool> done[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
     if (!done[dev].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) return false;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes) != cudaSuccess) return false;
         done[dev].store(true, std::memory_order_release);
     }
     return true;

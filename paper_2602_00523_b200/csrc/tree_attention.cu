@@ -123,10 +123,10 @@ static int g_schedule = 0;     // 0: chosen per launch, 1 or 3: streaming, 2: sp
 // The split schedule (tree_attention_split.cu).
 namespace split {
 size_t workspace_size(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
-int launch(const void* q, int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,
+int launch(int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,
            const int32_t* seq_len, const int32_t* parent, const int32_t* node_offsets, int batch, int sum_nodes,
            int n_q_heads, int n_kv_heads, float sm_scale, void* out, void* ws, int32_t* status, long long wait_cycles,
-           int producer_off, const CUtensorMap& kmap, const CUtensorMap& vmap, cudaStream_t stream);
+           int producer_off, const CUtensorMap& qmap, const CUtensorMap& kmap, const CUtensorMap& vmap, cudaStream_t stream);
 }  // namespace split
 
 // The streaming schedule (tree_attention_stream.cu).
@@ -202,13 +202,13 @@ extern "C" int sage_tree_attention(const void* q, const void* k_pool, const void
     if (!streaming && (long long)n_layers * batch * n_kv_heads > 65535) return SAGE_ERR_UNSUPPORTED;    // grid limit of the split schedule
     CUtensorMap qmap, kmap, vmap;
     if (!make_pool_map(&kmap, k_pool, n_layers, n_pages, n_kv_heads, layer_stride_elems) ||
-        !make_pool_map(&vmap, v_pool, n_layers, n_pages, n_kv_heads, layer_stride_elems))
+        !make_pool_map(&vmap, v_pool, n_layers, n_pages, n_kv_heads, layer_stride_elems) ||
+        !make_q_map(&qmap, q, n_layers, sum_nodes, n_kv_heads, G))
         return SAGE_ERR_CUDA;
     if (!streaming)
-        return split::launch(q, n_layers, n_pages, page_table, max_pages_per_seq, seq_len, parent, node_offsets, batch,
+        return split::launch(n_layers, n_pages, page_table, max_pages_per_seq, seq_len, parent, node_offsets, batch,
                              sum_nodes, n_q_heads, n_kv_heads, sm_scale, out, ws, status, g_wait_cycles, g_producer_off,
-                             kmap, vmap, as_stream(stream));
-    if (!make_q_map(&qmap, q, n_layers, sum_nodes, n_kv_heads, G)) return SAGE_ERR_CUDA;
+                             qmap, kmap, vmap, as_stream(stream));
     return stream::launch(resident_ctas(), n_layers, n_pages, page_table, max_pages_per_seq, seq_len, parent, node_offsets,
                           batch, sum_nodes, n_q_heads, n_kv_heads, sm_scale, out, ws, status, g_wait_cycles, g_producer_off,
                           qmap, kmap, vmap, as_stream(stream));

@@ -242,14 +242,6 @@ __device__ __forceinline__ void store_rows(const AttnParams& p, const Seg& sg, u
         }
     }
 }
-__device__ __forceinline__ void pack_rows(const uint32_t (&o)[32], float f, uint4 (&v)[4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        v[i] = make_uint4(pack_bf16(__uint_as_float(o[8 * i + 0]) * f, __uint_as_float(o[8 * i + 1]) * f),
-                          pack_bf16(__uint_as_float(o[8 * i + 2]) * f, __uint_as_float(o[8 * i + 3]) * f),
-                          pack_bf16(__uint_as_float(o[8 * i + 4]) * f, __uint_as_float(o[8 * i + 5]) * f),
-                          pack_bf16(__uint_as_float(o[8 * i + 6]) * f, __uint_as_float(o[8 * i + 7]) * f));
-}
 // 32 columns of a partial result; po: the thread's place in the first column quad.
 __device__ __forceinline__ void store_partial(float4* po, const uint32_t (&o)[32]) {
 #pragma unroll
@@ -366,7 +358,7 @@ __device__ __forceinline__ void softmax(const AttnParams& p, Shared* sh, uint8_t
         float m_ref = -INFINITY, l_sum = 0.f;
         for (int i = t; i < n; i += 2) {
             const int j = sg.s0 + i;
-            ok = mbar_wait(&sh->s_full[t], nsteps & 1, sh, p);
+            ok = mbar_wait_warp(&sh->s_full[t], nsteps & 1, sh, p);
             if (!ok) break;
             ++nsteps;
             const int valid = sg.L + sg.N - j * kStepKeys;      // keys of this step that exist
@@ -376,7 +368,7 @@ __device__ __forceinline__ void softmax(const AttnParams& p, Shared* sh, uint8_t
                 // the rows; the writes are ordered before this warp's arrival, which the P V product waits for.  The V tile of step s0 + i lands with ring
                 // step i + kLag of the segment.
                 const int rcv = rc_seg + i + kLag;
-                ok = mbar_wait(&sh->kv_full[rcv % kRing], (rcv / kRing) & 1, sh, p);
+                ok = mbar_wait_warp(&sh->kv_full[rcv % kRing], (rcv / kRing) & 1, sh, p);
                 if (!ok) break;
                 uint8_t* vb = sV + ((vc_seg + i) % kVStages) * kTileBytes;
                 for (int c = q * 32 + lane; c < (kStepKeys - valid) * 16; c += 128) {
@@ -397,8 +389,8 @@ __device__ __forceinline__ void softmax(const AttnParams& p, Shared* sh, uint8_t
         }
         if (!ok) break;
         const bool has1 = n >= 2;                   // slot 1 took part in this segment
-        ok = mbar_wait(&sh->o_full[0], nseg & 1, sh, p);
-        if (ok && has1) ok = mbar_wait(&sh->o_full[1], nseg1 & 1, sh, p);
+        ok = mbar_wait_warp(&sh->o_full[0], nseg & 1, sh, p);
+        if (ok && has1) ok = mbar_wait_warp(&sh->o_full[1], nseg1 & 1, sh, p);
         ++nseg;
         if (has1) ++nseg1;
         if (!ok) break;
@@ -565,7 +557,7 @@ int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int
     // it would hold up the chain, 69 instead of 63 us for a layer of 60 nodes at 16k).  (One kernel with both inside took 61 instead of 57 us for a layer of 60 nodes at
     // 16k: the compiler did worse with the softmax loops.)
     const int most_nodes = sum_nodes < SAGE_MAX_NODES ? sum_nodes : SAGE_MAX_NODES;
-    if (!allow_shared_memory<tree_attention_alt_kernel>() ||
+    if (!allow_shared_memory<kSmemBytes>(tree_attention_alt_kernel) ||
         sage::launch(tree_attention_alt_kernel, dim3(p.n_ctas), kAttnThreads, kSmemBytes, stream, 0, p, qmap, kmap, vmap) != cudaSuccess)
         return SAGE_ERR_CUDA;
     if (most_nodes * G > kRowTile && !launch_rows(p, qmap, kmap, vmap, stream)) return SAGE_ERR_CUDA;

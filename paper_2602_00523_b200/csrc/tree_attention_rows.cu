@@ -212,7 +212,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
             }
             float m_ref = -INFINITY, l_sum = 0.f;
             for (int j = sg.s0; j < sg.s1; ++j) {
-                ok = mbar_wait(&sh->s_full[t], nsteps & 1, sh, p);
+                ok = mbar_wait_warp(&sh->s_full[t], nsteps & 1, sh, p);
                 if (!ok) break;
                 const int valid = sg.L + sg.N - j * kStepKeys;      // keys of this step that exist
                 if (valid < kStepKeys) {
@@ -222,7 +222,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                     // warp's arrival, which the P V product waits for.  The V tile of step j lands with ring
                     // step j - s0 + 1 of the segment.
                     const int rcv = rc_seg + (j - sg.s0) + 1;
-                    ok = mbar_wait(&sh->kv_full[rcv % kRing], (rcv / kRing) & 1, sh, p);
+                    ok = mbar_wait_warp(&sh->kv_full[rcv % kRing], (rcv / kRing) & 1, sh, p);
                     if (!ok) break;
                     uint8_t* vb = sV + ((vc_seg + (j - sg.s0)) % kVStages) * kTileBytes;
                     for (int c = (warp & 3) * 32 + lane; c < (kStepKeys - valid) * 16; c += 128) {
@@ -303,7 +303,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
             }
             if (!ok) break;
             // ---- epilogue: O_t / l -> bf16 output, or unnormalised partials for the merge
-            ok = mbar_wait(&sh->o_full[t], nseg & 1, sh, p);
+            ok = mbar_wait_warp(&sh->o_full[t], nseg & 1, sh, p);
             ++nseg;
             if (!ok) break;
             tc_fence_after();
@@ -359,7 +359,7 @@ bool launch_rows(const AttnParams& p, const CUtensorMap& qmap, const CUtensorMap
     // The two CTAs of a gang are launched as a cluster, which puts them side by side: they read the same K and V.  (Left to
     // itself, the order in which SMs become free behind the kernel before decides, and a gang spread over both dies
     // costs power: 60 nodes, 80 layers x 16k keys at the power limit, 3000 -> 2815 us.)
-    return allow_shared_memory<tree_attention_rows_kernel>() &&
+    return allow_shared_memory<kSmemBytes>(tree_attention_rows_kernel) &&
            sage::launch(tree_attention_rows_kernel, dim3(p.n_ctas), kAttnThreads, kSmemBytes, stream, p.n_rp, p, qmap, kmap, vmap) == cudaSuccess;
 }
 
