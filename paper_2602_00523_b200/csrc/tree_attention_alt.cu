@@ -434,19 +434,21 @@ tree_attention_alt_kernel(const AttnParams p, const __grid_constant__ CUtensorMa
 }
 
 // Merge of the items that a range boundary cut into segments.  Only a boundary between two gangs' ranges can cut an
-// item, so the grid holds a block per boundary and 32 rows of a gang's CTAs: the block finds the item its boundary falls into,
-// leaves if the boundary coincides with the item's start or if an earlier boundary already lies inside the same item
-// (that block does the work), and otherwise combines the item's segments: which gangs hold them, and in which of their
-// two partial slots, follows from the positions alone.  One lane per row, 16 output columns per warp; the loads of four
-// segments are in flight together (one segment after the other took 20 us for one layer at 16k keys).
-__global__ void __launch_bounds__(256) attention_merge_kernel(AttnParams p) {
+// item, so the grid holds kMergeParts blocks per boundary and CTA of a gang.  A block finds the item its boundary falls into
+// and leaves if the boundary coincides with the item's start; the blocks of all boundaries inside the item share its output
+// columns, and combine the item's segments: which gangs hold them, and in which of their two partial slots, follows from
+// the positions alone.  One thread per row; eight 16-byte loads of two segments in flight together.  Finding the item costs a
+// block some 2 us whatever it merges, so all blocks are resident at once (a block per 32 rows, with the item's first boundary
+// doing all the work, came in four waves: 14 us for a layer of 60 nodes at 16k keys).
+constexpr int kMergeParts = 4;
+__global__ void __launch_bounds__(kRowsPerCta, 4) attention_merge_kernel(AttnParams p) {
     __shared__ Plan s_plan;
     __shared__ Place s_at;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, row = threadIdx.x;
     if (warp == 0) {
         int err = 0;
         const Plan pl = make_plan(p, lane, &err);
-        const int k = blockIdx.x / (pl.n_rp * (kRowsPerCta / 32)) + 1;
+        const int k = blockIdx.x / pl.n_rp + 1;
         Place at{0, 0, 0, 0};
         if (pl.W > 0 && k < pl.n_act) at = locate(p, pl, lane, gang_begin(pl, k));
         if (lane == 0) { s_plan = pl; s_at = at; }
@@ -454,71 +456,71 @@ __global__ void __launch_bounds__(256) attention_merge_kernel(AttnParams p) {
     __syncthreads();
     const Plan pl = s_plan;
     const Place at = s_at;
-    const int k_cut = blockIdx.x / (pl.n_rp * (kRowsPerCta / 32)) + 1;  // boundary between gang k_cut - 1 and gang k_cut
+    const int k_cut = blockIdx.x / pl.n_rp + 1;         // boundary between gang k_cut - 1 and gang k_cut
     if (pl.W <= 0 || k_cut >= pl.n_act || at.s0 == 0) return;           // no such boundary, or it falls between two items
-    const int chunk = blockIdx.x % (pl.n_rp * (kRowsPerCta / 32));
-    const int member = chunk / (kRowsPerCta / 32), row = chunk % (kRowsPerCta / 32) * 32 + lane;
+    const int member = blockIdx.x % pl.n_rp;
     int err = 0;
     const Item it = load_item(p, at.b, &err);
     const long long a = gang_begin(pl, k_cut) - at.s0;  // position of the item's first step
     const int k_first = gang_of(pl, a), k_last = gang_of(pl, a + it.steps - 1);
-    if (k_first != k_cut - 1) return;                   // an earlier boundary cuts the same item
+    const int part = (k_cut - 1 - k_first) * kMergeParts + blockIdx.y, parts = (k_last - k_first) * kMergeParts;
+    if (part >= kHeadDim / 16) return;
     const bool first_mid_range = (a != gang_begin(pl, k_first));
     const bool pair = pl.n_rp == 2 && it.rp == 1;
     const int g = pair ? 2 * at.u + member : at.u;
     const int R = row + (it.rp == 2 ? row_pair_of(member, at.u, at.b) * kRowsPerCta : 0);
-    if (g >= p.Hkv) return;
-    const bool row_ok = R < it.N * p.G;
-    if (!__any_sync(0xffffffffu, row_ok)) return;
+    if (g >= p.Hkv || R >= it.N * p.G) return;
     // (up to here only inputs have been read, which were complete before the attention kernel let this one be brought up)
     after_previous_kernel();
-    auto slot_of = [&](int k) { return (size_t)(k * pl.n_rp + member) * 2 + (k == k_first && first_mid_range ? 1 : 0); };
-    // (rows past the tree were not written: they are read all the same, as lanes of a warp with live rows, and dropped)
+    auto slot_of = [&](int k) { return (k * pl.n_rp + member) * 2 + (k == k_first && first_mid_range ? 1 : 0); };
     float mx = -INFINITY;
-    for (int k0 = k_first; k0 <= k_last; k0 += 8) {
-        float2 ml[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) ml[u] = p.part_ml[slot_of(min(k0 + u, k_last)) * kRowsPerCta + row];
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (row_ok && ml[u].y > 0.f) mx = fmaxf(mx, ml[u].x);
-    }
-    float lsum = 0.f;
-    float4 acc[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int k0 = k_first; k0 <= k_last; k0 += 4) {
-        float w[4];
-        float4 v[4][4];
+        float2 ml[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const size_t slot = slot_of(min(k0 + u, k_last));
-            const float2 ml = p.part_ml[slot * kRowsPerCta + row];
-            w[u] = (row_ok && k0 + u <= k_last && ml.y > 0.f) ? exp2f(ml.x - mx) : 0.f;
-            lsum = fmaf(w[u] > 0.f ? ml.y : 0.f, w[u], lsum);
+        for (int u = 0; u < 4; ++u) ml[u] = p.part_ml[slot_of(min(k0 + u, k_last)) * kRowsPerCta + row];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) v[u][i] = p.part_o[(slot * (kHeadDim / 4) + warp * 4 + i) * kRowsPerCta + row];
-        }
+        for (int u = 0; u < 4; ++u)
+            if (ml[u].y > 0.f) mx = fmaxf(mx, ml[u].x);
+    }
+    const size_t orow = (size_t)(it.n0 + R / p.G) * p.Hq + g * p.G + R % p.G;
+    uint4* out = reinterpret_cast<uint4*>(p.out + ((size_t)at.layer * p.sum_nodes * p.Hq + orow) * kHeadDim);
+#pragma unroll 1
+    for (int q0 = part * 4; q0 < kHeadDim / 4; q0 += parts * 4) {      // 16 output columns
+        const float4* po = p.part_o + (size_t)q0 * kRowsPerCta + row;
+        float lsum = 0.f;
+        float4 acc[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (w[u] > 0.f) {
+        for (int i = 0; i < 4; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k0 = k_first; k0 <= k_last; k0 += 2) {
+            float2 ml[2];
+            float4 v[2][4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    acc[i].x = fmaf(w[u], v[u][i].x, acc[i].x); acc[i].y = fmaf(w[u], v[u][i].y, acc[i].y);
-                    acc[i].z = fmaf(w[u], v[u][i].z, acc[i].z); acc[i].w = fmaf(w[u], v[u][i].w, acc[i].w);
+            for (int u = 0; u < 2; ++u) {
+                const int slot = slot_of(min(k0 + u, k_last));
+                ml[u] = p.part_ml[slot * kRowsPerCta + row];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[u][i] = po[((size_t)slot * (kHeadDim / 4) + i) * kRowsPerCta];
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (k0 + u <= k_last && ml[u].y > 0.f) {
+                    const float w = exp2f(ml[u].x - mx);
+                    lsum = fmaf(ml[u].y, w, lsum);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        acc[i].x = fmaf(w, v[u][i].x, acc[i].x); acc[i].y = fmaf(w, v[u][i].y, acc[i].y);
+                        acc[i].z = fmaf(w, v[u][i].z, acc[i].z); acc[i].w = fmaf(w, v[u][i].w, acc[i].w);
+                    }
                 }
             }
         }
-    }
-    if (!row_ok) return;
-    const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
-    const size_t orow = (size_t)(it.n0 + R / p.G) * p.Hq + g * p.G + R % p.G;
-    uint4* out = reinterpret_cast<uint4*>(p.out + ((size_t)at.layer * p.sum_nodes * p.Hq + orow) * kHeadDim + warp * 16);
+        const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-        out[h] = make_uint4(pack_bf16(acc[2 * h].x * inv, acc[2 * h].y * inv), pack_bf16(acc[2 * h].z * inv, acc[2 * h].w * inv),
-                            pack_bf16(acc[2 * h + 1].x * inv, acc[2 * h + 1].y * inv),
-                            pack_bf16(acc[2 * h + 1].z * inv, acc[2 * h + 1].w * inv));
+        for (int h = 0; h < 2; ++h)
+            out[q0 / 2 + h] = make_uint4(pack_bf16(acc[2 * h].x * inv, acc[2 * h].y * inv), pack_bf16(acc[2 * h].z * inv, acc[2 * h].w * inv),
+                                         pack_bf16(acc[2 * h + 1].x * inv, acc[2 * h + 1].y * inv),
+                                         pack_bf16(acc[2 * h + 1].z * inv, acc[2 * h + 1].w * inv));
+    }
 }
 
 // The kernel for trees of more than one row tile (tree_attention_rows.cu).
@@ -562,9 +564,8 @@ int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int
         return SAGE_ERR_CUDA;
     if (most_nodes * G > kRowTile && !launch_rows(p, qmap, kmap, vmap, stream)) return SAGE_ERR_CUDA;
     if (p.n_ctas > 1) {
-        // one block per possible boundary between two gangs' ranges and 32 rows; those that find no cut item leave
-        dim3 mg((unsigned)(p.n_ctas * (kRowsPerCta / 32)));
-        if (sage::launch(attention_merge_kernel, mg, 256, 0, stream, 0, p) != cudaSuccess) return SAGE_ERR_CUDA;
+        // (a gang's boundaries and members: as many as CTAs; blocks that find no cut item leave)
+        if (sage::launch(attention_merge_kernel, dim3(p.n_ctas, kMergeParts), kRowsPerCta, 0, stream, 0, p) != cudaSuccess) return SAGE_ERR_CUDA;
     }
     return launch_status();
 }
