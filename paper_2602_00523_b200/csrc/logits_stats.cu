@@ -9,11 +9,12 @@
 //     most 8 below the largest element so far) in fp32 over its elements: about seven instructions
 //     per logit, loads included.
 //  2. The K best.  After batches 0, 1, 3, 7, ... the CTA takes a threshold from its threads' largest
-//     elements: with r = 1 (K <= 8) or 2, the q-th largest of the warps' r-th largest thread maxima,
-//     q = ceil(K / r), so that at least K elements reach it.  Elements that reach the threshold go to the
-//     warp's sorted queue, whose K-th value raises the threshold for the whole CTA too; the rest of the
-//     stream only compares each thread's largest element of a batch with it.  Keys order by value (with
-//     -0 == +0) and then by lowest index, so every merge order gives the same answer.
+//     elements: the q-th largest of the warps' r-th largest thread maxima, q = ceil(K / r), so that at
+//     least K elements reach it.  Elements that reach the threshold are appended to the CTA's list, some
+//     50 in all; the rest of the stream only compares each thread's largest element of a batch with
+//     it.  When the list is full (ascending data), the warps' sorted queues take over, whose K-th value
+//     raises the threshold for the whole CTA too.  Keys order by value (with -0 == +0) and then by
+//     lowest index, so every merge order gives the same answer.
 //  3. Moments (in fp64) and the K best keys of every CTA go to the first CTA of the cluster through
 //     distributed shared memory; it ranks them, derives lse, entropies, log-probs and alpha, and
 //     hands the row's tokens to the children of the row's node.
@@ -36,6 +37,7 @@ constexpr int kBatch = 4;                        // 16-byte pieces of a batch pe
 constexpr int kStages = 3;                       // batches on their way per thread
 constexpr int kStreamBytes = kStages * kBatch * kThreads * 16;
 constexpr int kCtasPerSm = 4;
+constexpr int kListCap = 256;                    // candidates a CTA takes down before its warps' queues take over
 
 __device__ __forceinline__ uint32_t order_key(float x) {
     x += 0.0f;                                   // -0 -> +0
@@ -214,15 +216,17 @@ __device__ __forceinline__ void hand_tokens(const ExpandParams& p, int row, int 
 }
 
 // A threshold that at least K of the CTA's elements reach (see the top of the file), as a value key; 0 lets everything
-// pass.  top_key: key of this thread's largest element so far; *most: the largest of the warps' values.
+// pass.  top_key: key of this thread's largest element so far; *most: the largest of the warps' values.  r: the choice that
+// lets the fewest elements pass (ten batches of normal data: K = 4, r = 1 / 2: 17 / 24; K = 8, r = 1 / 2 / 3: 76 / 42 / 57;
+// K = 10, r = 2 / 3: 52 / 72; K = 16, r = 2 / 3 / 4: 119 / 100 / 98).
 __device__ __forceinline__ uint32_t cta_threshold(int K, uint32_t top_key, uint32_t* s_wtop, uint32_t* most, int lane, int warp) {
-    const int r_th = K <= kWarps ? 1 : 2;
+    const int r_th = K <= 5 ? 1 : K <= 12 ? 2 : 3;
     const int q_th = (K + r_th - 1) / r_th;
     uint32_t wt = __reduce_max_sync(0xffffffffu, top_key);
-    if (r_th == 2) {
-        const unsigned b = __ballot_sync(0xffffffffu, top_key == wt);
-        const uint32_t second = __reduce_max_sync(0xffffffffu, top_key == wt ? 0u : top_key);
-        if (__popc(b) == 1) wt = second;
+    for (int n = __popc(__ballot_sync(0xffffffffu, top_key == wt)); n < r_th;) {
+        top_key = top_key == wt ? 0u : top_key;
+        wt = __reduce_max_sync(0xffffffffu, top_key);
+        n += __popc(__ballot_sync(0xffffffffu, top_key == wt));
     }
     if (lane == 0) s_wtop[warp] = wt;
     __syncthreads();
@@ -257,8 +261,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
     __shared__ uint32_t s_wtop[2][kWarps];
     __shared__ float s_wref[kWarps];
     __shared__ double s_ws[kWarps], s_wt[kWarps];
-    __shared__ __align__(16) uint64_t s_list[kWarps * SAGE_MAX_TOPK];
-    __shared__ int s_n;
+    __shared__ __align__(16) uint64_t s_list[kListCap + kWarps * SAGE_MAX_TOPK];   // candidates; what the queues hold
+    __shared__ int s_n, s_nq;                                    // of both (s_n goes on counting past kListCap)
     // written by every CTA of the cluster in its first CTA
     __shared__ uint64_t s_stat[kMaxChunks][3];                   // moments (M, S, T), as doubles
     __shared__ __align__(16) uint64_t s_ckeys[kMaxChunks * SAGE_MAX_TOPK];     // K best keys of every CTA, 0 where there are fewer
@@ -285,8 +289,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
 #pragma unroll
     for (int b = 0; b < kStages; ++b) start(b);
     // (read and raised after the barrier in the first cta_threshold)
-    if (tid < kWarps * SAGE_MAX_TOPK) s_list[tid] = 0;
-    if (tid == 0) { s_n = 0; s_thr = 0; }
+    for (int i = tid; i < kListCap + kWarps * SAGE_MAX_TOPK; i += kThreads) s_list[i] = 0;
+    if (tid == 0) { s_n = 0; s_nq = 0; s_thr = 0; }
     // (the other half of this barrier, before the first store to the first CTA's memory: that CTA runs by then)
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
@@ -323,9 +327,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
             thr = max(thr, *(volatile uint32_t*)&s_thr);
             const float thr_x = thr ? key_value(thr) : -INFINITY;
             if (__any_sync(0xffffffffu, mx >= thr_x && mx != -INFINITY)) {
-                __syncwarp();                                    // the whole warp reads what its lanes' copies left in shared memory
-                // this thread's elements that reach the threshold, one bit each; they are looked at one by one, the
-                // last lane's first: in ascending data that fills the queue with values that stay
+                // this thread's elements that reach the threshold, one bit each
                 uint32_t mask = 0;
 #pragma unroll
                 for (int u = 0; u < kBatch; ++u) {
@@ -333,22 +335,37 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
                         mask |= ((v[u].x >= thr_x ? 1u : 0u) | (v[u].y >= thr_x ? 2u : 0u) | (v[u].z >= thr_x ? 4u : 0u) |
                                  (v[u].w >= thr_x ? 8u : 0u)) << (4 * u);
                 }
-                unsigned todo = __ballot_sync(0xffffffffu, mask != 0);
-                while (todo) {
-                    const int src = 31 - __clz(todo);
-                    uint32_t m = __shfl_sync(0xffffffffu, mask, src);
-                    while (m) {
-                        const int e = 31 - __clz(m);
-                        m &= ~(1u << e);
-                        const int at = (e >> 2) * kThreads + warp * 32 + src;
-                        const float x = reinterpret_cast<const float*>(buf + at)[e & 3];
-                        const uint64_t key = make_key(x, begin + 4 * (b * kBatch * kThreads + at) + (e & 3));
-                        if (key > wq.kth) wq.insert(key, lane);
+                if (mask) {
+                    int at = atomicAdd(&s_n, __popc(mask));
+                    for (; mask != 0 && at < kListCap; ++at) {
+                        const int e = __ffs(mask) - 1;
+                        mask &= mask - 1;
+                        const int piece = (e >> 2) * kThreads + tid;
+                        s_list[at] = make_key(reinterpret_cast<const float*>(buf + piece)[e & 3],
+                                              begin + 4 * (b * kBatch * kThreads + piece) + (e & 3));
                     }
-                    todo &= ~(1u << src);
                 }
-                if (lane == 0 && (uint32_t)(wq.kth >> 32) > thr) atomicMax(&s_thr, (uint32_t)(wq.kth >> 32));
-                __syncwarp();
+                unsigned todo = __ballot_sync(0xffffffffu, mask != 0);
+                if (todo) {
+                    // The list is full (ascending data, many equal values): the warp's queue takes the rest one by one, the
+                    // last lane's first, which fills the queue with values that stay.
+                    __syncwarp();                                // the whole warp reads what its lanes' copies left in shared memory
+                    while (todo) {
+                        const int src = 31 - __clz(todo);
+                        uint32_t m = __shfl_sync(0xffffffffu, mask, src);
+                        while (m) {
+                            const int e = 31 - __clz(m);
+                            m &= ~(1u << e);
+                            const int at = (e >> 2) * kThreads + warp * 32 + src;
+                            const float x = reinterpret_cast<const float*>(buf + at)[e & 3];
+                            const uint64_t key = make_key(x, begin + 4 * (b * kBatch * kThreads + at) + (e & 3));
+                            if (key > wq.kth) wq.insert(key, lane);
+                        }
+                        todo &= ~(1u << src);
+                    }
+                    if (lane == 0 && (uint32_t)(wq.kth >> 32) > thr) atomicMax(&s_thr, (uint32_t)(wq.kth >> 32));
+                    __syncwarp();
+                }
             }
             mo.rise(mx);
             start(b + kStages);                                  // (into the slots just read)
@@ -371,42 +388,25 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
                 if (lane == j) mo.add1(x);
             }
         }
+        const unsigned have = __ballot_sync(0xffffffffu, wq.q != 0);
+        if (have) {
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&s_nq, __popc(have));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (wq.q != 0) s_list[kListCap + at + lane] = wq.q;
+        }
+    }
+    // the warp's moments, in fp64 under the warp's reference
+    {
         float wr = mo.m;
         for (int o = 16; o > 0; o >>= 1) wr = fmaxf(wr, __shfl_xor_sync(0xffffffffu, wr, o));
-        const unsigned have = __ballot_sync(0xffffffffu, wq.q != 0);
-        int at = 0;
-        if (lane == 0) {
-            s_wref[warp] = wr;
-            if (have) at = atomicAdd(&s_n, __popc(have));
-        }
-        at = __shfl_sync(0xffffffffu, at, 0);
-        if (wq.q != 0) s_list[at + lane] = wq.q;
-    }
-    __syncthreads();
-    // ---- 3. the K best keys of this CTA go to the first CTA of the cluster, ...
-    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-    {
-        const int n = s_n;
-        const uint32_t keys = lead_addr(&s_ckeys[chunk * SAGE_MAX_TOPK]);
-        if (tid < n) {
-            const uint64_t mine = s_list[tid];
-            const int rank = rank_of(s_list, (n + 7) & ~7, mine);        // keys are unique
-            if (rank < p.K) st_cluster(keys + rank * 8, mine);
-        }
-        if (tid >= min(n, p.K) && tid < SAGE_MAX_TOPK) st_cluster(keys + tid * 8, 0);
-    }
-    // ... and its moments, in fp64 under the CTA's reference
-    float ref = s_wref[0];
-#pragma unroll
-    for (int w = 1; w < kWarps; ++w) ref = fmaxf(ref, s_wref[w]);
-    {
         float s0, s1, t0, t1;
         f2_unpack(mo.s2, s0, s1);
         f2_unpack(mo.t2, t0, t1);
         double ds = (double)s0 + (double)s1, dt = (double)t0 + (double)t1;
-        if (!__all_sync(0xffffffffu, mo.m == ref)) {
+        if (!__all_sync(0xffffffffu, mo.m == wr)) {
             if (ds > 0.0) {
-                const double dm = (double)mo.m - (double)ref;
+                const double dm = (double)mo.m - (double)wr;
                 const double c = exp(dm);
                 dt = c * (dt + dm * ds);
                 ds *= c;
@@ -416,24 +416,51 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
             ds += __shfl_xor_sync(0xffffffffu, ds, o);
             dt += __shfl_xor_sync(0xffffffffu, dt, o);
         }
-        if (lane == 0) { s_ws[warp] = ds; s_wt[warp] = dt; }
+        if (lane == 0) { s_wref[warp] = wr; s_ws[warp] = ds; s_wt[warp] = dt; }
     }
     __syncthreads();
-    if (tid < 3) {
-        double v = (double)ref;
-        if (tid > 0) {
-            const double* part = tid == 1 ? s_ws : s_wt;
-            v = ((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]));
+    // ---- 3. the moments of this CTA (the last warp) and its K best keys (the others) go to the first CTA of the cluster
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    if (warp == kWarps - 1) {
+        const int w = lane & (kWarps - 1);
+        const float wr = s_wref[w];
+        float ref = wr;
+        for (int o = kWarps / 2; o > 0; o >>= 1) ref = fmaxf(ref, __shfl_xor_sync(0xffffffffu, ref, o));
+        double ds = s_ws[w], dt = s_wt[w];
+        if (!__all_sync(0xffffffffu, wr == ref)) {
+            if (ds > 0.0) {
+                const double dm = (double)wr - (double)ref;
+                const double c = exp(dm);
+                dt = c * (dt + dm * ds);
+                ds *= c;
+            }
         }
-        st_cluster(lead_addr(&s_stat[chunk][tid]), (uint64_t)__double_as_longlong(v));
+        for (int o = kWarps / 2; o > 0; o >>= 1) {
+            ds += __shfl_xor_sync(0xffffffffu, ds, o);
+            dt += __shfl_xor_sync(0xffffffffu, dt, o);
+        }
+        if (lane < 3)
+            st_cluster(lead_addr(&s_stat[chunk][lane]), (uint64_t)__double_as_longlong(lane == 0 ? (double)ref : lane == 1 ? ds : dt));
+    } else {
+        const int n = min(s_n, kListCap), nq = s_nq;
+        const uint32_t keys = lead_addr(&s_ckeys[chunk * SAGE_MAX_TOPK]);
+        for (int i = tid; i < n + nq; i += kThreads - 32) {
+            const uint64_t mine = s_list[i < n ? i : kListCap + i - n];
+            int rank = rank_of(s_list, (n + 7) & ~7, mine);              // keys are unique
+            if (nq) rank += rank_of(s_list + kListCap, (nq + 7) & ~7, mine);
+            if (rank < p.K) st_cluster(keys + rank * 8, mine);
+        }
+        if (tid >= min(n + nq, p.K) && tid < SAGE_MAX_TOPK) st_cluster(keys + tid * 8, 0);
     }
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (chunk != 0) return;
 
-    // ---- the row: lse and entropy in warp 0 while the others rank every CTA's keys among all
-    double lse = 0.0;
+    // ---- the row: lse and entropy in warp 0; meanwhile four warps rank every CTA's keys among all, and one of them goes on
+    // with the entropy of the best ones, which needs no lse
+    if (warp > 4) return;
     if (warp == 0) {
+        double lse;
         double Mc = -INFINITY, Sc = 0.0, Tc = 0.0;
         if (lane < n_chunks) {
             Mc = __longlong_as_double((long long)s_stat[lane][0]);
@@ -462,7 +489,12 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
             if (p.lse) p.lse[row] = (float)lse;
             if (p.entropy_full) p.entropy_full[row] = (float)(lnS - T / S);
         }
-    } else if (tid - 32 < n_chunks * SAGE_MAX_TOPK) {
+        asm volatile("bar.sync 1, 160;" ::: "memory");                   // the keys are ranked
+        if (lane < p.k && p.topk_logprob)
+            p.topk_logprob[(size_t)row * p.k + lane] = (float)((double)key_value((uint32_t)(s_best[lane] >> 32)) - lse);
+        return;
+    }
+    if (tid - 32 < n_chunks * SAGE_MAX_TOPK) {
         const uint64_t mine = s_ckeys[tid - 32];
         if (mine != 0) {
             const int rank = rank_of(s_ckeys, n_chunks * SAGE_MAX_TOPK, mine);
@@ -472,14 +504,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
             }
         }
     }
-    __syncthreads();
-    if (warp == 0) {
-        if (lane < p.k) {
-            p.topk_idx[(size_t)row * p.k + lane] = s_idx[lane];
-            if (p.topk_logprob)
-                p.topk_logprob[(size_t)row * p.k + lane] = (float)((double)key_value((uint32_t)(s_best[lane] >> 32)) - lse);
-        }
-    } else if (warp == 1) {
+    asm volatile("bar.arrive 1, 160;" ::: "memory");
+    asm volatile("bar.sync 2, 128;" ::: "memory");
+    if (warp == 1) {
+        if (lane < p.k) p.topk_idx[(size_t)row * p.k + lane] = s_idx[lane];
         if (p.draft_token) hand_tokens(p, row, lane, s_idx);
     } else if (warp == 2 && (p.entropy_topk || p.alpha)) {
         const double v = lane < p.k_entropy ? (double)key_value((uint32_t)(s_best[lane] >> 32)) : 0.0;
