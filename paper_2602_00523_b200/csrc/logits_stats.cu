@@ -18,8 +18,8 @@
 //  3. Moments (in fp64) and the K best keys of every CTA go to the first CTA of the cluster through
 //     distributed shared memory; it ranks them, derives lse, entropies, log-probs and alpha, and
 //     hands the row's tokens to the children of the row's node.
-// What bounds it: HBM for many rows (960 rows x 152064, K = 10: 158 -> 97 us, 6.0 TB/s), the chain
-// launch -> load -> select -> merge for few (60 rows: 41 -> 17.5 us; 15 rows x 32000, K = 4: 13 -> 5.9 us).
+// What bounds it: HBM for many rows (960 rows x 152064, K = 10: 158 -> 94 us, 6.2 TB/s), the chain
+// launch -> load -> select -> merge for few (60 rows: 41 -> 15.6 us; 15 rows x 32000, K = 4: 13 -> 5.3 us).
 // The form before this one offered every element to per-warp queues that started empty, 67 thread
 // instructions per logit at K = 10, and took two more launches to merge and to gather the tokens.
 #include <math.h>
@@ -544,18 +544,21 @@ static bool allow_stream_buffer() {
     return true;
 }
 
-// CTAs per row (a power of two, each with at least one batch of elements).  About 200 CTAs when the rows are few:
-// more, shorter chunks only add selecting and merging (60 rows x 152064, K = 10: 4 CTAs per row 17.5 us, 8 19.4 us;
-// 120 rows: 2 / 4 / 8 give 24.7 / 25.4 / 30.6 us).  A launch of one wave of resident CTAs and a part of a second takes
-// as long as two: twice the CTAs fill the second (672 rows, K = 1: 1 / 2 CTAs per row 82 / 72 us; 4 take 77).
+// CTAs per row.  Up to 148 rows: as many as fit two to an SM, since two CTAs of an SM take little longer than one and three
+// nearly twice as long (clusters of three and more do not pack the SMs quite full).  us at K = 10, 152064 words: 36 rows, 6 / 7 /
+// 8 CTAs: 12.8 / 13.1 / 15.9; 56 rows, 4 / 5 / 6: 15.5 / 14.6 / 18.1; 88 rows, 2 / 3 / 4: 21.9 / 19.5 / 22.6; 148 rows, 1 / 2 / 3:
+// 27.3 / 22.9 / 26.7.  Beyond that long rows are cut where it makes up for SMs that would wait: 180 rows, 1 / 3: 34.1 /
+// 27.2; 400 rows, 1 / 2: 55.1 / 49.0; 560 rows: 59.5 / 62.6; 672 rows, K = 1: 83.2 / 69.1; 800 rows: 85.0 / 86.9.  (Rows of
+// 32000 gain nothing there: 180 rows, 1 / 3: 12.7 / 13.7; 640 rows, 1 / 2: 21.9 / 24.3.)
 static int pick_chunks(int rows, int vocab) {
+    constexpr int kSms = 148;
     const int batch = kBatch * 4 * kThreads;
-    const long wave = 148 * kCtasPerSm;
-    auto can_double = [&](int c) { return c < kMaxChunks && (2 * c - 1) * batch < vocab; };
-    int c = 1;
-    while (c * rows < 200 && can_double(c)) c *= 2;
-    if ((long)c * rows > wave && (long)c * rows < 2 * wave && can_double(c)) c *= 2;
-    return c;
+    for (int c = kMaxChunks; c >= 2; --c) {                      // (every CTA gets at least one batch of elements)
+        if ((c - 1) * batch < vocab && (long)c * rows <= (c > 2 ? 272 : 2 * kSms)) return c;
+    }
+    if (vocab < 16 * batch) return 1;
+    if (3 * (long)rows <= 544) return 3;
+    return (rows > 2 * kSms && rows <= 3 * kSms) || (rows > 4 * kSms && rows <= 5 * kSms) ? 2 : 1;
 }
 
 // Scratch that callers hand in: the size that they were always asked for (24 bytes of moments and SAGE_MAX_TOPK keys

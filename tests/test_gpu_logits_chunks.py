@@ -25,10 +25,12 @@ def expand(lg, k, ke, **tree):
     return {n: t.cpu().numpy() for n, t in o.items()}, int(st.item())
 
 
-# (rows, vocab): blocks per row 1, 2, 4, 8 and, for the many-row case, a doubled count
+# (rows, vocab): every number of blocks per row from 1 to 8, and the counts of the many-row cases
 @pytest.mark.parametrize("rows,vocab", [(1, 1), (2, 3), (3, 5), (201, 9), (1, BATCH - 1), (1, BATCH + 1), (2, 2 * BATCH),
                                         (1, 4 * BATCH + 3), (30, 8 * BATCH - 2), (70, 3 * BATCH + 1), (120, 5 * BATCH),
-                                        (200, 7 * BATCH + 2), (25, 15 * BATCH + 1), (601, 2 * BATCH + 5)])
+                                        (200, 7 * BATCH + 2), (25, 15 * BATCH + 1), (601, 2 * BATCH + 5),
+                                        (37, 9 * BATCH + 6), (45, 7 * BATCH - 1), (54, 5 * BATCH + 1), (90, 3 * BATCH),
+                                        (150, 16 * BATCH + 3), (300, 16 * BATCH)])
 @pytest.mark.parametrize("k", [1, 8, 9, 16])
 def test_chunk_edges(rows, vocab, k):
     k = min(k, vocab)
