@@ -309,8 +309,8 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kv_kernel(const Compa
 
 // ---------------------------------------------------------------------------
 // Dynamic tree construction, one level per launch (Section 3.2: hierarchical width
-// decay, Eq. 12, and "Dynamic Tree Construction").  One block per sequence, one
-// thread per frontier node.  A child of rank r of frontier node u joins the tree iff
+// decay, Eq. 12, and "Dynamic Tree Construction").  One block per sequence.
+// A child of rank r of frontier node u joins the tree iff
 // r < W_l and exp(cum_logprob) > theta_l; both tests only ever cut a suffix of the
 // (descending) candidate row, so each node contributes a prefix of its ranks, and the
 // children are laid out in breadth-first order by a prefix sum.  Decisions are taken
@@ -331,21 +331,44 @@ struct GrowParams {
     int32_t* status;
 };
 
-__global__ void __launch_bounds__(SAGE_MAX_NODES) grow_tree_kernel(GrowParams p) {
+// A launch is one short chain of dependent steps, so the chain is what is kept short: one round of loads for the sequence's
+// numbers, one for the nodes and their candidates, and a thread per candidate, 16 to a node, for the fp64 exponentials (one
+// thread per node went through up to 16 loads and exponentials in turn).
+constexpr int kGrowThreads = 512;                          // 32 frontier nodes at a time
+constexpr int kGrowNodes = kGrowThreads / SAGE_MAX_TOPK, kGrowTurns = SAGE_MAX_NODES / kGrowNodes;
+static_assert(SAGE_MAX_TOPK == 16 && SAGE_MAX_NODES == 64, "two nodes per warp, two counts per lane");
+__global__ void __launch_bounds__(kGrowThreads) grow_tree_kernel(GrowParams p) {
     after_previous_kernel();
     __shared__ int s_count[SAGE_MAX_NODES];
-    const int b = blockIdx.x, tid = threadIdx.x;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+    const int r = tid % SAGE_MAX_TOPK;                     // rank of this thread's candidates
     const int base = b * SAGE_MAX_NODES;
     const int n = p.n_nodes[b], fb = p.frontier_begin[b];
+    const double a = (double)p.alpha[p.alpha_row ? p.alpha_row[b] : b];
+    const double d_max = p.d_max_seq ? (double)p.d_max_seq[b] : (double)p.pol.d_max;
     if (n < 1 || n > p.n_max || fb < 0 || fb > n) {
         if (tid == 0) report_status(p.status, SAGE_STATUS_BAD_TREE);
         return;
     }
     if (fb == n) return;                                   // nothing left to expand
     const int level = p.depth[base + fb] + 1;
-    const double a = (double)p.alpha[p.alpha_row ? p.alpha_row[b] : b];
+    float cum_u[kGrowTurns], c[kGrowTurns];
+    int32_t word[kGrowTurns];
+#pragma unroll
+    for (int t = 0; t < kGrowTurns; ++t) {
+        const int node = fb + t * kGrowNodes + tid / SAGE_MAX_TOPK;
+        cum_u[t] = 0.f;
+        c[t] = 0.f;
+        word[t] = 0;
+        if (node < n) {
+            cum_u[t] = p.cum_logprob[base + node];
+            if (r < p.k) {
+                c[t] = p.topk_logprob[(size_t)(base + node) * p.k + r];
+                word[t] = p.topk_idx[(size_t)(base + node) * p.k + r];
+            }
+        }
+    }
     // explicit roundings: no fused multiply-add, so that a host check in plain fp64 sees the same D and W
-    const double d_max = p.d_max_seq ? (double)p.d_max_seq[b] : (double)p.pol.d_max;
     const double D = __dadd_rn((double)p.pol.d_min, __dmul_rn(a, d_max - (double)p.pol.d_min));
     const double W = __dadd_rn((double)p.pol.w_min, __dmul_rn(1.0 - a, (double)p.pol.w_max - (double)p.pol.w_min));
     if ((double)level > D) {                               // the tree has reached its depth
@@ -353,40 +376,35 @@ __global__ void __launch_bounds__(SAGE_MAX_NODES) grow_tree_kernel(GrowParams p)
         return;
     }
     const double theta = 0.1 * (double)level / D;
-    const int node = fb + tid;
-    int count = 0;
-    float cum_u = 0.f;
-    if (node < n) {
-        cum_u = p.cum_logprob[base + node];
-        const double p_parent = exp((double)cum_u);
-        const double w_l = (level == 1) ? W : W / (double)level * (0.5 + p_parent);
-        const float* lp = p.topk_logprob + (size_t)(base + node) * p.k;
-        for (int r = 0; r < p.k; ++r) {
-            if (!((double)r < w_l)) break;
-            const float c = __fadd_rn(cum_u, lp[r]);
-            if (!(exp((double)c) > theta)) break;
-            ++count;
+    int count[kGrowTurns];
+#pragma unroll
+    for (int t = 0; t < kGrowTurns; ++t) {
+        bool in = false;
+        if (fb + t * kGrowNodes + tid / SAGE_MAX_TOPK < n && r < p.k) {
+            const double w_l = (level == 1) ? W : W / (double)level * (0.5 + exp((double)cum_u[t]));
+            c[t] = __fadd_rn(cum_u[t], c[t]);
+            in = (double)r < w_l && exp((double)c[t]) > theta;
         }
+        // the node's children are its ranks up to the first that fails
+        const unsigned out = ~__ballot_sync(0xffffffffu, in) >> (lane & SAGE_MAX_TOPK);
+        count[t] = __ffs(out | (1u << SAGE_MAX_TOPK)) - 1;
+        if (r == 0) s_count[t * kGrowNodes + tid / SAGE_MAX_TOPK] = count[t];
     }
-    s_count[tid] = count;
     __syncthreads();
-    int before = 0, total = 0;
-    for (int i = 0; i < SAGE_MAX_NODES; ++i) {
-        const int c = s_count[i];
-        if (i < tid) before += c;
-        total += c;
-    }
-    if (node < n) {
-        const float* lp = p.topk_logprob + (size_t)(base + node) * p.k;
-        const int32_t* ix = p.topk_idx + (size_t)(base + node) * p.k;
-        for (int r = 0; r < count; ++r) {
-            const int pos = n + before + r;
-            if (pos >= p.n_max) break;                     // node budget: breadth-first prefix
-            p.parent[base + pos] = node;
+    const int c0 = s_count[lane], c1 = s_count[lane + 32];
+    const int total = __reduce_add_sync(0xffffffffu, c0 + c1);
+#pragma unroll
+    for (int t = 0; t < kGrowTurns; ++t) {
+        // children of the nodes in front of this thread's
+        const int first = t * kGrowNodes + tid / 32 * 2;   // the warp's first node
+        const int before = __reduce_add_sync(0xffffffffu, (lane < first ? c0 : 0) + (lane + 32 < first ? c1 : 0));
+        const int pos = n + before + (lane >= SAGE_MAX_TOPK ? s_count[first] : 0) + r;
+        if (r < count[t] && pos < p.n_max) {               // node budget: breadth-first prefix
+            p.parent[base + pos] = fb + first + lane / SAGE_MAX_TOPK;
             p.rank[base + pos] = r;
             p.depth[base + pos] = level;
-            p.token[base + pos] = ix[r];
-            p.cum_logprob[base + pos] = __fadd_rn(cum_u, lp[r]);
+            p.token[base + pos] = word[t];
+            p.cum_logprob[base + pos] = c[t];
         }
     }
     if (tid == 0) {
@@ -512,7 +530,7 @@ extern "C" int sage_grow_tree(const int32_t* topk_idx, const float* topk_logprob
     if (batch == 0) return SAGE_OK;
     GrowParams p{topk_idx, topk_logprob, k, alpha, alpha_row, *policy, n_max, parent, rank, depth, token,
                  cum_logprob, n_nodes, frontier_begin, d_max_seq, status};
-    (void)launch(grow_tree_kernel, dim3(batch), SAGE_MAX_NODES, 0, as_stream(stream), 0, p);
+    (void)launch(grow_tree_kernel, dim3(batch), kGrowThreads, 0, as_stream(stream), 0, p);
     return launch_status();
 }
 
