@@ -43,12 +43,13 @@ WORKLOAD = "config4: qwen2.5-vl-72b layer shape 64/8/128 bf16, 16384-token prefi
            "page 64 shuffled, 60-node tree, 80 layers, logits 60x152064 fp32"
 
 
-# DRAM bytes per layer of the benchmark's attention launch (split schedule, 60-node tree) as counted by
-# ncu: dram__bytes_read.sum + dram__bytes_write.sum = 615.30 MB + 3.81 MB over 9 layers
-# (profiles/tree_attention_split_kernel_config4_9layers.md).  Traffic grows in proportion to the layer
+# DRAM bytes per layer of the benchmark's attention launch (streaming schedule, 60-node tree) as counted by
+# ncu: dram__bytes_read.sum + dram__bytes_write.sum = 622.99 MB + 18.85 MB over 9 layers
+# (profiles/tree_attention_rows_kernel_9layers.md; part of the writes are the partial results of cut items, whose number
+# does not grow with the layers).  Traffic grows in proportion to the layer
 # count: every layer streams its own K/V once.  Set to None whenever that kernel changes until the
 # counters are taken again.
-ATTN_DRAM_BYTES_PER_LAYER = 619.11e6 / 9
+ATTN_DRAM_BYTES_PER_LAYER = 641.84e6 / 9
 
 
 def load_peaks():
@@ -451,7 +452,7 @@ def run_cuda(args):
 
     def graph_time_us(fn, passes=3):
         """GPU time of one call of fn(): its launches are captured in a CUDA graph once and replayed, so that
-        the host's per-call cost (Python, ctypes, tensor views) does not sit between the kernels."""
+        the host's per-call cost (Python, argument marshalling, the launch) does not sit between the kernels."""
         fn()                                          # first call outside the capture (per-device set-up, tensor maps)
         torch.cuda.synchronize()
         side = torch.cuda.Stream(device=dev)
@@ -621,11 +622,10 @@ def run_cuda(args):
                             "sample": f"{sample_s:.1f} s of oracle work: the whole logits side (60 draft + 60 target "
                                       f"rows), attention, acceptance and compaction of 1 of the {N_LAYERS} layers; "
                                       "the other layers are extrapolated"}
-        # expand (3), select + hand-over (2), attention (5: the library starts the kernels for trees of one row
-        # tile (+ merge), two row tiles (+ merge) and more, and the tree size found on the device leaves the last
-        # one running; at this shape it has one context slice per CTA, so no merge of its own), target top-1 (2),
-        # accept (1), compact + advance (2).  With --layers below 9 the launch is short and only one kernel starts.
-        launches = 3 + 2 + 5 + 2 + 1 + 2
+        # expand (1), select + hand-over (2), attention (3: the streaming schedule starts the kernel for trees of one row
+        # tile and the one for more, of which the tree size found on the device leaves the second one running, and the
+        # merge; with --layers below 4 the split schedule runs, kernel and merge), target top-1 (1), accept (1), compact (1).
+        launches = 1 + 2 + (3 if N_LAYERS >= 4 else 2) + 1 + 1 + 1
         # Which tensor peak applies: the burst figure when the SM clock stayed at its maximum through the
         # timed region, the sustained one when the power cap pulled it down.  Both fractions are printed.
         sm, sm_max = clocks.get("sm_mhz"), clocks.get("sm_max_mhz")
@@ -684,13 +684,13 @@ def run_cuda(args):
                 "expand_topk_draft_k10": None if not other_us["expand_draft"] else {
                     "us": other_us["expand_draft"], "gbs": logits_bytes / (other_us["expand_draft"] * 1e-6) / 1e9,
                     "frac_hbm": logits_bytes / (other_us["expand_draft"] * 1e-6) / 1e9 / peaks["hbm_gbs"],
-                    "algorithmic_bytes": logits_bytes, "launches": 3},
+                    "algorithmic_bytes": logits_bytes, "launches": 1},
                 "expand_topk_target_k1": None if not other_us["expand_target"] else {
                     "us": other_us["expand_target"], "gbs": logits_bytes / (other_us["expand_target"] * 1e-6) / 1e9,
                     "frac_hbm": logits_bytes / (other_us["expand_target"] * 1e-6) / 1e9 / peaks["hbm_gbs"],
-                    "algorithmic_bytes": logits_bytes, "launches": 2},
+                    "algorithmic_bytes": logits_bytes, "launches": 1},
                 "accept_compact": None if not other_us["accept_compact"] else {
-                    "us": other_us["accept_compact"], "launches": 3,
+                    "us": other_us["accept_compact"], "launches": 2,
                     "note": f"{N_LAYERS} layers; at most 9 rows x 8 heads x 256 B x 2 pools moved per layer: latency-bound"}},
             "attention_per_layer": None if layer_us is None else {
                 "us_per_call": layer_us, "tflops": flops / N_LAYERS / (layer_us * 1e-6) / 1e12,
