@@ -1,6 +1,8 @@
 // Tree-side kernels of the SAGE decode round: template selection, ancestor
 // bitsets, draft-token expansion, greedy acceptance and KV compaction.
 // All of them are latency-bound (a few hundred bytes to a few MB per round).
+#include <atomic>
+
 #include "sage_common.cuh"
 
 namespace sage {
@@ -190,8 +192,9 @@ __global__ void accept_kernel(const int32_t* __restrict__ parent, const int32_t*
 // walking the moves upwards with "read a batch, then write it" needs no barrier.
 // The length advances in the same launch: the cluster's barrier says when every block has
 // read the old one.  Latency-bound (a few MB at most): all loads of a batch are in flight
-// together.  80 layers, 4 sequences, with the acceptance before it: 17.3 us as two launches
-// with one thread planning (4.5 + 2.9 us of kernels), 15.0 us as this one.
+// together, and what an SM can keep in flight limits a sequence: 80 layers, 9 entries, one
+// sequence 10.9 us with 8 blocks, 7.5 us with 16; four 11.3 and 8.3 us.  (Two launches, one for the
+// length, with one thread planning: 17.3 us for four with the acceptance before it; one launch 15.0.)
 // ---------------------------------------------------------------------------
 struct CompactParams {
     __nv_bfloat16* k_pool;
@@ -207,7 +210,7 @@ struct CompactParams {
 };
 
 constexpr int kCompactThreads = 512;
-constexpr int kCompactCluster = 8;               // blocks of a sequence at most (the portable limit)
+constexpr int kCompactCluster = 16;              // blocks of a sequence at most (sm_100a allows 16 on request)
 constexpr int kColumns = 3;                      // columns a thread works on at a time
 constexpr int kMoves = 4;                        // moves of a batch
 
@@ -305,6 +308,18 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kv_kernel(const Compa
     }
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
     if (part == 0 && tid == 0 && s_len >= 0) p.seq_len[b] = s_len;
+}
+
+// Clusters of more than 8 blocks are a per-device opt-in of the kernel.
+static bool allow_large_cluster() {
+    static std::atomic<bool> done[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    if (!done[dev].load(std::memory_order_acquire)) {
+        if (cudaFuncSetAttribute(compact_kv_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+        done[dev].store(true, std::memory_order_release);
+    }
+    return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -509,6 +524,7 @@ extern "C" int sage_compact_kv(void* k_pool, void* v_pool, int64_t layer_stride_
     while (blocks < kCompactCluster && (int64_t)blocks * kCompactThreads < columns) blocks *= 2;
     CompactParams p{(__nv_bfloat16*)k_pool, (__nv_bfloat16*)v_pool, layer_stride_elems, n_layers, n_pages,
                     max_pages_per_seq, max_path, n_kv_heads, blocks, page_table, seq_len, path, path_len, status};
+    if (blocks > 8 && !allow_large_cluster()) return SAGE_ERR_CUDA;
     if (launch(compact_kv_kernel, dim3((unsigned)(blocks * batch)), kCompactThreads, 0, as_stream(stream), blocks, p) != cudaSuccess)
         return SAGE_ERR_CUDA;
     return launch_status();
