@@ -555,9 +555,9 @@ int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int
     p.wait_cycles = wait_cycles;
     p.producer_off = producer_off;
     // Where the host's bound on the tree sizes (the capacity of the node arrays) allows both kernels, both are started and the
-    // one that is not meant leaves after its plan (the usually shorter one first: between the other and the merge
-    // it would hold up the chain, 69 instead of 63 us for a layer of 60 nodes at 16k).  (One kernel with both inside took 61 instead of 57 us for a layer of 60 nodes at
-    // 16k: the compiler did worse with the softmax loops.)
+    // one that is not meant leaves after its plan; the usually shorter one first, since between the other and the merge it
+    // would hold up the chain (69 instead of 63 us for a layer of 60 nodes at 16k).  One kernel with both inside saves
+    // less than the compiler loses on the softmax loops (57 -> 61 us; as functions, 80 layers: 2.72 -> 2.80 ms).
     const int most_nodes = sum_nodes < SAGE_MAX_NODES ? sum_nodes : SAGE_MAX_NODES;
     if (!allow_shared_memory<kSmemBytes>(tree_attention_alt_kernel) ||
         sage::launch(tree_attention_alt_kernel, dim3(p.n_ctas), kAttnThreads, kSmemBytes, stream, 0, p, qmap, kmap, vmap) != cudaSuccess)

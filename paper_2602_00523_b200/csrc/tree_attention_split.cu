@@ -68,7 +68,7 @@ struct __align__(8) Barriers {
 constexpr int kSplitSmemBytes = 1024 /*align*/ + 2 * kQTileBytes + 2 * kPageStages * kPageBytes + (int)sizeof(Barriers);
 
 // 64 scores of a page for one query row per thread: probabilities (bf16, over the first 32 columns of the S buffer), running
-// reference and sum.  As softmax_step in attention_stream.cuh; pv_done / parity: the P V product of the page before.
+// reference and sum.  The reference works as in the streaming kernels (see softmax_step in tree_attention_alt.cu); pv_done / parity: the P V product of the page before.
 __device__ __forceinline__ bool softmax_page(const SplitParams& p, Barriers* bars, uint64_t* pv_done, uint32_t pv_parity, uint32_t s_taddr,
                                              uint32_t o_taddr, bool first, bool masked, int pos0, int L, int N, uint64_t anc,
                                              float& m_ref, float& l_sum) {
