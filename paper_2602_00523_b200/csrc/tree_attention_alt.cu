@@ -169,9 +169,10 @@ __device__ __forceinline__ void issue(const AttnParams& p, Shared* sh, uint8_t* 
 
 // =========================== softmax ===========================
 // One step of one query row per thread: scores of S_t -> probabilities (bf16, over the first 64 columns of S_t), running
-// reference and sum.  first: nothing has been accumulated yet; masked: the step reaches into the tree part (or past the end).
-__device__ __forceinline__ void softmax_step(uint32_t s_taddr, uint32_t o_taddr, float scale, bool first, bool masked, int pos0,
-                                             int L, int N, uint64_t anc, float& m_ref, float& l_sum) {
+// reference and sum.  first: nothing has been accumulated yet; masked: the step reaches into the tree part (or past
+// the end), jt0: tree slot of its first key.
+__device__ __forceinline__ void softmax_step(uint32_t s_taddr, uint32_t o_taddr, float scale, bool first, bool masked, int jt0,
+                                             uint64_t anc, float& m_ref, float& l_sum) {
     uint32_t sr[128];
     // Probabilities are taken against the row's reference of the steps before: any reference within some 2^60
     // of the row's maximum gives the same result, so a step need not look for its maximum first.  It shows in
@@ -197,7 +198,7 @@ __device__ __forceinline__ void softmax_step(uint32_t s_taddr, uint32_t o_taddr,
         load_scores(s_taddr, sr);
         if (masked) {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) mask_chunk(sr + 32 * c, pos0 + 32 * c, L, N, anc);
+            for (int c = 0; c < 4; ++c) mask_chunk(sr + 32 * c, jt0 + 32 * c, anc);
         }
         float mx = -INFINITY;
 #pragma unroll
@@ -237,7 +238,7 @@ __device__ __forceinline__ void store_rows(const AttnParams& p, const Seg& sg, u
     for (int i = 0; i < 4; ++i) {
         const int R = row0 + (lane & ~3) + i;
         if (R < M) {
-            const size_t row = (size_t)(sg.n0 + R / p.G) * p.Hq + sg.g * p.G + R % p.G;
+            const size_t row = (size_t)(sg.n0 + (R >> p.g_shift)) * p.Hq + sg.g * p.G + (R & (p.G - 1));
             reinterpret_cast<uint4*>(p.out + ((size_t)sg.layer * p.sum_nodes * p.Hq + row) * kHeadDim + col)[lane & 3] = v[i];
         }
     }
@@ -338,6 +339,8 @@ __device__ __forceinline__ void softmax(const AttnParams& p, Shared* sh, uint8_t
     Seg sg;
     int nsteps = 0, nseg = 0, nseg1 = 0;            // steps this slot has been through; segments; those with work for the slot (for slot 1, alternating)
     int rc0 = 0, vc0 = 0;                           // ring steps / V tiles of the CTA before the current segment
+    int anc_b = -1;                                 // the sequence that anc belongs to
+    uint64_t anc = 0;
     bool ok = true;
     while (ok && it.next(p, sg)) {
         const int M = sg.N * p.G, n = sg.s1 - sg.s0;
@@ -345,12 +348,15 @@ __device__ __forceinline__ void softmax(const AttnParams& p, Shared* sh, uint8_t
         rc0 += n + kLag;
         vc0 += n;
         const bool row_ok = r < M;
-        const int node = row_ok ? r / p.G : 0;
         const bool warp_live = q * 32 < M;
-        uint64_t anc = 0;
-        if (sg.s1 * kStepKeys > sg.L && row_ok) {
+        if (sg.b != anc_b) {
+            anc_b = sg.b;
+            anc = 0;
+        }
+        if (sg.s1 * kStepKeys > sg.L && row_ok && anc == 0) {
             // the segment reaches the tree part: this row's ancestor bitset (the G rows of a node
-            // walk the same parent chain, at most N - 1 cached loads deep)
+            // walk the same parent chain, at most N - 1 loads deep; kept for the sequence's next heads and layers)
+            const int node = r >> p.g_shift;
             bool bad = false;
             anc = ancestor_bits(p.parent + sg.n0, sg.N, node, &bad);
             if (bad) { report_status(p.status, SAGE_STATUS_BAD_TREE); anc = 1ull << node; }
@@ -381,8 +387,8 @@ __device__ __forceinline__ void softmax(const AttnParams& p, Shared* sh, uint8_t
             // rows, which are zero, as they are; their outputs are never stored)
             if (warp_live) {
                 tc_fence_after();
-                const int pos0 = j * kStepKeys;
-                softmax_step(s_taddr, o_taddr, p.scale_log2, i < 2, pos0 + kStepKeys > sg.L, pos0, sg.L, sg.N, anc, m_ref, l_sum);
+                const int jt0 = j * kStepKeys - sg.L;           // tree slot of the step's first key
+                softmax_step(s_taddr, o_taddr, p.scale_log2, i < 2, jt0 + kStepKeys > 0, jt0, anc, m_ref, l_sum);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh->p_full[t]);
@@ -482,7 +488,7 @@ __global__ void __launch_bounds__(kRowsPerCta, 4) attention_merge_kernel(AttnPar
         for (int u = 0; u < 4; ++u)
             if (ml[u].y > 0.f) mx = fmaxf(mx, ml[u].x);
     }
-    const size_t orow = (size_t)(it.n0 + R / p.G) * p.Hq + g * p.G + R % p.G;
+    const size_t orow = (size_t)(it.n0 + (R >> p.g_shift)) * p.Hq + g * p.G + (R & (p.G - 1));
     uint4* out = reinterpret_cast<uint4*>(p.out + ((size_t)at.layer * p.sum_nodes * p.Hq + orow) * kHeadDim);
 #pragma unroll 1
     for (int q0 = part * 4; q0 < kHeadDim / 4; q0 += parts * 4) {      // 16 output columns
@@ -550,7 +556,7 @@ int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int
     p.page_table = page_table; p.seq_len = seq_len; p.parent = parent; p.node_offsets = node_offsets;
     p.status = status;
     p.n_layers = n_layers; p.batch = batch; p.sum_nodes = sum_nodes; p.n_pages = n_pages;
-    p.max_pages = max_pages_per_seq; p.Hq = n_q_heads; p.Hkv = n_kv_heads; p.G = G;
+    p.max_pages = max_pages_per_seq; p.Hq = n_q_heads; p.Hkv = n_kv_heads; p.G = G; p.g_shift = __builtin_ctz(G);
     p.scale_log2 = sm_scale * 1.4426950408889634f;
     p.wait_cycles = wait_cycles;
     p.producer_off = producer_off;

@@ -49,7 +49,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                 for (int t = 0; t < n_rt; ++t)
                     for (int h = 0; h < 2; ++h)
                         tma_load_5d(smem_u32(sQ + t * kQTileBytes + h * kQHalfBytes), &qmap, h * 64, 0, sg.g,
-                                    sg.n0 + (sg.row0 + t * kRowTile) / p.G, sg.layer, &sh->q_ready);
+                                    sg.n0 + ((sg.row0 + t * kRowTile) >> p.g_shift), sg.layer, &sh->q_ready);
                 ++nq;
                 int ids_prev[2] = {0, 0}, npg_prev = 0;
                 for (int i = 0; i <= n; ++i) {
@@ -191,6 +191,8 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
         Seg sg;
         int nsteps = 0, nseg = 0;                       // steps / segments this row tile has been through
         int rc0 = 0, vc0 = 0;                           // ring steps / V tiles of the CTA before the current segment
+        int anc_b = -1;                                 // the sequence that anc_of (by half of the rows) belongs to
+        uint64_t anc_of[2] = {0, 0};
         bool ok = true;
         while (ok && it.next(p, sg)) {
             const int M = sg.N * p.G;
@@ -200,15 +202,21 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
             if (t == 1 && M - sg.row0 <= kRowTile) continue;
             const int R = sg.row0 + t * kRowTile + r;
             const bool row_ok = R < M;
-            const int node = row_ok ? R / p.G : 0;
             const bool warp_live = sg.row0 + t * kRowTile + (warp & 3) * 32 < M;
-            uint64_t anc = 0;
-            if (sg.s1 * kStepKeys > sg.L && row_ok) {
-                // the segment reaches the tree part: this row's ancestor bitset (the G rows of a node
-                // walk the same parent chain, at most N - 1 cached loads deep)
+            if (sg.b != anc_b) {
+                anc_b = sg.b;
+                anc_of[0] = anc_of[1] = 0;
+            }
+            uint64_t anc = sg.row0 == 0 ? anc_of[0] : anc_of[1];
+            if (sg.s1 * kStepKeys > sg.L && row_ok && anc == 0) {
+                // the segment reaches the tree part: this row's ancestor bitset (the G rows of a node walk the same
+                // parent chain, at most N - 1 loads deep; kept for the sequence's next heads and layers)
+                const int node = R >> p.g_shift;
                 bool bad = false;
                 anc = ancestor_bits(p.parent + sg.n0, sg.N, node, &bad);
                 if (bad) { report_status(p.status, SAGE_STATUS_BAD_TREE); anc = 1ull << node; }
+                if (sg.row0 == 0) anc_of[0] = anc;
+                else anc_of[1] = anc;
             }
             float m_ref = -INFINITY, l_sum = 0.f;
             for (int j = sg.s0; j < sg.s1; ++j) {
@@ -240,8 +248,8 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                     continue;
                 }
                 tc_fence_after();
-                const int pos0 = j * kStepKeys;
-                const bool masked = pos0 + kStepKeys > sg.L;     // reaches into the tree part (or past the end)
+                const int jt0 = j * kStepKeys - sg.L;            // tree slot of the step's first key
+                const bool masked = jt0 + kStepKeys > 0;     // reaches into the tree part (or past the end)
                 uint32_t sr[128];
                 // Probabilities are taken against the row's reference of the steps before: any reference within some 2^60
                 // of the row's maximum gives the same result, so a step need not look for its maximum first.  It shows in
@@ -267,7 +275,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                     load_scores(s_taddr, sr);
                     if (masked) {
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) mask_chunk(sr + 32 * c, pos0 + 32 * c, sg.L, sg.N, anc);
+                        for (int c = 0; c < 4; ++c) mask_chunk(sr + 32 * c, jt0 + 32 * c, anc);
                     }
                     float mx = -INFINITY;
 #pragma unroll
@@ -336,7 +344,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                         for (int i = 0; i < 4; ++i) {
                             const int Ri = sg.row0 + t * kRowTile + (warp & 3) * 32 + (lane & ~3) + i;
                             if (Ri < M) {
-                                const size_t row = (size_t)(sg.n0 + Ri / p.G) * p.Hq + sg.g * p.G + Ri % p.G;
+                                const size_t row = (size_t)(sg.n0 + (Ri >> p.g_shift)) * p.Hq + sg.g * p.G + (Ri & (p.G - 1));
                                 reinterpret_cast<uint4*>(p.out + ((size_t)sg.layer * p.sum_nodes * p.Hq + row) * kHeadDim + c * 32)[lane & 3] = v[i];
                             }
                         }

@@ -48,7 +48,7 @@ struct SplitParams {
     const int32_t* node_offsets;
     int32_t* status;
     int n_layers, batch, sum_nodes, n_pages, max_pages;
-    int Hq, Hkv, G, n_splits;
+    int Hq, Hkv, G, g_shift, n_splits;     // G = 1 << g_shift query heads per KV head
     float scale_log2;  // sm_scale * log2(e)
     long long wait_cycles;     // budget of every on-device wait
     int producer_off;          // diagnostics: the TMA warp issues no copies (every consumer wait then runs out)
@@ -70,7 +70,7 @@ constexpr int kSplitSmemBytes = 1024 /*align*/ + 2 * kQTileBytes + 2 * kPageStag
 // 64 scores of a page for one query row per thread: probabilities (bf16, over the first 32 columns of the S buffer), running
 // reference and sum.  The reference works as in the streaming kernels (see softmax_step in tree_attention_alt.cu); pv_done / parity: the P V product of the page before.
 __device__ __forceinline__ bool softmax_page(const SplitParams& p, Barriers* bars, uint64_t* pv_done, uint32_t pv_parity, uint32_t s_taddr,
-                                             uint32_t o_taddr, bool first, bool masked, int pos0, int L, int N, uint64_t anc,
+                                             uint32_t o_taddr, bool first, bool masked, int jt0, uint64_t anc,
                                              float& m_ref, float& l_sum) {
     uint32_t sr[64];
     bool by_max = masked || first;
@@ -92,8 +92,8 @@ __device__ __forceinline__ bool softmax_page(const SplitParams& p, Barriers* bar
         tmem_ld32(s_taddr + 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[32]));
         tmem_wait_ld();
         if (masked) {
-            mask_chunk(sr, pos0, L, N, anc);
-            mask_chunk(sr + 32, pos0 + 32, L, N, anc);
+            mask_chunk(sr, jt0, anc);
+            mask_chunk(sr + 32, jt0 + 32, anc);
         }
         float mx = -INFINITY;
         max_chunk(sr, mx);
@@ -199,7 +199,7 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
             for (int t = 0; t < n_rtiles; ++t)
                 for (int h = 0; h < 2; ++h)
                     tma_load_5d(smem_u32(sQ + t * kQTileBytes + h * kQHalfBytes), &qmap, h * 64, 0, g,
-                                n0 + (rpair * kRowsPerCta + t * kRowTile) / p.G, layer, &bars->q_ready);
+                                n0 + ((rpair * kRowsPerCta + t * kRowTile) >> p.g_shift), layer, &bars->q_ready);
             int issued_k = 0, issued_v = 0;
             int next = pages[0];
             for (int j = 0; j < ns; ++j) {
@@ -329,7 +329,7 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
         const int row0 = rpair * kRowsPerCta + t * kRowTile;
         const int R = row0 + r;
         const bool row_ok = R < M;
-        const int node = row_ok ? R / p.G : 0;
+        const int node = row_ok ? R >> p.g_shift : 0;
         const bool warp_live = row0 + (warp & 3) * 32 < M;
         uint64_t anc = 0;
         if ((pg_begin + ns) * kPageSize > L && row_ok) {
@@ -349,9 +349,9 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
             // these rows as they are; their outputs are never stored)
             if (warp_live) {
                 tc_fence_after();
-                const int pos0 = (pg_begin + j) * kPageSize;
-                ok = softmax_page(p, bars, &bars->pv_done[t], (j - 1) & 1, s_taddr + x * 64, o_taddr, j == 0, pos0 + kPageSize > L, pos0, L, N,
-                                  anc, m_ref, l_sum);
+                const int jt0 = (pg_begin + j) * kPageSize - L;     // tree slot of the page's first key
+                ok = softmax_page(p, bars, &bars->pv_done[t], (j - 1) & 1, s_taddr + x * 64, o_taddr, j == 0, jt0 + kPageSize > 0, jt0, anc,
+                                  m_ref, l_sum);
                 if (!ok) break;
             }
             __syncwarp();
@@ -362,7 +362,7 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
         if (ok && warp_live) {
             tc_fence_after();
             const size_t rows_total = (size_t)p.sum_nodes * p.Hq;
-            const size_t row = (size_t)(n0 + node) * p.Hq + g * p.G + (row_ok ? R % p.G : 0);
+            const size_t row = (size_t)(n0 + node) * p.Hq + g * p.G + (row_ok ? R & (p.G - 1) : 0);
             const size_t part = (size_t)layer * p.n_splits + split;
             const float inv = (l_sum > 0.f) ? 1.0f / l_sum : 0.f;
             if (p.n_splits > 1 && row_ok) p.part_ml[part * rows_total + row] = make_float2(m_ref, l_sum);
@@ -380,7 +380,7 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
                     for (int i = 0; i < 4; ++i) {
                         const int Ri = R - lane + (lane & ~3) + i;
                         if (Ri < M) {
-                            const size_t orow = (size_t)(n0 + Ri / p.G) * p.Hq + g * p.G + Ri % p.G;
+                            const size_t orow = (size_t)(n0 + (Ri >> p.g_shift)) * p.Hq + g * p.G + (Ri & (p.G - 1));
                             reinterpret_cast<uint4*>(p.out + ((size_t)layer * rows_total + orow) * kHeadDim + c * 32)[lane & 3] = v[i];
                         }
                     }
@@ -522,7 +522,7 @@ int launch(int n_layers, int n_pages, const int32_t* page_table, int max_pages_p
     p.page_table = page_table; p.seq_len = seq_len; p.parent = parent; p.node_offsets = node_offsets;
     p.status = status;
     p.n_layers = n_layers; p.batch = batch; p.sum_nodes = sum_nodes; p.n_pages = n_pages;
-    p.max_pages = max_pages_per_seq; p.Hq = n_q_heads; p.Hkv = n_kv_heads; p.G = G; p.n_splits = S;
+    p.max_pages = max_pages_per_seq; p.Hq = n_q_heads; p.Hkv = n_kv_heads; p.G = G; p.g_shift = __builtin_ctz(G); p.n_splits = S;
     p.scale_log2 = sm_scale * 1.4426950408889634f;
     p.wait_cycles = wait_cycles;
     p.producer_off = producer_off;
