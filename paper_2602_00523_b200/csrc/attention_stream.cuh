@@ -94,6 +94,7 @@ struct __align__(16) Shared {
     int n_rp, heads_all;       // of the plan
     uint32_t tmem_base;
     volatile int abort;
+    int parked[8][24];         // alternating: what a softmax warp knows of its segment and need not hold in registers
 };
 constexpr int kSmemBytes = 1024 /*align*/ + 7 * kTileBytes + (int)sizeof(Shared);
 static_assert(kSmemBytes <= 232448, "shared memory budget of one CTA exceeded");

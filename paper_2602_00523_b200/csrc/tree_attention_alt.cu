@@ -334,19 +334,33 @@ __device__ __forceinline__ void softmax(const AttnParams& p, Shared* sh, uint8_t
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;            // r: row inside the tile == TMEM lane, q: its quadrant
     const uint32_t s_taddr = tmem + lane_base + t * 128;
     const uint32_t o_taddr = tmem + lane_base + 256 + t * 128;
-    SegIter it;
-    it.init(sh);
-    Seg sg;
+    // A step needs all registers for its scores: where the warp is in its range, and what only the epilogue needs of the
+    // segment, waits in shared memory (as spilled registers it went to L2 and back, see the kernel).
+    struct Parked { SegIter it; Seg sg; };
+    static_assert(sizeof(Parked) <= sizeof(sh->parked[0]), "parked state outgrew its place");
+    Parked* parked = reinterpret_cast<Parked*>(sh->parked[t * 4 + q]);
+    if (lane == 0) {
+        SegIter it;
+        it.init(sh);
+        parked->it = it;
+        parked->sg.b = -1;
+    }
     int nsteps = 0, nseg = 0, nseg1 = 0;            // steps this slot has been through; segments; those with work for the slot (for slot 1, alternating)
-    int rc0 = 0, vc0 = 0;                           // ring steps / V tiles of the CTA before the current segment
+    int vc0 = 0;                                    // V tiles of the CTA before the current segment
     int anc_b = -1;                                 // the sequence that anc belongs to
     uint64_t anc = 0;
     bool ok = true;
-    while (ok && it.next(p, sg)) {
+    while (ok) {
+        __syncwarp();
+        Seg sg = parked->sg;
+        {
+            SegIter it = parked->it;
+            if (!it.next(p, sg)) break;
+            __syncwarp();
+            if (lane == 0) { parked->it = it; parked->sg = sg; }
+            __syncwarp();
+        }
         const int M = sg.N * p.G, n = sg.s1 - sg.s0;
-        const int rc_seg = rc0, vc_seg = vc0;       // this segment's first ring step / V tile
-        rc0 += n + kLag;
-        vc0 += n;
         const bool row_ok = r < M;
         const bool warp_live = q * 32 < M;
         if (sg.b != anc_b) {
@@ -373,10 +387,10 @@ __device__ __forceinline__ void softmax(const AttnParams& p, Shared* sh, uint8_t
                 // copied): zero them so that 0 * V stays 0.  Each warp of the warpgroup takes a quarter of
                 // the rows; the writes are ordered before this warp's arrival, which the P V product waits for.  The V tile of step s0 + i lands with ring
                 // step i + kLag of the segment.
-                const int rcv = rc_seg + i + kLag;
+                const int rcv = vc0 + (nseg + 1) * kLag + i;    // (a segment of n steps takes n + kLag ring steps)
                 ok = mbar_wait_warp(&sh->kv_full[rcv % kRing], (rcv / kRing) & 1, sh, p);
                 if (!ok) break;
-                uint8_t* vb = sV + ((vc_seg + i) % kVStages) * kTileBytes;
+                uint8_t* vb = sV + ((vc0 + i) % kVStages) * kTileBytes;
                 for (int c = q * 32 + lane; c < (kStepKeys - valid) * 16; c += 128) {
                     const int vr = valid + c / 16, ch = c % 16;
                     *reinterpret_cast<uint4*>(vb + (ch >> 3) * kTileHalfBytes + vr * 128 + ((ch & 7) << 4)) = make_uint4(0, 0, 0, 0);
@@ -399,10 +413,12 @@ __device__ __forceinline__ void softmax(const AttnParams& p, Shared* sh, uint8_t
         if (ok && has1) ok = mbar_wait_warp(&sh->o_full[1], nseg1 & 1, sh, p);
         ++nseg;
         if (has1) ++nseg1;
+        vc0 += n;
         if (!ok) break;
         if (warp_live) {
             tc_fence_after();
-            ok = finish_slots(p, sh, sg, tmem, lane_base, t, q, r, lane, has1, (uint32_t)nseg, m_ref, l_sum);
+            asm volatile("" ::: "memory");
+            ok = finish_slots(p, sh, parked->sg, tmem, lane_base, t, q, r, lane, has1, (uint32_t)nseg, m_ref, l_sum);
             if (!ok) break;
         }
         tc_fence_before();                          // the next segment's first P V products overwrite O_0 and O_1
@@ -424,16 +440,19 @@ tree_attention_alt_kernel(const AttnParams p, const __grid_constant__ CUtensorMa
     uint32_t tmem;
     if (!set_up<true>(p, sh, warp, lane, qmap, kmap, vmap, &tmem)) return;
     // Registers move from the copy / MMA warpgroup (which needs few) to the softmax warpgroups:
-    // 4 warps give up 168 - 72 registers per thread, 8 warps take 216 - 168 each.
+    // 4 warps give up 168 - 40 registers per thread, 8 warps take 232 - 168 each.  (With 72 and 216 the softmax
+    // warps kept part of a segment's state in local memory, which L1 is too small to hold beside this much shared memory:
+    // a segment's epilogue and the way to the next one took 12 000 clocks.  80 layers of 4k keys, 12 nodes: 288 -> 270 us,
+    // and 254 with the state that is parked in shared memory.  The kernel for more rows spills nothing with 72 and 216.)
     if (warp >= 8) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
         if (warp == 8) {
             if (lane == 0) produce(p, sh, smem, qmap, kmap, vmap);
         } else if (warp == 9) {
             issue(p, sh, smem, tmem, lane);
         }
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
         softmax(p, sh, smem, tmem, warp >> 2, warp & 3, tid & 127, lane);
     }
     tear_down(tmem, warp);
