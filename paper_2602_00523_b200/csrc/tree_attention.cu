@@ -144,16 +144,16 @@ int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int
 //   split: grid over (context slice, row pair, layer x sequence x KV head), 64-key steps: shorter set-up and no plan, for
 //     launches too short to give every SM a long stream (single layers, short contexts: fixed costs dominate).
 // The line lies where both take the same time (us, split / streaming; steps per SM in brackets; 8 KV heads of 8 queries):
-//   one sequence, up to one row pair: 24 nodes, 16k keys, 3 layers (21) 65/86, 4 (28) 89/101, 8 (56) 170/170; 12 nodes, 4k
-//     keys, 32 layers (57) 125/129, 64 (114) 257/237;
-//   one sequence whose node arrays have room for two row pairs: 60 nodes, 16k keys, 2 layers (14) 84/93, 4 (28) 157/159;
-//     but nine nodes in such arrays, for which half of the split grid is empty, 4 layers (28) 98/87;
+//   one sequence, up to one row pair: 24 nodes, 16k keys, 4 layers (28) 86/93, 8 (56) 164/164; 12 nodes, 4k keys, 16 layers
+//     (28) 56/65, 24 (43) 102/90, 32 (57) 118/112;
+//   one sequence whose node arrays have room for two row pairs: 60 nodes, 16k keys, 3 layers (21) 115/119, 4 (28) 156/153;
+//     but nine nodes in such arrays, for which half of the split grid is empty, 2 layers (14) 55/55, 4 (28) 92/74;
 //   several sequences: the split grid is as uneven as their lengths.  1k to 8k keys, 24 to 60 nodes: four sequences
-//     (12) 68/70, eight (25) 116/94, sixteen of 24 nodes (54) 122/101.
+//     (12.5) 68/61, eight (25) 110/82, sixteen of 24 nodes (54) 117/84; eight of 2k keys, 36 nodes (7) 38/56.
 static bool use_streaming(int n_layers, int batch, int n_kv_heads, int max_pages_per_seq, int rows) {
     if (g_schedule) return g_schedule != 2;
     const long long steps = (long long)n_layers * batch * n_kv_heads * ((max_pages_per_seq + 1) / 2);   // upper bound
-    const int line = batch > 1 ? 16 : rows > 256 ? 24 : 48;
+    const int line = batch > 1 ? 12 : rows > 256 ? 24 : 40;
     return steps >= (long long)line * resident_ctas();
 }
 
@@ -205,7 +205,8 @@ extern "C" int sage_tree_attention(const void* q, const void* k_pool, const void
     const size_t need = sage_tree_attention_workspace_size(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads,
                                                            head_dim, max_pages_per_seq);
     if (!ws || ws_bytes < need || ((uintptr_t)ws & 15)) return SAGE_ERR_WORKSPACE;
-    const bool streaming = use_streaming(n_layers, batch, n_kv_heads, max_pages_per_seq, (sum_nodes < SAGE_MAX_NODES ? sum_nodes : SAGE_MAX_NODES) * G);
+    const int most_rows = (sum_nodes < SAGE_MAX_NODES ? sum_nodes : SAGE_MAX_NODES) * G;
+    const bool streaming = use_streaming(n_layers, batch, n_kv_heads, max_pages_per_seq, most_rows);
     if (!streaming && (long long)n_layers * batch * n_kv_heads > 65535) return SAGE_ERR_UNSUPPORTED;    // grid limit of the split schedule
     CUtensorMap qmap, kmap, vmap;
     if (!make_pool_map(&kmap, k_pool, n_layers, n_pages, n_kv_heads, layer_stride_elems) ||
