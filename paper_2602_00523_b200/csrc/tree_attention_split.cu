@@ -496,6 +496,7 @@ static int pick_splits(int n_layers, int batch, int n_kv_heads, int G, int max_p
     double best_cost = 0.0;
     for (int s = 1; s <= s_max; ++s) {
         const long waves = (base * s + 147) / 148;
+        if (s > 1 && waves > 4) break;                      // (the last wave matters little by then, partial results do)
         const double cost = (double)waves * (6 + (max_pages + s - 1) / s) + (s > 1 ? 4.0 + 0.25 * s : 0.0);
         if (s == 1 || cost < best_cost - 1e-9) { best_cost = cost; best = s; }
     }
