@@ -479,6 +479,9 @@ __global__ void __launch_bounds__(kRowsPerCta, 4) attention_merge_kernel(AttnPar
         if (lane == 0) { s_plan = pl; s_at = at; }
     }
     __syncthreads();
+    // Before any block leaves: the kernel behind this one waits for this one only, and where no boundary cuts an item
+    // every block would be gone before the attention kernel is.
+    after_previous_kernel();
     const Plan pl = s_plan;
     const Place at = s_at;
     const int k_cut = blockIdx.x / pl.n_rp + 1;         // boundary between gang k_cut - 1 and gang k_cut
@@ -495,8 +498,6 @@ __global__ void __launch_bounds__(kRowsPerCta, 4) attention_merge_kernel(AttnPar
     const int g = pair ? 2 * at.u + member : at.u;
     const int R = row + (it.rp == 2 ? row_pair_of(member, at.u, at.b) * kRowsPerCta : 0);
     if (g >= p.Hkv || R >= it.N * p.G) return;
-    // (up to here only inputs have been read, which were complete before the attention kernel let this one be brought up)
-    after_previous_kernel();
     auto slot_of = [&](int k) { return (k * pl.n_rp + member) * 2 + (k == k_first && first_mid_range ? 1 : 0); };
     float mx = -INFINITY;
     for (int k0 = k_first; k0 <= k_last; k0 += 4) {

@@ -54,3 +54,49 @@ def test_attention_edges(schedule, layers, heads, G, Ls, Ns, ramp, spare):
         # Probabilities are rounded to bf16: at most 2^-9 of the largest value in play (below 5) = 0.0098 per output
         # before its own rounding, for which the half unit is added.
         check_attention(got[layer, :nodes], want, bf16_slack=True)
+
+
+@pytest.mark.parametrize("layers,heads,G,L,N,batch,width", [
+    (80, 8, 8, 100, 12, 1, 19),             # items of one step
+    (80, 8, 8, 90, 36, 1, 19),              # the same with trees of two row pairs
+    (1, 8, 8, 200, 12, 16, 28),             # two steps, a thread block for each item
+    (1, 8, 8, 200, 30, 37, 6)])             # two whole items per thread block
+def test_launches_in_which_no_range_cuts_an_item(layers, heads, G, L, N, batch, width):
+    """Nothing to merge: every block of the merge leaves at once, and what follows in the stream must find the attention
+    finished all the same.  Rounds of attention, then compaction of the very rows that it reads, without a pause."""
+    r = np.random.Generator(np.random.Philox(layers * 1000 + batch + N))
+    tree = random_tree(r, N)
+    used = (L + N + 63) // 64
+    kv = make_kv_cache(r, [L] * batch, [N] * batch, [L // 2] * batch, heads, n_layers=layers, shuffle=True, spare_frac=0.1)
+    table = np.full((batch, width), -1, np.int32)
+    table[:, :used] = kv["page_table"][:, :used]
+    path = np.full((batch, 9), -1, np.int32)         # the last node's root path: its rows have the furthest to go
+    chain = [N - 1]
+    while chain[-1]:
+        chain.append(int(tree["parent"][chain[-1]]))
+    path[:, :len(chain)] = chain[::-1][:9]
+    length = np.full(batch, min(9, len(chain)), np.int32)
+    q = make_q(r, batch * N, heads * G, n_layers=layers)
+    parent, off = np.tile(tree["parent"], batch).astype(np.int32), (np.arange(batch + 1) * N).astype(np.int32)
+    st, dev = sage.new_status(), dict(q=dev_bf16(q), table=dev_i32(table), parent=dev_i32(parent), off=dev_i32(off),
+                                      path=dev_i32(path), length=dev_i32(length), L=dev_i32(kv["seq_len"]))
+    k0, v0 = dev_bf16(kv["k_pool"]), dev_bf16(kv["v_pool"])
+    outs = [torch.zeros_like(dev["q"]) for _ in range(4)]
+    sage.sage_debug_attention_schedule(1)
+    try:
+        for out in outs:
+            k, v, seq = k0.clone(), v0.clone(), dev["L"].clone()
+            sage.sage_tree_attention(dev["q"], k, v, dev["table"], seq, dev["parent"], dev["off"], 128 ** -0.5, out=out, status=st)
+            sage.sage_compact_kv(k, v, dev["table"], seq, dev["path"], dev["length"], status=st)
+        torch.cuda.synchronize()
+    finally:
+        sage.sage_debug_attention_schedule(0)
+    assert int(st.item()) == 0
+    assert np.array_equal(seq.cpu().numpy(), kv["seq_len"] + length)
+    for out in outs[1:]:
+        assert torch.equal(out.view(torch.int16), outs[0].view(torch.int16))
+    got = host_bits(outs[0])
+    for layer in sorted({0, layers // 2, layers - 1}):
+        want = oracle.tree_attention(q[layer], kv["k_pool"][layer], kv["v_pool"][layer], table, kv["seq_len"], parent, off,
+                                     heads * G, heads, 128, 64, 128 ** -0.5)
+        check_attention(got[layer], want, bf16_slack=True)       # (bound: see test_attention_edges)

@@ -1,0 +1,40 @@
+"""Rules that every kernel keeps because each is launched while the one before it still runs, checked on the sources: no GPU
+shows reliably what breaks when one is forgotten."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2602_00523_b200", "csrc")
+WAIT = "after_previous_kernel();"
+
+
+def kernels():
+    """(name, body without comments) of every __global__ function."""
+    found = []
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        text = re.sub(r"//[^\n]*", "", open(path).read())
+        for m in re.finditer(r"__global__\s+void\s+(?:__launch_bounds__\([^)]*\)\s*)?(\w+)\s*\(", text):
+            at = text.index("{", m.end())
+            depth, end = 1, at + 1
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[end], 0)
+                end += 1
+            found.append((m.group(1), text[at:end]))
+    return found
+
+
+KERNELS = kernels()
+
+
+def test_all_kernels_are_found():
+    assert len(KERNELS) == 13 and {"attention_merge_kernel", "expand_topk_kernel", "tree_attention_rows_kernel"} <= {n for n, _ in KERNELS}
+
+
+@pytest.mark.parametrize("name,body", KERNELS, ids=[n for n, _ in KERNELS])
+def test_no_thread_leaves_before_the_wait(name, body):
+    """A kernel waits for its direct predecessor only, so stream order holds as long as no kernel can finish without
+    having waited for its own."""
+    assert body.count(WAIT) == 1
+    assert not re.search(r"\breturn\b", body[:body.index(WAIT)])
