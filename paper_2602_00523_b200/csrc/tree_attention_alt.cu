@@ -467,6 +467,7 @@ tree_attention_alt_kernel(const AttnParams p, const __grid_constant__ CUtensorMa
 // doing all the work, came in four waves: 14 us for a layer of 60 nodes at 16k keys).
 constexpr int kMergeParts = 4;
 __global__ void __launch_bounds__(kRowsPerCta, 4) attention_merge_kernel(AttnParams p) {
+    after_previous_kernel();
     __shared__ Plan s_plan;
     __shared__ Place s_at;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, row = threadIdx.x;
@@ -479,9 +480,6 @@ __global__ void __launch_bounds__(kRowsPerCta, 4) attention_merge_kernel(AttnPar
         if (lane == 0) { s_plan = pl; s_at = at; }
     }
     __syncthreads();
-    // Before any block leaves: the kernel behind this one waits for this one only, and where no boundary cuts an item
-    // every block would be gone before the attention kernel is.
-    after_previous_kernel();
     const Plan pl = s_plan;
     const Place at = s_at;
     const int k_cut = blockIdx.x / pl.n_rp + 1;         // boundary between gang k_cut - 1 and gang k_cut

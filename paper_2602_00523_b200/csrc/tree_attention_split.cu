@@ -404,6 +404,7 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
 constexpr int kMaxSplits = 32;
 template <int kMaxS>
 __global__ void __launch_bounds__(256) attention_split_merge_kernel(const SplitParams p) {
+    after_previous_kernel();
     constexpr bool kShare = kMaxS > 8;
     constexpr int kMl = kShare ? kMaxS / 8 : kMaxS;         // weights per thread
     constexpr int kBatch = kMaxS < 16 ? kMaxS : 16;         // slices in flight
@@ -411,9 +412,7 @@ __global__ void __launch_bounds__(256) attention_split_merge_kernel(const SplitP
     const size_t rows_total = (size_t)p.sum_nodes * p.Hq;
     const size_t row = (size_t)blockIdx.x * 32 + lane;
     const int layer = blockIdx.y, S = p.n_splits, quad = blockIdx.z * 8 + warp;
-    // (inputs only: complete before the attention kernel let this one be brought up)
     const bool ok = row < rows_total && row < (size_t)p.node_offsets[p.batch] * p.Hq;   // rows past the live nodes were never written
-    after_previous_kernel();
     if (!__any_sync(0xffffffffu, ok)) return;               // the same for all warps
     const size_t r = ok ? row : (size_t)blockIdx.x * 32;
     const float2* ml = p.part_ml + (size_t)layer * S * rows_total + r;

@@ -38,3 +38,11 @@ def test_no_thread_leaves_before_the_wait(name, body):
     having waited for its own."""
     assert body.count(WAIT) == 1
     assert not re.search(r"\breturn\b", body[:body.index(WAIT)])
+
+
+@pytest.mark.parametrize("name,body", KERNELS, ids=[n for n, _ in KERNELS])
+def test_nothing_in_global_memory_is_touched_before_the_wait(name, body):
+    """Node offsets, lengths and page tables are written on the device every round, and only the wait makes the writes of
+    earlier kernels visible."""
+    ahead = body[:body.index(WAIT)]
+    assert not re.search(r"p\.\w+\s*\[|node_offsets|seq_len|page_table|parent|part_|load_item|make_plan|locate|atomic|report_status", ahead)
