@@ -17,9 +17,9 @@
 // TMEM map (512 columns): tile t owns S_t,even [128t, 128t+64), S_t,odd [128t+64, 128t+128)
 // (P overlays the first 32 columns of its S buffer) and O_t [256+128t, 384+128t).
 // Slices are merged by attention_split_merge_kernel.
-// These launches are bound by fixed costs, so the way to the first MMA is kept short: tensor memory is allocated and
-// tensor maps are fetched while the kernel before still runs, then one round of loads (the sequence's offsets and length),
-// the barriers, and the copies start; what is left of the set-up (page ids, ancestors) happens in the roles.  Before, query
+// These launches are bound by fixed costs, so the way to the first MMA is kept short: tensor maps are fetched while the
+// kernel before still runs, then one round of loads (the sequence's offsets and length) beside the allocation of tensor
+// memory, the barriers, and the copies start; what is left of the set-up (page ids, ancestors) happens in the roles.  Before, query
 // rows went through registers, partial results were written row by row (32 lines per store) and merged one warp per row:
 // one layer, 8 KV heads of 8 queries, 60 nodes: 2k keys 23.5 -> 16.5 us, 16k keys 49.7 -> 40.0; 24 nodes, 16k: 37.3 -> 27.4.
 // With two row tiles a page costs 1650 clocks, of which the tensor pipe is busy for 1536 (a 64-key score product takes it
@@ -142,17 +142,20 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
     const int b = (blockIdx.z / p.Hkv) % p.batch;
     const int layer = blockIdx.z / (p.Hkv * p.batch);
 
-    // ---- before the kernel in front has finished: nothing here touches global memory
-    if (warp == 9) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(&bars->tmem_base)), "r"(512) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    } else if (warp == 8 && lane == 0) {
+    // before the kernel in front has finished: nothing here touches global memory
+    if (warp == 8 && lane == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(&kmap) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&vmap) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&qmap) : "memory");
     }
     after_previous_kernel();
+    // Not earlier: held while this block waits for the kernel in front, the tensor memory would be missing to a block of that
+    // kernel (any kernel, of the caller's too) that shares the SM and asks for its own only after it has let this one start.
+    if (warp == 9) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(&bars->tmem_base)), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
     const int n0 = p.node_offsets[b];
     const int N = p.node_offsets[b + 1] - n0;
     const int L = p.seq_len[b];

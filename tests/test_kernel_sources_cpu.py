@@ -46,3 +46,11 @@ def test_nothing_in_global_memory_is_touched_before_the_wait(name, body):
     earlier kernels visible."""
     ahead = body[:body.index(WAIT)]
     assert not re.search(r"p\.\w+\s*\[|node_offsets|seq_len|page_table|parent|part_|load_item|make_plan|locate|atomic|report_status", ahead)
+
+
+@pytest.mark.parametrize("name,body", KERNELS, ids=[n for n, _ in KERNELS])
+def test_no_tensor_memory_is_held_while_waiting(name, body):
+    """A block that holds it while it waits for the kernel in front can keep a block of that kernel on the same SM from ever
+    getting its own."""
+    ahead = body[:body.index(WAIT)]
+    assert "tcgen05" not in ahead and "set_up" not in ahead
