@@ -170,9 +170,10 @@ __device__ __forceinline__ void issue(const AttnParams& p, Shared* sh, uint8_t* 
 // =========================== softmax ===========================
 // One step of one query row per thread: scores of S_t -> probabilities (bf16, over the first 64 columns of S_t), running
 // reference and sum.  first: nothing has been accumulated yet; masked: the step reaches into the tree part (or past
-// the end), jt0: tree slot of its first key.
-__device__ __forceinline__ void softmax_step(uint32_t s_taddr, uint32_t o_taddr, float scale, bool first, bool masked, int jt0,
-                                             uint64_t anc, float& m_ref, float& l_sum) {
+// the end), jt0: tree slot of its first key.  row_ok: the row exists (others, spare rows or the next sequence's, have no say in
+// how the rows beside them are computed).
+__device__ __forceinline__ void softmax_step(uint32_t s_taddr, uint32_t o_taddr, float scale, bool row_ok, bool first, bool masked,
+                                             int jt0, uint64_t anc, float& m_ref, float& l_sum) {
     uint32_t sr[128];
     // Probabilities are taken against the row's reference of the steps before: any reference within some 2^60
     // of the row's maximum gives the same result, so a step need not look for its maximum first.  It shows in
@@ -191,7 +192,7 @@ __device__ __forceinline__ void softmax_step(uint32_t s_taddr, uint32_t o_taddr,
         float sum_a, sum_b;
         f2_unpack(f2_add(acc[0], acc[1]), sum_a, sum_b);
         const float sum = sum_a + sum_b;
-        by_max = __any_sync(0xffffffffu, !(sum < kMaxSum));
+        by_max = __any_sync(0xffffffffu, row_ok && !(sum < kMaxSum));
         if (!by_max) l_sum += sum;
     }
     if (by_max) {
@@ -402,7 +403,7 @@ __device__ __forceinline__ void softmax(const AttnParams& p, Shared* sh, uint8_t
             if (warp_live) {
                 tc_fence_after();
                 const int jt0 = j * kStepKeys - sg.L;           // tree slot of the step's first key
-                softmax_step(s_taddr, o_taddr, p.scale_log2, i < 2, jt0 + kStepKeys > 0, jt0, anc, m_ref, l_sum);
+                softmax_step(s_taddr, o_taddr, p.scale_log2, row_ok, i < 2, jt0 + kStepKeys > 0, jt0, anc, m_ref, l_sum);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh->p_full[t]);

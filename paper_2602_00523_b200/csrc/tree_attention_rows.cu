@@ -254,7 +254,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                 // Probabilities are taken against the row's reference of the steps before: any reference within some 2^60
                 // of the row's maximum gives the same result, so a step need not look for its maximum first.  It shows in
                 // the step's sum whether the reference still serves; the first step of a segment, steps with masked
-                // scores and steps whose sum has grown beyond 2^30 go through the maximum.
+                // scores and steps whose sum has grown beyond 2^30 go through the maximum (rows that do not exist have no say).
                 bool by_max = masked || j == sg.s0;
                 if (!by_max) {
                     uint64_t acc[2] = {0ull, 0ull};
@@ -268,7 +268,7 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                     float sum_a, sum_b;
                     f2_unpack(f2_add(acc[0], acc[1]), sum_a, sum_b);
                     const float sum = sum_a + sum_b;
-                    by_max = __any_sync(0xffffffffu, !(sum < kMaxSum));
+                    by_max = __any_sync(0xffffffffu, row_ok && !(sum < kMaxSum));
                     if (!by_max) l_sum += sum;
                 }
                 if (by_max) {

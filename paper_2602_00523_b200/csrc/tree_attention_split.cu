@@ -70,7 +70,7 @@ constexpr int kSplitSmemBytes = 1024 /*align*/ + 2 * kQTileBytes + 2 * kPageStag
 // 64 scores of a page for one query row per thread: probabilities (bf16, over the first 32 columns of the S buffer), running
 // reference and sum.  The reference works as in the streaming kernels (see softmax_step in tree_attention_alt.cu); pv_done / parity: the P V product of the page before.
 __device__ __forceinline__ bool softmax_page(const SplitParams& p, Barriers* bars, uint64_t* pv_done, uint32_t pv_parity, uint32_t s_taddr,
-                                             uint32_t o_taddr, bool first, bool masked, int jt0, uint64_t anc,
+                                             uint32_t o_taddr, bool row_ok, bool first, bool masked, int jt0, uint64_t anc,
                                              float& m_ref, float& l_sum) {
     uint32_t sr[64];
     bool by_max = masked || first;
@@ -84,7 +84,7 @@ __device__ __forceinline__ bool softmax_page(const SplitParams& p, Barriers* bar
         float sum_a, sum_b;
         f2_unpack(f2_add(acc[0], acc[1]), sum_a, sum_b);
         const float sum = sum_a + sum_b;
-        by_max = __any_sync(0xffffffffu, !(sum < kMaxSum));
+        by_max = __any_sync(0xffffffffu, row_ok && !(sum < kMaxSum));
         if (!by_max) l_sum += sum;
     }
     if (by_max) {
@@ -353,7 +353,7 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
             if (warp_live) {
                 tc_fence_after();
                 const int jt0 = (pg_begin + j) * kPageSize - L;     // tree slot of the page's first key
-                ok = softmax_page(p, bars, &bars->pv_done[t], (j - 1) & 1, s_taddr + x * 64, o_taddr, j == 0, jt0 + kPageSize > 0, jt0, anc,
+                ok = softmax_page(p, bars, &bars->pv_done[t], (j - 1) & 1, s_taddr + x * 64, o_taddr, row_ok, j == 0, jt0 + kPageSize > 0, jt0, anc,
                                   m_ref, l_sum);
                 if (!ok) break;
             }

@@ -100,3 +100,35 @@ def test_launches_in_which_no_range_cuts_an_item(layers, heads, G, L, N, batch, 
         want = oracle.tree_attention(q[layer], kv["k_pool"][layer], kv["v_pool"][layer], table, kv["seq_len"], parent, off,
                                      heads * G, heads, 128, 64, 128 ** -0.5)
         check_attention(got[layer], want, bf16_slack=True)       # (bound: see test_attention_edges)
+
+
+@pytest.mark.parametrize("schedule", [1, 2], ids=["streaming", "split"])
+@pytest.mark.parametrize("N", [5, 21, 37])
+@pytest.mark.parametrize("behind", ["spare", "sequence"])
+def test_rows_behind_a_tree_do_not_change_a_bit_of_it(schedule, N, behind):
+    """The last warp of a tree's rows also holds rows that are not the tree's: spare capacity, or the next sequence's.  Rows
+    beside it that have to move their softmax reference must not make a row of the tree go another way."""
+    r = np.random.Generator(np.random.Philox(N))
+    heads, G, L = 2, 8, 1500
+    Ns = [N] if behind == "spare" else [N, 8]
+    kv = make_kv_cache(r, [L] * len(Ns), Ns, [0] * len(Ns), heads, shuffle=True)
+    for i, page in enumerate(kv["page_table"][0, :(L + N + 63) // 64]):      # scores that grow and fall along the context
+        kv["k_pool"][:, page] = bf16_bits((widen(kv["k_pool"][:, page]) * (1 + i // 2 % 12 / 2)).astype(np.float32))
+    parent = np.concatenate([random_tree(r, n)["parent"] for n in (N, 8)]).astype(np.int32)
+    off = np.concatenate([[0], np.cumsum(Ns)]).astype(np.int32)
+    q = make_q(r, N + 8, heads * G)
+    got = []
+    sage.sage_debug_attention_schedule(schedule)
+    try:
+        for f in (0.0, 30.0):
+            q_f = q.copy()
+            q_f[:, N:] = bf16_bits((widen(q[:, N:]) * f).astype(np.float32))
+            st = sage.new_status()
+            out = sage.sage_tree_attention(dev_bf16(q_f), dev_bf16(kv["k_pool"]), dev_bf16(kv["v_pool"]), dev_i32(kv["page_table"]),
+                                           dev_i32(kv["seq_len"]), dev_i32(parent), dev_i32(off), 128 ** -0.5, status=st)
+            torch.cuda.synchronize()
+            assert int(st.item()) == 0
+            got.append(host_bits(out)[0, :N])
+    finally:
+        sage.sage_debug_attention_schedule(0)
+    np.testing.assert_array_equal(got[0], got[1])
