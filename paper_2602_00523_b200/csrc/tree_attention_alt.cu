@@ -175,10 +175,10 @@ __device__ __forceinline__ void issue(const AttnParams& p, Shared* sh, uint8_t* 
 __device__ __forceinline__ void softmax_step(uint32_t s_taddr, uint32_t o_taddr, float scale, bool row_ok, bool first, bool masked,
                                              int jt0, uint64_t anc, float& m_ref, float& l_sum) {
     uint32_t sr[128];
-    // Probabilities are taken against the row's reference of the steps before: any reference within some 2^60
-    // of the row's maximum gives the same result, so a step need not look for its maximum first.  It shows in
-    // the step's sum whether the reference still serves; the first step of a segment, steps with masked
-    // scores and steps whose sum has grown beyond 2^30 go through the maximum.
+    // Probabilities are taken against the row's reference of the steps before, which moves only when a score exceeds
+    // it by more than 2^8, so a step need not look for its maximum first.  It shows in the step's sum whether the
+    // reference still serves; the first step of a segment, steps with masked scores and steps whose sum has grown to
+    // kMaxSum go through the maximum.
     bool by_max = masked || first;
     if (!by_max) {
         uint64_t acc[2] = {0ull, 0ull};

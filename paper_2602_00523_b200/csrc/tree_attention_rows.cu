@@ -251,10 +251,10 @@ tree_attention_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorM
                 const int jt0 = j * kStepKeys - sg.L;            // tree slot of the step's first key
                 const bool masked = jt0 + kStepKeys > 0;     // reaches into the tree part (or past the end)
                 uint32_t sr[128];
-                // Probabilities are taken against the row's reference of the steps before: any reference within some 2^60
-                // of the row's maximum gives the same result, so a step need not look for its maximum first.  It shows in
-                // the step's sum whether the reference still serves; the first step of a segment, steps with masked
-                // scores and steps whose sum has grown beyond 2^30 go through the maximum (rows that do not exist have no say).
+                // Probabilities are taken against the row's reference of the steps before, which moves only when a score exceeds
+                // it by more than 2^8, so a step need not look for its maximum first.  It shows in the step's sum whether the
+                // reference still serves; the first step of a segment, steps with masked scores and steps whose sum has grown to
+                // kMaxSum go through the maximum (rows that do not exist have no say).
                 bool by_max = masked || j == sg.s0;
                 if (!by_max) {
                     uint64_t acc[2] = {0ull, 0ull};
