@@ -5,8 +5,8 @@
 // HBM.  Every thread copies its own 16-byte pieces asynchronously to shared memory, three batches
 // ahead, and is the only one to read them: no barrier in the stream, and 48 KB per CTA in flight
 // without registers to hold them.
-//  1. Every thread keeps softmax moments (s = sum e^(x-m), t = sum (x-m) e^(x-m), m a reference at
-//     most 8 below the largest element so far) in fp32 over its elements: about seven instructions
+//  1. Every thread keeps softmax moments (s = sum e^(x-m), t = sum (x-m) e^(x-m), m the largest
+//     element so far or larger) in fp32 over its elements: about seven instructions
 //     per logit, loads included.
 //  2. The K best.  After batches 0, 1, 3, 7, ... the CTA takes a threshold from its threads' largest
 //     elements: the q-th largest of the warps' r-th largest thread maxima, q = ceil(K / r), so that at
@@ -91,10 +91,11 @@ struct Moments {
     float m;           // reference, -1e30 before the first element
     uint64_t s2, t2;   // (even, odd) partial sums
     __device__ __forceinline__ void init() { m = -1e30f; s2 = 0; t2 = 0; }
-    // The reference only moves when an element exceeds it by more than 8 (any reference is exact; e^8 keeps
-    // the sums far from overflow), which after the first batch hardly ever happens: no divergent rescaling.
+    // The reference moves with the largest element, whose e^(x - m) is exactly 1 then (left up to 8 below it, a confident row's
+    // log-probability and entropy took the rounding of e^8).  After the first batch, whose maximum the CTA shares,
+    // that hardly ever happens: no divergent rescaling.
     __device__ __forceinline__ void rise(float mx) {
-        if (mx > m + 8.0f) {
+        if (mx > m) {
             const float c = expf(m - mx);
             float s0, s1, t0, t1;
             f2_unpack(s2, s0, s1);
@@ -104,18 +105,31 @@ struct Moments {
             m = mx;
         }
     }
-    __device__ __forceinline__ void add(float x0, float x1, uint64_t nm2) {
-        const uint64_t d2 = f2_add(f2_pack(x0, x1), nm2);
-        float y0, y1;
-        f2_unpack(f2_mul(d2, f2_pack(kLog2e, kLog2e)), y0, y1);
-        const uint64_t e2 = f2_pack(ex2(y0), ex2(y1));
-        s2 = f2_add(s2, e2);
-        t2 = f2_fma(d2, e2, t2);
-    }
-    __device__ __forceinline__ void add4(const float4& v) {
+    // The 16 elements of a batch are summed by themselves and then added: a long row's sums then take one rounding per batch at
+    // their full size instead of eight (148 rows of 152064 with a peak, error of the entropy against 64 bits, root mean
+    // square: 5.1e-7 -> 2.8e-7; 3.3e-7 if a row is cut into 32 chunks instead).
+    // kAll: every piece is there, else the first `n` of them.
+    template <bool kAll>
+    __device__ __forceinline__ void add_batch(const float4 (&v)[kBatch], int n) {
         const uint64_t nm2 = f2_pack(-m, -m);
-        add(v.x, v.y, nm2);
-        add(v.z, v.w, nm2);
+        uint64_t s = 0, t = 0;
+        auto add = [&](float x0, float x1) {
+            const uint64_t d2 = f2_add(f2_pack(x0, x1), nm2);
+            float y0, y1;
+            f2_unpack(f2_mul(d2, f2_pack(kLog2e, kLog2e)), y0, y1);
+            const uint64_t e2 = f2_pack(ex2(y0), ex2(y1));
+            s = f2_add(s, e2);
+            t = f2_fma(d2, e2, t);
+        };
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            if (kAll || u < n) {
+                add(v[u].x, v[u].y);
+                add(v[u].z, v[u].w);
+            }
+        }
+        s2 = f2_add(s2, s);
+        t2 = f2_add(t2, t);
     }
     __device__ __forceinline__ void add1(float x) {
         rise(x);
@@ -369,14 +383,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
             }
             mo.rise(mx);
             start(b + kStages);                                  // (into the slots just read)
-            if ((b + 1) * kBatch * kThreads <= n4) {
-#pragma unroll
-                for (int u = 0; u < kBatch; ++u) mo.add4(v[u]);
-            } else {
-#pragma unroll
-                for (int u = 0; u < kBatch; ++u)
-                    if (i0 + u * kThreads < n4) mo.add4(v[u]);
-            }
+            if ((b + 1) * kBatch * kThreads <= n4) mo.add_batch<true>(v, kBatch);
+            else mo.add_batch<false>(v, i0 < n4 ? (n4 - 1 - i0) / kThreads + 1 : 0);
         }
         copy_wait<0>();
         if (warp == 0) {
