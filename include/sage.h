@@ -82,6 +82,8 @@ typedef struct sage_tree_policy {
  *     Section 3.1) in entropy_topk[r], and alpha[r] = 1 - H / ln(k_entropy) clamped to
  *     [0,1] (Eq. 9); alpha = 1 when k_entropy == 1.
  * Any of entropy_full / entropy_topk / alpha / lse / topk_logprob may be NULL.
+ * Masked words of -inf are ranked behind all others, the lowest index first, and lse counts them as nothing; entropies
+ * of such rows, and alpha where one of them is among the k_entropy best, are not defined.
  * Optional expansion (Section 2.2 "Tree-based Drafting", Section 3.2 "Dynamic Tree
  * Construction"): when draft_token != NULL, logits row r belongs to global node r and
  *   draft_token[i] = topk_idx[(n0 + parent[i])*k + rank[i]]  for non-root nodes,

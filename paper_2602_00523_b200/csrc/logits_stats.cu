@@ -305,6 +305,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
     // (read and raised after the barrier in the first cta_threshold)
     for (int i = tid; i < kListCap + kWarps * SAGE_MAX_TOPK; i += kThreads) s_list[i] = 0;
     if (tid == 0) { s_n = 0; s_nq = 0; s_thr = 0; }
+    if (tid < SAGE_MAX_TOPK) { s_best[tid] = 0; s_idx[tid] = -1; }       // (stays where a row has fewer candidates, all others NaN)
     // (the other half of this barrier, before the first store to the first CTA's memory: that CTA runs by then)
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
@@ -340,7 +341,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
             }
             thr = max(thr, *(volatile uint32_t*)&s_thr);
             const float thr_x = thr ? key_value(thr) : -INFINITY;
-            if (__any_sync(0xffffffffu, mx >= thr_x && mx != -INFINITY)) {
+            if (__any_sync(0xffffffffu, mx >= thr_x)) {
                 // this thread's elements that reach the threshold, one bit each
                 uint32_t mask = 0;
 #pragma unroll
@@ -349,6 +350,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
                         mask |= ((v[u].x >= thr_x ? 1u : 0u) | (v[u].y >= thr_x ? 2u : 0u) | (v[u].z >= thr_x ? 4u : 0u) |
                                  (v[u].w >= thr_x ? 8u : 0u)) << (4 * u);
                 }
+                // (-inf counts, the lowest indices first, until the warp's queue is full of what lies in front of it)
+                if (mx == -INFINITY && wq.kth != 0) mask = 0;
                 if (mask) {
                     int at = atomicAdd(&s_n, __popc(mask));
                     for (; mask != 0 && at < kListCap; ++at) {
@@ -392,7 +395,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
                 const int i = begin + 4 * n4 + j;
                 const float x = rowp[i];
                 const uint64_t key = make_key(x, i);
-                if (key > wq.kth) wq.insert(key, lane);
+                if (x == x && key > wq.kth) wq.insert(key, lane);
                 if (lane == j) mo.add1(x);
             }
         }
@@ -518,10 +521,11 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
         if (lane < p.k) p.topk_idx[(size_t)row * p.k + lane] = s_idx[lane];
         if (p.draft_token) hand_tokens(p, row, lane, s_idx);
     } else if (warp == 2 && (p.entropy_topk || p.alpha)) {
-        const double v = lane < p.k_entropy ? (double)key_value((uint32_t)(s_best[lane] >> 32)) : 0.0;
+        const bool have = lane < p.k_entropy && s_best[lane] != 0;
+        const double v = have ? (double)key_value((uint32_t)(s_best[lane] >> 32)) : 0.0;
         const double v1 = __shfl_sync(0xffffffffu, v, 0);
         double w = 0.0, wd = 0.0;                        // w_j = P_j / P_1
-        if (lane < p.k_entropy) {
+        if (have) {
             const double d = v - v1;
             w = exp(d);
             wd = w * d;

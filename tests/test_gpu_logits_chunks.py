@@ -103,3 +103,33 @@ def test_rows_with_peaks_are_as_exact_as_32_bit_sums_allow(peaks, entropy_bound,
     rms = lambda e: float(np.sqrt((e ** 2).mean()))                                              # noqa: E731
     assert rms(got["entropy_full"] - H) <= entropy_bound
     assert rms(got["topk_logprob"][:, 0] - (lg.max(axis=1).astype(np.float64) - lse)) <= logprob_bound
+
+
+@pytest.mark.parametrize("rows_more", [0, 148])
+def test_rows_with_few_finite_logits_give_real_indices(rows_more):
+    """Masks of -inf that leave fewer elements than candidates (allowed tokens of a grammar): the finite ones first, then the
+    lowest of the masked indices.  Elements that are no number are never candidates; without any other the index is -1."""
+    V, k = 6 * BATCH + 3, 10
+    r = np.random.Generator(np.random.Philox(14))
+    lg = np.full((8 + rows_more, V), -np.inf, np.float32)
+    lg[1, [V - 1, 5, 2 * BATCH + 77]] = 3.0, 1.0, 2.0
+    lg[2, [V - 2, BATCH]] = -1.0, 4.0
+    lg[3, r.permutation(V)[:9]] = r.standard_normal(9)
+    lg[4, 3 * BATCH:3 * BATCH + 9] = 2.5
+    lg[5, -k:] = r.standard_normal(k)                # as many as are asked for
+    lg[6, :BATCH] = r.standard_normal(BATCH)         # whole blocks without a finite element
+    lg[7] = np.nan
+    lg[7, [40, V - 1]] = 1.0, 2.0
+    lg[8:] = r.standard_normal((rows_more, V))
+    got, st = expand(lg, k, k)
+    assert st == 0
+    ok = np.arange(len(lg)) != 7
+    np.testing.assert_array_equal(got["topk_idx"][ok], oracle.topk(lg[ok], k))
+    assert list(got["topk_idx"][7]) == [V - 1, 40] + [-1] * 8
+    some = ok & (np.arange(len(lg)) > 0)
+    x = lg[some].astype(np.float64)
+    lse = x.max(axis=1) + np.log(np.exp(x - x.max(axis=1, keepdims=True)).sum(axis=1))
+    np.testing.assert_allclose(got["lse"][some], lse, rtol=1e-6, atol=1e-6)
+    want = np.take_along_axis(x, got["topk_idx"][some].astype(np.int64), 1) - lse[:, None]
+    np.testing.assert_allclose(got["topk_logprob"][some], want, rtol=1e-5, atol=1e-5)
+    assert np.abs(got["alpha"][5:7] - oracle.confidence(lg[5:7], k)[1]).max() <= 1e-5
