@@ -699,9 +699,9 @@ template <int kBytes, typename K>
 static bool allow_shared_memory(K kernel) {
     static std::atomic<bool> done[64];
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    if (!succeeded(cudaGetDevice(&dev)) || dev < 0 || dev >= 64) return false;
     if (!done[dev].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes) != cudaSuccess) return false;
+        if (!succeeded(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes))) return false;
         done[dev].store(true, std::memory_order_release);
     }
     return true;

@@ -547,10 +547,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
 static bool allow_stream_buffer() {
     static std::atomic<bool> done[64];
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    if (!succeeded(cudaGetDevice(&dev)) || dev < 0 || dev >= 64) return false;
     if (!done[dev].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(expand_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStreamBytes) != cudaSuccess)
-            return false;
+        if (!succeeded(cudaFuncSetAttribute(expand_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStreamBytes))) return false;
         done[dev].store(true, std::memory_order_release);
     }
     return true;
@@ -590,9 +589,7 @@ static int launch_expand(const ExpandParams& p, cudaStream_t stream) {
     const int C = pick_chunks(p.rows, p.vocab);
     ExpandParams q = p;
     q.chunk_len = (((p.vocab + C - 1) / C) + 3) & ~3;
-    if (launch(expand_topk_kernel, dim3((unsigned)C, (unsigned)p.rows), kThreads, kStreamBytes, stream, C, q) != cudaSuccess)
-        return SAGE_ERR_CUDA;
-    return launch_status();
+    return launch_status(launch(expand_topk_kernel, dim3((unsigned)C, (unsigned)p.rows), kThreads, kStreamBytes, stream, C, q));
 }
 
 }  // namespace sage

@@ -75,6 +75,13 @@ inline cudaError_t launch(void (*kernel)(Params...), dim3 grid, int threads, siz
 
 inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
-inline int launch_status() { return cudaGetLastError() == cudaSuccess ? SAGE_OK : SAGE_ERR_CUDA; }
+// A call's result as the entry points return it.  The runtime also keeps a failure as the thread's last error: it is taken
+// away here, so that no later call can mistake it for its own.
+inline bool succeeded(cudaError_t e) {
+    if (e == cudaSuccess) return true;
+    (void)cudaGetLastError();
+    return false;
+}
+inline int launch_status(cudaError_t e) { return succeeded(e) ? SAGE_OK : SAGE_ERR_CUDA; }
 
 }  // namespace sage

@@ -23,7 +23,7 @@ static EncodeTiledFn encode_fn() {
     if (!fn) {
         void* sym = nullptr;
         cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &qres) == cudaSuccess &&
+        if (succeeded(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &qres)) &&
             qres == cudaDriverEntryPointSuccess)
             fn = reinterpret_cast<EncodeTiledFn>(sym);
     }
@@ -102,16 +102,10 @@ static bool make_q_map(CUtensorMap* map, const void* q, int n_layers, int sum_no
 static int resident_ctas() {
     static int cached[64] = {};
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
-        (void)cudaGetLastError();
-        return 148;
-    }
+    if (!succeeded(cudaGetDevice(&dev)) || dev < 0 || dev >= 64) return 148;
     if (!cached[dev]) {
         int n = 0;
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) {
-            (void)cudaGetLastError();
-            return 148;
-        }
+        if (!succeeded(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) || n < 1) return 148;
         cached[dev] = n;
     }
     return cached[dev];

@@ -585,14 +585,12 @@ int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int
     // less than the compiler loses on the softmax loops (57 -> 61 us; as functions, 80 layers: 2.72 -> 2.80 ms).
     const int most_nodes = sum_nodes < SAGE_MAX_NODES ? sum_nodes : SAGE_MAX_NODES;
     if (!allow_shared_memory<kSmemBytes>(tree_attention_alt_kernel) ||
-        sage::launch(tree_attention_alt_kernel, dim3(p.n_ctas), kAttnThreads, kSmemBytes, stream, 0, p, qmap, kmap, vmap) != cudaSuccess)
+        !succeeded(sage::launch(tree_attention_alt_kernel, dim3(p.n_ctas), kAttnThreads, kSmemBytes, stream, 0, p, qmap, kmap, vmap)))
         return SAGE_ERR_CUDA;
     if (most_nodes * G > kRowTile && !launch_rows(p, qmap, kmap, vmap, stream)) return SAGE_ERR_CUDA;
-    if (p.n_ctas > 1) {
-        // (a gang's boundaries and members: as many as CTAs; blocks that find no cut item leave)
-        if (sage::launch(attention_merge_kernel, dim3(p.n_ctas, kMergeParts), kRowsPerCta, 0, stream, 0, p) != cudaSuccess) return SAGE_ERR_CUDA;
-    }
-    return launch_status();
+    if (p.n_ctas <= 1) return SAGE_OK;
+    // (a gang's boundaries and members: as many as CTAs; blocks that find no cut item leave)
+    return launch_status(sage::launch(attention_merge_kernel, dim3(p.n_ctas, kMergeParts), kRowsPerCta, 0, stream, 0, p));
 }
 
 }  // namespace stream

@@ -368,7 +368,7 @@ bool launch_rows(const AttnParams& p, const CUtensorMap& qmap, const CUtensorMap
     // itself, the order in which SMs become free behind the kernel before decides, and a gang spread over both dies
     // costs power: 60 nodes, 80 layers x 16k keys at the power limit, 3000 -> 2815 us.)
     return allow_shared_memory<kSmemBytes>(tree_attention_rows_kernel) &&
-           sage::launch(tree_attention_rows_kernel, dim3(p.n_ctas), kAttnThreads, kSmemBytes, stream, p.n_rp, p, qmap, kmap, vmap) == cudaSuccess;
+           succeeded(sage::launch(tree_attention_rows_kernel, dim3(p.n_ctas), kAttnThreads, kSmemBytes, stream, p.n_rp, p, qmap, kmap, vmap));
 }
 
 }  // namespace stream

@@ -531,15 +531,13 @@ int launch(int n_layers, int n_pages, const int32_t* page_table, int max_pages_p
     p.producer_off = producer_off;
     const dim3 grid(S, row_pairs_for(sum_nodes, G), n_layers * batch * n_kv_heads);
     if (!allow_shared_memory<kSplitSmemBytes>(tree_attention_split_kernel) ||
-        sage::launch(tree_attention_split_kernel, grid, kSplitThreads, kSplitSmemBytes, stream, 0, p, qmap, kmap, vmap) != cudaSuccess)
+        !succeeded(sage::launch(tree_attention_split_kernel, grid, kSplitThreads, kSplitSmemBytes, stream, 0, p, qmap, kmap, vmap)))
         return SAGE_ERR_CUDA;
-    if (S > 1) {
-        const size_t rows_total = (size_t)sum_nodes * n_q_heads;
-        const dim3 mg((unsigned)((rows_total + 31) / 32), n_layers, 4);
-        const auto merge = S <= 4 ? attention_split_merge_kernel<4> : S <= 8 ? attention_split_merge_kernel<8> : attention_split_merge_kernel<kMaxSplits>;
-        if (sage::launch(merge, mg, 256, 0, stream, 0, p) != cudaSuccess) return SAGE_ERR_CUDA;
-    }
-    return launch_status();
+    if (S == 1) return SAGE_OK;
+    const size_t rows_total = (size_t)sum_nodes * n_q_heads;
+    const dim3 mg((unsigned)((rows_total + 31) / 32), n_layers, 4);
+    const auto merge = S <= 4 ? attention_split_merge_kernel<4> : S <= 8 ? attention_split_merge_kernel<8> : attention_split_merge_kernel<kMaxSplits>;
+    return launch_status(sage::launch(merge, mg, 256, 0, stream, 0, p));
 }
 
 }  // namespace split

@@ -314,9 +314,9 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kv_kernel(const Compa
 static bool allow_large_cluster() {
     static std::atomic<bool> done[64];
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    if (!succeeded(cudaGetDevice(&dev)) || dev < 0 || dev >= 64) return false;
     if (!done[dev].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(compact_kv_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+        if (!succeeded(cudaFuncSetAttribute(compact_kv_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1))) return false;
         done[dev].store(true, std::memory_order_release);
     }
     return true;
@@ -480,17 +480,16 @@ extern "C" int sage_select_tree(const float* alpha, const int32_t* alpha_row, in
     if (batch == 0) return SAGE_OK;
     SelectParams p{alpha, alpha_row, batch, *policy, template_id, depth_cont, width_cont, bank_parent,
                    bank_rank, bank_n_nodes, next_parent, next_rank, next_node_offsets, status};
-    (void)launch(select_tree_kernel, dim3((batch + 127) / 128), 128, 0, as_stream(stream), 0, p);
-    if (handover) (void)launch(handover_trees_kernel, dim3(1), 256, 0, as_stream(stream), 0, p);
-    return launch_status();
+    const int code = launch_status(launch(select_tree_kernel, dim3((batch + 127) / 128), 128, 0, as_stream(stream), 0, p));
+    if (code != SAGE_OK || !handover) return code;
+    return launch_status(launch(handover_trees_kernel, dim3(1), 256, 0, as_stream(stream), 0, p));
 }
 
 extern "C" int sage_build_ancestor_mask(const int32_t* parent, const int32_t* node_offsets, int batch,
                                         uint64_t* anc, int32_t* status, void* stream) {
     if (!parent || !node_offsets || !anc || batch < 0) return SAGE_ERR_INVALID_ARG;
     if (batch == 0) return SAGE_OK;
-    (void)launch(ancestor_mask_kernel, dim3(batch), SAGE_MAX_NODES, 0, as_stream(stream), 0, parent, node_offsets, anc, status);
-    return launch_status();
+    return launch_status(launch(ancestor_mask_kernel, dim3(batch), SAGE_MAX_NODES, 0, as_stream(stream), 0, parent, node_offsets, anc, status));
 }
 
 extern "C" int sage_accept(const int32_t* parent, const int32_t* draft_token, const int32_t* target_argmax,
@@ -501,9 +500,8 @@ extern "C" int sage_accept(const int32_t* parent, const int32_t* draft_token, co
     if (batch < 0 || max_path < 1) return SAGE_ERR_INVALID_ARG;
     if (batch == 0) return SAGE_OK;
     const int wpb = 4;
-    (void)launch(accept_kernel, dim3((batch + wpb - 1) / wpb), wpb * 32, 0, as_stream(stream), 0, parent, draft_token,
-                 target_argmax, node_offsets, batch, max_path, path, path_len, bonus_token, status);
-    return launch_status();
+    return launch_status(launch(accept_kernel, dim3((batch + wpb - 1) / wpb), wpb * 32, 0, as_stream(stream), 0, parent, draft_token,
+                 target_argmax, node_offsets, batch, max_path, path, path_len, bonus_token, status));
 }
 
 extern "C" int sage_compact_kv(void* k_pool, void* v_pool, int64_t layer_stride_elems, int n_layers, int n_pages,
@@ -525,9 +523,7 @@ extern "C" int sage_compact_kv(void* k_pool, void* v_pool, int64_t layer_stride_
     CompactParams p{(__nv_bfloat16*)k_pool, (__nv_bfloat16*)v_pool, layer_stride_elems, n_layers, n_pages,
                     max_pages_per_seq, max_path, n_kv_heads, blocks, page_table, seq_len, path, path_len, status};
     if (blocks > 8 && !allow_large_cluster()) return SAGE_ERR_CUDA;
-    if (launch(compact_kv_kernel, dim3((unsigned)(blocks * batch)), kCompactThreads, 0, as_stream(stream), blocks, p) != cudaSuccess)
-        return SAGE_ERR_CUDA;
-    return launch_status();
+    return launch_status(launch(compact_kv_kernel, dim3((unsigned)(blocks * batch)), kCompactThreads, 0, as_stream(stream), blocks, p));
 }
 
 extern "C" int sage_grow_tree(const int32_t* topk_idx, const float* topk_logprob, int k, const float* alpha,
@@ -546,8 +542,7 @@ extern "C" int sage_grow_tree(const int32_t* topk_idx, const float* topk_logprob
     if (batch == 0) return SAGE_OK;
     GrowParams p{topk_idx, topk_logprob, k, alpha, alpha_row, *policy, n_max, parent, rank, depth, token,
                  cum_logprob, n_nodes, frontier_begin, d_max_seq, status};
-    (void)launch(grow_tree_kernel, dim3(batch), kGrowThreads, 0, as_stream(stream), 0, p);
-    return launch_status();
+    return launch_status(launch(grow_tree_kernel, dim3(batch), kGrowThreads, 0, as_stream(stream), 0, p));
 }
 
 extern "C" int sage_update_history(const int32_t* path_len, int batch, const sage_history_policy* policy,
@@ -559,9 +554,8 @@ extern "C" int sage_update_history(const int32_t* path_len, int batch, const sag
         return SAGE_ERR_INVALID_ARG;
     if (policy->window > 1024) return SAGE_ERR_UNSUPPORTED;
     if (batch == 0) return SAGE_OK;
-    (void)launch(update_history_kernel, dim3((batch + 127) / 128), 128, 0, as_stream(stream), 0, path_len, batch, *policy,
-                 window_buf, count, d_max, status);
-    return launch_status();
+    return launch_status(launch(update_history_kernel, dim3((batch + 127) / 128), 128, 0, as_stream(stream), 0, path_len, batch, *policy,
+                 window_buf, count, d_max, status));
 }
 
 extern "C" const char* sage_status_string(int code) {
