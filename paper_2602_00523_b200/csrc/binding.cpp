@@ -74,22 +74,43 @@ struct Names {
 } N;
 
 struct Missing {};                                  // `out` lacks an entry
-PyObject* entry(PyObject* dict, PyObject* name) {
-    PyObject* v = PyDict_GetItemWithError(dict, name);
-    if (v == nullptr) {
-        if (PyErr_Occurred()) throw Failed{};
-        throw Missing{};
+// A dict, or any other mapping, of tensors; what another mapping hands out is held until the call has been made.
+class Tensors {
+public:
+    explicit Tensors(PyObject* o) : o_(o), dict_(PyDict_Check(o)) {
+        if (!dict_ && !PyMapping_Check(o)) fail(PyExc_TypeError, "a dict of tensors is expected");
     }
-    return v;
-}
-PyObject* entry_or_none(PyObject* dict, PyObject* name) {
-    PyObject* v = PyDict_GetItemWithError(dict, name);
-    if (v == nullptr && PyErr_Occurred()) throw Failed{};
-    return v;
-}
-void want_dict(PyObject* o) {
-    if (!PyDict_Check(o)) fail(PyExc_TypeError, "a dict of tensors is expected");
-}
+    ~Tensors() {
+        for (int i = 0; i < n_held_; ++i) Py_DECREF(held_[i]);
+    }
+    Tensors(const Tensors&) = delete;
+    Tensors& operator=(const Tensors&) = delete;
+    PyObject* get(PyObject* name) {                 // nullptr where there is none
+        if (dict_) {
+            PyObject* v = PyDict_GetItemWithError(o_, name);
+            if (v == nullptr && PyErr_Occurred()) throw Failed{};
+            return v;
+        }
+        PyObject* v = PyObject_GetItem(o_, name);
+        if (v == nullptr) {
+            if (!PyErr_ExceptionMatches(PyExc_KeyError)) throw Failed{};
+            PyErr_Clear();
+            return nullptr;
+        }
+        return held_[n_held_++] = v;
+    }
+    PyObject* operator[](PyObject* name) {
+        PyObject* v = get(name);
+        if (v == nullptr) throw Missing{};
+        return v;
+    }
+
+private:
+    PyObject* o_;
+    bool dict_;
+    int n_held_ = 0;
+    PyObject* held_[8];                             // (no call asks for more)
+};
 
 template <typename F>
 PyObject* guarded(Py_ssize_t n_args, Py_ssize_t want, F body) {
@@ -123,14 +144,13 @@ PyObject* expand_topk(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const at::Tensor& lg = tensor(a[0]);
         if (lg.scalar_type() != at::kFloat || lg.dim() != 2 || lg.stride(1) != 1)
             fail(PyExc_AssertionError, "logits: fp32 [rows, vocab] with contiguous rows");
-        PyObject* o = a[7];
-        want_dict(o);
+        Tensors o(a[7]);
         const int k = integer(a[1]), ke = integer(a[2]);
         const bool tree = a[3] != Py_None, is_static = a[11] == Py_True;
-        int32_t* idx = ptr<int32_t>(entry(o, N.topk_idx));
-        float *lp = ptr<float>(entry(o, N.topk_logprob)), *hf = ptr<float>(entry(o, N.entropy_full)),
-              *ht = ptr<float>(entry(o, N.entropy_topk)), *al = ptr<float>(entry(o, N.alpha)), *ls = ptr<float>(entry(o, N.lse));
-        int32_t* tok = ptr<int32_t>(tree ? entry(o, N.draft_token) : entry_or_none(o, N.draft_token));
+        int32_t* idx = ptr<int32_t>(o[N.topk_idx]);
+        float *lp = ptr<float>(o[N.topk_logprob]), *hf = ptr<float>(o[N.entropy_full]),
+              *ht = ptr<float>(o[N.entropy_topk]), *al = ptr<float>(o[N.alpha]), *ls = ptr<float>(o[N.lse]);
+        int32_t* tok = ptr<int32_t>(tree ? o[N.draft_token] : o.get(N.draft_token));
         if (!is_static && a[8] == Py_None) throw Missing{};
         const int batch = tree ? size32(length(a[5]) - 1) : 0;
         const int32_t *parent = ptr<int32_t>(a[3]), *rank = ptr<int32_t>(a[4]), *offs = ptr<int32_t>(a[5]), *root = ptr<int32_t>(a[6]);
@@ -153,15 +173,14 @@ PyObject* expand_topk(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // alpha, alpha_row, batch, policy, out, bank_parent, bank_rank, bank_n_nodes, handover?, status, stream
 PyObject* select_tree(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 11, [&]() -> int {
-        PyObject* o = a[4];
-        want_dict(o);
+        Tensors o(a[4]);
         const sage_tree_policy pol = structure<sage_tree_policy>(a[3]);
         const bool handover = PyObject_IsTrue(a[8]) == 1;
-        int32_t* id = ptr<int32_t>(entry(o, N.template_id));
-        float *d = ptr<float>(entry(o, N.depth_cont)), *w = ptr<float>(entry(o, N.width_cont));
-        int32_t* np = ptr<int32_t>(handover ? entry(o, N.next_parent) : entry_or_none(o, N.next_parent));
-        int32_t* nr = ptr<int32_t>(handover ? entry(o, N.next_rank) : entry_or_none(o, N.next_rank));
-        int32_t* no = ptr<int32_t>(handover ? entry(o, N.next_node_offsets) : entry_or_none(o, N.next_node_offsets));
+        int32_t* id = ptr<int32_t>(o[N.template_id]);
+        float *d = ptr<float>(o[N.depth_cont]), *w = ptr<float>(o[N.width_cont]);
+        int32_t* np = ptr<int32_t>(handover ? o[N.next_parent] : o.get(N.next_parent));
+        int32_t* nr = ptr<int32_t>(handover ? o[N.next_rank] : o.get(N.next_rank));
+        int32_t* no = ptr<int32_t>(handover ? o[N.next_node_offsets] : o.get(N.next_node_offsets));
         const float* alpha = ptr<float>(a[0]);
         const int32_t *row = ptr<int32_t>(a[1]), *bp = ptr<int32_t>(a[5]), *br = ptr<int32_t>(a[6]), *bn = ptr<int32_t>(a[7]);
         const int batch = a[2] != Py_None ? integer(a[2]) : size32(a[1] != Py_None ? length(a[1]) : length(a[0]));
@@ -174,20 +193,19 @@ PyObject* select_tree(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // topk_idx, topk_logprob, alpha, policy, tree, alpha_row, n_max, d_max_seq, status, stream
 PyObject* grow_tree(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 10, [&]() -> int {
-        PyObject* t = a[4];
-        want_dict(t);
+        Tensors t(a[4]);
         const sage_tree_policy pol = structure<sage_tree_policy>(a[3]);
         const at::Tensor& idx = tensor(a[0]);
         if (idx.dim() != 2) fail(PyExc_AssertionError, "topk_idx: [slots, k]");
-        PyObject* nn = entry(t, N.n_nodes);
+        PyObject* nn = t[N.n_nodes];
         const int batch = size32(length(nn)), k = size32(idx.size(1)), n_max = integer(a[6]);
         const int32_t* ix = ptr<int32_t>(a[0]);
         const float *lp = ptr<float>(a[1]), *alpha = ptr<float>(a[2]), *dm = ptr<float>(a[7]);
         const int32_t* row = ptr<int32_t>(a[5]);
-        int32_t *parent = ptr<int32_t>(entry(t, N.parent)), *rank = ptr<int32_t>(entry(t, N.rank)),
-                *depth = ptr<int32_t>(entry(t, N.depth)), *token = ptr<int32_t>(entry(t, N.token));
-        float* cum = ptr<float>(entry(t, N.cum_logprob));
-        int32_t *nodes = ptr<int32_t>(nn), *fb = ptr<int32_t>(entry(t, N.frontier_begin)), *status = ptr<int32_t>(a[8]);
+        int32_t *parent = ptr<int32_t>(t[N.parent]), *rank = ptr<int32_t>(t[N.rank]),
+                *depth = ptr<int32_t>(t[N.depth]), *token = ptr<int32_t>(t[N.token]);
+        float* cum = ptr<float>(t[N.cum_logprob]);
+        int32_t *nodes = ptr<int32_t>(nn), *fb = ptr<int32_t>(t[N.frontier_begin]), *status = ptr<int32_t>(a[8]);
         void* stream = stream_of(a[9]);
         return without_gil([&] {
             return sage_grow_tree(ix, lp, k, alpha, row, batch, &pol, n_max, parent, rank, depth, token, cum, nodes, fb, dm, status, stream);
@@ -266,10 +284,9 @@ PyObject* tree_attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // parent, draft_token, target_argmax, node_offsets, max_path, out, status, stream
 PyObject* accept(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded(n, 8, [&]() -> int {
-        PyObject* o = a[5];
-        want_dict(o);
-        int32_t *path = ptr<int32_t>(entry(o, N.path)), *pl = ptr<int32_t>(entry(o, N.path_len)),
-                *bonus = ptr<int32_t>(entry(o, N.bonus_token));
+        Tensors o(a[5]);
+        int32_t *path = ptr<int32_t>(o[N.path]), *pl = ptr<int32_t>(o[N.path_len]),
+                *bonus = ptr<int32_t>(o[N.bonus_token]);
         const int32_t *parent = ptr<int32_t>(a[0]), *draft = ptr<int32_t>(a[1]), *target = ptr<int32_t>(a[2]), *offs = ptr<int32_t>(a[3]);
         const int batch = size32(length(a[3]) - 1), max_path = integer(a[4]);
         int32_t* status = ptr<int32_t>(a[6]);

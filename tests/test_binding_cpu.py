@@ -1,4 +1,6 @@
 """The marshalling of calls rejects what the kernels could not take, before anything is enqueued (no GPU needed)."""
+from collections import UserDict, defaultdict
+
 import pytest
 import torch
 
@@ -22,3 +24,21 @@ def test_host_tensors_and_wrong_types_are_rejected():
 def test_static_variant_allocates_nothing():
     with pytest.raises(KeyError, match="topk_idx"):
         sage.sage_expand_topk_static(torch.zeros(2, 8), 2, 2, out={})
+
+
+@pytest.mark.parametrize("kind", [dict, UserDict, lambda d: defaultdict(lambda: torch.zeros(4), d)])
+def test_outputs_and_trees_may_be_any_mapping(kind):
+    """Anything with items by name serves: the calls below get as far as the check of where the tensors are."""
+    x, i = torch.zeros(2, 8), torch.zeros(2, dtype=torch.int32)
+    names = ["topk_idx", "topk_logprob", "entropy_full", "entropy_topk", "alpha", "lse"]
+    with pytest.raises(ValueError, match="device tensors only"):
+        sage.sage_expand_topk_static(x, 2, 2, out=kind({n: x for n in names}))
+    tree = {n: i for n in ("parent", "rank", "depth", "token", "n_nodes", "frontier_begin")}
+    with pytest.raises(ValueError, match="device tensors only"):
+        sage.sage_grow_tree(torch.zeros(128, 4, dtype=torch.int32), x, x, sage.make_policy([]), kind({**tree, "cum_logprob": x}))
+    with pytest.raises(ValueError, match="device tensors only"):
+        sage.sage_accept(i, i, i, i, 4, out=kind({"path": i, "path_len": i, "bonus_token": i}))
+    with pytest.raises(KeyError):
+        sage.sage_grow_tree(torch.zeros(128, 4, dtype=torch.int32), x, x, sage.make_policy([]), UserDict(parent=i))
+    with pytest.raises(TypeError):
+        sage.sage_accept(i, i, i, i, 4, out=3)
