@@ -12,8 +12,8 @@
 //     elements: the q-th largest of the warps' r-th largest thread maxima, q = ceil(K / r), so that at
 //     least K elements reach it.  Elements that reach the threshold are appended to the CTA's list, some
 //     50 in all; the rest of the stream only compares each thread's largest element of a batch with
-//     it.  When the list is full (ascending data), the warps' sorted queues take over, whose K-th value
-//     raises the threshold for the whole CTA too.  Keys order by value (with -0 == +0) and then by
+//     it.  When the list is full (ascending data, many equal values), the warps' sorted queues take
+//     over, whose K-th value raises the threshold for the whole CTA too.  Keys order by value (with -0 == +0) and then by
 //     lowest index, so every merge order gives the same answer.
 //  3. Moments (in fp64) and the K best keys of every CTA go to the first CTA of the cluster through
 //     distributed shared memory; it ranks them, derives lse, entropies, log-probs and alpha, and
@@ -316,7 +316,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
     wq.init(p.K);
     {
         const int n_batch = (n4 + kBatch * kThreads - 1) / (kBatch * kThreads);
-        uint32_t thr = 0;
+        // Value key that this warp's elements still have to reach: above what K elements in front of them reach already, since
+        // of equal values the lowest index counts.
+        uint32_t least = 0;
         float top = -INFINITY;                                   // this thread's largest element so far
         for (int b = 0; b < n_batch; ++b) {
             copy_wait<kStages - 1>();
@@ -332,10 +334,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
             }
             const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
             top = fmaxf(top, mx);
+            uint32_t thr = least;
             if ((b & (b + 1)) == 0) {
                 // after batches 0, 1, 3, 7, ...: as many elements pass in each doubling of the stream
                 uint32_t most;
-                thr = max(thr, cta_threshold(p.K, top == -INFINITY ? 0u : order_key(top), s_wtop[__popc(b) & 1], &most, lane, warp));
+                const uint32_t reached = cta_threshold(p.K, top == -INFINITY ? 0u : order_key(top), s_wtop[__popc(b) & 1], &most, lane, warp);
+                thr = max(thr, reached);
+                least = max(least, reached ? reached + 1 : 0);   // (from the next batch on)
                 // threads share their first reference, so that the sums hardly ever need rescaling when they are merged
                 if (b == 0 && most) mo.m = fmaxf(mo.m, key_value(most));
             }
@@ -350,8 +355,19 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
                         mask |= ((v[u].x >= thr_x ? 1u : 0u) | (v[u].y >= thr_x ? 2u : 0u) | (v[u].z >= thr_x ? 4u : 0u) |
                                  (v[u].w >= thr_x ? 8u : 0u)) << (4 * u);
                 }
-                // (-inf counts, the lowest indices first, until the warp's queue is full of what lies in front of it)
-                if (mx == -INFINITY && wq.kth != 0) mask = 0;
+                if (__reduce_add_sync(0xffffffffu, __popc(mask)) > 2 * 32) {
+                    // Many at a time, equal ones most likely (masked words): of those at the threshold itself only the first K
+                    // count, and whole pieces in front of an element, in this warp, tell most of the others.
+                    int before = 0;
+#pragma unroll
+                    for (int u = 0; u < kBatch; ++u) {
+                        const unsigned whole = __ballot_sync(0xffffffffu, ((mask >> (4 * u)) & 15u) == 15u);
+                        if (before + 4 * __popc(whole & ((1u << lane) - 1u)) >= p.K)
+                            mask &= ~(((v[u].x == thr_x ? 1u : 0u) | (v[u].y == thr_x ? 2u : 0u) | (v[u].z == thr_x ? 4u : 0u) |
+                                       (v[u].w == thr_x ? 8u : 0u)) << (4 * u));
+                        before += 4 * __popc(whole);
+                    }
+                }
                 if (mask) {
                     int at = atomicAdd(&s_n, __popc(mask));
                     for (; mask != 0 && at < kListCap; ++at) {
@@ -362,26 +378,35 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) expand_topk_kernel(const
                                               begin + 4 * (b * kBatch * kThreads + piece) + (e & 3));
                     }
                 }
-                unsigned todo = __ballot_sync(0xffffffffu, mask != 0);
-                if (todo) {
-                    // The list is full (ascending data, many equal values): the warp's queue takes the rest one by one, the
-                    // last lane's first, which fills the queue with values that stay.
-                    __syncwarp();                                // the whole warp reads what its lanes' copies left in shared memory
-                    while (todo) {
-                        const int src = 31 - __clz(todo);
-                        uint32_t m = __shfl_sync(0xffffffffu, mask, src);
-                        while (m) {
-                            const int e = 31 - __clz(m);
-                            m &= ~(1u << e);
-                            const int at = (e >> 2) * kThreads + warp * 32 + src;
-                            const float x = reinterpret_cast<const float*>(buf + at)[e & 3];
-                            const uint64_t key = make_key(x, begin + 4 * (b * kBatch * kThreads + at) + (e & 3));
-                            if (key > wq.kth) wq.insert(key, lane);
+                if (__any_sync(0xffffffffu, mask != 0)) {
+                    // The list is full (ascending or masked data, many equal values): the warp's queue takes the rest, the best
+                    // of all lanes first, so that a batch costs it K insertions at most.
+                    const int at0 = begin + 4 * (b * kBatch * kThreads + tid);
+                    auto best_left = [&]() {
+                        uint64_t best = 0;
+                        for (uint32_t m = mask; m; m &= m - 1) {
+                            const int e = __ffs(m) - 1, piece = (e >> 2) * kThreads;
+                            const uint64_t key = make_key(reinterpret_cast<const float*>(buf + piece + tid)[e & 3], at0 + 4 * piece + (e & 3));
+                            best = key > best ? key : best;
                         }
-                        todo &= ~(1u << src);
+                        return best;
+                    };
+                    uint64_t mine = best_left();
+                    while (true) {
+                        const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(mine >> 32));
+                        const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(mine >> 32) == hi ? (uint32_t)mine : 0u);
+                        const uint64_t best = ((uint64_t)hi << 32) | lo;
+                        if (best <= wq.kth) break;
+                        wq.insert(best, lane);
+                        if (mine == best) {
+                            const int off = (int)(0xffffffffu - lo) - at0;       // 4 * piece + element
+                            mask &= ~(1u << (off / (4 * kThreads) * 4 + (off & 3)));
+                            mine = best_left();
+                        }
                     }
-                    if (lane == 0 && (uint32_t)(wq.kth >> 32) > thr) atomicMax(&s_thr, (uint32_t)(wq.kth >> 32));
-                    __syncwarp();
+                    const uint32_t kth = (uint32_t)(wq.kth >> 32);
+                    if (kth) least = max(least, kth + 1);
+                    if (lane == 0 && kth > thr) atomicMax(&s_thr, kth);
                 }
             }
             mo.rise(mx);
@@ -564,7 +589,7 @@ static bool allow_stream_buffer() {
 static int pick_chunks(int rows, int vocab) {
     constexpr int kSms = 148;
     const int batch = kBatch * 4 * kThreads;
-    for (int c = kMaxChunks; c >= 2; --c) {                      // (every CTA gets at least one batch of elements)
+    for (int c = kMaxChunks; c >= 2; --c) {                      // (a CTA gets more than (c - 1) / c of a batch)
         if ((c - 1) * batch < vocab && (long)c * rows <= (c > 2 ? 272 : 2 * kSms)) return c;
     }
     if (vocab < 16 * batch) return 1;
