@@ -54,10 +54,11 @@ constexpr int kTileBytes = 2 * kTileHalfBytes;              // K or V tile of on
 constexpr int kQTileBytes = kRowTile * kHeadDim * 2;        // 32 KB
 constexpr int kQHalfBytes = kRowTile * 64 * 2;              // one 64-wide d-half of a Q tile: 16 KB
 constexpr int kAttnThreads = 384;              // 2 softmax warpgroups + one warpgroup of TMA warp, MMA warp and two idle warps
-// A step whose sum of probabilities stays below this keeps its reference: none of its scores exceeds it by 2^8 then, which is
-// where the maximum would move it.  (With 2^30 the dominant key of a row whose scores grow had a probability rounded to bf16
-// instead of an exact one: error 1.8e-3 -> 2.15e-3 of the outputs' norm.  Normal scores rarely reach 2^8: no time lost.)
-constexpr float kMaxSum = 256.f;
+// A row's step whose probabilities sum to this or more goes through its maximum, to which the reference then moves.  Lower, rows of
+// widely spread scores compute many steps twice (one layer, 60 nodes, 16k keys of three times the usual spread: 54.8 us at 2^8,
+// 49.2 at 2^10, 44.7 here, 40.5 for the usual); higher, the dominant probability of a row is rounded to bf16 more often where it
+// would be exactly 1 (error on growing scores 1.92e-3 of the outputs' norm at 2^8, 1.95e-3 here, 1.98e-3 at 2^14, 2.15e-3 at 2^30).
+constexpr float kMaxSum = 4096.f;
 constexpr int kMinSteps = 2;                   // no range shorter than this (short contexts are latency-bound)
 
 struct AttnParams {

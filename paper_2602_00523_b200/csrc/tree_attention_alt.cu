@@ -175,11 +175,10 @@ __device__ __forceinline__ void issue(const AttnParams& p, Shared* sh, uint8_t* 
 __device__ __forceinline__ void softmax_step(uint32_t s_taddr, uint32_t o_taddr, float scale, bool row_ok, bool first, bool masked,
                                              int jt0, uint64_t anc, float& m_ref, float& l_sum) {
     uint32_t sr[128];
-    // Probabilities are taken against the row's reference of the steps before, which moves only when a score exceeds
-    // it by more than 2^8, so a step need not look for its maximum first.  It shows in the step's sum whether the
-    // reference still serves; the first step of a segment, steps with masked scores and steps whose sum has grown to
-    // kMaxSum go through the maximum.
-    bool by_max = masked || first;
+    // Probabilities are taken against the row's reference of the steps before, so a step need not look for its maximum
+    // first.  It shows in the step's sum whether the reference still serves; the first step of a segment, steps with
+    // masked scores and steps whose sum has grown to kMaxSum go through the maximum.
+    bool by_max = masked || first, outgrown = false;
     if (!by_max) {
         uint64_t acc[2] = {0ull, 0ull};
         tmem_ld32(s_taddr, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
@@ -192,7 +191,8 @@ __device__ __forceinline__ void softmax_step(uint32_t s_taddr, uint32_t o_taddr,
         float sum_a, sum_b;
         f2_unpack(f2_add(acc[0], acc[1]), sum_a, sum_b);
         const float sum = sum_a + sum_b;
-        by_max = __any_sync(0xffffffffu, row_ok && !(sum < kMaxSum));
+        outgrown = !(sum < kMaxSum);
+        by_max = __any_sync(0xffffffffu, row_ok && outgrown);
         if (!by_max) l_sum += sum;
     }
     if (by_max) {
@@ -204,9 +204,9 @@ __device__ __forceinline__ void softmax_step(uint32_t s_taddr, uint32_t o_taddr,
         float mx = -INFINITY;
 #pragma unroll
         for (int c = 0; c < 4; ++c) max_chunk(sr + 32 * c, mx);
-        // the reference moves only when the row max grew by more than 2^8 over it
+        // the reference moves where the row's sum asked for it, else only when its maximum grew by more than 2^8
         const float m_cand = mx * scale;
-        const bool grow = m_cand > m_ref + 8.0f;
+        const bool grow = m_cand > m_ref + (outgrown ? 0.f : 8.0f);
         float alpha = 1.0f;
         if (grow) {
             alpha = fast_exp2(m_ref - m_cand);              // 0 when m_ref was -inf

@@ -73,7 +73,7 @@ __device__ __forceinline__ bool softmax_page(const SplitParams& p, Barriers* bar
                                              uint32_t o_taddr, bool row_ok, bool first, bool masked, int jt0, uint64_t anc,
                                              float& m_ref, float& l_sum) {
     uint32_t sr[64];
-    bool by_max = masked || first;
+    bool by_max = masked || first, outgrown = false;
     if (!by_max) {
         uint64_t acc[2] = {0ull, 0ull};
         tmem_ld32(s_taddr, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
@@ -84,7 +84,8 @@ __device__ __forceinline__ bool softmax_page(const SplitParams& p, Barriers* bar
         float sum_a, sum_b;
         f2_unpack(f2_add(acc[0], acc[1]), sum_a, sum_b);
         const float sum = sum_a + sum_b;
-        by_max = __any_sync(0xffffffffu, row_ok && !(sum < kMaxSum));
+        outgrown = !(sum < kMaxSum);
+        by_max = __any_sync(0xffffffffu, row_ok && outgrown);
         if (!by_max) l_sum += sum;
     }
     if (by_max) {
@@ -99,7 +100,7 @@ __device__ __forceinline__ bool softmax_page(const SplitParams& p, Barriers* bar
         max_chunk(sr, mx);
         max_chunk(sr + 32, mx);
         const float m_cand = mx * p.scale_log2;
-        const bool grow = m_cand > m_ref + 8.0f;
+        const bool grow = m_cand > m_ref + (outgrown ? 0.f : 8.0f);
         float alpha = 1.0f;
         if (grow) {
             alpha = fast_exp2(m_ref - m_cand);              // 0 when m_ref was -inf
