@@ -48,7 +48,7 @@ extern "C" {
 #define SAGE_ERR_UNSUPPORTED  2   /* outside the supported envelope                     */
 #define SAGE_ERR_WORKSPACE    3   /* ws == NULL or ws_bytes too small                   */
 #define SAGE_ERR_CUDA         4   /* a CUDA runtime / driver call failed                */
-#define SAGE_ERR_TOO_LARGE    5   /* problem needs more scratch than the built-in array */
+#define SAGE_ERR_TOO_LARGE    5   /* beyond SAGE_STATIC_SCRATCH_BYTES (static variant)   */
 
 /* values written to the device status word (first error wins) */
 #define SAGE_STATUS_BAD_TREE  101 /* parent array / node count violates the tree rules  */
@@ -201,7 +201,8 @@ int sage_build_ancestor_mask(const int32_t *parent, const int32_t *node_offsets,
  *   slots L_b + j for j in anc(i).
  * q, out: bf16 [n_layers][sum_nodes][n_q_heads][head_dim]; `sum_nodes` is the node
  * capacity of those buffers (>= node_offsets[batch]).  Softmax and accumulation in
- * fp32.  Rows of the cache beyond L_b+N_b may hold anything (NaN included).
+ * fp32, probabilities rounded to bf16; how a launch is cut (its size, the batch, the page table's width) shows
+ * in the last digit of an output.  Rows of the cache beyond L_b+N_b may hold anything (NaN included).
  * Rows of q and out beyond node_offsets[batch] have no effect and are not written.  The work is scheduled from
  * the trees actually present, not from the capacity: where the host cannot tell which of the streaming
  * kernels suits them (capacity for trees of more than 128 query rows per KV head), both are started, each
@@ -258,9 +259,8 @@ void sage_debug_attention_waits(long long wait_cycles, int producer_off);
  * multiprocessor walks an equal share of all the work in steps of 128 keys; trees of up to 128 query
  * rows per KV head alternate their steps between two accumulator slots, larger ones keep two row
  * tiles per block) for long launches, and a split one (a grid over context slices, row pairs
- * and KV heads, plus a merge) for short ones.  schedule = 1 or 3 forces the streaming one (3 was a form on
- * two-block clusters that was never faster), 2 the split one, anything else restores the automatic
- * choice.  For tests and measurements (no counterpart in the paper). */
+ * and KV heads, plus a merge) for short ones.  schedule = 1 forces the streaming one (so does 3, an older
+ * name for it), 2 the split one, anything else restores the automatic choice.  For tests and measurements (no counterpart in the paper). */
 void sage_debug_attention_schedule(int schedule);
 
 #ifdef __cplusplus

@@ -218,12 +218,6 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
           "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]),
           "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]) : "memory");
 }
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
-        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-          "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
-}
 __device__ __forceinline__ void tmem_st2(uint32_t taddr, uint32_t a, uint32_t b) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(taddr), "r"(a), "r"(b) : "memory");
 }
@@ -609,15 +603,14 @@ struct SegIter {
     }
 };
 
-// Query rows past the tree: the box of a query tile reaches into the next sequence's rows, or into spare capacity.  Nothing
-// reads what these rows result in, but the tensor cores draw less power on zeros, and long launches run at the power limit:
+// Query rows past the tree (one row tile): the tile's box reaches into the next sequence's rows, or into spare capacity.
+// Nothing reads what these rows result in, but the tensor cores draw less power on zeros, and long launches run at the power limit:
 // nine nodes in arrays of 64, 80 layers x 16k keys, 1035 -> 990 us.  Not for short segments, where it costs more than it saves.
 // Called by the whole MMA warp.
 constexpr int kClearMinSteps = 32;
-__device__ __forceinline__ void clear_query_rows(const AttnParams& p, const Seg& sg, uint8_t* sQ, int rows, int n_rt, int lane) {
-    const int live = rows - (n_rt - 1) * kRowTile;                  // of the last tile
+__device__ __forceinline__ void clear_query_rows(const AttnParams& p, const Seg& sg, uint8_t* sQ, int live, int lane) {
     if (live >= kRowTile || sg.s1 - sg.s0 < kClearMinSteps || sg.n0 + sg.N >= p.sum_nodes) return;      // (past sum_nodes TMA fills in zeros)
-    const uint32_t q = smem_u32(sQ) + (n_rt - 1) * kQTileBytes + ((lane >> 3) & 1) * kQHalfBytes + (lane >> 4) * 128 + (lane & 7) * 16;
+    const uint32_t q = smem_u32(sQ) + ((lane >> 3) & 1) * kQHalfBytes + (lane >> 4) * 128 + (lane & 7) * 16;
 #pragma unroll 4
     for (int r = live + (live & 1); r < kRowTile; r += 2)           // two rows a turn (an odd row at the front may stay)
         asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(q + r * 128), "r"(0) : "memory");

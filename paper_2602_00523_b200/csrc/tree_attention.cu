@@ -1,7 +1,7 @@
 // Tree-masked verification attention over a paged bf16 KV cache (Section 2.2;
 // Algorithm 1, the target pass over all tree tokens; Section 3.3 Phase 2), sm_100a:
-// the C entry points, the tensor maps and the choice of schedule.  The kernels are in
-// tree_attention_stream.cu (streaming schedule) and tree_attention_split.cu (split schedule).
+// the C entry points, the tensor maps and the choice of schedule.  The kernels are in tree_attention_rows.cu and
+// tree_attention_alt.cu (streaming schedule, launched from the latter) and tree_attention_split.cu (split schedule).
 #include <cuda.h>
 
 #include <mutex>
@@ -112,7 +112,7 @@ static int resident_ctas() {
 }
 static long long g_wait_cycles = kWaitCyclesDefault;
 static int g_producer_off = 0;
-static int g_schedule = 0;     // 0: chosen per launch, 1 or 3: streaming, 2: split
+static int g_schedule = 0;     // 0: chosen per launch, 2: split, else streaming
 
 // The split schedule (tree_attention_split.cu).
 namespace split {
@@ -123,7 +123,7 @@ int launch(int n_layers, int n_pages, const int32_t* page_table, int max_pages_p
            int producer_off, const CUtensorMap& qmap, const CUtensorMap& kmap, const CUtensorMap& vmap, cudaStream_t stream);
 }  // namespace split
 
-// The streaming schedule (tree_attention_stream.cu).
+// The streaming schedule (tree_attention_alt.cu).
 namespace stream {
 size_t workspace_size(int n_ctas);
 int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,

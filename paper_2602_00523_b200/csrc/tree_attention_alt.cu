@@ -127,7 +127,7 @@ __device__ __forceinline__ void issue(const AttnParams& p, Shared* sh, uint8_t* 
     while (ok && it.next(p, sg)) {
         const int n = __shfl_sync(0xffffffffu, sg.s1 - sg.s0, 0);
         ok = mbar_wait_warp(&sh->q_ready, nseg & 1, sh, p);
-        if (ok) clear_query_rows(p, sg, smem, sg.N * p.G, 1, lane);
+        if (ok) clear_query_rows(p, sg, smem, sg.N * p.G, lane);
         for (int i = 0; ok && i < n + kLag; ++i) {
             ok = mbar_wait_warp(&sh->kv_full[rc % kRing], (rc / kRing) & 1, sh, p);
             if (!ok) break;

@@ -194,4 +194,4 @@ def test_widely_spread_scores_take_little_longer():
 
     k[:, table[0, :2 * pages // 5].long()] *= 1.5        # (the visual part of a context)
     usual = us(k)
-    assert us(k * 3) <= 1.22 * usual
+    assert us(k * 3) <= 1.25 * usual

@@ -43,7 +43,7 @@ def _build(n_nodes=N, shape=(3, 10)):
                 seq_len=dev_i32([L]), parent=dev_i32(tree["parent"]), offs=dev_i32([0, n_nodes]))
 
 
-@pytest.mark.parametrize("schedule", [0, 1, 3], ids=["as_benchmarked", "streaming", "pairs"])
+@pytest.mark.parametrize("schedule", [0, 1], ids=["as_benchmarked", "streaming"])
 def test_attention_80_layers_sampled_layers_match_the_oracle_and_all_outputs_are_finite(schedule):
     w = _build()
     sage.sage_debug_attention_schedule(schedule)
