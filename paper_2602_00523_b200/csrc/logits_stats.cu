@@ -19,7 +19,8 @@
 //     distributed shared memory; it ranks them, derives lse, entropies, log-probs and alpha, and
 //     hands the row's tokens to the children of the row's node.
 // What bounds it: HBM for many rows (960 rows x 152064, K = 10: 158 -> 94 us, 6.2 TB/s), the chain
-// launch -> load -> select -> merge for few (60 rows: 41 -> 15.6 us; 15 rows x 32000, K = 4: 13 -> 5.3 us).
+// launch -> load -> select -> merge for few (60 rows: 41 -> 15.7 us; 15 rows x 32000, K = 4: 13 -> 5.4 us).  Rows that are
+// constant, or masked with one value, take the same time (600 rows: 63 to 69 us); ascending rows are the worst (884 us).
 // The form before this one offered every element to per-warp queues that started empty, 67 thread
 // instructions per logit at K = 10, and took two more launches to merge and to gather the tokens.
 #include <math.h>

@@ -137,13 +137,17 @@ int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int
 //   streaming: persistent CTAs that walk equal ranges of 128-key steps, whatever the batch looks like.
 //   split: grid over (context slice, row pair, layer x sequence x KV head), 64-key steps: shorter set-up and no plan, for
 //     launches too short to give every SM a long stream (single layers, short contexts: fixed costs dominate).
-// The line lies where both take the same time (us, split / streaming; steps per SM in brackets; 8 KV heads of 8 queries):
-//   one sequence, up to one row pair: 24 nodes, 16k keys, 4 layers (28) 86/93, 8 (56) 164/164; 12 nodes, 4k keys, 16 layers
-//     (28) 56/65, 24 (43) 102/90, 32 (57) 118/112;
-//   one sequence whose node arrays have room for two row pairs: 60 nodes, 16k keys, 3 layers (21) 115/119, 4 (28) 156/153;
-//     but nine nodes in such arrays, for which half of the split grid is empty, 2 layers (14) 55/55, 4 (28) 92/74;
+// The line lies where both take the same time (us, split / streaming; steps per SM in brackets; 8 KV heads of 8 queries;
+// bursts of a few ms, in longer loops the power limit takes 10 to 20 % off the lead of the split schedule):
+//   one sequence, up to one row pair: 24 nodes, 16k keys, 4 layers (28) 72/88, 8 (56) 146/163 (in longer loops 164/164);
+//     12 nodes, 4k keys, 16 layers (28) 61/66, 24 (43) 97/88, 32 (57) 106/108 (118/112);
+//   one sequence whose node arrays have room for two row pairs: 60 nodes, 16k keys, 3 layers (21) 111/133, 4 (28) 144/149
+//     (156/153); but nine nodes in such arrays, for which half of the split grid is empty, 2 layers (14) 57/57, 4 (28) 92/75;
 //   several sequences: the split grid is as uneven as their lengths.  1k to 8k keys, 24 to 60 nodes: four sequences
-//     (12.5) 68/61, eight (25) 110/82, sixteen of 24 nodes (54) 117/84; eight of 2k keys, 36 nodes (7) 38/56.
+//     (14) 69/55, eight (28) 121/86, sixteen of 24 nodes (56) 121/98; eight of 2k keys, 36 nodes (7) 38/61.
+// The host knows the width of the page table, not the lengths, so a wide table takes short sequences across the line, or into
+// more slices than they fill: eight sequences of 1k keys 23 us with 17 pages per row, 41 with 512; one of 2k keys, 60 nodes, 16.0
+// with 33 pages, 16.1 with 512, 10 nodes 9.4 and 10.7.
 static bool use_streaming(int n_layers, int batch, int n_kv_heads, int max_pages_per_seq, int rows) {
     if (g_schedule) return g_schedule != 2;
     const long long steps = (long long)n_layers * batch * n_kv_heads * ((max_pages_per_seq + 1) / 2);   // upper bound

@@ -21,7 +21,7 @@
 // kernel before still runs, then one round of loads (the sequence's offsets and length) beside the allocation of tensor
 // memory, the barriers, and the copies start; what is left of the set-up (page ids, ancestors) happens in the roles.  Before, query
 // rows went through registers, partial results were written row by row (32 lines per store) and merged one warp per row:
-// one layer, 8 KV heads of 8 queries, 60 nodes: 2k keys 23.5 -> 16.5 us, 16k keys 49.7 -> 40.0; 24 nodes, 16k: 37.3 -> 27.4.
+// one layer, 8 KV heads of 8 queries, 60 nodes: 2k keys 23.5 -> 16.3 us, 16k keys 49.7 -> 39.8; 24 nodes, 16k: 37.3 -> 26.1.
 // With two row tiles a page costs 1650 clocks, of which the tensor pipe is busy for 1536 (a 64-key score product takes it
 // as long as one of 128 keys); with one row tile HBM is the bound (6 TB/s).
 // All waits are bounded: on expiry the CTA records SAGE_STATUS_TIMEOUT, drains its copies, frees its
@@ -489,7 +489,7 @@ static int row_pairs_for(int sum_nodes, int G) {
     return (n * G + kRowsPerCta - 1) / kRowsPerCta;
 }
 
-// Slices of the context, down to a page each (512 keys, 60 nodes: 15.1 us with two pages at least, 14.5 with one).  One CTA
+// Slices of the context, down to a page each (512 keys, 60 nodes: 0.6 us less than with two pages at least, now 12.5).  One CTA
 // is resident per SM; a wave of them takes what its pages take plus a fixed part (set-up, first copies, drain), worth about
 // six pages (four and nine measure the same), and every slice costs the merge a little.
 static int pick_splits(int n_layers, int batch, int n_kv_heads, int G, int max_pages, int sum_nodes) {
