@@ -279,6 +279,7 @@ __device__ __forceinline__ bool finish_slots(const AttnParams& p, Shared* sh, co
     if (!seen) {
         const long long t0 = clock64();
         while (true) {
+#pragma unroll 1
             for (int k = 0; k < 64 && !seen; ++k) seen = (*flag == eseq);
             if (seen || sh->abort) break;
             if (clock64() - t0 > p.wait_cycles) {
