@@ -61,6 +61,15 @@ constexpr int kAttnThreads = 384;              // 2 softmax warpgroups + one war
 constexpr float kMaxSum = 4096.f;
 constexpr int kMinSteps = 2;                   // no range shorter than this (short contexts are latency-bound)
 
+// The boundary in front of a CTA's range as the merge kernel needs it: which item it cuts, and which gangs hold the item.
+struct __align__(16) Cut {
+    int n_rp;                       // CTAs per gang
+    int s0;                         // step inside the item that the boundary falls on; 0: between two items, or there is no boundary
+    int layer, u, b, n0, N, steps;  // the item
+    int k_first, k_last;            // gangs that hold it
+    int mid;                        // it begins in the middle of the first one's range
+    int pad;
+};
 struct AttnParams {
     __nv_bfloat16* out;
     // Partial results, one slot per CTA for the head and one for the tail of its range.  Four output columns of
@@ -68,6 +77,7 @@ struct AttnParams {
     // row-major slots took 32 separate lines (an epilogue of 6 000 to 10 000 clocks; now 1 500 to 3 000).
     float4* part_o;    // [CTA][2][32 column quads][256 rows]   unnormalised
     float2* part_ml;   // [CTA][2][256 rows]                    (reference in log2 units, l)
+    Cut* cuts;         // [CTA]
     const int32_t* page_table;
     const int32_t* seq_len;
     const int32_t* parent;
@@ -81,6 +91,15 @@ struct AttnParams {
     int producer_off;          // diagnostics: the TMA warp issues no copies (every consumer wait then runs out)
 };
 
+// How a launch's work is laid out (see make_plan).
+struct Plan {
+    int n_rp;               // CTAs per gang
+    int heads_all;          // units that every sequence takes part in; the others are for trees of two row pairs only
+    int steps_all, steps_big;   // steps of all sequences, and of those with two row pairs
+    int n_act;              // gangs with work
+    int one_tile;           // no tree has more than one row tile
+    long long steps_layer, W;   // steps of a layer, of the launch
+};
 struct Place { int layer, u, b, s0; };     // layer, unit, sequence and step of a position in the launch's work
 struct __align__(16) Shared {
     uint64_t kv_full[kRing];   // ring step r: its K tile and its V tile have landed
@@ -94,6 +113,7 @@ struct __align__(16) Shared {
     uint64_t drain;            // abort path: everything issued so far has retired
     volatile uint32_t eflag[2][4];     // alternating: [slot][quadrant] segment number whose (reference, sum) this warp has posted
     long long range_begin, range_end;
+    Plan plan;
     Place first;               // where the range begins
     int n_rp, heads_all;       // of the plan
     uint32_t tmem_base;
@@ -461,15 +481,7 @@ __device__ __forceinline__ Item load_item(const AttnParams& p, int b, int* err) 
 // gang a unit is a KV head.  With two (some tree of the batch has more than 256 rows) it is a KV head for the trees of
 // two row pairs, one per CTA, and two KV heads, one per CTA, for the trees of one: both CTAs always have rows to work on
 // (with a head per unit throughout, one of them idled through the small trees of a mixed batch).
-struct Plan {
-    int n_rp;               // CTAs per gang
-    int heads_all;          // units that every sequence takes part in; the others are for trees of two row pairs only
-    int steps_all, steps_big;   // steps of all sequences, and of those with two row pairs
-    int n_act;              // gangs with work
-    int one_tile;           // no tree has more than one row tile
-    long long steps_layer, W;   // steps of a layer, of the launch
-};
-// Called by a whole warp; the same answer in every CTA and in the merge kernel.
+// Called by a whole warp; the same answer in every CTA.
 __device__ __forceinline__ Plan make_plan(const AttnParams& p, int lane, int* err) {
     Plan pl;
     int mx = 0, all = 0, big = 0;
@@ -641,6 +653,8 @@ __device__ __forceinline__ bool set_up(const AttnParams& p, Shared* sh, int warp
         }
         if (lane == 0) {
             sh->range_begin = begin; sh->range_end = end;
+            if (end <= begin && pl.one_tile == (kOneTile ? 1 : 0)) p.cuts[blockIdx.x] = Cut{pl.n_rp};
+            sh->plan = pl;
             sh->first = at;
             sh->n_rp = pl.n_rp; sh->heads_all = pl.heads_all;
         }
@@ -677,6 +691,21 @@ __device__ __forceinline__ bool set_up(const AttnParams& p, Shared* sh, int warp
         return false;
     }
     *tmem_out = tmem;
+    if (warp == 11 && lane == 0) {                          // (idle otherwise) what the merge kernel has to know of the range's beginning
+        const Plan pl = sh->plan;
+        const Place at = sh->first;
+        Cut c{pl.n_rp, at.s0, at.layer, at.u, at.b};
+        if (at.s0 > 0) {
+            int err = 0;
+            const Item it = load_item(p, at.b, &err);
+            const long long a = sh->range_begin - at.s0;    // position of the item's first step
+            c.n0 = it.n0; c.N = it.N; c.steps = it.steps;
+            c.k_first = gang_of(pl, a);
+            c.k_last = gang_of(pl, a + it.steps - 1);
+            c.mid = a != gang_begin(pl, c.k_first);
+        }
+        p.cuts[blockIdx.x] = c;
+    }
     return true;
 }
 

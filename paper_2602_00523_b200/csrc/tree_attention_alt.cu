@@ -461,55 +461,45 @@ tree_attention_alt_kernel(const AttnParams p, const __grid_constant__ CUtensorMa
 }
 
 // Merge of the items that a range boundary cut into segments.  Only a boundary between two gangs' ranges can cut an
-// item, so the grid holds kMergeParts blocks per boundary and CTA of a gang.  A block finds the item its boundary falls into
-// and leaves if the boundary coincides with the item's start; the blocks of all boundaries inside the item share its output
-// columns, and combine the item's segments: which gangs hold them, and in which of their two partial slots, follows from
-// the positions alone.  One thread per row; eight 16-byte loads of two segments in flight together.  Finding the item costs a
-// block some 2 us whatever it merges, so all blocks are resident at once (a block per 32 rows, with the item's first boundary
-// doing all the work, came in four waves: 14 us for a layer of 60 nodes at 16k keys).
+// item, so the grid holds kMergeParts blocks per boundary and CTA of a gang.  A block is told which item its boundary falls into by the
+// gang behind it (Cut) and leaves if the boundary coincides with the item's start; the blocks of all boundaries inside the item share
+// its output columns, and combine the item's segments: which of a gang's two partial slots holds one follows from the positions.  One
+// thread per row.  The kernel is a chain of latencies at the end of a launch, so all that an item of two segments (the usual one) needs is
+// asked for at once.  Blocks that made the plan, looked their item up and read the sums first, one after the other, took four times the
+// code: sixteen ragged sequences of 1k to 8k keys 151 -> 145 us, sixteen of up to 4k and 12 nodes 62.7 -> 57.7, a layer of forty 98 -> 90.
+// (Warps that finish a cut item themselves when the next gang's part is already there: 146, the reading only moves.)
 constexpr int kMergeParts = 4;
 __global__ void __launch_bounds__(kRowsPerCta, 4) attention_merge_kernel(AttnParams p) {
     after_previous_kernel();
-    __shared__ Plan s_plan;
-    __shared__ Place s_at;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, row = threadIdx.x;
-    if (warp == 0) {
-        int err = 0;
-        const Plan pl = make_plan(p, lane, &err);
-        const int k = blockIdx.x / pl.n_rp + 1;
-        Place at{0, 0, 0, 0};
-        if (pl.W > 0 && k < pl.n_act) at = locate(p, pl, lane, gang_begin(pl, k));
-        if (lane == 0) { s_plan = pl; s_at = at; }
-    }
-    __syncthreads();
-    const Plan pl = s_plan;
-    const Place at = s_at;
-    const int k_cut = blockIdx.x / pl.n_rp + 1;         // boundary between gang k_cut - 1 and gang k_cut
-    if (pl.W <= 0 || k_cut >= pl.n_act || at.s0 == 0) return;           // no such boundary, or it falls between two items
-    const int member = blockIdx.x % pl.n_rp;
-    int err = 0;
-    const Item it = load_item(p, at.b, &err);
-    const long long a = gang_begin(pl, k_cut) - at.s0;  // position of the item's first step
-    const int k_first = gang_of(pl, a), k_last = gang_of(pl, a + it.steps - 1);
-    const int part = (k_cut - 1 - k_first) * kMergeParts + blockIdx.y, parts = (k_last - k_first) * kMergeParts;
+    const int row = threadIdx.x;
+    const int n_rp = p.cuts[blockIdx.x].n_rp;
+    const Cut c1 = p.cuts[min((int)blockIdx.x + 1, p.n_ctas - 1)], c2 = p.cuts[min((int)blockIdx.x + 2, p.n_ctas - 1)];
+    const Cut c = n_rp == 2 ? c2 : c1;
+    const int k_cut = blockIdx.x / n_rp + 1;            // boundary between gang k_cut - 1 and gang k_cut
+    if ((int)blockIdx.x + n_rp >= p.n_ctas || c.s0 == 0) return;        // no such boundary, or it falls between two items
+    const int member = blockIdx.x % n_rp;
+    const int part = (k_cut - 1 - c.k_first) * kMergeParts + blockIdx.y, parts = (c.k_last - c.k_first) * kMergeParts;
     if (part >= kHeadDim / 16) return;
-    const bool first_mid_range = (a != gang_begin(pl, k_first));
-    const bool pair = pl.n_rp == 2 && it.rp == 1;
-    const int g = pair ? 2 * at.u + member : at.u;
-    const int R = row + (it.rp == 2 ? row_pair_of(member, at.u, at.b) * kRowsPerCta : 0);
+    Item it{c.n0, c.N, 0, c.steps, (c.N * p.G + kRowsPerCta - 1) / kRowsPerCta};
+    const bool pair = n_rp == 2 && it.rp == 1;
+    const int g = pair ? 2 * c.u + member : c.u;
+    const int R = row + (it.rp == 2 ? row_pair_of(member, c.u, c.b) * kRowsPerCta : 0);
     if (g >= p.Hkv || R >= it.N * p.G) return;
-    auto slot_of = [&](int k) { return (k * pl.n_rp + member) * 2 + (k == k_first && first_mid_range ? 1 : 0); };
-    float mx = -INFINITY;
-    for (int k0 = k_first; k0 <= k_last; k0 += 4) {
-        float2 ml[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) ml[u] = p.part_ml[slot_of(min(k0 + u, k_last)) * kRowsPerCta + row];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (ml[u].y > 0.f) mx = fmaxf(mx, ml[u].x);
-    }
+    auto slot_of = [&](int k) { return (k * n_rp + member) * 2 + (k == c.k_first && c.mid ? 1 : 0); };
     const size_t orow = (size_t)(it.n0 + (R >> p.g_shift)) * p.Hq + g * p.G + (R & (p.G - 1));
-    uint4* out = reinterpret_cast<uint4*>(p.out + ((size_t)at.layer * p.sum_nodes * p.Hq + orow) * kHeadDim);
+    uint4* out = reinterpret_cast<uint4*>(p.out + ((size_t)c.layer * p.sum_nodes * p.Hq + orow) * kHeadDim);
+    const bool two = c.k_last == c.k_first + 1;
+    float mx = -INFINITY;
+    if (!two) {
+        for (int k0 = c.k_first; k0 <= c.k_last; k0 += 4) {
+            float2 ml[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) ml[u] = p.part_ml[slot_of(min(k0 + u, c.k_last)) * kRowsPerCta + row];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (ml[u].y > 0.f) mx = fmaxf(mx, ml[u].x);
+        }
+    }
 #pragma unroll 1
     for (int q0 = part * 4; q0 < kHeadDim / 4; q0 += parts * 4) {      // 16 output columns
         const float4* po = p.part_o + (size_t)q0 * kRowsPerCta + row;
@@ -517,19 +507,20 @@ __global__ void __launch_bounds__(kRowsPerCta, 4) attention_merge_kernel(AttnPar
         float4 acc[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int k0 = k_first; k0 <= k_last; k0 += 2) {
+        for (int k0 = c.k_first; k0 <= c.k_last; k0 += 2) {
             float2 ml[2];
             float4 v[2][4];
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                const int slot = slot_of(min(k0 + u, k_last));
+                const int slot = slot_of(min(k0 + u, c.k_last));
                 ml[u] = p.part_ml[slot * kRowsPerCta + row];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) v[u][i] = po[((size_t)slot * (kHeadDim / 4) + i) * kRowsPerCta];
             }
+            if (two) mx = fmaxf(ml[0].y > 0.f ? ml[0].x : -INFINITY, ml[1].y > 0.f ? ml[1].x : -INFINITY);
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                if (k0 + u <= k_last && ml[u].y > 0.f) {
+                if (k0 + u <= c.k_last && ml[u].y > 0.f) {
                     const float w = exp2f(ml[u].x - mx);
                     lsum = fmaf(ml[u].y, w, lsum);
 #pragma unroll
@@ -558,8 +549,8 @@ static int row_pairs(int sum_nodes, int G) {
     return (n * G + kRowsPerCta - 1) / kRowsPerCta;
 }
 
-// Two partial slots (head and tail of its range) per resident CTA, independent of the problem size.
-size_t workspace_size(int n_ctas) { return (size_t)n_ctas * 2 * kRowsPerCta * (kHeadDim + 2) * sizeof(float); }
+// Two partial slots (head and tail of its range) and the boundary in front of it per resident CTA, independent of the problem size.
+size_t workspace_size(int n_ctas) { return (size_t)n_ctas * (2 * kRowsPerCta * (kHeadDim + 2) * sizeof(float) + sizeof(Cut)); }
 
 int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,
            const int32_t* seq_len, const int32_t* parent, const int32_t* node_offsets, int batch, int sum_nodes,
@@ -573,6 +564,7 @@ int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int
     p.out = (__nv_bfloat16*)out;
     p.part_o = (float4*)ws;
     p.part_ml = (float2*)((float*)ws + (size_t)n_ctas * 2 * kRowsPerCta * kHeadDim);
+    p.cuts = (Cut*)(p.part_ml + (size_t)n_ctas * 2 * kRowsPerCta);
     p.page_table = page_table; p.seq_len = seq_len; p.parent = parent; p.node_offsets = node_offsets;
     p.status = status;
     p.n_layers = n_layers; p.batch = batch; p.sum_nodes = sum_nodes; p.n_pages = n_pages;
