@@ -60,6 +60,12 @@ constexpr int kAttnThreads = 384;              // 2 softmax warpgroups + one war
 // would be exactly 1 (error on growing scores 1.92e-3 of the outputs' norm at 2^8, 1.95e-3 here, 1.98e-3 at 2^14, 2.15e-3 at 2^30).
 constexpr float kMaxSum = 4096.f;
 constexpr int kMinSteps = 2;                   // no range shorter than this (short contexts are latency-bound)
+// What an item costs beyond its steps, in steps: the step that holds the tree takes longer, and between two segments lie an epilogue, new
+// query rows and a first step.  Without it ranges of equally many steps take as much longer as they hold more ends of items (sixteen
+// sequences of 1k to 8k keys: a CTA's 53 steps took 122 us on average, 134 at most).  Measured with 0 / 1 / 2 / 3 / 4, us: those 145.0 / 143.7 /
+// 142.8 / 142.1 / 144.6; sixteen of 1k to 4k, 12 nodes 57.7 / 57.0 / 54.1 / 56.1 / 56.6; forty of 64 to 1000 89.9 / 83.8 / 80.0 / 79.4 / 77.6;
+// one of 4k, 80 layers 257 / 259 / 256 / 257 / 257.
+constexpr int kItemExtra = 2;
 
 // The boundary in front of a CTA's range as the merge kernel needs it: which item it cuts, and which gangs hold the item.
 struct __align__(16) Cut {
@@ -95,7 +101,7 @@ struct AttnParams {
 struct Plan {
     int n_rp;               // CTAs per gang
     int heads_all;          // units that every sequence takes part in; the others are for trees of two row pairs only
-    int steps_all, steps_big;   // steps of all sequences, and of those with two row pairs
+    int steps_all, steps_big;   // steps of all sequences, and of those with two row pairs (here and below: with kItemExtra for each item)
     int n_act;              // gangs with work
     int one_tile;           // no tree has more than one row tile
     long long steps_layer, W;   // steps of a layer, of the launch
@@ -489,8 +495,9 @@ __device__ __forceinline__ Plan make_plan(const AttnParams& p, int lane, int* er
         Item it{0, 0, 0, 0, 0};
         if (b0 + lane < p.batch) it = load_item(p, b0 + lane, err);
         if (it.steps) mx = max(mx, it.N * p.G);
-        all += it.steps;
-        big += it.rp > 1 ? it.steps : 0;
+        const int cost = it.steps ? it.steps + kItemExtra : 0;
+        all += cost;
+        big += it.rp > 1 ? cost : 0;
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
     pl.steps_all = __reduce_add_sync(0xffffffffu, all);
@@ -513,8 +520,10 @@ __device__ __forceinline__ long long gang_begin(const Plan& pl, int gang) {
 // Gang whose range holds position pos: the largest k with gang_begin(k) <= pos.
 __device__ __forceinline__ int gang_of(const Plan& pl, long long pos) { return (int)(((pos + 1) * pl.n_act - 1) / pl.W); }
 
-// Layer, unit, sequence and step inside it of position pos < W; whole warp.
-__device__ __forceinline__ Place locate(const AttnParams& p, const Plan& pl, int lane, long long pos) {
+// Layer, unit, sequence and step inside it of position pos < W; whole warp.  The extra of an item lies behind its steps: a position there
+// is moved to the start of the next item (which may be W; the place is then past the last layer).
+__device__ __forceinline__ Place locate(const AttnParams& p, const Plan& pl, int lane, long long* position) {
+    const long long pos = *position;
     Place at;
     unsigned r;
     if (pl.W < (1ll << 31)) {
@@ -537,7 +546,7 @@ __device__ __forceinline__ Place locate(const AttnParams& p, const Plan& pl, int
         int s = 0;
         if (b0 + lane < p.batch) {
             const Item it = load_item(p, b0 + lane, &err);
-            if (!big_only || it.rp > 1) s = it.steps;
+            if (it.steps && (!big_only || it.rp > 1)) s = it.steps + kItemExtra;
         }
         int inc = s;
         for (int o = 1; o < 32; o <<= 1) {
@@ -550,6 +559,14 @@ __device__ __forceinline__ Place locate(const AttnParams& p, const Plan& pl, int
             const int incl = __shfl_sync(0xffffffffu, inc, l), sl = __shfl_sync(0xffffffffu, s, l);
             at.b = b0 + l;
             at.s0 = off - (run + incl - sl);
+            if (at.s0 >= sl - kItemExtra) {
+                *position += sl - at.s0;
+                at.s0 = 0;
+                if (++at.b == p.batch) {
+                    at.b = 0;
+                    if (++at.u == p.Hkv) { at.u = 0; ++at.layer; }
+                }
+            }
             break;
         }
         run += __shfl_sync(0xffffffffu, inc, 31);
@@ -564,7 +581,7 @@ struct Seg { int layer, g, b, n0, N, L, s0, s1, steps, row0; bool at_range_begin
 
 // Walks the segments of a CTA's range; every thread that needs them runs its own copy.
 struct SegIter {
-    int remaining;      // steps of the range still to hand out
+    int remaining;      // of the range, still to hand out (steps, and kItemExtra for each end of an item)
     int layer, u, b, s0;
     int n_rp, heads_all, member;
     bool fresh;         // nothing handed out yet
@@ -600,7 +617,7 @@ struct SegIter {
                 next_sequence(p);
                 continue;
             }
-            const int s1 = (it.steps - s0 <= remaining) ? it.steps : s0 + remaining;
+            const int s1 = (it.steps - s0 <= remaining) ? it.steps : s0 + remaining;      // (the range may end in the item's extra)
             const bool pair = n_rp == 2 && it.rp == 1;              // two heads of a small tree, one per CTA
             sg.layer = layer; sg.b = b;
             sg.g = pair ? 2 * u + member : u;
@@ -609,7 +626,7 @@ struct SegIter {
             sg.s0 = s0; sg.s1 = s1; sg.steps = it.steps;
             sg.at_range_begin = fresh;
             fresh = false;
-            remaining -= s1 - s0;
+            remaining -= s1 - s0 + (s1 == it.steps ? kItemExtra : 0);
             if (s1 == it.steps) next_sequence(p);
             else s0 = s1;
             if (sg.g < p.Hkv) return true;
@@ -649,7 +666,7 @@ __device__ __forceinline__ bool set_up(const AttnParams& p, Shared* sh, int warp
         if (pl.W > 0 && gang < pl.n_act && pl.one_tile == (kOneTile ? 1 : 0)) {
             begin = gang_begin(pl, gang);
             end = gang_begin(pl, gang + 1);
-            if (end > begin) at = locate(p, pl, lane, begin);
+            if (end > begin) at = locate(p, pl, lane, &begin);
         }
         if (lane == 0) {
             sh->range_begin = begin; sh->range_end = end;
@@ -702,7 +719,7 @@ __device__ __forceinline__ bool set_up(const AttnParams& p, Shared* sh, int warp
             c.n0 = it.n0; c.N = it.N; c.steps = it.steps;
             c.k_first = gang_of(pl, a);
             c.k_last = gang_of(pl, a + it.steps - 1);
-            c.mid = a != gang_begin(pl, c.k_first);
+            c.mid = gang_begin(pl, c.k_first) < a - kItemExtra;      // (more than the extra of the item in front lies before it)
         }
         p.cuts[blockIdx.x] = c;
     }
