@@ -35,6 +35,7 @@ using namespace stream;
 
 constexpr int kPageStages = 5;                 // depth of the K ring and of the V ring, in pages
 constexpr int kPageBytes = kPageSize * kHeadDim * 2;        // one (page, head) tile: 16 KB
+constexpr int kTablePages = 256;               // page tables of up to so many pages are read ahead of the lengths that say which part is needed
 constexpr int kSplitThreads = 352;             // 2 softmax warpgroups + TMA warp + one MMA warp per row tile
 constexpr uint32_t kIdescPageQK = idesc_f16(kPageSize);     // S (128 x 64): A, B both K-major
 
@@ -64,6 +65,7 @@ struct __align__(8) Barriers {
     uint64_t q_ready;          // the query tiles are in shared memory
     uint32_t tmem_base;
     volatile int abort;
+    int pages[kTablePages];    // the sequence's row of the page table, where that is no longer
 };
 constexpr int kSplitSmemBytes = 1024 /*align*/ + 2 * kQTileBytes + 2 * kPageStages * kPageBytes + (int)sizeof(Barriers);
 
@@ -160,6 +162,19 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
     const int n0 = p.node_offsets[b];
     const int N = p.node_offsets[b + 1] - n0;
     const int L = p.seq_len[b];
+    // The whole row of the page table in the same round of loads, not the slice's part in a second one once the length is known (one
+    // layer of ten nodes at 2k keys 9.18 -> 8.94 us, 60 nodes 16.0 -> 15.8, 15 nodes at 627 keys 9.42 -> 9.02, 24 at 4k 14.8 -> 14.5).
+    const bool table = p.max_pages <= kTablePages;
+    if (warp == 8 && table) {
+        const int32_t* pages = p.page_table + (size_t)b * p.max_pages;
+        int ids[kTablePages / 32];
+#pragma unroll
+        for (int i = 0; i < kTablePages / 32; ++i)
+            if (lane + 32 * i < p.max_pages) ids[i] = pages[lane + 32 * i];
+#pragma unroll
+        for (int i = 0; i < kTablePages / 32; ++i)
+            if (lane + 32 * i < p.max_pages) bars->pages[lane + 32 * i] = ids[i];
+    }
     const bool bad_tree = N < 1 || N > SAGE_MAX_NODES || n0 < 0 || n0 + N > p.sum_nodes;
     const bool bad_page = !bad_tree && (L < 0 || L + N > p.max_pages * kPageSize);
     const int T = L + N;
@@ -198,7 +213,7 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
     if (warp == 8) {
         // =========================== TMA producer ===========================
         if (lane == 0 && ns > 0 && !p.producer_off) {
-            const int32_t* pages = p.page_table + (size_t)b * p.max_pages + pg_begin;
+            const int32_t* pages = table ? bars->pages + pg_begin : p.page_table + (size_t)b * p.max_pages + pg_begin;
             mbar_expect_tx(&bars->q_ready, n_rtiles * kQTileBytes);
             for (int t = 0; t < n_rtiles; ++t)
                 for (int h = 0; h < 2; ++h)
