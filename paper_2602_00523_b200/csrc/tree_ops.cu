@@ -105,6 +105,8 @@ __global__ void ancestor_mask_kernel(const int32_t* __restrict__ parent, const i
 // of matching nodes this is (anc(i) & ~match) == 0.  Because parent < child, a
 // root path read in increasing node index is the path itself, so "longest, then
 // lexicographically smallest" is the maximum of (depth, bit-reversed anc(i)).
+// A chain of latencies: two rounds of loads (offsets, nodes), the rest in registers and shuffles.  Walking up the parents in memory, a
+// node at a time, and looking tokens up behind that took 2.88 us instead of 2.06 (four trees, back to back in a graph).
 // ---------------------------------------------------------------------------
 __global__ void accept_kernel(const int32_t* __restrict__ parent, const int32_t* __restrict__ draft_token,
                               const int32_t* __restrict__ target_argmax, const int32_t* __restrict__ node_offsets,
@@ -119,18 +121,29 @@ __global__ void accept_kernel(const int32_t* __restrict__ parent, const int32_t*
     const int n = node_offsets[b + 1] - n0;
     int32_t* my_path = path + (size_t)b * max_path;
     bool bad_tree = (n < 1 || n > SAGE_MAX_NODES);
-    uint64_t anc[2] = {0, 0};
-    bool match[2] = {false, false};
-    if (!bad_tree) {
-        for (int u = 0; u < 2; ++u) {
-            const int i = lane + 32 * u;
-            if (i < n) {
-                bool bad = false;
-                anc[u] = ancestor_bits(parent + n0, n, i, &bad);
-                bad_tree |= bad;
-                if (!bad) match[u] = (i == 0) || (draft_token[n0 + i] == target_argmax[n0 + parent[n0 + i]]);
-            }
-        }
+    // Everything about the nodes in one round of loads; a parent's part of it comes from the lane that has it.
+    const int count = bad_tree ? 0 : n;
+    int par[2], draft[2], target[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int i = lane + 32 * u;
+        par[u] = i < count ? parent[n0 + i] : -1;
+        draft[u] = i < count ? draft_token[n0 + i] : 0;
+        target[u] = i < count ? target_argmax[n0 + i] : 0;
+    }
+    auto of = [](const auto (&v)[2], int node) {
+        const auto lo = __shfl_sync(0xffffffffu, v[0], node & 31), hi = __shfl_sync(0xffffffffu, v[1], node & 31);
+        return node < 32 ? lo : hi;
+    };
+    uint64_t anc[2];
+    int up[2];
+    bool match[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int i = lane + 32 * u;
+        if (i < count && (i == 0 ? par[u] != -1 : par[u] < 0 || par[u] >= i)) bad_tree = true;
+        up[u] = i < count && i > 0 ? par[u] : 0;
+        anc[u] = 1ull << i;
     }
     bad_tree = __any_sync(0xffffffffu, bad_tree);
     if (bad_tree) {
@@ -142,6 +155,22 @@ __global__ void accept_kernel(const int32_t* __restrict__ parent, const int32_t*
         for (int j = lane; j < max_path; j += 32) my_path[j] = -1;
         return;
     }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int i = lane + 32 * u, at_parent = of(target, up[u]);
+        match[u] = i < n && (i == 0 || draft[u] == at_parent);
+    }
+    // ancestors by doubling: what a node has collected so far, and how far up that reaches
+    while (__any_sync(0xffffffffu, (up[0] | up[1]) != 0)) {
+        const uint64_t a0 = of(anc, up[0]), a1 = of(anc, up[1]);
+        const int u0 = of(up, up[0]), u1 = of(up, up[1]);
+        anc[0] |= a0;
+        anc[1] |= a1;
+        up[0] = u0;
+        up[1] = u1;
+    }
+    anc[0] |= 1ull;
+    anc[1] |= 1ull;
     const uint64_t match_bits = (uint64_t)__ballot_sync(0xffffffffu, match[0]) |
                                 ((uint64_t)__ballot_sync(0xffffffffu, match[1]) << 32);
     // best key over accepted nodes: depth first, then bit-reversed ancestor set
@@ -178,9 +207,10 @@ __global__ void accept_kernel(const int32_t* __restrict__ parent, const int32_t*
         }
         my_path[j] = node;
     }
+    const int bonus = of(target, 63 - __clzll((long long)best_anc));
     if (lane == 0) {
         path_len[b] = len;
-        bonus_token[b] = target_argmax[n0 + (63 - __clzll((long long)best_anc))];
+        bonus_token[b] = bonus;
     }
 }
 
@@ -223,6 +253,8 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kv_kernel(const Compa
     if (tid < 32) {
         // Checks the accepted path and turns it into moves, two entries per lane.  A path or a page id that is not
         // valid leaves the sequence exactly as it is (nothing moves, its length does not advance).
+        // (the path's first entries are asked for beside the lengths)
+        const int ahead = lane < p.max_path ? p.path[(size_t)b * p.max_path + lane] : SAGE_MAX_NODES;
         const int L = p.seq_len[b];
         const int plen = p.path_len[b];
         const bool whole_bad = plen < 0 || plen > p.max_path || plen > SAGE_MAX_NODES || L < 0;
@@ -230,7 +262,7 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kv_kernel(const Compa
         int moves = 0, before = -1;              // before: the last node of the previous 32 entries
         for (int j0 = 0; j0 < (whole_bad ? 0 : plen); j0 += 32) {
             const int j = j0 + lane;
-            const int node = j < plen ? p.path[(size_t)b * p.max_path + j] : SAGE_MAX_NODES;
+            const int node = j >= plen ? SAGE_MAX_NODES : j0 == 0 ? ahead : p.path[(size_t)b * p.max_path + j];
             int prev = __shfl_up_sync(0xffffffffu, node, 1);
             if (lane == 0) prev = before;
             before = __shfl_sync(0xffffffffu, node, 31);
