@@ -116,6 +116,7 @@ static int g_schedule = 0;     // 0: chosen per launch, 2: split, else streaming
 
 // The split schedule (tree_attention_split.cu).
 namespace split {
+double estimate(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
 size_t workspace_size(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
 int launch(int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,
            const int32_t* seq_len, const int32_t* parent, const int32_t* node_offsets, int batch, int sum_nodes,
@@ -143,16 +144,31 @@ int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int
 //     12 nodes, 4k keys, 16 layers (28) 61/66, 24 (43) 97/88, 32 (57) 106/108 (118/112);
 //   one sequence whose node arrays have room for two row pairs: 60 nodes, 16k keys, 3 layers (21) 111/133, 4 (28) 144/149
 //     (156/153); but nine nodes in such arrays, for which half of the split grid is empty, 2 layers (14) 57/57, 4 (28) 92/75;
-//   several sequences: the split grid is as uneven as their lengths.  1k to 8k keys, 24 to 60 nodes: four sequences
+//   several sequences, long: the split grid is as uneven as their lengths.  1k to 8k keys, 24 to 60 nodes: four sequences
 //     (14) 69/55, eight (28) 121/86, sixteen of 24 nodes (56) 121/98; eight of 2k keys, 36 nodes (7) 38/61.
+// Several sequences under page tables of up to 40 pages: an item is no longer than the tile loop's way in and out, and what decides is how
+// full the last wave of the split grid is, a block per item and slice.  Both schedules are estimated in pages of 64 keys (split::estimate;
+// streaming: the items' pages and extra over the SMs, and 21 for plan, first copies and merge).  From 12 steps per SM the split schedule
+// is taken when it is ahead by a twentieth, below the streaming one when it is ahead at all (not under 20 pages, where the estimate
+// is too high for split, nor for one row tile).  8 KV heads of 8 queries, split / streaming: 16 sequences of 2k keys, 12 nodes 32/47, 24 nodes
+// 41/54, 60 nodes 75/85; 19: 55/52, 68/61, 103/96 (one item too many for a wave); 36: 66/75, 86/95, 155/169; 28 of 1k keys 36/47, 44/55; 18 of up
+// to 2k, 24 nodes 38/52; 12 of 2k, 60 nodes 88/70, 24 nodes 49/46; 9 of 2k, 60 nodes 40/58; 11 of up to 2.5k, mixed 61/54.
 // The host knows the width of the page table, not the lengths, so a wide table takes short sequences across the line, or into
 // more slices than they fill: eight sequences of 1k keys 23 us with 17 pages per row, 41 with 512; one of 2k keys, 60 nodes, 16.0
 // with 33 pages, 16.1 with 512, 10 nodes 9.4 and 10.7.
-static bool use_streaming(int n_layers, int batch, int n_kv_heads, int max_pages_per_seq, int rows) {
+static bool use_streaming(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq) {
     if (g_schedule) return g_schedule != 2;
-    const long long steps = (long long)n_layers * batch * n_kv_heads * ((max_pages_per_seq + 1) / 2);   // upper bound
+    const int G = n_q_heads / n_kv_heads;
+    const int rows = (sum_nodes < SAGE_MAX_NODES ? sum_nodes : SAGE_MAX_NODES) * G;      // most that a tree can have
+    const long long items = (long long)n_layers * batch * n_kv_heads;
+    const long long steps = items * ((max_pages_per_seq + 1) / 2);   // upper bound
     const int line = batch > 1 ? 12 : rows > 256 ? 24 : 40;
-    return steps >= (long long)line * resident_ctas();
+    const bool is_long = steps >= (long long)line * resident_ctas();
+    const int rows_avg = sum_nodes / batch * G;
+    if (batch == 1 || max_pages_per_seq > 40 || items > 65535) return is_long;       // (the split schedule's grid ends there)
+    if (!is_long && (max_pages_per_seq <= 20 || rows_avg <= kRowTile)) return false;
+    const double streaming = (double)items * (rows_avg > 256 ? 2 : 1) * (max_pages_per_seq + 4) / resident_ctas() + 21.0;
+    return streaming < (is_long ? 1.05 : 1.0) * split::estimate(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq);
 }
 
 }  // namespace sage
@@ -203,8 +219,7 @@ extern "C" int sage_tree_attention(const void* q, const void* k_pool, const void
     const size_t need = sage_tree_attention_workspace_size(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads,
                                                            head_dim, max_pages_per_seq);
     if (!ws || ws_bytes < need || ((uintptr_t)ws & 15)) return SAGE_ERR_WORKSPACE;
-    const int most_rows = (sum_nodes < SAGE_MAX_NODES ? sum_nodes : SAGE_MAX_NODES) * G;
-    const bool streaming = use_streaming(n_layers, batch, n_kv_heads, max_pages_per_seq, most_rows);
+    const bool streaming = use_streaming(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq);
     if (!streaming && (long long)n_layers * batch * n_kv_heads > 65535) return SAGE_ERR_UNSUPPORTED;    // grid limit of the split schedule
     CUtensorMap qmap, kmap, vmap;
     if (!make_pool_map(&kmap, k_pool, n_layers, n_pages, n_kv_heads, layer_stride_elems) ||

@@ -195,3 +195,29 @@ def test_widely_spread_scores_take_little_longer():
     k[:, table[0, :2 * pages // 5].long()] *= 1.5        # (the visual part of a context)
     usual = us(k)
     assert us(k * 3) <= 1.25 * usual
+
+
+@pytest.mark.parametrize("heads,Ns", [(8, [12]), (8, [40, 12, 20, 9]), (7, [36, 5]), (3, [24])], ids=["one_tile", "mixed", "odd_heads", "two_tiles"])
+def test_ranges_that_end_at_the_end_of_an_item(heads, Ns):
+    """Items of one to nine steps, ranges of about as many: boundaries fall on every step of an item, and into the extra that stands for
+    its end, where the range ends with the item and the next one starts with the next item."""
+    r = np.random.Generator(np.random.Philox(heads * 100 + len(Ns)))
+    batch, G = 24, 8
+    Ns = [Ns[b % len(Ns)] for b in range(batch)]
+    Ls = [int(v) for v in r.integers(1, 1100, batch)]
+    kv = make_kv_cache(r, Ls, Ns, [0] * batch, heads, shuffle=True)
+    q = make_q(r, sum(Ns), heads * G)
+    parent = np.concatenate([random_tree(r, n)["parent"] for n in Ns]).astype(np.int32)
+    off = np.concatenate([[0], np.cumsum(Ns)]).astype(np.int32)
+    st = sage.new_status()
+    sage.sage_debug_attention_schedule(1)
+    try:
+        out = sage.sage_tree_attention(dev_bf16(q), dev_bf16(kv["k_pool"]), dev_bf16(kv["v_pool"]), dev_i32(kv["page_table"]),
+                                       dev_i32(kv["seq_len"]), dev_i32(parent), dev_i32(off), 128 ** -0.5, status=st)
+        torch.cuda.synchronize()
+    finally:
+        sage.sage_debug_attention_schedule(0)
+    assert int(st.item()) == 0
+    want = oracle.tree_attention(q[0], kv["k_pool"][0], kv["v_pool"][0], kv["page_table"], kv["seq_len"], parent, off, heads * G, heads,
+                                 128, 64, 128 ** -0.5)
+    check_attention(host_bits(out)[0], want, bf16_slack=True)       # (bound: see test_attention_edges)
