@@ -5,13 +5,13 @@
 //
 // Work decomposition.  The N tree nodes x G query heads that share one KV head form
 // M = N*G query rows (<= 512).  An *item* is one (layer, sequence, KV head); its work
-// is measured in steps of 128 keys (two 64-token pages).  All items are laid end to
-// end and cut into equal ranges of steps, one range per *gang*; a gang is the 1 or 2
+// is measured in steps of 128 keys (two 64-token pages), its end counts as kItemExtra
+// more.  All items are laid end to end and cut into equal ranges, one range per *gang*; a gang is the 1 or 2
 // CTAs (one per 256 query rows) that walk the same range side by side, so that the
 // second CTA finds the K/V of the first in L2.  A kernel launch is one resident CTA
 // per SM that loops over the segments of its range: whole items write their output
 // directly, items cut by a range boundary leave unnormalised partial results that
-// the merge kernel combines.  Nothing waits on another CTA.
+// the merge kernel combines, told by a record per range which item that is.  Nothing waits on another CTA.
 //
 // Inside a CTA (384 threads): tensor memory holds two slots t of (S_t 128 x 128 fp32 scores,
 // O_t 128 x 128 fp32 accumulator): S_t in columns [128t, 128t+128), O_t in [256+128t, 384+128t).
@@ -28,8 +28,8 @@
 //   tree_attention_alt.cu (up to 128 rows): both slots belong to the same rows and take the even and the odd steps
 //     of a segment, each with its own accumulator and running (reference, sum); combined in the epilogue.
 //     (With one slot per row tile the chain scores -> softmax -> P V would be strictly serial.)
-// A 128 x 64 score MMA occupies the tensor pipe exactly as long as a 128 x 128 one (64 clocks
-// per K=16 slice, measured), hence the 128-key step.
+// Clocks per K=16 slice, measured (128 rows, N columns): N/2 with the A operand in TMEM; with both in shared memory 32 + N/4 up to
+// N = 128, which is what reading them takes, so scores of 64 keys cost 48 and of 128 keys 64: hence the 128-key step.
 // All waits are bounded: on expiry the CTA records SAGE_STATUS_TIMEOUT, waits (bounded) for
 // its copies and MMAs in flight, frees its TMEM and returns.
 #pragma once

@@ -44,8 +44,8 @@ __device__ __forceinline__ uint64_t ancestor_bits(const int32_t* __restrict__ pa
 // writes are visible, before it touches global memory, and then lets the next kernel of the stream be brought up.
 // No block leaves without passing it: a kernel waits for its direct predecessor only, and that one's end has to mean that
 // its own predecessor has ended.
-// The merges of the attention pay for it (0.4 us of a layer's 9 at 2k keys, 2 of 156 for sixteen ragged sequences: the
-// chain of loads that finds their work used to run before the wait), but what a kernel reads ahead of it need not be visible yet.
+// The split schedule's merge pays for it (0.4 us of a layer's 9 at 2k keys: the loads that find its work used to run before the
+// wait), but what a kernel reads ahead of it need not be visible yet.
 // Between dependent kernels of a few microseconds this hides most of the gap: eight levels of tree growth
 // (sixteen sequences) and the history update 45 -> 33 us.
 __device__ __forceinline__ void after_previous_kernel() {

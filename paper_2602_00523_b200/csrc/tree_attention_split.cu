@@ -22,8 +22,8 @@
 // memory, the barriers, and the copies start; what is left of the set-up (page ids, ancestors) happens in the roles.  Before, query
 // rows went through registers, partial results were written row by row (32 lines per store) and merged one warp per row:
 // one layer, 8 KV heads of 8 queries, 60 nodes: 2k keys 23.5 -> 16.3 us, 16k keys 49.7 -> 39.8; 24 nodes, 16k: 37.3 -> 26.1.
-// With two row tiles a page costs 1650 clocks, of which the tensor pipe is busy for 1536 (a 64-key score product takes it
-// as long as one of 128 keys); with one row tile HBM is the bound (6 TB/s).
+// With two row tiles a page costs 1650 clocks, of which the tensor pipe is busy for 1280 (a 64-key score product costs 48
+// clocks per K=16 slice where one of 128 keys costs 64); with one row tile HBM is the bound (6 TB/s).
 // All waits are bounded: on expiry the CTA records SAGE_STATUS_TIMEOUT, drains its copies, frees its
 // TMEM and returns.
 #include "attention_stream.cuh"
@@ -163,7 +163,8 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
     const int N = p.node_offsets[b + 1] - n0;
     const int L = p.seq_len[b];
     // The whole row of the page table in the same round of loads, not the slice's part in a second one once the length is known (one
-    // layer of ten nodes at 2k keys 9.18 -> 8.94 us, 60 nodes 16.0 -> 15.8, 15 nodes at 627 keys 9.42 -> 9.02, 24 at 4k 14.8 -> 14.5).
+    // layer of ten nodes at 2k keys 9.18 -> 8.94 us, 60 nodes 16.0 -> 15.8, 15 nodes at 627 keys 9.42 -> 9.02, 24 at 4k 14.8 -> 14.5; of 35
+    // batches of short sequences, 1 to 8 query heads a KV head, 32 gain 2 to 4 %, three of one head and mixed trees lose as much, 11.0 -> 11.3).
     const bool table = p.max_pages <= kTablePages;
     if (warp == 8 && table) {
         const int32_t* pages = p.page_table + (size_t)b * p.max_pages;
