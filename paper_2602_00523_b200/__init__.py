@@ -17,6 +17,7 @@ _BINDING_NAMES = (
     "sage_build_ancestor_mask", "sage_grow_tree", "sage_update_history", "make_history_policy",
     "SageHistoryPolicy", "sage_tree_attention", "sage_tree_attention_workspace_size",
     "sage_accept", "sage_compact_kv", "sage_debug_attention_waits", "sage_debug_attention_schedule",
+    "sage_debug_attention_plan",
     "SAGE_OK", "SAGE_ERR_INVALID_ARG", "SAGE_ERR_UNSUPPORTED", "SAGE_ERR_WORKSPACE", "SAGE_ERR_CUDA",
     "SAGE_ERR_TOO_LARGE", "SAGE_STATIC_SCRATCH_BYTES",
     "SAGE_STATUS_BAD_TREE", "SAGE_STATUS_BAD_PAGE", "SAGE_STATUS_TIMEOUT", "SAGE_STATUS_BAD_PATH",

@@ -98,6 +98,8 @@ _lib.sage_debug_attention_waits.restype = None
 _lib.sage_debug_attention_waits.argtypes = [ctypes.c_longlong, _i]
 _lib.sage_debug_attention_schedule.restype = None
 _lib.sage_debug_attention_schedule.argtypes = [_i]
+_lib.sage_debug_attention_plan.restype = _i
+_lib.sage_debug_attention_plan.argtypes = [_i, _i, _i, _i, _i, _i, ctypes.POINTER(_i)]
 _lib.sage_status_string.restype = ctypes.c_char_p
 _lib.sage_status_string.argtypes = [_i]
 
@@ -265,6 +267,14 @@ def sage_debug_attention_waits(wait_cycles: int = 0, producer_off: bool = False)
 def sage_debug_attention_schedule(schedule: int = 0) -> None:
     """0: the library picks the attention schedule per launch; 1: streaming; 2: split."""
     _lib.sage_debug_attention_schedule(int(schedule))
+
+
+def sage_debug_attention_plan(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages) -> dict:
+    """What sage_tree_attention would do with a launch of these sizes: the schedule, 1 streaming or 2 split, and the split one's
+    context slices."""
+    plan = (_i * 2)()
+    _check(_lib.sage_debug_attention_plan(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages, plan), "sage_debug_attention_plan")
+    return {"schedule": plan[0], "slices": plan[1]}
 
 
 def sage_accept(parent, draft_token, target_argmax, node_offsets, max_path: int, *, out=None, status=None, stream=None):

@@ -117,6 +117,7 @@ static int g_schedule = 0;     // 0: chosen per launch, 2: split, else streaming
 // The split schedule (tree_attention_split.cu).
 namespace split {
 double estimate(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
+int slices(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
 size_t workspace_size(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
 int launch(int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,
            const int32_t* seq_len, const int32_t* parent, const int32_t* node_offsets, int batch, int sum_nodes,
@@ -146,13 +147,16 @@ int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int
 //     (156/153); but nine nodes in such arrays, for which half of the split grid is empty, 2 layers (14) 57/57, 4 (28) 92/75;
 //   several sequences, long: the split grid is as uneven as their lengths.  1k to 8k keys, 24 to 60 nodes: four sequences
 //     (14) 69/55, eight (28) 121/86, sixteen of 24 nodes (56) 121/98; eight of 2k keys, 36 nodes (7) 38/61.
-// Several sequences under page tables of up to 40 pages: an item is no longer than the tile loop's way in and out, and what decides is how
-// full the last wave of the split grid is, a block per item and slice.  Both schedules are estimated in pages of 64 keys (split::estimate;
-// streaming: the items' pages and extra over the SMs, and 21 for plan, first copies and merge).  From 12 steps per SM the split schedule
-// is taken when it is ahead by a twentieth, below the streaming one when it is ahead at all (not under 20 pages, where the estimate
-// is too high for split, nor for one row tile).  8 KV heads of 8 queries, split / streaming: 16 sequences of 2k keys, 12 nodes 32/47, 24 nodes
+// Above the line, several sequences under page tables of up to 40 pages: an item is no longer than the tile loop's way in and out, and
+// what decides is how full the last wave of the split grid is, a block per item and slice.  Both schedules are estimated in pages of 64 keys
+// (split::estimate; streaming: the items' pages and extra over the SMs, and 21 for plan, first copies and merge), and the split schedule
+// is taken when it is ahead by a twentieth.  8 KV heads of 8 queries, split / streaming: 16 sequences of 2k keys, 12 nodes 32/47, 24 nodes
 // 41/54, 60 nodes 75/85; 19: 55/52, 68/61, 103/96 (one item too many for a wave); 36: 66/75, 86/95, 155/169; 28 of 1k keys 36/47, 44/55; 18 of up
-// to 2k, 24 nodes 38/52; 12 of 2k, 60 nodes 88/70, 24 nodes 49/46; 9 of 2k, 60 nodes 40/58; 11 of up to 2.5k, mixed 61/54.
+// to 2k, 24 nodes 38/52.
+// Below the line the split schedule runs, whatever the estimates say.  They know what a table and the node arrays can hold, not what they
+// do hold, and a streaming launch takes 20 us however little there is to do: 27 sequences in tables of 21 pages an eighth full, one KV head of 8
+// queries, 3 layers 12/29; twelve chains of nine nodes in arrays of 64 each, 21 full pages 22/32.  (Tight and uneven batches pay for it:
+// twelve sequences of 2k keys, 60 nodes 88/70.)
 // The host knows the width of the page table, not the lengths, so a wide table takes short sequences across the line, or into
 // more slices than they fill: eight sequences of 1k keys 23 us with 17 pages per row, 41 with 512; one of 2k keys, 60 nodes, 16.0
 // with 33 pages, 16.1 with 512, 10 nodes 9.4 and 10.7.
@@ -163,12 +167,11 @@ static bool use_streaming(int n_layers, int batch, int sum_nodes, int n_q_heads,
     const long long items = (long long)n_layers * batch * n_kv_heads;
     const long long steps = items * ((max_pages_per_seq + 1) / 2);   // upper bound
     const int line = batch > 1 ? 12 : rows > 256 ? 24 : 40;
-    const bool is_long = steps >= (long long)line * resident_ctas();
+    if (steps < (long long)line * resident_ctas()) return false;
+    if (batch == 1 || max_pages_per_seq > 40 || items > 65535) return true;          // (the split schedule's grid ends there)
     const int rows_avg = sum_nodes / batch * G;
-    if (batch == 1 || max_pages_per_seq > 40 || items > 65535) return is_long;       // (the split schedule's grid ends there)
-    if (!is_long && (max_pages_per_seq <= 20 || rows_avg <= kRowTile)) return false;
     const double streaming = (double)items * (rows_avg > 256 ? 2 : 1) * (max_pages_per_seq + 4) / resident_ctas() + 21.0;
-    return streaming < (is_long ? 1.05 : 1.0) * split::estimate(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq);
+    return streaming < 1.05 * split::estimate(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq);
 }
 
 }  // namespace sage
@@ -194,6 +197,14 @@ extern "C" void sage_debug_attention_waits(long long wait_cycles, int producer_o
 }
 
 extern "C" void sage_debug_attention_schedule(int schedule) { g_schedule = (schedule >= 1 && schedule <= 3) ? schedule : 0; }
+
+extern "C" int sage_debug_attention_plan(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq, int* plan) {
+    if (n_layers < 1 || batch < 1 || sum_nodes < 1 || n_q_heads < 1 || n_kv_heads < 1 || max_pages_per_seq < 1 || n_q_heads % n_kv_heads || !plan)
+        return SAGE_ERR_INVALID_ARG;
+    plan[0] = use_streaming(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq) ? 1 : 2;
+    plan[1] = plan[0] == 1 ? 0 : split::slices(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq);
+    return SAGE_OK;
+}
 
 extern "C" int sage_tree_attention(const void* q, const void* k_pool, const void* v_pool, int64_t layer_stride_elems,
                                    int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,

@@ -532,6 +532,10 @@ double estimate(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_
     return wave_cost((long)n_layers * batch * n_kv_heads * (sum_nodes / batch * G > kRowsPerCta ? 2 : 1), max_pages_per_seq, S);
 }
 
+int slices(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq) {
+    return pick_splits(n_layers, batch, n_kv_heads, n_q_heads / n_kv_heads, max_pages_per_seq, sum_nodes);
+}
+
 size_t workspace_size(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq) {
     const int S = pick_splits(n_layers, batch, n_kv_heads, n_q_heads / n_kv_heads, max_pages_per_seq, sum_nodes);
     if (S == 1) return 16;

@@ -1,0 +1,35 @@
+"""Which schedule sage_tree_attention gives a launch: host arithmetic, for 148 multiprocessors where there is no GPU to ask."""
+import pytest
+
+import paper_2602_00523_b200 as sage
+
+STREAMING, SPLIT = 1, 2
+
+
+def schedule(layers, batch, nodes, heads, pages):
+    return sage.sage_debug_attention_plan(layers, batch, batch * nodes, heads[0], heads[1], pages)["schedule"]
+
+
+@pytest.mark.parametrize("layers,batch,nodes,heads,pages", [
+    (3, 27, 42, (8, 1), 21), (1, 12, 64, (64, 8), 21), (2, 10, 42, (64, 8), 21), (1, 8, 24, (64, 8), 33), (1, 13, 36, (64, 8), 33),
+    (1, 39, 64, (8, 1), 40), (1, 11, 60, (64, 8), 40)])
+def test_short_launches_are_split_whatever_table_and_arrays_could_hold(layers, batch, nodes, heads, pages):
+    """Fewer than twelve steps of 128 keys per multiprocessor even if every table is full: how little there is may not show in the
+    sizes, and a streaming launch costs its twenty microseconds all the same."""
+    assert layers * batch * heads[1] * -(-pages // 2) < 12 * 148
+    assert schedule(layers, batch, nodes, heads, pages) == SPLIT
+
+
+def test_long_launches():
+    assert schedule(80, 1, 60, (64, 8), 257) == STREAMING
+    assert schedule(1, 1, 60, (64, 8), 257) == SPLIT
+    assert schedule(1, 16, 42, (64, 8), 129) == STREAMING
+    assert schedule(1, 70000, 1, (8, 1), 20) == STREAMING           # more items than the split grid takes
+    assert schedule(1, 36, 12, (64, 8), 17) == SPLIT                # a wave and most of another, short items
+
+
+def test_sizes_that_no_call_takes_are_refused():
+    with pytest.raises(sage.SageError):
+        sage.sage_debug_attention_plan(1, 1, 8, 60, 8, 4)
+    with pytest.raises(sage.SageError):
+        sage.sage_debug_attention_plan(1, 0, 8, 64, 8, 4)
