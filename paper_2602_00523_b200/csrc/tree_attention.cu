@@ -147,12 +147,16 @@ int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int
 //     (156/153); but nine nodes in such arrays, for which half of the split grid is empty, 2 layers (14) 57/57, 4 (28) 92/75;
 //   several sequences, long: the split grid is as uneven as their lengths.  1k to 8k keys, 24 to 60 nodes: four sequences
 //     (14) 69/55, eight (28) 121/86, sixteen of 24 nodes (56) 121/98; eight of 2k keys, 36 nodes (7) 38/61.
-// Above the line, several sequences under page tables of up to 40 pages: an item is no longer than the tile loop's way in and out, and
-// what decides is how full the last wave of the split grid is, a block per item and slice.  Both schedules are estimated in pages of 64 keys
-// (split::estimate; streaming: the items' pages and extra over the SMs, and 21 for plan, first copies and merge), and the split schedule
-// is taken when it is ahead by a twentieth.  8 KV heads of 8 queries, split / streaming: 16 sequences of 2k keys, 12 nodes 32/47, 24 nodes
-// 41/54, 60 nodes 75/85; 19: 55/52, 68/61, 103/96 (one item too many for a wave); 36: 66/75, 86/95, 155/169; 28 of 1k keys 36/47, 44/55; 18 of up
-// to 2k, 24 nodes 38/52.
+// Above the line, several sequences under narrow page tables: what decides is how full the last wave of the split grid is, a block per item
+// and slice.  Both schedules are estimated in pages of 64 keys (split::estimate; streaming: the items' pages and extra over the SMs, and 21
+// for plan, first copies and merge), and the split schedule is taken when it is ahead by a twentieth.  8 KV heads of 8 queries, split /
+// streaming: 16 sequences of 1.7k keys, 12 nodes 28/43, 24 nodes 35/50, 60 nodes 63/76; 19: 46/48, 57/56, 88/86 (one item too many for a
+// wave); 36: 63/72, 75/87, 144/162; 28 of 1k keys 38/50, 46/59; 18 of up to 1.7k, 24 nodes 42/51.
+// Narrow: the estimates know the table's width, not the lengths, and if a single sequence fills it while the others are short, a split launch
+// takes what the pages of that one take a block of its own (0.7 us each), a streaming one hardly more than its least.  So only as far as
+// that is no loss: 16 sequences, one long and the others a tenth of it, 12 nodes, one query head per KV head, 27 pages 25/21, 33
+// pages 27/21, 37 pages 30/21 (full tables 25/33, 29/36, 32/39); eight, whose ends of items cost more, 28 pages 24/24, 33 pages 28/25,
+// 37 pages 30/26 (full tables 28/43, 32/47, 34/50; the streaming schedule's 25 and 26 were 29 when this was first chosen).
 // Below the line the split schedule runs, whatever the estimates say.  They know what a table and the node arrays can hold, not what they
 // do hold, and a streaming launch takes 20 us however little there is to do: 27 sequences in tables of 21 pages an eighth full, one KV head of 8
 // queries, 3 layers 12/29; twelve chains of nine nodes in arrays of 64 each, 21 full pages 22/32.  (Tight and uneven batches pay for it:
@@ -168,7 +172,8 @@ static bool use_streaming(int n_layers, int batch, int sum_nodes, int n_q_heads,
     const long long steps = items * ((max_pages_per_seq + 1) / 2);   // upper bound
     const int line = batch > 1 ? 12 : rows > 256 ? 24 : 40;
     if (steps < (long long)line * resident_ctas()) return false;
-    if (batch == 1 || max_pages_per_seq > 40 || items > 65535) return true;          // (the split schedule's grid ends there)
+    const int narrow = G >= 4 ? 33 : 24;
+    if (batch == 1 || max_pages_per_seq > narrow || items > 65535) return true;      // (the split schedule's grid ends there)
     const int rows_avg = sum_nodes / batch * G;
     const double streaming = (double)items * (rows_avg > 256 ? 2 : 1) * (max_pages_per_seq + 4) / resident_ctas() + 21.0;
     return streaming < 1.05 * split::estimate(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq);

@@ -20,6 +20,14 @@ def test_short_launches_are_split_whatever_table_and_arrays_could_hold(layers, b
     assert schedule(layers, batch, nodes, heads, pages) == SPLIT
 
 
+@pytest.mark.parametrize("heads,narrow,batch", [((64, 8), 33, 18), ((32, 8), 33, 18), ((16, 8), 24, 36), ((8, 8), 24, 36)])
+def test_only_narrow_tables_are_split_for_several_long_sequences(heads, narrow, batch):
+    """One sequence may fill the table while the others are short: the split launch then takes what that one takes a block of its own,
+    the streaming one next to nothing."""
+    for pages in (narrow - 1, narrow, narrow + 1, narrow + 4, 40, 41, 129):
+        assert schedule(1, batch, 12, heads, pages) == (SPLIT if pages <= narrow else STREAMING), pages
+
+
 def test_long_launches():
     assert schedule(80, 1, 60, (64, 8), 257) == STREAMING
     assert schedule(1, 1, 60, (64, 8), 257) == SPLIT
