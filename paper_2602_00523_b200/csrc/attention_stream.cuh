@@ -59,7 +59,10 @@ constexpr int kAttnThreads = 384;              // 2 softmax warpgroups + one war
 // 49.2 at 2^10, 44.7 here, 40.5 for the usual); higher, the dominant probability of a row is rounded to bf16 more often where it
 // would be exactly 1 (error on growing scores 1.92e-3 of the outputs' norm at 2^8, 1.95e-3 here, 1.98e-3 at 2^14, 2.15e-3 at 2^30).
 constexpr float kMaxSum = 4096.f;
-constexpr int kMinSteps = 2;                   // no range shorter than this (short contexts are latency-bound)
+// No more ranges than one for so many steps (the extra of ends of items counts, so one may hold fewer).  And where items have no more on
+// average, and there is a gang for each, ranges are as many as items: with 147 items of two steps on 148 gangs every boundary cut one into two
+// single steps (23.0 us instead of 18.4; 72 items on 74 pairs of CTAs 28.0 instead of 22.2).
+constexpr int kMinSteps = 2;
 // What an item costs beyond its steps, in steps: the step that holds the tree takes longer, and between two segments lie an epilogue, new
 // query rows and a first step.  Without it ranges of equally many steps take as much longer as they hold more ends of items (sixteen
 // sequences of 1k to 8k keys: a CTA's 53 steps took 122 us on average, 134 at most).  Measured with 0 / 1 / 2 / 3 / 4, us: those 145.0 / 143.7 /
@@ -102,7 +105,7 @@ struct Plan {
     int n_rp;               // CTAs per gang
     int heads_all;          // units that every sequence takes part in; the others are for trees of two row pairs only
     int steps_all, steps_big;   // steps of all sequences, and of those with two row pairs (here and below: with kItemExtra for each item)
-    int n_act;              // gangs with work
+    int n_act;              // gangs that get a range (which may turn out empty, see locate)
     int one_tile;           // no tree has more than one row tile
     long long steps_layer, W;   // steps of a layer, of the launch
 };
@@ -510,9 +513,13 @@ __device__ __forceinline__ Plan make_plan(const AttnParams& p, int lane, int* er
     const long long a = pl.W / kMinSteps;
     const int gangs = p.n_ctas / pl.n_rp;
     pl.n_act = a < 1 ? 1 : a < gangs ? (int)a : gangs;
+    // (the number of items: trees of one and of two row pairs in a batch make it more, skipped sequences less)
+    const long long items = (long long)p.n_layers * p.batch * (pl.steps_big == pl.steps_all ? p.Hkv : pl.heads_all);
+    if (a > gangs && items < gangs && pl.W <= (kMinSteps + kItemExtra) * items) pl.n_act = (int)items;
     return pl;
 }
-// First step of a gang's range.  (32-bit division where the numbers allow it: the 64-bit one takes some hundred clocks.)
+// Where a gang's range begins, before locate has moved it out of an item's extra.  (32-bit division where the numbers allow it: the 64-bit
+// one takes some hundred clocks.)
 __device__ __forceinline__ long long gang_begin(const Plan& pl, int gang) {
     if (pl.W < (1 << 23)) return (unsigned)gang * (unsigned)pl.W / (unsigned)pl.n_act;      // gang <= 148 < 2^9
     return (long long)gang * pl.W / pl.n_act;

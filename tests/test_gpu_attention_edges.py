@@ -221,3 +221,27 @@ def test_ranges_that_end_at_the_end_of_an_item(heads, Ns):
     want = oracle.tree_attention(q[0], kv["k_pool"][0], kv["v_pool"][0], kv["page_table"], kv["seq_len"], parent, off, heads * G, heads,
                                  128, 64, 128 ** -0.5)
     check_attention(host_bits(out)[0], want, bf16_slack=True)       # (bound: see test_attention_edges)
+
+
+@pytest.mark.parametrize("G,N,batch,heads", [(4, 24, 21, 7), (8, 60, 9, 8), (1, 12, 16, 8)], ids=["147_items", "72_pairs", "128_items"])
+def test_items_of_two_steps_are_not_cut_while_there_is_a_gang_for_each(G, N, batch, heads):
+    """Nearly as many items as thread blocks (or pairs of them): equal ranges would cut every one.  An item that is not cut has the bits that
+    it has in a launch of its own."""
+    r = np.random.Generator(np.random.Philox(batch))
+    L = 250 - N
+    kv = make_kv_cache(r, [L] * batch, [N] * batch, [0] * batch, heads, shuffle=True)
+    q, parent = make_q(r, batch * N, heads * G), random_tree(r, N)["parent"].astype(np.int32)
+    k, v, qd = dev_bf16(kv["k_pool"]), dev_bf16(kv["v_pool"]), dev_bf16(q)
+    st = sage.new_status()
+
+    def attention(b0, b1):
+        return sage.sage_tree_attention(qd[:, b0 * N:b1 * N].contiguous(), k, v, dev_i32(kv["page_table"][b0:b1]), dev_i32(kv["seq_len"][b0:b1]),
+                                        dev_i32(np.tile(parent, b1 - b0)), dev_i32(np.arange(b1 - b0 + 1) * N), 128 ** -0.5, status=st)
+    sage.sage_debug_attention_schedule(1)
+    try:
+        together, alone = attention(0, batch), torch.cat([attention(b, b + 1) for b in range(batch)], dim=1)
+        torch.cuda.synchronize()
+    finally:
+        sage.sage_debug_attention_schedule(0)
+    assert int(st.item()) == 0
+    np.testing.assert_array_equal(host_bits(together), host_bits(alone))
