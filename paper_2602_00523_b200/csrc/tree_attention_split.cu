@@ -59,7 +59,7 @@ struct __align__(8) Barriers {
     uint64_t k_full[kPageStages], k_empty[kPageStages];
     uint64_t v_full[kPageStages], v_empty[kPageStages];
     uint64_t s_full[2][2];     // [row tile][page parity]: scores of a page are in TMEM
-    uint64_t p_full[2][2];     // [row tile][page parity]: probabilities of a page are in TMEM
+    uint64_t p_full[2][2];     // [row tile][page parity]: probabilities of a page are in TMEM (an arrival per warp that has rows)
     uint64_t pv_done[2];       // [row tile]: completes once per page, when its P V product has finished
     uint64_t o_full[2];        // [row tile]: every MMA of the tile has finished
     uint64_t q_ready;          // the query tiles are in shared memory
@@ -189,7 +189,8 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
             mbar_init(&bars->v_full[i], 1); mbar_init(&bars->v_empty[i], n_rtiles);
         }
         for (int t = 0; t < 2; ++t) {
-            for (int x = 0; x < 2; ++x) { mbar_init(&bars->s_full[t][x], 1); mbar_init(&bars->p_full[t][x], 4); }
+            const int warps = max(1, min(4, (M - rpair * kRowsPerCta - t * kRowTile + 31) / 32));      // of the tile, with rows of the tree
+            for (int x = 0; x < 2; ++x) { mbar_init(&bars->s_full[t][x], 1); mbar_init(&bars->p_full[t][x], warps); }
             mbar_init(&bars->pv_done[t], 1);
             mbar_init(&bars->o_full[t], 1);
         }
@@ -360,26 +361,25 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
             if (bad) { report_status(p.status, SAGE_STATUS_BAD_TREE); anc = 1ull << node; }
         }
         float m_ref = -INFINITY, l_sum = 0.f;
-        bool ok = (t < n_rtiles);
+        // A warp none of whose 32 rows exists takes no part: the probabilities of these rows stay what their scores were, and their outputs are never
+        // stored.  (Left to keep the barriers going, three such warps polled beside the tile's one and held it up: nine sequences of 1.5k keys, 17
+        // nodes x 8 queries 28.6 -> 25.5 us, 24 nodes, two warps of the second tile, 27.8 -> 26.6.)
+        bool ok = t < n_rtiles && warp_live;
         for (int j = 0; ok && j < ns; ++j) {
             const int x = j & 1;
             ok = mbar_wait_warp(&bars->s_full[t][x], (j >> 1) & 1, bars, p);
             if (!ok) break;
-            // (a warp none of whose 32 rows exists keeps the barrier protocol going and leaves the probabilities of
-            // these rows as they are; their outputs are never stored)
-            if (warp_live) {
-                tc_fence_after();
-                const int jt0 = (pg_begin + j) * kPageSize - L;     // tree slot of the page's first key
-                ok = softmax_page(p, bars, &bars->pv_done[t], (j - 1) & 1, s_taddr + x * 64, o_taddr, row_ok, j == 0, jt0 + kPageSize > 0, jt0, anc,
-                                  m_ref, l_sum);
-                if (!ok) break;
-            }
+            tc_fence_after();
+            const int jt0 = (pg_begin + j) * kPageSize - L;     // tree slot of the page's first key
+            ok = softmax_page(p, bars, &bars->pv_done[t], (j - 1) & 1, s_taddr + x * 64, o_taddr, row_ok, j == 0, jt0 + kPageSize > 0, jt0, anc,
+                              m_ref, l_sum);
+            if (!ok) break;
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars->p_full[t][x]);
         }
         // ---- epilogue: O_t / l -> bf16 output, or unnormalised partials for the merge
         if (ok && ns > 0) ok = mbar_wait_warp(&bars->o_full[t], 0, bars, p);
-        if (ok && warp_live) {
+        if (ok) {
             tc_fence_after();
             const size_t rows_total = (size_t)p.sum_nodes * p.Hq;
             const size_t row = (size_t)(n0 + node) * p.Hq + g * p.G + (row_ok ? R & (p.G - 1) : 0);

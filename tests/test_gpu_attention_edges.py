@@ -245,3 +245,60 @@ def test_items_of_two_steps_are_not_cut_while_there_is_a_gang_for_each(G, N, bat
         sage.sage_debug_attention_schedule(0)
     assert int(st.item()) == 0
     np.testing.assert_array_equal(host_bits(together), host_bits(alone))
+
+
+def test_a_nearly_empty_row_tile_costs_no_more_than_a_half_empty_one():
+    """Seventeen nodes of eight queries leave the second row tile eight rows, in one warp; twenty-four leave it two warps of rows.  While
+    warps without rows polled beside the working ones, the smaller trees took 1.03 times as long as the larger, now 0.96 times."""
+    L, batch, heads, G = 24 * 64 - 64, 9, 8, 8
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(4)
+    k, v = (torch.randn(4, batch * 24, heads, 64, 128, generator=gen, device="cuda").bfloat16() for _ in range(2))     # (beyond L2)
+    table = torch.randperm(batch * 24, generator=gen, device="cuda").to(torch.int32).reshape(batch, 24)
+    seq, times = dev_i32([L] * batch), {}
+    st = sage.new_status()
+    sage.sage_debug_attention_schedule(2)
+    try:
+        calls = {}
+        for N in (17, 24):
+            q = torch.randn(1, batch * N, heads * G, 128, generator=gen, device="cuda").bfloat16()
+            parent = dev_i32(np.tile(random_tree(np.random.Generator(np.random.Philox(1)), N)["parent"], batch))
+            off, out = dev_i32(np.arange(batch + 1) * N), torch.empty_like(q)
+            ws = torch.empty(max(16, sage.sage_tree_attention_workspace_size(1, batch, batch * N, heads * G, heads, 128, 24)),
+                             dtype=torch.uint8, device="cuda")
+            calls[N] = (q, parent, off, out, ws)
+        for _ in range(8):                               # in turn
+            for N, (q, parent, off, out, ws) in calls.items():
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                for i in range(40):
+                    sage.sage_tree_attention(q, k[i % 4:i % 4 + 1], v[i % 4:i % 4 + 1], table, seq, parent, off, 128 ** -0.5, out=out, ws=ws, status=st)
+                b.record()
+                torch.cuda.synchronize()
+                times[N] = min(times.get(N, 1e9), a.elapsed_time(b))
+    finally:
+        sage.sage_debug_attention_schedule(0)
+    assert int(st.item()) == 0
+    assert times[17] <= times[24], times
+
+
+@pytest.mark.parametrize("N", [1, 4, 5, 9, 13, 17, 20, 21, 25, 29, 33, 49, 53, 57])
+def test_row_tiles_of_one_to_four_warps(N):
+    """The split schedule with one to four warps of rows in the first to the fourth row tile; warps without rows take no part."""
+    r = np.random.Generator(np.random.Philox(300 + N))
+    heads, G, Ls = 2, 8, [300, 700]
+    kv = make_kv_cache(r, Ls, [N, N], [0, 0], heads, shuffle=True)
+    q = make_q(r, 2 * N, heads * G)
+    parent, off = np.concatenate([random_tree(r, N)["parent"] for _ in Ls]).astype(np.int32), np.array([0, N, 2 * N], np.int32)
+    st = sage.new_status()
+    sage.sage_debug_attention_schedule(2)
+    try:
+        out = sage.sage_tree_attention(dev_bf16(q), dev_bf16(kv["k_pool"]), dev_bf16(kv["v_pool"]), dev_i32(kv["page_table"]),
+                                       dev_i32(kv["seq_len"]), dev_i32(parent), dev_i32(off), 128 ** -0.5, status=st)
+        torch.cuda.synchronize()
+    finally:
+        sage.sage_debug_attention_schedule(0)
+    assert int(st.item()) == 0
+    want = oracle.tree_attention(q[0], kv["k_pool"][0], kv["v_pool"][0], kv["page_table"], kv["seq_len"], parent, off, heads * G, heads,
+                                 128, 64, 128 ** -0.5)
+    check_attention(host_bits(out)[0], want, bf16_slack=True)       # (bound: see test_attention_edges)
