@@ -116,10 +116,10 @@ static int g_schedule = 0;     // 0: chosen per launch, 2: split, else streaming
 
 // The split schedule (tree_attention_split.cu).
 namespace split {
-double estimate(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
-int slices(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
-size_t workspace_size(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
-int launch(int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,
+double estimate(int n_sms, int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
+int slices(int n_sms, int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
+size_t workspace_size(int n_sms, int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
+int launch(int n_sms, int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,
            const int32_t* seq_len, const int32_t* parent, const int32_t* node_offsets, int batch, int sum_nodes,
            int n_q_heads, int n_kv_heads, float sm_scale, void* out, void* ws, int32_t* status, long long wait_cycles,
            int producer_off, const CUtensorMap& qmap, const CUtensorMap& kmap, const CUtensorMap& vmap, cudaStream_t stream);
@@ -176,7 +176,7 @@ static bool use_streaming(int n_layers, int batch, int sum_nodes, int n_q_heads,
     if (batch == 1 || max_pages_per_seq > narrow || items > 65535) return true;      // (the split schedule's grid ends there)
     const int rows_avg = sum_nodes / batch * G;
     const double streaming = (double)items * (rows_avg > 256 ? 2 : 1) * (max_pages_per_seq + 4) / resident_ctas() + 21.0;
-    return streaming < 1.05 * split::estimate(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq);
+    return streaming < 1.05 * split::estimate(resident_ctas(), n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq);
 }
 
 }  // namespace sage
@@ -192,7 +192,7 @@ extern "C" size_t sage_tree_attention_workspace_size(int n_layers, int batch, in
     // streaming: two partial slots (head and tail of its range) per resident CTA, independent of the problem size;
     // split: one partial per context slice.  Either may run, so the larger is asked for.
     const size_t streaming = stream::workspace_size(resident_ctas());
-    const size_t split_ws = split::workspace_size(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq);
+    const size_t split_ws = split::workspace_size(resident_ctas(), n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq);
     return streaming > split_ws ? streaming : split_ws;
 }
 
@@ -207,7 +207,7 @@ extern "C" int sage_debug_attention_plan(int n_layers, int batch, int sum_nodes,
     if (n_layers < 1 || batch < 1 || sum_nodes < 1 || n_q_heads < 1 || n_kv_heads < 1 || max_pages_per_seq < 1 || n_q_heads % n_kv_heads || !plan)
         return SAGE_ERR_INVALID_ARG;
     plan[0] = use_streaming(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq) ? 1 : 2;
-    plan[1] = plan[0] == 1 ? 0 : split::slices(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq);
+    plan[1] = plan[0] == 1 ? 0 : split::slices(resident_ctas(), n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq);
     return SAGE_OK;
 }
 
@@ -243,7 +243,7 @@ extern "C" int sage_tree_attention(const void* q, const void* k_pool, const void
         !make_q_map(&qmap, q, n_layers, sum_nodes, n_kv_heads, G))
         return SAGE_ERR_CUDA;
     if (!streaming)
-        return split::launch(n_layers, n_pages, page_table, max_pages_per_seq, seq_len, parent, node_offsets, batch,
+        return split::launch(resident_ctas(), n_layers, n_pages, page_table, max_pages_per_seq, seq_len, parent, node_offsets, batch,
                              sum_nodes, n_q_heads, n_kv_heads, sm_scale, out, ws, status, g_wait_cycles, g_producer_off,
                              qmap, kmap, vmap, as_stream(stream));
     return stream::launch(resident_ctas(), n_layers, n_pages, page_table, max_pages_per_seq, seq_len, parent, node_offsets,

@@ -508,47 +508,47 @@ static int row_pairs_for(int sum_nodes, int G) {
 // Slices of the context, down to a page each (512 keys, 60 nodes: 0.6 us less than with two pages at least, now 12.5).  One CTA
 // is resident per SM; a wave of them takes what its pages take plus a fixed part (set-up, first copies, drain), worth about
 // six pages (four and nine measure the same), and every slice costs the merge a little.
-static double wave_cost(long blocks, int pages, int s) {
-    return (double)((blocks * s + 147) / 148) * (6 + (pages + s - 1) / s) + (s > 1 ? 4.0 + 0.25 * s : 0.0);
+static double wave_cost(int n_sms, long blocks, int pages, int s) {
+    return (double)((blocks * s + n_sms - 1) / n_sms) * (6 + (pages + s - 1) / s) + (s > 1 ? 4.0 + 0.25 * s : 0.0);
 }
-static int pick_splits(int n_layers, int batch, int n_kv_heads, int G, int max_pages, int sum_nodes) {
+static int pick_splits(int n_sms, int n_layers, int batch, int n_kv_heads, int G, int max_pages, int sum_nodes) {
     const long base = (long)n_layers * batch * n_kv_heads * row_pairs_for(sum_nodes, G);
     const int s_max = max_pages < kMaxSplits ? max_pages : kMaxSplits;
     int best = 1;
     double best_cost = 0.0;
     for (int s = 1; s <= s_max; ++s) {
-        const long waves = (base * s + 147) / 148;
+        const long waves = (base * s + n_sms - 1) / n_sms;
         if (s > 1 && waves > 4) break;                      // (the last wave matters little by then, partial results do)
-        const double cost = wave_cost(base, max_pages, s);
+        const double cost = wave_cost(n_sms, base, max_pages, s);
         if (s == 1 || cost < best_cost - 1e-9) { best_cost = cost; best = s; }
     }
     return best;
 }
 
 // What a launch takes, in pages of 64 keys, if its trees are of the average size (blocks for rows that a tree does not have leave at once).
-double estimate(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq) {
+double estimate(int n_sms, int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq) {
     const int G = n_q_heads / n_kv_heads;
-    const int S = pick_splits(n_layers, batch, n_kv_heads, G, max_pages_per_seq, sum_nodes);
-    return wave_cost((long)n_layers * batch * n_kv_heads * (sum_nodes / batch * G > kRowsPerCta ? 2 : 1), max_pages_per_seq, S);
+    const int S = pick_splits(n_sms, n_layers, batch, n_kv_heads, G, max_pages_per_seq, sum_nodes);
+    return wave_cost(n_sms, (long)n_layers * batch * n_kv_heads * (sum_nodes / batch * G > kRowsPerCta ? 2 : 1), max_pages_per_seq, S);
 }
 
-int slices(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq) {
-    return pick_splits(n_layers, batch, n_kv_heads, n_q_heads / n_kv_heads, max_pages_per_seq, sum_nodes);
+int slices(int n_sms, int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq) {
+    return pick_splits(n_sms, n_layers, batch, n_kv_heads, n_q_heads / n_kv_heads, max_pages_per_seq, sum_nodes);
 }
 
-size_t workspace_size(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq) {
-    const int S = pick_splits(n_layers, batch, n_kv_heads, n_q_heads / n_kv_heads, max_pages_per_seq, sum_nodes);
+size_t workspace_size(int n_sms, int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq) {
+    const int S = pick_splits(n_sms, n_layers, batch, n_kv_heads, n_q_heads / n_kv_heads, max_pages_per_seq, sum_nodes);
     if (S == 1) return 16;
     return (size_t)n_layers * S * sum_nodes * n_q_heads * (kHeadDim + 2) * sizeof(float);
 }
 
 // Arguments have been validated by sage_tree_attention.
-int launch(int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,
+int launch(int n_sms, int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,
            const int32_t* seq_len, const int32_t* parent, const int32_t* node_offsets, int batch, int sum_nodes,
            int n_q_heads, int n_kv_heads, float sm_scale, void* out, void* ws, int32_t* status, long long wait_cycles,
            int producer_off, const CUtensorMap& qmap, const CUtensorMap& kmap, const CUtensorMap& vmap, cudaStream_t stream) {
     const int G = n_q_heads / n_kv_heads;
-    const int S = pick_splits(n_layers, batch, n_kv_heads, G, max_pages_per_seq, sum_nodes);
+    const int S = pick_splits(n_sms, n_layers, batch, n_kv_heads, G, max_pages_per_seq, sum_nodes);
     SplitParams p{};
     p.out = (__nv_bfloat16*)out;
     p.part_o = (float4*)ws;
