@@ -264,7 +264,8 @@ void sage_debug_attention_waits(long long wait_cycles, int producer_off);
 void sage_debug_attention_schedule(int schedule);
 
 /* What sage_tree_attention would do with a launch of these sizes: plan[0] the schedule (1 streaming, 2 split), plan[1] the
- * context slices of the split one.  Host arithmetic only.  For tests (no counterpart in the paper). */
+ * context slices of the split one, plan[2] whether their merge is brought up while they are still being worked on.  Host
+ * arithmetic only.  For tests (no counterpart in the paper). */
 int sage_debug_attention_plan(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq,
                               int *plan);
 

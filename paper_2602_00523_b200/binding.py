@@ -270,11 +270,11 @@ def sage_debug_attention_schedule(schedule: int = 0) -> None:
 
 
 def sage_debug_attention_plan(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages) -> dict:
-    """What sage_tree_attention would do with a launch of these sizes: the schedule, 1 streaming or 2 split, and the split one's
-    context slices."""
-    plan = (_i * 2)()
+    """What sage_tree_attention would do with a launch of these sizes: the schedule, 1 streaming or 2 split, the split one's
+    context slices, and whether their merge is brought up while they are still being worked on."""
+    plan = (_i * 3)()
     _check(_lib.sage_debug_attention_plan(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages, plan), "sage_debug_attention_plan")
-    return {"schedule": plan[0], "slices": plan[1]}
+    return {"schedule": plan[0], "slices": plan[1], "merge_overlaps": bool(plan[2])}
 
 
 def sage_accept(parent, draft_token, target_argmax, node_offsets, max_path: int, *, out=None, status=None, stream=None):

@@ -73,6 +73,16 @@ inline cudaError_t launch(void (*kernel)(Params...), dim3 grid, int threads, siz
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
 }
 
+// The same without the overlap: the kernel is brought up once the one before it has ended, with the whole chip to spread over.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_in_order(void (*kernel)(Params...), dim3 grid, int threads, cudaStream_t stream, const Args&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = stream;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
 // A call's result as the entry points return it.  The runtime also keeps a failure as the thread's last error: it is taken

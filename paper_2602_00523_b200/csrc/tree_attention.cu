@@ -118,6 +118,7 @@ static int g_schedule = 0;     // 0: chosen per launch, 2: split, else streaming
 namespace split {
 double estimate(int n_sms, int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
 int slices(int n_sms, int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
+bool merge_overlaps(int n_sms, int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int S);
 size_t workspace_size(int n_sms, int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq);
 int launch(int n_sms, int n_layers, int n_pages, const int32_t* page_table, int max_pages_per_seq,
            const int32_t* seq_len, const int32_t* parent, const int32_t* node_offsets, int batch, int sum_nodes,
@@ -208,6 +209,7 @@ extern "C" int sage_debug_attention_plan(int n_layers, int batch, int sum_nodes,
         return SAGE_ERR_INVALID_ARG;
     plan[0] = use_streaming(n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq) ? 1 : 2;
     plan[1] = plan[0] == 1 ? 0 : split::slices(resident_ctas(), n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, max_pages_per_seq);
+    plan[2] = plan[1] > 1 && split::merge_overlaps(resident_ctas(), n_layers, batch, sum_nodes, n_q_heads, n_kv_heads, plan[1]) ? 1 : 0;
     return SAGE_OK;
 }
 

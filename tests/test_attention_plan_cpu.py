@@ -28,6 +28,19 @@ def test_only_narrow_tables_are_split_for_several_long_sequences(heads, narrow, 
         assert schedule(1, batch, 12, heads, pages) == (SPLIT if pages <= narrow else STREAMING), pages
 
 
+@pytest.mark.parametrize("layers,batch,sum_nodes,heads,pages,overlaps", [
+    (1, 1, 10, (32, 8), 33, True),          # 88 split blocks, 40 merge blocks on the 60 multiprocessors left
+    (1, 4, 168, (8, 8), 8, False),          # 128, 168 on 20
+    (1, 5, 210, (8, 8), 9, False),          # 120, 212 on 28
+    (1, 2, 24, (8, 8), 8, True),            # 64, 24 on 84
+    (1, 1, 60, (64, 8), 257, False),        # 144, 480 on 4
+    (2, 3, 72, (64, 8), 42, True),          # 288: more than one wave
+    (1, 1, 60, (64, 8), 1, False)])         # one slice: no merge
+def test_a_merge_waits_on_free_multiprocessors_only_if_its_blocks_are_few(layers, batch, sum_nodes, heads, pages, overlaps):
+    plan = sage.sage_debug_attention_plan(layers, batch, sum_nodes, heads[0], heads[1], pages)
+    assert plan["schedule"] == SPLIT and plan["merge_overlaps"] == overlaps, plan
+
+
 def test_long_launches():
     assert schedule(80, 1, 60, (64, 8), 257) == STREAMING
     assert schedule(1, 1, 60, (64, 8), 257) == SPLIT
