@@ -369,17 +369,19 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
             const int x = j & 1;
             ok = mbar_wait_warp(&bars->s_full[t][x], (j >> 1) & 1, bars, p);
             if (!ok) break;
-            tc_fence_after();
-            const int jt0 = (pg_begin + j) * kPageSize - L;     // tree slot of the page's first key
-            ok = softmax_page(p, bars, &bars->pv_done[t], (j - 1) & 1, s_taddr + x * 64, o_taddr, row_ok, j == 0, jt0 + kPageSize > 0, jt0, anc,
-                              m_ref, l_sum);
-            if (!ok) break;
+            if (warp_live) {                                        // (always; told so, the compiler lays the loop out better: short launches 8.5 -> 8.3 us)
+                tc_fence_after();
+                const int jt0 = (pg_begin + j) * kPageSize - L;     // tree slot of the page's first key
+                ok = softmax_page(p, bars, &bars->pv_done[t], (j - 1) & 1, s_taddr + x * 64, o_taddr, row_ok, j == 0, jt0 + kPageSize > 0, jt0, anc,
+                                  m_ref, l_sum);
+                if (!ok) break;
+            }
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars->p_full[t][x]);
         }
         // ---- epilogue: O_t / l -> bf16 output, or unnormalised partials for the merge
         if (ok && ns > 0) ok = mbar_wait_warp(&bars->o_full[t], 0, bars, p);
-        if (ok) {
+        if (ok && warp_live) {
             tc_fence_after();
             const size_t rows_total = (size_t)p.sum_nodes * p.Hq;
             const size_t row = (size_t)(n0 + node) * p.Hq + g * p.G + (row_ok ? R & (p.G - 1) : 0);
