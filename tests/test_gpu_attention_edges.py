@@ -302,3 +302,28 @@ def test_row_tiles_of_one_to_four_warps(N):
     want = oracle.tree_attention(q[0], kv["k_pool"][0], kv["v_pool"][0], kv["page_table"], kv["seq_len"], parent, off, heads * G, heads,
                                  128, 64, 128 ** -0.5)
     check_attention(host_bits(out)[0], want, bf16_slack=True)       # (bound: see test_attention_edges)
+
+
+@pytest.mark.parametrize("pages", [1, 31, 32, 33, 224, 225, 255, 256, 257])
+def test_page_tables_that_are_read_ahead_and_wider_ones(pages):
+    """The split schedule reads rows of up to 256 page ids whole, 32 at a time, wider ones where it needs them.  Two sequences, the second
+    of which uses its row to the last slot of the last page."""
+    r = np.random.Generator(np.random.Philox(400 + pages))
+    heads, G, N = 1, 8, 6
+    Ls = [max(0, pages * 32 - 5), pages * 64 - N]
+    kv = make_kv_cache(r, Ls, [N, N], [0, 0], heads, shuffle=True)
+    assert kv["page_table"].shape[1] == pages and (kv["page_table"][1] >= 0).all()
+    q = make_q(r, 2 * N, heads * G)
+    parent, off = np.concatenate([random_tree(r, N)["parent"] for _ in Ls]).astype(np.int32), np.array([0, N, 2 * N], np.int32)
+    st = sage.new_status()
+    sage.sage_debug_attention_schedule(2)
+    try:
+        out = sage.sage_tree_attention(dev_bf16(q), dev_bf16(kv["k_pool"]), dev_bf16(kv["v_pool"]), dev_i32(kv["page_table"]),
+                                       dev_i32(kv["seq_len"]), dev_i32(parent), dev_i32(off), 128 ** -0.5, status=st)
+        torch.cuda.synchronize()
+    finally:
+        sage.sage_debug_attention_schedule(0)
+    assert int(st.item()) == 0
+    want = oracle.tree_attention(q[0], kv["k_pool"][0], kv["v_pool"][0], kv["page_table"], kv["seq_len"], parent, off, heads * G, heads,
+                                 128, 64, 128 ** -0.5)
+    check_attention(host_bits(out)[0], want, bf16_slack=True)       # (bound: see test_attention_edges)

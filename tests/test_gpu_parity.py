@@ -436,6 +436,50 @@ def test_accept_chain_of_64_and_templates():
             np.testing.assert_array_equal(g, w)
 
 
+def _malformed(parent, kind):
+    p = parent.copy()
+    n = len(p)
+    i = {"low": 5, "high": 40}.get(kind.split("_")[-1], 0)
+    if kind == "root":
+        p[0] = 0
+    elif kind.startswith("itself"):
+        p[i] = i
+    elif kind.startswith("forward"):
+        p[i] = i + 1
+    elif kind.startswith("outside"):
+        p[i] = n + 1000000
+    elif kind.startswith("orphan"):
+        p[i] = -1
+    elif kind.startswith("negative"):
+        p[i] = -7
+    return p
+
+
+@pytest.mark.parametrize("kind", ["root", "itself_low", "itself_high", "forward_low", "forward_high", "outside_low", "outside_high",
+                                  "orphan_low", "orphan_high", "negative_high", "empty", "too_large"])
+def test_accept_rejects_malformed_trees_beside_valid_ones(kind):
+    r = rng(900)
+    trees = [random_tree(r, n)["parent"] for n in (24, 48, 1, 64, 33)]
+    bad = {"empty": np.zeros(0, np.int32), "too_large": np.arange(-1, 64, dtype=np.int32)}.get(kind)
+    if bad is None:
+        bad = _malformed(random_tree(r, 50)["parent"], kind)
+    trees.insert(2, bad)
+    parent = np.concatenate(trees).astype(np.int32)
+    offs = np.concatenate([[0], np.cumsum([len(t) for t in trees])]).astype(np.int32)
+    draft, target = r.integers(0, 2, len(parent)).astype(np.int32), r.integers(0, 2, len(parent)).astype(np.int32)
+    st = sage.new_status()
+    o = sage.sage_accept(dev_i32(parent), dev_i32(draft), dev_i32(target), dev_i32(offs), 9, status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == sage.SAGE_STATUS_BAD_TREE
+    path, plen, bonus = (o[n].cpu().numpy() for n in ("path", "path_len", "bonus_token"))
+    assert plen[2] == 0 and bonus[2] == -1 and (path[2] == -1).all()
+    for b in (0, 1, 3, 4, 5):
+        s = slice(offs[b], offs[b + 1])
+        want = oracle.accept(parent[s], draft[s], target[s], np.array([0, len(trees[b])], np.int32), 9)
+        for g, w in zip((path[b], plen[b], bonus[b]), want):
+            np.testing.assert_array_equal(g, w[0])
+
+
 # ------------------------------------------------------------------ compaction
 def run_compaction(kv, paths, plen, n_layers):
     k, v = dev_bf16(kv["k_pool"]), dev_bf16(kv["v_pool"])
