@@ -39,8 +39,8 @@ __device__ __forceinline__ uint64_t ancestor_bits(const int32_t* __restrict__ pa
     return a;
 }
 
-// Every kernel is launched to overlap its launch with the end of the kernel before it (programmatic stream
-// serialization) and starts with after_previous_kernel(): it waits there until that kernel has completed and its
+// Every kernel (but for merges that launch_in_order is for) is launched to overlap its launch with the end of the kernel before it
+// (programmatic stream serialization), and all start with after_previous_kernel(): it waits there until that kernel has completed and its
 // writes are visible, before it touches global memory, and then lets the next kernel of the stream be brought up.
 // No block leaves without passing it: a kernel waits for its direct predecessor only, and that one's end has to mean that
 // its own predecessor has ended.

@@ -142,28 +142,28 @@ int launch(int n_ctas, int n_layers, int n_pages, const int32_t* page_table, int
 //     launches too short to give every SM a long stream (single layers, short contexts: fixed costs dominate).
 // The line lies where both take the same time (us, split / streaming; steps per SM in brackets; 8 KV heads of 8 queries;
 // bursts of a few ms, in longer loops the power limit takes 10 to 20 % off the lead of the split schedule):
-//   one sequence, up to one row pair: 24 nodes, 16k keys, 4 layers (28) 72/88, 8 (56) 146/163 (in longer loops 164/164);
-//     12 nodes, 4k keys, 16 layers (28) 61/66, 24 (43) 97/88, 32 (57) 106/108 (118/112);
-//   one sequence whose node arrays have room for two row pairs: 60 nodes, 16k keys, 3 layers (21) 111/133, 4 (28) 144/149
-//     (156/153); but nine nodes in such arrays, for which half of the split grid is empty, 2 layers (14) 57/57, 4 (28) 92/75;
-//   several sequences, long: the split grid is as uneven as their lengths.  1k to 8k keys, 24 to 60 nodes: four sequences
-//     (14) 69/55, eight (28) 121/86, sixteen of 24 nodes (56) 121/98; eight of 2k keys, 36 nodes (7) 38/61.
+//   one sequence, up to one row pair: 24 nodes, 16k keys, 4 layers (28) 71/74, 8 (56) 157/150; 12 nodes, 4k keys, 16 layers (28) 60/62,
+//     24 (43) 107/86, 32 (57) 124/106;
+//   one sequence whose node arrays have room for two row pairs: 60 nodes, 16k keys, 3 layers (21) 110/121, 4 (28) 155/148; but nine
+//     nodes in such arrays, for which half of the split grid is empty, 2 layers (14) 53/52, 4 (28) 93/69;
+//   several sequences, long: the split grid is as uneven as their lengths.  1k to 8k keys, 24 to 60 nodes: four sequences (14) 66/48,
+//     eight (28) 116/91, sixteen of 24 nodes (56) 138/103; eight of 2k keys, 36 nodes (7) 40/56.
 // Above the line, several sequences under narrow page tables: what decides is how full the last wave of the split grid is, a block per item
 // and slice.  Both schedules are estimated in pages of 64 keys (split::estimate; streaming: the items' pages and extra over the SMs, and 21
 // for plan, first copies and merge), and the split schedule is taken when it is ahead by a twentieth.  8 KV heads of 8 queries, split /
-// streaming: 16 sequences of 1.7k keys, 12 nodes 28/43, 24 nodes 35/50, 60 nodes 63/76; 19: 46/48, 57/56, 88/86 (one item too many for a
-// wave); 36: 63/72, 75/87, 144/162; 28 of 1k keys 38/50, 46/59; 18 of up to 1.7k, 24 nodes 42/51.
+// streaming: 16 sequences of 1.7k keys, 12 nodes 28/43, 24 nodes 34/51, 60 nodes 67/83; 19: 54/51, 58/57, 94/94 (one item too many for a
+// wave); 36: 61/70, 79/94, 147/169; 28 of 1k keys 41/52, 45/59; 18 of up to 1.7k, 24 nodes 36/46.
 // Narrow: the estimates know the table's width, not the lengths, and if a single sequence fills it while the others are short, a split launch
 // takes what the pages of that one take a block of its own (0.7 us each), a streaming one hardly more than its least.  So only as far as
-// that is no loss: 16 sequences, one long and the others a tenth of it, 12 nodes, one query head per KV head, 27 pages 25/21, 33
-// pages 27/21, 37 pages 30/21 (full tables 25/33, 29/36, 32/39); eight, whose ends of items cost more, 28 pages 24/24, 33 pages 28/25,
-// 37 pages 30/26 (full tables 28/43, 32/47, 34/50; the streaming schedule's 25 and 26 were 29 when this was first chosen).
+// that is no loss: 16 sequences, one long and the others a tenth of it, 12 nodes, one query head per KV head, 27 pages 23/19, 33
+// pages 26/21, 37 pages 29/21 (full tables 24/32, 28/36, 30/38); eight, whose ends of items cost more, 28 pages 24/24, 33 pages 28/25,
+// 37 pages 30/26 (full tables 28/43, 32/47, 34/49; the streaming schedule's 25 and 26 were 29 before its ends of items were weighed).
 // Below the line the split schedule runs, whatever the estimates say.  They know what a table and the node arrays can hold, not what they
 // do hold, and a streaming launch takes 20 us however little there is to do: 27 sequences in tables of 21 pages an eighth full, one KV head of 8
-// queries, 3 layers 12/29; twelve chains of nine nodes in arrays of 64 each, 21 full pages 22/32.  (Tight and uneven batches pay for it:
-// twelve sequences of 2k keys, 60 nodes 88/70.)
+// queries, 3 layers 12/29; twelve chains of nine nodes in arrays of 64 each, 21 full pages 22/32.  (Tight batches may pay for it: twelve
+// sequences of 2k keys, 60 nodes 86/74.)
 // The host knows the width of the page table, not the lengths, so a wide table takes short sequences across the line, or into
-// more slices than they fill: eight sequences of 1k keys 23 us with 17 pages per row, 41 with 512; one of 2k keys, 60 nodes, 16.0
+// more slices than they fill: eight sequences of 1k keys 22 us with 17 pages per row, 41 with 512; one of 2k keys, 60 nodes, 16.2
 // with 33 pages, 16.1 with 512, 10 nodes 9.4 and 10.7.
 static bool use_streaming(int n_layers, int batch, int sum_nodes, int n_q_heads, int n_kv_heads, int max_pages_per_seq) {
     if (g_schedule) return g_schedule != 2;

@@ -163,8 +163,8 @@ tree_attention_split_kernel(const SplitParams p, const __grid_constant__ CUtenso
     const int N = p.node_offsets[b + 1] - n0;
     const int L = p.seq_len[b];
     // The whole row of the page table in the same round of loads, not the slice's part in a second one once the length is known (one
-    // layer of ten nodes at 2k keys 9.18 -> 8.94 us, 60 nodes 16.0 -> 15.8, 15 nodes at 627 keys 9.42 -> 9.02, 24 at 4k 14.8 -> 14.5; of 35
-    // batches of short sequences, 1 to 8 query heads a KV head, 32 gain 2 to 4 %, three of one head and mixed trees lose as much, 11.0 -> 11.3).
+    // layer of ten nodes at 2k keys 9.18 -> 8.94 us, 60 nodes 16.0 -> 15.8, 15 nodes at 627 keys 9.42 -> 9.02, 24 at 4k 14.8 -> 14.5).  A prefix
+    // of 16k keys and any tree have 257 pages: reading 320 ahead instead of 256 measured the same.
     const bool table = p.max_pages <= kTablePages;
     if (warp == 8 && table) {
         const int32_t* pages = p.page_table + (size_t)b * p.max_pages;
