@@ -49,6 +49,13 @@ def test_long_launches():
     assert schedule(1, 36, 12, (64, 8), 17) == SPLIT                # a wave and most of another, short items
 
 
+@pytest.mark.parametrize("nodes", [26, 44, 54])
+def test_the_long_launches_of_the_parity_tests_are_streamed(nodes):
+    """26 layers of three sequences of 33 pages, one row tile to more than two: those tests leave the choice to the library and are about the
+    streaming kernels, of which the trees on the device decide."""
+    assert sage.sage_debug_attention_plan(26, 3, nodes, 16, 2, 33)["schedule"] == STREAMING
+
+
 def test_sizes_that_no_call_takes_are_refused():
     with pytest.raises(sage.SageError):
         sage.sage_debug_attention_plan(1, 1, 8, 60, 8, 4)
